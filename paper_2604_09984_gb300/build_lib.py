@@ -12,7 +12,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 OUT = os.path.join(HERE, "libugks.so")
-SOURCES = ["ugks_kernels.cu", "ugks_tile.cu", "ugks_sweep.cu", "ugks_overset.cu", "ugks_api.cu", "ugks_static.cu",
+SOURCES = ["ugks_kernels.cu", "ugks_macro.cu", "ugks_tile.cu", "ugks_sweep.cu", "ugks_overset.cu", "ugks_api.cu", "ugks_static.cu",
            "ugks_probe.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # -ftz=true: FP32 subnormals flush to zero (none of the path's FP32 values is

@@ -120,7 +120,8 @@ struct Sizes {
   int nc = 0, nf = 0, nn = 0, nv = 0, nvp = 0, nseg = 0, nring = 0, max_nj = 0, ntiles = 0;
   int nvx = 0, nvy = 0;
   int iy0 = 0, nv_all = 0, nvp_all = 0;   // velocity shard: first row; the whole grid
-  size_t nmrec32 = 0;   // FP32 macro records: (ni + nj - 1) nj per block (diagonal-major)
+  size_t nmrec = 0;     // macro-sweep records of all blocks
+  int mpad = 0;         // their padding diagonals
 };
 
 int validate(const ugks_params *p, int nb, const ugks_block_desc *b, Sizes &s, std::string &why) {
@@ -168,8 +169,9 @@ int validate(const ugks_params *p, int nb, const ugks_block_desc *b, Sizes &s, s
     s.nf += B.nj * (B.periodic_i ? B.ni : B.ni + 1) + B.ni * (B.nj + 1);
     if (B.nj > s.max_nj) s.max_nj = B.nj;
     s.ntiles += tile_count(B.ni, B.nj);
-    s.nmrec32 += (size_t)(B.ni + B.nj - 1) * B.nj;
   }
+  s.mpad = macro_pad(s.max_nj, p->precision != UGKS_FP64);
+  for (int i = 0; i < nb; ++i) s.nmrec += macro_cells(b[i].ni, b[i].nj, s.mpad);
   return UGKS_OK;
 }
 
@@ -306,8 +308,8 @@ size_t carve(char *base, const Sizes &s, int nb, int fp32, int fbf, int nwork, i
   d.mpart = c.take<double>((size_t)MET_NQ * MET_BLOCKS);
   d.mout = c.take<double>(MET_NQ);
   d.TW = c.take<double>(4 * (size_t)s.nc); d.Fc = c.take<double>(4 * (size_t)s.nc);
-  d.dW = c.take<double>(4 * (size_t)s.nc); d.Wp = c.take<double>(4 * (size_t)s.nc);
-  d.mrec = c.take<char>(fp32 ? sizeof(float) * NMR32 * s.nmrec32 : sizeof(double) * NMR * (size_t)s.nc);
+  d.Wp = c.take<double>(4 * (size_t)s.nc);
+  d.mrec = c.take<char>(macro_record_bytes(fp32) * s.nmrec);
   d.mrec_off = c.take<int>((size_t)nb + 1);
   d.cpar = c.take<double>(NCP * (size_t)s.nc); d.cparn = c.take<double>(NCP * (size_t)s.nc);
   d.shp = c.take<char>(tsz * NSH * (size_t)s.nc); d.shn = c.take<char>(tsz * NSH * (size_t)s.nc);
@@ -1026,6 +1028,7 @@ int ugks_init_mesh(ugks_ctx *ctx, int nblocks, const ugks_block_desc *blocks, co
   d.dt = 1.0; d.idt = 1.0; d.idt_f = 1.0f;
   ctx->launches += upload_step_size(ctx);
   d.wait_polls = kWaitPolls;
+  d.mpad = s.mpad;
   d.vbox[0] = ctx->p.vx_min; d.vbox[1] = ctx->p.vx_max; d.vbox[2] = ctx->p.vy_min; d.vbox[3] = ctx->p.vy_max;
   {
     double lam = 1.0 / (2.0 * ctx->p.farfield[3]);
@@ -1096,7 +1099,7 @@ int ugks_init_mesh(ugks_ctx *ctx, int nblocks, const ugks_block_desc *blocks, co
   }
   d.ntiles = s.ntiles;
   tile_setup();
-  sweep_setup();
+  macro_setup();
   wsweep_setup();
   if ((r = up(ctx, (void *)d.vx, vx))) return r;
   if ((r = up(ctx, (void *)d.vy, vy))) return r;
@@ -1177,9 +1180,11 @@ int ugks_init_mesh(ugks_ctx *ctx, int nblocks, const ugks_block_desc *blocks, co
   if ((r = up(ctx, (void *)d.node_off, ctx->node_off))) return r;
   if ((r = up(ctx, (void *)d.blk_info, T.blk_info))) return r;
   {
-    std::vector<int> mo(nblocks + 1, 0);     // diagonal-major FP32 macro records per block
-    for (int b = 0; b < nblocks; ++b) mo[b + 1] = mo[b] + (blocks[b].ni + blocks[b].nj - 1) * blocks[b].nj;
+    std::vector<int> mo(nblocks + 1, 0);     // first macro-sweep record per block
+    for (int b = 0; b < nblocks; ++b) mo[b + 1] = mo[b] + (int)macro_cells(blocks[b].ni, blocks[b].nj, s.mpad);
     if ((r = up(ctx, (void *)d.mrec_off, mo))) return r;
+    launch_macro_pad(d, ctx->st, ctx->fp32);
+    ctx->launches += nblocks;
   }
   if ((r = up(ctx, (void *)ctx->blk_order, order))) return r;
   if ((r = up(ctx, (void *)ctx->work, work))) return r;

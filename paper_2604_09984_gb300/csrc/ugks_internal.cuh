@@ -77,7 +77,8 @@ struct Dev {
   float4 *jinvf;             // nc: the same in FP32
   void *fgeo;                // nf*NFG face geometry record (arithmetic type)
   void *srec;                // nc*NSR sweep record (layout at NSR)
-  int *mrec_off;             // nblocks+1: first FP32 macro record of each block (diagonal-major)
+  int *mrec_off;             // nblocks+1: first macro-sweep record of each block (padded diagonals x rows)
+  int mpad;                  // diagonals of padding on both sides of a block's macro-sweep records
   double vbox[4];            // velocity box (vx_min, vx_max, vy_min, vy_max)
   double *affine;            // nblocks*6
   // state
@@ -92,8 +93,7 @@ struct Dev {
                              // kernels read it there, so a captured step graph stays valid when dt changes)
   double *TW;                // nc*4 extensive level-n macro term
   double *Fc;                // nc*4 macro flux divergence of the last flux
-  double *dW;                // nc*4 macro increment
-  void *mrec;                // nc*41 macro-sweep records (arithmetic type)
+  void *mrec;                // macro-sweep records (arithmetic type, layout in ugks_macro.cu)
   double *Wp;                // nc*4 macro predictor W'
   double *cpar;              // nc*NCP cell parameters (predictor / level n)
   double *cparn;
@@ -163,9 +163,6 @@ enum { FG_SNX = 0, FG_SNY, FG_SUN, FG_UFX, FG_UFY, FG_DXLX, FG_DXLY, FG_DXRX, FG
 // micro-sweep diagonal base at SR_DBASE and the neighbour mask (int bits) at
 // SR_MASK; 16 values so a record is a whole number of 16-byte chunks
 enum { SR_DBASE = 12, SR_MASK = 13, NSR = 16 };
-
-// values per cell of the macro-sweep record (FP64 packed, FP32 padded to 256 B)
-enum { NMR = 41, NMR32 = 64 };
 
 // per-cell parameter record (from W' or W^n)
 enum { CP_RHO = 0, CP_UX, CP_UY, CP_LAM, CP_QX, CP_QY, CP_ITAU, CP_DBASE, NCP = 8 };

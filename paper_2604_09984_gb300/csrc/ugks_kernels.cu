@@ -651,451 +651,6 @@ template <typename T> __global__ void k_cell_params(Dev d, const double *Wsrc, d
   write_shrec<T>(d, o, d.vol_old[c], reinterpret_cast<T *>(d.shn) + (size_t)NSH * c);
 }
 
-// ----------------------------------------------------- macro LU-SGS sweep
-// Per-cell record of the macro sweep (gathered in parallel before it):
-// R (4), 1/diag, then per face slot: neighbour W (4), outward normal (2),
-// U.n, S/4, Gamma.
-enum { MR_R = 0, MR_IDIAG = 4, MR_SLOT = 5, MR_SW = 9 };
-
-// (1/4) S (dF_E,j - Gamma dW_j) across one face slot of the record.  FP64:
-// the difference F_E(W + dW) - F_E(W) evaluated directly.  FP32 (mixed
-// path): the same difference rewritten exactly in terms of dW (every term is
-// O(dW)), so no cancellation occurs when dW << W.
-// Off-diagonal coupling (1/4 S)(Delta F_E . n - Gamma dW) of a neighbour
-// with state W (slot record r: W (4), n (2), U.n, S/4, Gamma) and increment
-// dW, the flux variation written out as a difference (one division, no
-// cancellation between the two fluxes): with d(ab/rho) = (da b rho + a db
-// rho + da db rho - a b drho) / (rho (rho + drho)) and p = (gamma-1)(E -
-// |m|^2/(2 rho)).
-__device__ __forceinline__ void macro_off(const double *r, const double *dW, int Keff, double out[4]) {
-  const double rho = r[0], m1 = r[1], m2 = r[2], E = r[3], nx = r[4], ny = r[5], un = r[6];
-  const double dr = dW[0], d1 = dW[1], d2 = dW[2], dE = dW[3];
-  const double g1 = 2.0 / (2.0 + (double)Keff);          // gamma - 1
-  const double mn = m1 * nx + m2 * ny, dmn = d1 * nx + d2 * ny;
-  const double den = 1.0 / (rho * (rho + dr));
-  const double dq11 = (2.0 * (m1 * d1 + m2 * d2) * rho + (d1 * d1 + d2 * d2) * rho - (m1 * m1 + m2 * m2) * dr) * den;
-  const double dp = g1 * (dE - 0.5 * dq11);
-  const double p = g1 * (E - 0.5 * (m1 * m1 + m2 * m2) * ((rho + dr) * den));
-  const double dv = (dmn * rho - mn * dr) * den;
-  const double dF0 = dmn - dr * un;
-  const double dF1 = (d1 * mn * rho + m1 * dmn * rho + d1 * dmn * rho - m1 * mn * dr) * den - d1 * un + dp * nx;
-  const double dF2 = (d2 * mn * rho + m2 * dmn * rho + d2 * dmn * rho - m2 * mn * dr) * den - d2 * un + dp * ny;
-  const double dF3 = (dE * mn * rho + E * dmn * rho + dE * dmn * rho - E * mn * dr) * den - dE * un +
-                     dp * (mn + dmn) * (rho * den) + p * dv;
-  const double q = r[7], g = r[8];
-  out[0] = q * (dF0 - g * dr);
-  out[1] = q * (dF1 - g * d1);
-  out[2] = q * (dF2 - g * d2);
-  out[3] = q * (dF3 - g * dE);
-}
-
-__device__ __forceinline__ void macro_off(const float *rr, const float *dWn, int Keff, float out[4]) {
-  float4 s0 = reinterpret_cast<const float4 *>(rr)[0], s1 = reinterpret_cast<const float4 *>(rr)[1];
-  float gam = rr[8];
-  float4 dw = *reinterpret_cast<const float4 *>(dWn);
-  float r = s0.x, m1 = s0.y, m2 = s0.z, E = s0.w;
-  float nx = s1.x, ny = s1.y, un = s1.z;
-  float dr = dw.x, d1 = dw.y, d2 = dw.z, dE = dw.w;
-  float g1 = __fdividef(2.0f, 2.0f + (float)Keff);    // gamma - 1
-  float mn = m1 * nx + m2 * ny, dmn = d1 * nx + d2 * ny;
-  float den = __fdividef(1.0f, r * (r + dr));          // 1/(rho (rho + drho))
-  // d(a b / rho) = [da b rho + a db rho + da db rho - a b drho] / (rho (rho + drho))
-  float dq11 = (2.0f * (m1 * d1 + m2 * d2) * r + (d1 * d1 + d2 * d2) * r -
-                (m1 * m1 + m2 * m2) * dr) * den;
-  float dp = g1 * (dE - 0.5f * dq11);
-  float p = g1 * (E - 0.5f * (m1 * m1 + m2 * m2) * ((r + dr) * den));
-  float dv = (dmn * r - mn * dr) * den;               // d(mn / rho)
-  float dF0 = dmn - dr * un;
-  float dF1 = (d1 * mn * r + m1 * dmn * r + d1 * dmn * r - m1 * mn * dr) * den - d1 * un + dp * nx;
-  float dF2 = (d2 * mn * r + m2 * dmn * r + d2 * dmn * r - m2 * mn * dr) * den - d2 * un + dp * ny;
-  float dF3 = (dE * mn * r + E * dmn * r + dE * dmn * r - E * mn * dr) * den - dE * un +
-              dp * (mn + dmn) * (r * den) + p * dv;
-  float q = s1.w, g = gam;
-  out[0] = q * (dF0 - g * dr);
-  out[1] = q * (dF1 - g * d1);
-  out[2] = q * (dF2 - g * d2);
-  out[3] = q * (dF3 - g * dE);
-}
-
-// Gather the sweep record of every solved cell (parallel).  The FP64 record
-// is the packed layout above.  The FP32 record (64 floats, 256 bytes) keeps
-// every group 16-byte aligned for 128-bit shared-memory reads: R (4), 1/diag,
-// the neighbour mask, then per face slot 12 values (neighbour W (4); normal
-// (2), U.n, S/4; Gamma, 3 unused) and the increment of the sweep (4).
-enum { M32_R = 0, M32_IDIAG = 4, M32_MASK = 5, M32_SLOT = 8, M32_SW = 12, M32_DWS = 56 };
-template <typename MT> struct MacroRec;
-template <> struct MacroRec<double> {
-  static constexpr int R = MR_R, IDIAG = MR_IDIAG, SLOT = MR_SLOT, SW = MR_SW, STRIDE = NMR;
-};
-template <> struct MacroRec<float> {
-  static constexpr int R = M32_R, IDIAG = M32_IDIAG, SLOT = M32_SLOT, SW = M32_SW, STRIDE = NMR32;
-};
-
-// FP32 records are diagonal-major per block: the record of cell (i, j) of
-// block b is number mrec_off[b] + (i + j) nj + j, so the records of one
-// diagonal are contiguous and a sweep step fetches them with one bulk copy.
-__device__ __forceinline__ size_t mrec32_index(const Dev &d, int c) {
-  int b = d.cell_block[c];
-  int ni = d.blk_info[8 * b], nj = d.blk_info[8 * b + 1];
-  int loc = c - d.cell_off[b];
-  int i = loc % ni, j = loc / ni;
-  return (size_t)d.mrec_off[b] + (size_t)(i + j) * nj + j;
-}
-
-template <typename MT> __global__ void k_macro_prep(Dev d, MT *rec) {
-  typedef MacroRec<MT> L;
-  int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= d.nc) return;
-  MT *o = rec + (size_t)L::STRIDE * (sizeof(MT) == 4 ? mrec32_index(d, c) : (size_t)c);
-  int mask = d.cmask[c];
-  if (sizeof(MT) == 4) o[M32_MASK] = __int_as_float(mask);
-  if (!(mask & 1)) return;
-  double vol = d.vol_new[c], idt = 1.0 / d.stepc[0];
-  for (int m = 0; m < 4; ++m)
-    o[L::R + m] = (MT)(d.TW[4 * c + m] - vol * idt * d.W[4 * c + m] - 0.5 * d.Fc[4 * c + m]);
-  double diag = vol * (d.cfl_s / (d.cfl_pseudo * d.dts[c]) + idt);
-  for (int s = 0; s < 4; ++s) {
-    int f = d.cell_faces[4 * c + s];
-    diag += 0.25 * d.S[f] * d.gam[f];
-    double sg = (double)d.cell_sgn[4 * c + s];
-    int nb = (sg > 0) ? d.face_R[f] : d.face_L[f];
-    MT *q = o + L::SLOT + L::SW * s;
-    // missing neighbour: a harmless positive state (its increment is zero)
-    for (int m = 0; m < 4; ++m) q[m] = nb >= 0 ? (MT)d.W[4 * nb + m] : (m == 0 || m == 3 ? MT(1) : MT(0));
-    q[4] = (MT)(sg * d.nrm[2 * f]);
-    q[5] = (MT)(sg * d.nrm[2 * f + 1]);
-    q[6] = (MT)(sg * d.SUn[f] / d.S[f]);
-    q[7] = (MT)(0.25 * d.S[f]);
-    q[8] = (MT)d.gam[f];
-  }
-  o[L::IDIAG] = (MT)(1.0 / diag);
-}
-
-// shared memory of the FP32 macro sweep ahead of its buffers: the mbarriers
-// of the ring stages (floats)
-constexpr int MACRO_SMEM_HEAD = 16;
-
-// FP32 macro sweep: as k_macro_sweep below, with TPR threads per row (each
-// evaluates the couplings of face slots s = sub, sub + TPR, ...; a shuffle
-// within the row's lanes sums them).  The records of the next NS-1 diagonals
-// are in flight in a ring in shared memory, one bulk copy per diagonal
-// completing on the stage's mbarrier (bounded waits), and the part of the
-// next record a thread uses is moved into registers before the barrier that
-// ends a diagonal, so after the barrier only the coupling arithmetic remains.
-// The forward increment is stored into the record for the backward pass.
-// NS = 0: no ring, records read from global memory (blocks too tall for a
-// two-stage ring).
-__device__ __forceinline__ void macro_off_v(float4 s0, float4 s1, float gam, float4 dw, int Keff,
-                                            float out[4]) {
-  __align__(16) float rr[12] = {s0.x, s0.y, s0.z, s0.w, s1.x, s1.y, s1.z, s1.w, gam, 0.f, 0.f, 0.f};
-  __align__(16) float dv[4] = {dw.x, dw.y, dw.z, dw.w};
-  macro_off(rr, dv, Keff, out);
-}
-
-// PM (with TPR = 2): the two threads of a row take the two face slots that
-// couple in this pass -- forward the lower neighbours (slots 0 and 2),
-// backward the upper ones (1 and 3) -- and the first thread also the
-// periodic wrap slot (1 forward at i = n_i - 1, 0 backward at i = 0) where it
-// applies; couplings that are not evaluated are exact zeros in the TPR = 4
-// form, so the sums are the same.
-template <int NS, int TPR, bool PM = false>
-__global__ void __launch_bounds__(512) k_macro_sweep_f32(Dev d, float *rec) {
-  static_assert(!PM || TPR == 2, "pass-dependent slots pair two threads a row");
-  constexpr int NSL = PM ? 1 : 4 / TPR;         // face slots per thread (PM: plus the wrap)
-  constexpr int NSR_ = NS > 0 ? NS : 1;
-  extern __shared__ __align__(16) float smf[];
-  unsigned long long *mb = reinterpret_cast<unsigned long long *>(smf);   // one mbarrier per stage
-  int rows = blockDim.x / TPR;
-  float *buf0 = smf + MACRO_SMEM_HEAD, *buf1 = buf0 + 4 * rows;
-  float *ring = buf1 + 4 * rows;                 // NS * rows * NMR32
-  int b = blockIdx.x;
-  const int *bi = d.blk_info + 8 * b;
-  int ni = bi[0], nj = bi[1], per = bi[2];
-  const float *rb = rec + (size_t)NMR32 * d.mrec_off[b];          // this block's records
-  float *rbw = rec + (size_t)NMR32 * d.mrec_off[b];
-  int row = threadIdx.x / TPR, sub = threadIdx.x % TPR;
-  unsigned rmask = (TPR == 1 ? 1u : (1u << TPR) - 1u) << (threadIdx.x & 31 & ~(TPR - 1));
-  int nd = ni + nj - 1;
-  if (NS > 0 && threadIdx.x == 0) {
-    for (int s = 0; s < NSR_; ++s) mbar_init(&mb[s], 1);
-    mbar_fence_init();
-  }
-  if (sub == 0)
-    for (int m = 0; m < 4; ++m) { buf0[4 * row + m] = 0.f; buf1[4 * row + m] = 0.f; }
-  __syncthreads();
-  const unsigned diag_bytes = (unsigned)nj * NMR32 * sizeof(float);
-  bool to = false;                   // this thread's bounded wait ran out
-  int issued = -1, waited = -1;      // thread 0: last stage copied into / waited for
-  for (int pass = 0; pass < 2; ++pass) {
-    float4 prev = make_float4(0.f, 0.f, 0.f, 0.f), first = prev;
-    // face slot of this thread's q-th coupling
-    auto slot_of = [&](int q) {
-      if (!PM) return q * TPR + sub;
-      return sub == 0 ? (pass == 0 ? 0 : 1) : (pass == 0 ? 2 : 3);
-    };
-    // diagonal of step it, and its position in the ring (g = steps so far)
-    auto diag_of = [&](int it) { return pass == 0 ? it : nd - 1 - it; };
-    auto gstep = [&](int it) { return pass * nd + it; };
-    // thread 0 fetches the records of a whole diagonal with one bulk copy
-    auto issue = [&](int it) {
-      if (NS == 0 || threadIdx.x != 0 || it >= nd) return;
-      int s = gstep(it) % NSR_;
-      fence_proxy_async_shared();
-      mbar_arrive_expect_tx(&mb[s], diag_bytes);
-      bulk_g2s(ring + (size_t)s * rows * NMR32, rb + (size_t)diag_of(it) * nj * NMR32, diag_bytes, &mb[s]);
-      issued = gstep(it);
-    };
-    // a bounded wait; a thread that gives up marks `to`, and the CTA stops
-    // at the end of the diagonal (uniform decision at the barrier)
-    auto wait_stage = [&](int it) {
-      if (NS == 0 || it >= nd) return;
-      int g = gstep(it);
-      if (!mbar_wait(&mb[g % NSR_], (unsigned)(g / NSR_) & 1u, d.err, d.wait_polls)) to = true;
-      else if (threadIdx.x == 0) waited = g;
-    };
-    // registers of the next diagonal: mask, this thread's slot records,
-    // R (pass 0) or the forward increment (pass 1), 1/diag
-    int nmask = 0;
-    float4 nsa[NSL], nsb[NSL], nrv = make_float4(0.f, 0.f, 0.f, 0.f);
-    float ngam[NSL], nidg = 0.f;
-    auto fetch = [&](int it) {
-      nmask = 0;
-      if (it >= nd) return;
-      int t = diag_of(it), i = t - row;
-      if (!(row < nj && i >= 0 && i < ni)) return;
-      const float *r = NS > 0 ? ring + ((size_t)(gstep(it) % NSR_) * rows + row) * NMR32
-                              : rb + ((size_t)t * nj + row) * NMR32;
-      nmask = __float_as_int(r[M32_MASK]);
-#pragma unroll
-      for (int q = 0; q < NSL; ++q) {
-        const float *sr = r + M32_SLOT + M32_SW * slot_of(q);
-        nsa[q] = *reinterpret_cast<const float4 *>(sr);
-        nsb[q] = *reinterpret_cast<const float4 *>(sr + 4);
-        ngam[q] = sr[8];
-      }
-      nrv = *reinterpret_cast<const float4 *>(r + (pass == 0 ? M32_R : M32_DWS));
-      nidg = r[M32_IDIAG];
-    };
-#pragma unroll
-    for (int q = 0; q < NS - 1; ++q) issue(q);
-    wait_stage(0);
-    fetch(0);
-    int cur = 0;
-    for (int it = 0; it < nd; ++it) {
-      issue(it + NS - 1);
-      int t = diag_of(it);
-      int i = t - row;
-      bool act = row < nj && i >= 0 && i < ni;
-      int mask = nmask;
-      float4 val = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (mask & 1) {
-        const float *prv = cur ? buf0 : buf1;
-        float acc[4] = {0, 0, 0, 0};
-#pragma unroll
-        for (int q = 0; q < NSL; ++q) {
-          int s = slot_of(q);
-          float4 dv = make_float4(0.f, 0.f, 0.f, 0.f);
-          bool use = !PM;                        // PM: only the couplings of this pass
-          if (mask & (2 << s)) {
-            if (pass == 0) {
-              if (s == 0 && i > 0) { dv = prev; use = true; }
-              else if (s == 1 && per && i == ni - 1) { dv = first; use = true; }
-              else if (s == 2 && row > 0) { dv = *reinterpret_cast<const float4 *>(prv + 4 * (row - 1)); use = true; }
-            } else {
-              if (s == 1 && i < ni - 1) { dv = prev; use = true; }
-              else if (s == 0 && per && i == 0) { dv = first; use = true; }
-              else if (s == 3 && row < nj - 1) { dv = *reinterpret_cast<const float4 *>(prv + 4 * (row + 1)); use = true; }
-            }
-          }
-          if (use) {
-            float o[4];
-            macro_off_v(nsa[q], nsb[q], ngam[q], dv, d.Keff, o);
-            // a plain (never contracted) sum: the same bits as the lanes'
-            // shuffle sums of the four-slot form
-            for (int m = 0; m < 4; ++m) acc[m] = __fadd_rn(acc[m], o[m]);
-          }
-        }
-        // PM: the periodic wrap (slot 1 forward at i = n_i - 1, slot 0
-        // backward at i = 0), rare: its record is read where it lies (the
-        // ring stage of this step is not reissued before the next step)
-        if (PM && sub == 0 && per && i == (pass == 0 ? ni - 1 : 0) && (mask & (2 << (pass == 0 ? 1 : 0)))) {
-          const float *r = NS > 0 ? ring + ((size_t)(gstep(it) % NSR_) * rows + row) * NMR32
-                                  : rb + ((size_t)t * nj + row) * NMR32;
-          const float *sr = r + M32_SLOT + M32_SW * (pass == 0 ? 1 : 0);
-          float o[4];
-          macro_off_v(*reinterpret_cast<const float4 *>(sr), *reinterpret_cast<const float4 *>(sr + 4), sr[8],
-                      first, d.Keff, o);
-          for (int m = 0; m < 4; ++m) acc[m] = __fadd_rn(acc[m], o[m]);
-        }
-#pragma unroll
-        for (int w = 1; w < TPR; w <<= 1)
-          for (int m = 0; m < 4; ++m) acc[m] += __shfl_xor_sync(rmask, acc[m], w);
-        float4 rv = nrv;
-        float idg = nidg;
-        if (pass == 0)
-          val = make_float4((rv.x - acc[0]) * idg, (rv.y - acc[1]) * idg, (rv.z - acc[2]) * idg,
-                            (rv.w - acc[3]) * idg);
-        else
-          val = make_float4(rv.x - acc[0] * idg, rv.y - acc[1] * idg, rv.z - acc[2] * idg,
-                            rv.w - acc[3] * idg);
-        // forward: the increment d* for the backward pass; backward: the
-        // final increment for the post-processing kernel
-        if (sub == 0) *reinterpret_cast<float4 *>(rbw + ((size_t)t * nj + row) * NMR32 + M32_DWS) = val;
-      }
-      if (act) {
-        prev = val;
-        if (i == (pass == 0 ? 0 : ni - 1)) first = val;
-      }
-      float *dst = cur ? buf1 : buf0;
-      if (sub == 0) *reinterpret_cast<float4 *>(dst + 4 * row) = val;
-      // the next diagonal's records, read into registers before the barrier
-      wait_stage(it + 1);
-      fetch(it + 1);
-      if (__syncthreads_or(to)) break;
-      cur ^= 1;
-    }
-    if (__syncthreads_or(to)) break;
-    // the increments stored above are read by the next pass's bulk copies
-    fence_proxy_async_global();
-    __threadfence_block();
-    if (sub == 0)
-      for (int m = 0; m < 4; ++m) { buf0[4 * row + m] = 0.f; buf1[4 * row + m] = 0.f; }
-    __syncthreads();
-  }
-  // after a timeout: no copy of this CTA may still be in flight when it
-  // exits, so thread 0 waits (default bound) for every stage it issued and
-  // nobody waited for; the results of the step are invalid (EF_TIMEOUT)
-  if (NS > 0 && threadIdx.x == 0 && issued > waited)
-    for (int g = waited + 1; g <= issued; ++g) mbar_wait(&mb[g % NSR_], (unsigned)(g / NSR_) & 1u, d.err);
-}
-
-// LU-SGS of Eq. dualTimeStepping_macro (Sec. 2.2), one CTA per block,
-// thread = row j; diagonals i + j in increasing (forward) then decreasing
-// (backward) order reproduce the lexicographic Gauss-Seidel exactly.  The
-// record of the next diagonal's cell is loaded before the barrier, so a
-// diagonal step costs the arithmetic of its lower/upper couplings only.
-template <typename MT> __global__ void __launch_bounds__(512) k_macro_sweep(Dev d, const MT *rec) {
-  extern __shared__ double sm[];
-  MT *buf0 = reinterpret_cast<MT *>(sm), *buf1 = buf0 + 4 * blockDim.x;
-  int b = blockIdx.x;
-  const int *bi = d.blk_info + 8 * b;
-  int ni = bi[0], nj = bi[1], per = bi[2];
-  int off = d.cell_off[b];
-  int row = threadIdx.x;
-  MT prev[4] = {0, 0, 0, 0}, first[4] = {0, 0, 0, 0};
-  int nd = ni + nj - 1;
-  for (int m = 0; m < 4; ++m) { buf0[4 * row + m] = 0; buf1[4 * row + m] = 0; }
-  __syncthreads();
-  for (int pass = 0; pass < 2; ++pass) {
-    int cur = 0;
-    // registers holding the record of the cell this thread handles next
-    MT r[NMR];
-    MT dws[4] = {0, 0, 0, 0};
-    int mask = 0;
-    auto load = [&](int it) {
-      int step = pass == 0 ? it : nd - 1 - it;
-      int i = step - row;
-      mask = 0;
-      if (it < nd && row < nj && i >= 0 && i < ni) {
-        int c = off + row * ni + i;
-        mask = d.cmask[c];
-        if (mask & 1) {
-          const MT *src = rec + (size_t)NMR * c;
-#pragma unroll
-          for (int m = 0; m < NMR; ++m) r[m] = src[m];
-          if (pass == 1)
-            for (int m = 0; m < 4; ++m) dws[m] = (MT)d.dW[4 * c + m];
-        }
-      }
-    };
-    // FP32: the next diagonal's record is loaded before the barrier; FP64
-    // (reference path) loads at the start of the step to bound registers
-    constexpr bool PF = sizeof(MT) == 4;
-    if (PF) load(0);
-    for (int it = 0; it < nd; ++it) {
-      if (!PF) load(it);
-      int step = pass == 0 ? it : nd - 1 - it;
-      int i = step - row;
-      bool act = row < nj && i >= 0 && i < ni;
-      MT val[4] = {0, 0, 0, 0};
-      if (act && (mask & 1)) {
-        int c = off + row * ni + i;
-        MT acc[4];
-        if (pass == 0) for (int m = 0; m < 4; ++m) acc[m] = r[MR_R + m];
-        else for (int m = 0; m < 4; ++m) acc[m] = 0;
-        MT *prv = cur ? buf0 : buf1;
-        const MT zero4[4] = {0, 0, 0, 0};
-        MT o[4][4];
-#pragma unroll
-        for (int s = 0; s < 4; ++s) {
-          const MT *dv = zero4;
-          if (mask & (2 << s)) {
-            if (pass == 0) {          // lower: i-1, wrap ni-1 -> 0, j-1
-              if (s == 0 && i > 0) dv = prev;
-              else if (s == 1 && per && i == ni - 1) dv = first;
-              else if (s == 2 && row > 0) dv = prv + 4 * (row - 1);
-            } else {                  // upper: i+1, wrap 0 -> ni-1, j+1
-              if (s == 1 && i < ni - 1) dv = prev;
-              else if (s == 0 && per && i == 0) dv = first;
-              else if (s == 3 && row < nj - 1) dv = prv + 4 * (row + 1);
-            }
-          }
-          // a zero increment couples to zero: only slots with a neighbour
-          // increment are evaluated (the FP64 pipe is this kernel's bound)
-          if (dv != zero4) macro_off(r + MR_SLOT + MR_SW * s, dv, d.Keff, o[s]);
-          else o[s][0] = o[s][1] = o[s][2] = o[s][3] = MT(0);
-        }
-#pragma unroll
-        for (int s = 0; s < 4; ++s)
-          for (int m = 0; m < 4; ++m) acc[m] += pass == 0 ? -o[s][m] : o[s][m];
-        MT idg = r[MR_IDIAG];
-        if (pass == 0) for (int m = 0; m < 4; ++m) val[m] = acc[m] * idg;
-        else for (int m = 0; m < 4; ++m) val[m] = dws[m] - acc[m] * idg;
-        for (int m = 0; m < 4; ++m) d.dW[4 * c + m] = (double)val[m];
-      }
-      if (act) {
-        for (int m = 0; m < 4; ++m) prev[m] = val[m];
-        if (i == (pass == 0 ? 0 : ni - 1)) for (int m = 0; m < 4; ++m) first[m] = val[m];
-      }
-      MT *dst = cur ? buf1 : buf0;
-      for (int m = 0; m < 4; ++m) dst[4 * row + m] = val[m];
-      if (PF) load(it + 1);     // next diagonal's record, in flight across the barrier
-      __syncthreads();
-      cur ^= 1;
-    }
-    for (int m = 0; m < 4; ++m) { prev[m] = 0; first[m] = 0; }
-    for (int m = 0; m < 4; ++m) { buf0[4 * row + m] = 0; buf1[4 * row + m] = 0; }
-    __syncthreads();
-  }
-}
-
-// W' = W + dW and the predictor cell record (Step 4 result) for Step 5.
-template <typename T> __global__ void k_macro_post(Dev d) {
-  int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= d.nc) return;
-  T *sr = reinterpret_cast<T *>(d.srec) + (size_t)NSR * c;
-  int mask = d.cmask[c];
-  *reinterpret_cast<int *>(sr + SR_MASK) = mask;
-  if (!(mask & 1)) {
-    for (int m = 0; m < 4; ++m) d.Wp[4 * c + m] = d.W[4 * c + m];
-    return;
-  }
-  if (sizeof(T) == 4) {
-    const float *inc = reinterpret_cast<const float *>(d.mrec) + (size_t)NMR32 * mrec32_index(d, c) + M32_DWS;
-    for (int m = 0; m < 4; ++m) d.Wp[4 * c + m] = d.W[4 * c + m] + (double)inc[m];
-  } else {
-    for (int m = 0; m < 4; ++m) d.Wp[4 * c + m] = d.W[4 * c + m] + d.dW[4 * c + m];
-  }
-  Prim p = primitive(d.Wp + 4 * c, d.Keff);
-  double *o = d.cpar + NCP * c;
-  o[CP_RHO] = p.rho; o[CP_UX] = p.ux; o[CP_UY] = p.uy; o[CP_LAM] = p.lam;
-  o[CP_QX] = d.q[2 * c]; o[CP_QY] = d.q[2 * c + 1];
-  o[CP_ITAU] = 1.0 / collision_time(p.rho, p.lam, d.mu_ref, d.omega);
-  o[CP_DBASE] = d.vol_new[c] * (d.cfl_s / (d.cfl_pseudo * d.dts[c]) + 1.0 / d.stepc[0] + 0.5 * o[CP_ITAU]);
-  sr[SR_DBASE] = (T)o[CP_DBASE];
-  write_shrec<T>(d, o, d.vol_new[c], reinterpret_cast<T *>(d.shp) + (size_t)NSH * c);
-}
-
 // Step 7 (one warp per cell): W^{s+1} = W' + sum V Psi (f^{s+1} - g(W')),
 // heat flux about V' (reading R7); flags non-physical states.
 template <typename T, int FB> __global__ void k_moments(Dev d) {
@@ -1437,74 +992,6 @@ void launch_cell_params(const Dev &d, cudaStream_t s, const double *W, double *o
   if (fp32) k_cell_params<float><<<nblk(d.nc, 256), 256, 0, s>>>(d, W, out);
   else k_cell_params<double><<<nblk(d.nc, 256), 256, 0, s>>>(d, W, out);
 }
-// dynamic shared memory of the sweeps: up to the 227 KB a CTA may use
-constexpr size_t kMacroSmem = 227 * 1024;
-// The sweep records are gathered on the caller's stream before the fork, so
-// the sweep kernel is the first work of the side stream: it then takes its
-// empty SMs before the flux kernel launched beside it fills the GPU.
-void launch_macro_prep(const Dev &d, cudaStream_t s, int fp32) {
-  if (fp32) k_macro_prep<float><<<nblk(d.nc, 256), 256, 0, s>>>(d, reinterpret_cast<float *>(d.mrec));
-  else k_macro_prep<double><<<nblk(d.nc, 256), 256, 0, s>>>(d, reinterpret_cast<double *>(d.mrec));
-}
-
-void launch_macro_sweep(const Dev &d, cudaStream_t s, int rows, int fp32) {
-  if (fp32) {
-    float *rec = reinterpret_cast<float *>(d.mrec);
-    size_t per = (size_t)rows * NMR32 * sizeof(float);
-    size_t base = (MACRO_SMEM_HEAD + 8 * (size_t)rows) * sizeof(float);
-    int NS = (int)((kMacroSmem - base) / per);
-    NS = NS > 4 ? 4 : (NS < 2 ? 0 : NS);
-    // two threads a row on the slots of the pass (PM) where the rows fit
-    int tpr = rows <= 256 ? 2 : 1;
-    bool pm = tpr == 2;
-    if (const char *env = getenv("UGKS_MACRO_TPR")) {   // tuning: threads per row (1, 2 or 4; plain slots)
-      int t = atoi(env);
-      if ((t == 1 || t == 2 || t == 4) && t * rows <= 512) { tpr = t; pm = false; }
-    }
-    // the whole shared memory of an SM: the sweep's SMs take no CTA of the
-    // kernels running beside it on the main stream
-    size_t sm = kMacroSmem;
-    int th = tpr * rows;
-#define UGKS_MACRO_F32(ns, tp) k_macro_sweep_f32<ns, tp><<<d.nblocks, th, sm, s>>>(d, rec)
-#define UGKS_MACRO_PM(ns) k_macro_sweep_f32<ns, 2, true><<<d.nblocks, th, sm, s>>>(d, rec)
-    if (pm) {
-      if (NS == 4) UGKS_MACRO_PM(4); else if (NS == 3) UGKS_MACRO_PM(3);
-      else if (NS == 2) UGKS_MACRO_PM(2); else UGKS_MACRO_PM(0);
-    } else if (tpr == 4) {
-      if (NS == 4) UGKS_MACRO_F32(4, 4); else if (NS == 3) UGKS_MACRO_F32(3, 4);
-      else if (NS == 2) UGKS_MACRO_F32(2, 4); else UGKS_MACRO_F32(0, 4);
-    } else if (tpr == 2) {
-      if (NS == 4) UGKS_MACRO_F32(4, 2); else if (NS == 3) UGKS_MACRO_F32(3, 2);
-      else if (NS == 2) UGKS_MACRO_F32(2, 2); else UGKS_MACRO_F32(0, 2);
-    } else {
-      if (NS == 4) UGKS_MACRO_F32(4, 1); else if (NS == 3) UGKS_MACRO_F32(3, 1);
-      else if (NS == 2) UGKS_MACRO_F32(2, 1); else UGKS_MACRO_F32(0, 1);
-    }
-#undef UGKS_MACRO_F32
-#undef UGKS_MACRO_PM
-  } else {
-    double *rec = reinterpret_cast<double *>(d.mrec);
-    k_macro_sweep<double><<<d.nblocks, rows, kMacroSmem, s>>>(d, rec);
-  }
-  if (fp32) k_macro_post<float><<<nblk(d.nc, 256), 256, 0, s>>>(d);
-  else k_macro_post<double><<<nblk(d.nc, 256), 256, 0, s>>>(d);
-}
-// shared memory of the macro sweeps exceeds the default 48 KB
-void sweep_setup() {
-  int ms = (int)kMacroSmem;
-  cudaFuncSetAttribute(k_macro_sweep<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, ms);
-#define UGKS_MACRO_ATTR(ns, tp) \
-  cudaFuncSetAttribute(k_macro_sweep_f32<ns, tp>, cudaFuncAttributeMaxDynamicSharedMemorySize, ms)
-  UGKS_MACRO_ATTR(4, 4); UGKS_MACRO_ATTR(3, 4); UGKS_MACRO_ATTR(2, 4); UGKS_MACRO_ATTR(0, 4);
-  UGKS_MACRO_ATTR(4, 2); UGKS_MACRO_ATTR(3, 2); UGKS_MACRO_ATTR(2, 2); UGKS_MACRO_ATTR(0, 2);
-  UGKS_MACRO_ATTR(4, 1); UGKS_MACRO_ATTR(3, 1); UGKS_MACRO_ATTR(2, 1); UGKS_MACRO_ATTR(0, 1);
-#undef UGKS_MACRO_ATTR
-#define UGKS_MACRO_ATTR_PM(ns) \
-  cudaFuncSetAttribute(k_macro_sweep_f32<ns, 2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, ms)
-  UGKS_MACRO_ATTR_PM(4); UGKS_MACRO_ATTR_PM(3); UGKS_MACRO_ATTR_PM(2); UGKS_MACRO_ATTR_PM(0);
-#undef UGKS_MACRO_ATTR_PM
-}
-
 void launch_moments_finish(const Dev &d, cudaStream_t s) { k_moments_finish<<<nblk(d.nc, 256), 256, 0, s>>>(d); }
 // Two cells (warps) a CTA: small CTAs fit beside the velocity reduction's
 // two CTAs an SM, with which this Step 7 runs concurrently.

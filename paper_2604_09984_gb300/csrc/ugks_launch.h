@@ -13,6 +13,12 @@ void launch_gradW(const Dev &d, cudaStream_t s);                            // t
 void launch_face_coef(const Dev &d, cudaStream_t s, int fp32);
 void launch_cell_macro(const Dev &d, cudaStream_t s, int level_n);
 void launch_cell_params(const Dev &d, cudaStream_t s, const double *W, double *out, int fp32);
+// macro LU-SGS (ugks_macro.cu); rows: of the tallest block
+int macro_pad(int rows, int fp32);                     // padding diagonals of the records
+size_t macro_cells(int ni, int nj, int pad);           // records of a block
+size_t macro_record_bytes(int fp32);
+void macro_setup();
+void launch_macro_pad(const Dev &d, cudaStream_t s, int fp32);              // once per mesh
 void launch_macro_prep(const Dev &d, cudaStream_t s, int fp32);
 void launch_macro_sweep(const Dev &d, cudaStream_t s, int rows, int fp32);   // sweep + post (after launch_macro_prep)
 // micro LU-SGS sweeps (ugks_sweep.cu): pass 0 forward, 1 backward; nw warps
@@ -23,7 +29,6 @@ void launch_wsweep(const Dev &d, cudaStream_t s, int pass, const int *work, int 
 void wsweep_setup();
 int wsweep_ql(int max_nj);
 int wsweep_fits(int fp32, int fbf, int vpt, int nw, int ns, int ql);
-void sweep_setup();
 void launch_moments(const Dev &d, cudaStream_t s, int fp32);
 void launch_moments_finish(const Dev &d, cudaStream_t s);   // sharded step, after the exchange
 // step metrics: stage 0 after the macro prep (|R|^2), 1 after the residual
