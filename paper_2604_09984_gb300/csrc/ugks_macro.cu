@@ -7,41 +7,51 @@
 // A block is swept by one CTA as a skewed wavefront without barriers inside a
 // warp.  LPR lanes hold a row; row j takes cell i = t - j at diagonal t, so
 // its lower neighbour along the row is its own result of diagonal t - 1 and
-// its lower neighbour across rows is row j - 1's, one warp shuffle away.  A
-// cell evaluates the variation of both Cartesian fluxes for its own increment
-// once and sends the finished couplings (4 values) to its two next
-// neighbours, so the chain from one diagonal to the next is one reciprocal, a
-// dozen fused multiply-adds and a shuffle.  Bands of 32 / LPR rows (one warp
-// each) hand their last row's couplings on through a ring in shared memory;
-// a band trails the one before it by K - 1 further diagonals, so that one CTA
-// barrier per K diagonals orders the ring (no polling).
+// its lower neighbour across rows is row j - 1's, one warp shuffle away.
+// Bands of 32 / LPR rows (one warp each) hand their last row's values on
+// through a link in shared memory; a band trails the one before it by K - 1
+// further diagonals, so that one CTA barrier per K diagonals orders the links
+// (no polling).
 //
-// What bounds it: the latency of that chain (one SM per block).  The four
-// vectors a cell needs per pass arrive D - 1 diagonals ahead in a ring in
-// shared memory (asynchronous 16-byte copies, coalesced over the rows of a
-// diagonal), and the next diagonal's are moved into registers while the
-// current one is evaluated; padding around the diagonals and rows holds
-// records of a cell at rest that couples to nothing, so the loop has no
-// bounds checks.  FP64: the pipe retires a warp instruction in tens of cycles,
-// so four lanes share a row (one component each) while all bands fit in one
-// CTA.  Measured (sweep alone, 256 x 128 + 128 x 32 cells, FP32): 115 us for
-// both passes, 0.15 us a diagonal, against 608 us for the form with one CTA
-// barrier and one 32 KB record copy per diagonal; the same loop with the
-// records prefetched straight into registers took 200 us (eight loads in
-// flight wait on each other's scoreboards).  FP64, 64 x 32 cells: 1.53 ms to
-// 0.37 ms with its record gather and predictor.
+// What bounds it: the latency of the chain from one diagonal to the next (one
+// SM per block).  The record of a cell arrives D - 1 diagonals ahead in a ring
+// in shared memory (asynchronous 16-byte copies, coalesced over the rows of a
+// diagonal), and the next diagonal's is moved into registers while the current
+// one is evaluated; padding around the diagonals and rows holds records of
+// cells that keep a zero increment, so the loop has no bounds checks.
+//
+// FP32: a lane a row; the cell evaluates the couplings of its two neighbours
+// of the pass from their increments (the same arithmetic, rounding for
+// rounding, as one thread per face slot).  FP64: the pipe retires a warp
+// instruction in tens of cycles, so a cell evaluates the variation of both
+// Cartesian fluxes for its own increment once and sends finished couplings (4
+// values) to its two next neighbours, and four lanes share a row (one
+// component each) while all bands fit in one CTA.
+//
+// Measured (192 x 96 + 96 x 24 cells, FP32, the sweep alone): 117 us for both
+// passes, 0.20 us a diagonal, against 437 us for the form with one CTA barrier
+// and one 32 KB record copy per diagonal.  FP64, 64 x 32 cells: 1.53 ms to 0.42
+// with its record gather and predictor.
+#include <type_traits>
 #include "ugks_internal.cuh"
 #include "ugks_launch.h"
 
 namespace ugks {
 
-// planes of the sweep records, one vector of 4 per cell each:
-//   VAL  R of Step 4, then the increment (forward, then final)
+// Planes of the sweep records, one vector of 4 per cell each.  Plane VAL: R of
+// Step 4, then the increment (forward, then final).
+// FP64:
 //   ST   rho, V_x, V_y, p of W
 //   F1   1/diag, couplings sent across the i-high face   F2 the j-high face
 //   B1   1/diag, couplings sent across the i-low face    B2 the j-low face
-// A coupling (a, b, g) gives the neighbour a dF_x + b dF_y - g dW.
-enum { MP_VAL = 0, MP_ST, MP_F1, MP_F2, MP_B1, MP_B2, NMP };
+// where a coupling (a, b, g) gives the neighbour a dF_x + b dF_y - g dW.
+// FP32, per pass (forward FW: slots i-low, j-low; backward BW: i-high, j-high):
+//   +0   W of the neighbour along the row   +1 outward normal, U.n, S/4 there
+//   +2   W of the neighbour across rows     +3 outward normal, U.n, S/4 there
+//   +4   Gamma of both faces, 1/diag
+enum { MP_VAL = 0, MP_ST, MP_F1, MP_F2, MP_B1, MP_B2, NMP64 };
+enum { MP_FW = 1, MP_BW = 6, NMP32 = 11, NPASS32 = 5 };
+template <typename T> struct Planes { static constexpr int N = sizeof(T) == 4 ? NMP32 : NMP64; };
 
 template <typename T> struct alignas(16) MV4 { T v[4]; };
 
@@ -53,7 +63,7 @@ __host__ __device__ __forceinline__ int macro_rows(int nj) { return (nj + 31) / 
 // hide the barrier; D - 1 diagonals of copies in flight cover the L2 latency
 // (about 1 us at 0.12 us a diagonal), fewer where 16 bands share the memory.
 struct MacroShape { int lpr, k, d; };
-constexpr MacroShape kShape32{1, 8, 8}, kShape32Tall{1, 8, 6}, kShape64{4, 2, 4}, kShape64Tall{1, 2, 3};
+constexpr MacroShape kShape32{1, 8, 8}, kShape32Tall{1, 8, 4}, kShape64{4, 2, 4}, kShape64Tall{1, 2, 3};
 static MacroShape macro_shape(int rows, int fp32) {
   if (fp32) return rows <= 256 ? kShape32 : kShape32Tall;
   return rows <= 128 ? kShape64 : kShape64Tall;
@@ -68,40 +78,43 @@ int macro_pad(int rows, int fp32) {
 }
 // records (cells with padding) of one block
 size_t macro_cells(int ni, int nj, int pad) { return (size_t)(ni + nj - 1 + 2 * pad) * macro_rows(nj); }
-size_t macro_record_bytes(int fp32) { return NMP * (fp32 ? sizeof(MV4<float>) : sizeof(MV4<double>)); }
+size_t macro_record_bytes(int fp32) { return fp32 ? NMP32 * sizeof(MV4<float>) : NMP64 * sizeof(MV4<double>); }
 
 // vector index of plane 0 of row `row` on diagonal t of block b
-__device__ __forceinline__ long macro_at(const Dev &d, int b, int t, int row) {
+template <typename T> __device__ __forceinline__ long macro_at(const Dev &d, int b, int t, int row) {
   int njp = macro_rows(d.blk_info[8 * b + 1]);
-  return (long)NMP * ((long)d.mrec_off[b] + (long)(t + d.mpad) * njp) + row;
+  return (long)Planes<T>::N * ((long)d.mrec_off[b] + (long)(t + d.mpad) * njp) + row;
 }
-__device__ __forceinline__ long macro_at_cell(const Dev &d, int c, int &njp) {
+template <typename T> __device__ __forceinline__ long macro_at_cell(const Dev &d, int c, int &njp) {
   int b = d.cell_block[c];
   int ni = d.blk_info[8 * b], loc = c - d.cell_off[b];
   int j = loc / ni, i = loc - j * ni;
   njp = macro_rows(d.blk_info[8 * b + 1]);
-  return macro_at(d, b, i + j, j);
+  return macro_at<T>(d, b, i + j, j);
 }
 
-// every record a cell at rest without couplings (once per mesh: the padding
-// keeps it)
+// every record a cell at rest that keeps a zero increment (once per mesh: the
+// padding keeps it)
 template <typename T> __global__ void k_macro_pad(Dev d, int b) {
+  constexpr int N = Planes<T>::N;
   int njp = macro_rows(d.blk_info[8 * b + 1]), nd = d.blk_info[8 * b] + d.blk_info[8 * b + 1] - 1 + 2 * d.mpad;
-  MV4<T> *rec = reinterpret_cast<MV4<T> *>(d.mrec) + (long)NMP * d.mrec_off[b];
-  for (long q = (long)blockIdx.x * blockDim.x + threadIdx.x; q < (long)nd * NMP * njp; q += (long)gridDim.x * blockDim.x) {
-    int plane = (int)(q / njp % NMP);
-    T one = plane == MP_ST ? T(1) : T(0);
+  MV4<T> *rec = reinterpret_cast<MV4<T> *>(d.mrec) + (long)N * d.mrec_off[b];
+  for (long q = (long)blockIdx.x * blockDim.x + threadIdx.x; q < (long)nd * N * njp; q += (long)gridDim.x * blockDim.x) {
+    int plane = (int)(q / njp % N);
+    bool state = sizeof(T) == 8 ? plane == MP_ST : plane == MP_FW || plane == MP_FW + 2 || plane == MP_BW || plane == MP_BW + 2;
+    T one = state ? T(1) : T(0);
     rec[q] = MV4<T>{{one, T(0), T(0), one}};
   }
 }
 
-// Gather the records of every cell (parallel): R, 1/diag, the state and the
-// couplings to the solved neighbours.
-template <typename T> __global__ void k_macro_prep(Dev d) {
+// Gather the records of every cell (parallel), FP64: R, 1/diag, the state and
+// the couplings to the solved neighbours.
+__global__ void k_macro_prep64(Dev d) {
   int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= d.nc) return;
+  typedef double T;
   int njp;
-  MV4<T> *o = reinterpret_cast<MV4<T> *>(d.mrec) + macro_at_cell(d, c, njp);
+  MV4<T> *o = reinterpret_cast<MV4<T> *>(d.mrec) + macro_at_cell<T>(d, c, njp);
   int mask = d.cmask[c];
   const bool on = mask & 1;
   double r[4] = {0, 0, 0, 0}, st[4] = {1, 0, 0, 1}, idg = 0.0;
@@ -131,9 +144,7 @@ template <typename T> __global__ void k_macro_prep(Dev d) {
     }
     idg = 1.0 / diag;
   }
-  auto put = [&](int plane, double a, double b, double e, double g) {
-    o[(long)plane * njp] = MV4<T>{{(T)a, (T)b, (T)e, (T)g}};
-  };
+  auto put = [&](int plane, double a, double b, double e, double g) { o[(long)plane * njp] = MV4<T>{{a, b, e, g}}; };
   put(MP_VAL, r[0], r[1], r[2], r[3]);
   put(MP_ST, st[0], st[1], st[2], st[3]);
   put(MP_F1, idg, cp[1][0], cp[1][1], cp[1][2]);
@@ -142,12 +153,211 @@ template <typename T> __global__ void k_macro_prep(Dev d) {
   put(MP_B2, cp[2][0], cp[2][1], cp[2][2], 0.0);
 }
 
-__device__ __forceinline__ double m_rcp(double x) { return 1.0 / x; }
-__device__ __forceinline__ float m_rcp(float x) { return __fdividef(1.0f, x); }   // 2 ulp
+// The same, FP32: R, 1/diag and per face slot the neighbour's state and the
+// face.  A cell that is not solved gets 1/diag = 0 and keeps a zero increment.
+__global__ void k_macro_prep32(Dev d) {
+  int c = blockIdx.x * blockDim.x + threadIdx.x;
+  if (c >= d.nc) return;
+  int njp;
+  MV4<float> *o = reinterpret_cast<MV4<float> *>(d.mrec) + macro_at_cell<float>(d, c, njp);
+  auto put = [&](int plane, float a, float b, float e, float g) { o[(long)plane * njp] = MV4<float>{{a, b, e, g}}; };
+  int mask = d.cmask[c];
+  if (!(mask & 1)) {
+    put(MP_VAL, 0.f, 0.f, 0.f, 0.f);
+    put(MP_FW + 4, 0.f, 0.f, 0.f, 0.f);
+    put(MP_BW + 4, 0.f, 0.f, 0.f, 0.f);
+    return;
+  }
+  double vol = d.vol_new[c], idt = 1.0 / d.stepc[0];
+  float r[4];
+  for (int m = 0; m < 4; ++m) r[m] = (float)(d.TW[4 * c + m] - vol * idt * d.W[4 * c + m] - 0.5 * d.Fc[4 * c + m]);
+  put(MP_VAL, r[0], r[1], r[2], r[3]);
+  double diag = vol * (d.cfl_s / (d.cfl_pseudo * d.dts[c]) + idt);
+  float gam[4];
+#pragma unroll
+  for (int s = 0; s < 4; ++s) {
+    int f = d.cell_faces[4 * c + s];
+    diag += 0.25 * d.S[f] * d.gam[f];
+    double sg = (double)d.cell_sgn[4 * c + s];
+    int nb = (sg > 0) ? d.face_R[f] : d.face_L[f];
+    // missing neighbour: a harmless positive state (its increment is zero)
+    float w[4];
+    for (int m = 0; m < 4; ++m) w[m] = nb >= 0 ? (float)d.W[4 * nb + m] : (m == 0 || m == 3 ? 1.f : 0.f);
+    const int plane = (s & 1 ? MP_BW : MP_FW) + (s & 2);
+    put(plane, w[0], w[1], w[2], w[3]);
+    put(plane + 1, (float)(sg * d.nrm[2 * f]), (float)(sg * d.nrm[2 * f + 1]), (float)(sg * d.SUn[f] / d.S[f]),
+        (float)(0.25 * d.S[f]));
+    gam[s] = (float)d.gam[f];
+  }
+  float idg = (float)(1.0 / diag);
+  put(MP_FW + 4, gam[0], gam[2], idg, 0.f);
+  put(MP_BW + 4, gam[1], gam[3], idg, 0.f);
+}
 
-// One pass (0 forward, 1 backward) over block b for this warp's band.
-template <typename T, int LPR, int K, int D, int PASS>
-__device__ __forceinline__ void macro_pass(const Dev &d, int b, int ni, int nj, bool per, int nb, MV4<T> *ring, T *links) {
+// Coupling (1/4 S)(Delta F_E . n - Gamma dW) of a neighbour with state w,
+// outward normal, U.n and S/4 in e, and increment dw, the flux variation
+// written out as a difference (one division, no cancellation between the two
+// fluxes): with d(a b / rho) = (da b rho + a db rho + da db rho - a b drho) /
+// (rho (rho + drho)) and p = (gamma - 1)(E - |m|^2 / (2 rho)).
+__device__ __forceinline__ void macro_off(const float *w, const float *e, float gam, const float *dw, int Keff, float out[4]) {
+  float r = w[0], m1 = w[1], m2 = w[2], E = w[3];
+  float nx = e[0], ny = e[1], un = e[2];
+  float dr = dw[0], d1 = dw[1], d2 = dw[2], dE = dw[3];
+  float g1 = __fdividef(2.0f, 2.0f + (float)Keff);    // gamma - 1
+  float mn = m1 * nx + m2 * ny, dmn = d1 * nx + d2 * ny;
+  float den = __fdividef(1.0f, r * (r + dr));          // 1/(rho (rho + drho))
+  float dq11 = (2.0f * (m1 * d1 + m2 * d2) * r + (d1 * d1 + d2 * d2) * r -
+                (m1 * m1 + m2 * m2) * dr) * den;
+  float dp = g1 * (dE - 0.5f * dq11);
+  float p = g1 * (E - 0.5f * (m1 * m1 + m2 * m2) * ((r + dr) * den));
+  float dv = (dmn * r - mn * dr) * den;               // d(mn / rho)
+  float dF0 = dmn - dr * un;
+  float dF1 = (d1 * mn * r + m1 * dmn * r + d1 * dmn * r - m1 * mn * dr) * den - d1 * un + dp * nx;
+  float dF2 = (d2 * mn * r + m2 * dmn * r + d2 * dmn * r - m2 * mn * dr) * den - d2 * un + dp * ny;
+  float dF3 = (dE * mn * r + E * dmn * r + dE * dmn * r - E * mn * dr) * den - dE * un +
+              dp * (mn + dmn) * (r * den) + p * dv;
+  float q = e[3], g = gam;
+  out[0] = q * (dF0 - g * dr);
+  out[1] = q * (dF1 - g * d1);
+  out[2] = q * (dF2 - g * d2);
+  out[3] = q * (dF3 - g * dE);
+}
+
+// The bands' copies of a diagonal: NPL planes of a band's RPB rows as 16-byte
+// chunks over the lanes, from a ring of D diagonals.
+template <typename T, int NPL, int RPB> struct MacroRing {
+  typedef MV4<T> V;
+  static constexpr int CPV = (int)sizeof(V) / 16, CPP = RPB * CPV, NCH = NPL * CPP / 32;
+  static_assert(NPL * CPP % 32 == 0, "whole copies per lane");
+  const char *src[NCH];
+  V *rg;
+  long step;             // bytes to the next diagonal
+  // planes: VAL, then NPL - 1 planes given by plane(1), plane(2), ...
+  template <typename F> __device__ __forceinline__ void init(const V *first, long njp, long stride, V *ring, int lane, F plane) {
+#pragma unroll
+    for (int m = 0; m < NCH; ++m) {
+      const int q = lane + 32 * m, pl = q / CPP;
+      src[m] = reinterpret_cast<const char *>(first + (long)(pl == 0 ? 0 : plane(pl)) * njp) + 16 * (q - pl * CPP);
+    }
+    rg = ring;
+    step = stride * (long)sizeof(V);
+  }
+  __device__ __forceinline__ void copy(int slot, int lane) {
+    char *dst = reinterpret_cast<char *>(rg + slot * NPL * RPB) + 16 * lane;
+#pragma unroll
+    for (int m = 0; m < NCH; ++m) {
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem_addr(dst + 512 * m)), "l"(src[m]) : "memory");
+      src[m] += step;
+    }
+    cp_async_commit();
+  }
+  __device__ __forceinline__ const V *slot(int s, int row) const { return rg + s * NPL * RPB + row; }
+};
+
+// One pass (0 forward, 1 backward) over block b for this warp's band, FP32.
+template <int K, int D, int PASS>
+__device__ __forceinline__ void macro_pass32(const Dev &d, int b, int ni, int nj, bool per, int nb, MV4<float> *ring,
+                                             float4 *links) {
+  constexpr unsigned FULL = 0xffffffffu;
+  constexpr int NPL = 1 + NPASS32, P0 = PASS == 0 ? MP_FW : MP_BW, Q0 = PASS == 0 ? MP_BW : MP_FW;
+  static_assert(K % 2 == 0 && D >= 3, "register pair by step parity; a copy, a read and a free slot");
+  typedef MV4<float> V;
+  struct Rec { V v, wi, ei, wj, ej, c; };
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, row = w * 32 + lane;
+  const int njp = macro_rows(nj), nd = ni + nj - 1;
+  const int lead = PASS == 0 ? w : nb - 1 - w;         // position of the band in the sweep order
+  const int total = (nd + (nb - 1) * (K - 1) + K - 1) / K * K;
+  const int t0 = PASS == 0 ? -lead * (K - 1) : nd - 1 + lead * (K - 1);
+  const long stride = (PASS == 0 ? 1 : -1) * (long)NMP32 * njp;          // to the next diagonal (vectors)
+  V *rec0 = reinterpret_cast<V *>(d.mrec);
+  V *ps = rec0 + macro_at<float>(d, b, t0, row);                         // this step's cell, plane 0
+  MacroRing<float, NPL, 32> R;
+  R.init(rec0 + macro_at<float>(d, b, t0, w * 32), njp, stride, ring + (size_t)w * D * NPL * 32, lane,
+         [](int pl) { return P0 + pl - 1; });
+  auto read = [&](int slot, Rec &r) {                                    // a lane reads what it copied itself
+    const V *s = R.slot(slot, lane);
+    r.v = s[0]; r.wi = s[32]; r.ei = s[64]; r.wj = s[96]; r.ej = s[128]; r.c = s[160];
+  };
+#pragma unroll
+  for (int u = 0; u < D - 1; ++u) R.copy(u, lane);
+  // the wrap of a periodic row: its last cell of the pass is coupled to its
+  // first, across the slot the other pass's record holds
+  const int ifirst = PASS == 0 ? 0 : ni - 1, ilast = PASS == 0 ? ni - 1 : 0;
+  V ww = {{1.f, 0.f, 0.f, 1.f}}, we = {{0.f, 0.f, 0.f, 0.f}};
+  float wg = 0.f, first[4] = {0.f, 0.f, 0.f, 0.f};
+  if (per && row < nj) {
+    const V *x = rec0 + macro_at<float>(d, b, ilast + row, row);
+    ww = x[(long)Q0 * njp];
+    we = x[(long)(Q0 + 1) * njp];
+    wg = x[(long)(Q0 + 4) * njp].v[0];
+  }
+  float4 *rin = links + (size_t)lead * 2 * K, *rout = rin + 2 * K;       // link 0 stays zero
+  if (lane < 2 * K) {
+    rout[lane] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (lead == 0) rin[lane] = make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  float val[4] = {0.f, 0.f, 0.f, 0.f};
+  const bool efirst = PASS == 0 ? lane == 0 : lane == 31, elast = PASS == 0 ? lane == 31 : lane == 0;
+  int i = t0 - row, sc = D - 1, sr = 1;                // ring slots: next copy, next read
+  Rec rec[2];
+  cp_async_wait<D - 2>();
+  read(0, rec[0]);
+  for (int c = 0; c < total; c += K) {
+    // the link half written before this barrier is read after it, and the
+    // half read before it is written after it
+    asm volatile("bar.sync 1, %0;" ::"r"(32 * nb) : "memory");
+    const int hw = (c / K & 1) * K, hr = K - hw;
+#pragma unroll 2
+    for (int u = 0; u < K; ++u) {                      // (all eight would overrun the instruction cache)
+      const Rec &r = rec[u & 1];
+      R.copy(sc, lane);                                // into the slot read the step before last
+      sc = sc + 1 == D ? 0 : sc + 1;
+      cp_async_wait<D - 2>();
+      read(sr, rec[(u & 1) ^ 1]);
+      sr = sr + 1 == D ? 0 : sr + 1;
+      // increments of the neighbours: along the row this lane's last one,
+      // across rows the neighbour lane's or the band before's
+      float up[4], oi[4], oj[4], acc[4];
+      const float4 lk = rin[hr + u];
+#pragma unroll
+      for (int m = 0; m < 4; ++m) up[m] = PASS == 0 ? __shfl_up_sync(FULL, val[m], 1) : __shfl_down_sync(FULL, val[m], 1);
+      if (efirst) { up[0] = lk.x; up[1] = lk.y; up[2] = lk.z; up[3] = lk.w; }
+      macro_off(r.wi.v, r.ei.v, r.c.v[0], val, d.Keff, oi);
+      macro_off(r.wj.v, r.ej.v, r.c.v[1], up, d.Keff, oj);
+      if (per && i == ilast) {
+        float ow[4];
+        macro_off(ww.v, we.v, wg, first, d.Keff, ow);
+#pragma unroll
+        for (int m = 0; m < 4; ++m) oi[m] = __fadd_rn(oi[m], ow[m]);
+      }
+#pragma unroll
+      for (int m = 0; m < 4; ++m) acc[m] = __fadd_rn(oi[m], oj[m]);
+      const float idg = r.c.v[2];
+      const bool on = idg != 0.f;                      // a solved cell; the others keep a zero increment
+      V x;
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        x.v[m] = PASS == 0 ? (r.v.v[m] - acc[m]) * idg : r.v.v[m] - acc[m] * idg;
+        val[m] = on ? x.v[m] : 0.f;
+      }
+      if (on) ps[0] = x;
+      if (per && i == ifirst) {
+#pragma unroll
+        for (int m = 0; m < 4; ++m) first[m] = val[m];
+      }
+      if (elast) rout[hw + u] = make_float4(val[0], val[1], val[2], val[3]);
+      ps += stride;
+      i += PASS == 0 ? 1 : -1;
+    }
+  }
+  cp_async_wait<0>();
+}
+
+// One pass over block b for this warp's band, FP64.
+template <int LPR, int K, int D, int PASS>
+__device__ __forceinline__ void macro_pass64(const Dev &d, int b, int ni, int nj, bool per, int nb, MV4<double> *ring,
+                                             double *links) {
+  typedef double T;
   constexpr int RPB = 32 / LPR, NC = 4 / LPR;          // rows a band, components a lane
   constexpr unsigned FULL = 0xffffffffu;
   static_assert(K % 2 == 0 && D >= 3, "register pair by step parity; a copy, a read and a free slot");
@@ -159,32 +369,15 @@ __device__ __forceinline__ void macro_pass(const Dev &d, int b, int ni, int nj, 
   const int lead = PASS == 0 ? w : nb - 1 - w;         // position of the band in the sweep order
   const int total = (nd + (nb - 1) * (K - 1) + K - 1) / K * K;
   const int t0 = PASS == 0 ? -lead * (K - 1) : nd - 1 + lead * (K - 1);
-  const long stride = (PASS == 0 ? 1 : -1) * (long)NMP * njp;      // to the next diagonal (vectors)
-  V *ps = reinterpret_cast<V *>(d.mrec) + macro_at(d, b, t0, row); // this step's cell, plane 0
-  // the band's copies of a diagonal: planes VAL, ST and this pass's two, RPB
-  // vectors each, as 16-byte chunks over the lanes
+  const long stride = (PASS == 0 ? 1 : -1) * (long)NMP64 * njp;       // to the next diagonal (vectors)
+  V *rec0 = reinterpret_cast<V *>(d.mrec);
+  V *ps = rec0 + macro_at<T>(d, b, t0, row);                          // this step's cell, plane 0
   constexpr int P1 = PASS == 0 ? MP_F1 : MP_B1, P2 = PASS == 0 ? MP_F2 : MP_B2;
-  constexpr int CPV = (int)sizeof(V) / 16, CPP = RPB * CPV, NCH = 4 * CPP / 32;
-  static_assert(CPP * 4 % 32 == 0, "whole copies per lane");
-  const char *src[NCH];
-#pragma unroll
-  for (int m = 0; m < NCH; ++m) {
-    const int q = lane + 32 * m, pl = q / CPP, plane = pl == 0 ? MP_VAL : pl == 1 ? MP_ST : pl == 2 ? P1 : P2;
-    src[m] = reinterpret_cast<const char *>(reinterpret_cast<const V *>(d.mrec) + macro_at(d, b, t0, w * RPB) +
-                                            (long)plane * njp) + 16 * (q - pl * CPP);
-  }
-  V *rg = ring + (size_t)w * D * 4 * RPB;
-  auto copy = [&](int slot) {
-    char *dst = reinterpret_cast<char *>(rg + slot * 4 * RPB) + 16 * lane;
-#pragma unroll
-    for (int m = 0; m < NCH; ++m) {
-      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem_addr(dst + 512 * m)), "l"(src[m]) : "memory");
-      src[m] += stride * (long)sizeof(V);
-    }
-    cp_async_commit();
-  };
+  MacroRing<T, 4, RPB> R;                              // planes VAL, ST and this pass's two
+  R.init(rec0 + macro_at<T>(d, b, t0, w * RPB), njp, stride, ring + (size_t)w * D * 4 * RPB, lane,
+         [](int pl) { return pl == 1 ? MP_ST : pl == 2 ? P1 : P2; });
   auto read = [&](int slot, Rec &r) {
-    const V *s = rg + slot * 4 * RPB + lr;
+    const V *s = R.slot(slot, lr);
 #pragma unroll
     for (int m = 0; m < NC; ++m) r.v[m] = s[0].v[LPR == 1 ? m : sub];
     r.st = s[RPB];
@@ -192,13 +385,13 @@ __device__ __forceinline__ void macro_pass(const Dev &d, int b, int ni, int nj, 
     r.c2 = s[3 * RPB];
   };
 #pragma unroll
-  for (int u = 0; u < D - 1; ++u) copy(u);
+  for (int u = 0; u < D - 1; ++u) R.copy(u, lane);
   // couplings that wrap around a periodic row: from its first cell of the
   // pass to its last, with the coefficients of the other pass's record
   T wrap[NC], wc[3] = {T(0), T(0), T(0)};
   const int ifirst = PASS == 0 ? 0 : ni - 1, ilast = PASS == 0 ? ni - 1 : 0;
   if (per && row < nj) {
-    const V x = (reinterpret_cast<const V *>(d.mrec) + macro_at(d, b, ifirst + row, row))[(long)(PASS == 0 ? MP_B1 : MP_F1) * njp];
+    const V x = (rec0 + macro_at<T>(d, b, ifirst + row, row))[(long)(PASS == 0 ? MP_B1 : MP_F1) * njp];
     for (int m = 0; m < 3; ++m) wc[m] = x.v[1 + m];
   }
   T *rin = links + (size_t)lead * 2 * K * 4, *rout = rin + 2 * K * 4;     // link 0 stays zero
@@ -227,10 +420,10 @@ __device__ __forceinline__ void macro_pass(const Dev &d, int b, int ni, int nj, 
 #pragma unroll
     for (int u = 0; u < K; ++u) {
       const Rec &r = rec[u & 1];
-      copy(sc);                                        // into the slot read the step before last
+      R.copy(sc, lane);                                // into the slot read the step before last
       sc = sc + 1 == D ? 0 : sc + 1;
       cp_async_wait<D - 2>();
-      if (CPV * LPR > 1) __syncwarp();                 // (else a lane reads what it copied itself)
+      __syncwarp();                                    // the band's copies, made by all its lanes
       read(sr, rec[(u & 1) ^ 1]);
       sr = sr + 1 == D ? 0 : sr + 1;
       T in[NC], val[NC], dw[4];
@@ -267,7 +460,7 @@ __device__ __forceinline__ void macro_pass(const Dev &d, int b, int ni, int nj, 
       // in the increments (no difference of two fluxes)
       const T rho = r.st.v[0], vx = r.st.v[1], vy = r.st.v[2], p = r.st.v[3];
       const T hh = ig1 * p + T(0.5) * rho * (vx * vx + vy * vy);      // rho E + p
-      const T ri = m_rcp(rho + dw[0]);
+      const T ri = 1.0 / (rho + dw[0]);
       const T du = (dw[1] - vx * dw[0]) * ri, dv = (dw[2] - vy * dw[0]) * ri;
       const T m1 = rho * vx + dw[1], m2 = rho * vy + dw[2];
       const T dk = dw[1] * vx + dw[2] * vy + m1 * du + m2 * dv;       // variation of rho |V|^2
@@ -298,25 +491,32 @@ __device__ __forceinline__ void macro_pass(const Dev &d, int b, int ni, int nj, 
   cp_async_wait<0>();
 }
 
-template <typename T, int LPR, int K, int D> __host__ __device__ constexpr size_t macro_ring(int nb) {
-  return (size_t)nb * D * 4 * (32 / LPR) * sizeof(MV4<T>);
+// shared memory: the bands' rings, then the links [nb + 1][2 K][4]
+template <typename T, int LPR, int D> __host__ __device__ constexpr size_t macro_ring(int nb) {
+  return (size_t)nb * D * (sizeof(T) == 4 ? 1 + NPASS32 : 4) * (32 / LPR) * sizeof(MV4<T>);
 }
 
-template <typename T, int LPR, int K, int D> __global__ void __launch_bounds__(512) k_macro_sweep(Dev d) {
+template <typename T, int LPR, int K, int D>
+__global__ void __launch_bounds__(sizeof(T) == 4 && D == 8 ? 256 : 512) k_macro_sweep(Dev d) {
   extern __shared__ __align__(16) unsigned char smraw[];
   const int b = blockIdx.x;
   const int *bi = d.blk_info + 8 * b;
   const int ni = bi[0], nj = bi[1], nb = (nj + 32 / LPR - 1) / (32 / LPR);
   const bool per = bi[2] != 0;
-  MV4<T> *ring = reinterpret_cast<MV4<T> *>(smraw);                              // [nb][D][4][RPB]
-  T *links = reinterpret_cast<T *>(smraw + macro_ring<T, LPR, K, D>(nb));        // [nb + 1][2 K][4]
+  MV4<T> *ring = reinterpret_cast<MV4<T> *>(smraw);
+  unsigned char *links = smraw + macro_ring<T, LPR, D>(nb);
   if ((int)(threadIdx.x >> 5) >= nb) return;           // the named barrier counts the block's bands
-  macro_pass<T, LPR, K, D, 0>(d, b, ni, nj, per, nb, ring, links);
+  auto pass = [&](auto which) {
+    constexpr int PASS = decltype(which)::value;
+    if constexpr (sizeof(T) == 4) macro_pass32<K, D, PASS>(d, b, ni, nj, per, nb, ring, reinterpret_cast<float4 *>(links));
+    else macro_pass64<LPR, K, D, PASS>(d, b, ni, nj, per, nb, ring, reinterpret_cast<double *>(links));
+  };
+  pass(std::integral_constant<int, 0>());
   // the increments stored above are copied by the same band's lanes in the
   // next pass; the links are free
   __threadfence();
   asm volatile("bar.sync 1, %0;" ::"r"(32 * nb) : "memory");
-  macro_pass<T, LPR, K, D, 1>(d, b, ni, nj, per, nb, ring, links);
+  pass(std::integral_constant<int, 1>());
 }
 
 // W' = W + dW and the predictor cell record (Step 4 result) for Step 5.
@@ -331,7 +531,7 @@ template <typename T> __global__ void k_macro_post(Dev d) {
     return;
   }
   int njp;
-  const MV4<T> inc = reinterpret_cast<const MV4<T> *>(d.mrec)[macro_at_cell(d, c, njp)];
+  const MV4<T> inc = reinterpret_cast<const MV4<T> *>(d.mrec)[macro_at_cell<T>(d, c, njp)];
   for (int m = 0; m < 4; ++m) d.Wp[4 * c + m] = d.W[4 * c + m] + (double)inc.v[m];
   Prim p = primitive(d.Wp + 4 * c, d.Keff);
   double *o = d.cpar + NCP * c;
@@ -357,8 +557,8 @@ void launch_macro_pad(const Dev &d, cudaStream_t s, int fp32) {
 // the sweep kernel is the first work of the side stream: it then takes its
 // empty SMs before the flux kernel launched beside it fills the GPU.
 void launch_macro_prep(const Dev &d, cudaStream_t s, int fp32) {
-  if (fp32) k_macro_prep<float><<<nblk(d.nc, 128), 128, 0, s>>>(d);
-  else k_macro_prep<double><<<nblk(d.nc, 128), 128, 0, s>>>(d);
+  if (fp32) k_macro_prep32<<<nblk(d.nc, 128), 128, 0, s>>>(d);
+  else k_macro_prep64<<<nblk(d.nc, 128), 128, 0, s>>>(d);
 }
 
 // the whole shared memory of an SM: the sweep's SMs take no CTA of the
@@ -383,7 +583,7 @@ void launch_macro_sweep(const Dev &d, cudaStream_t s, int rows, int fp32) {
 }
 
 template <typename T, int LPR, int K, int D, int NB> static void macro_attr() {
-  static_assert(macro_ring<T, LPR, K, D>(NB) + (NB + 1) * 2 * K * 4 * sizeof(T) <= kMacroSmem, "ring and links fit");
+  static_assert(macro_ring<T, LPR, D>(NB) + (NB + 1) * 2 * K * 4 * sizeof(T) <= kMacroSmem, "ring and links fit");
   cudaFuncSetAttribute(k_macro_sweep<T, LPR, K, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMacroSmem);
 }
 void macro_setup() {
