@@ -55,7 +55,6 @@ struct ugks_ctx {
   int nwork_cap = 0;                  // work-list capacity (largest tuning candidate)
   int sweep_vpt = 2;                  // micro sweeps: velocities per lane
   int ns_fwd = 4, ns_bwd = 4;         // prefetch ring depths (steps) of the two sweeps
-  int face_tile = 0;                  // tile shape of the face kernels (face_tile_shape)
   ugks_exchange_fn xfn = nullptr;     // velocity sharding: the caller's exchange
   void *xuser = nullptr;
   bool debug_sync = false, debug_failed = false;   // UGKS_DEBUG_SYNC
@@ -122,6 +121,7 @@ struct Sizes {
   int iy0 = 0, nv_all = 0, nvp_all = 0;   // velocity shard: first row; the whole grid
   size_t nmrec = 0;     // macro-sweep records of all blocks
   int mpad = 0;         // their padding diagonals
+  int nsplit = 1;       // CTAs per tile of the face kernels
 };
 
 int validate(const ugks_params *p, int nb, const ugks_block_desc *b, Sizes &s, std::string &why) {
@@ -171,6 +171,8 @@ int validate(const ugks_params *p, int nb, const ugks_block_desc *b, Sizes &s, s
     s.ntiles += tile_count(B.ni, B.nj);
   }
   s.mpad = macro_pad(s.max_nj, p->precision != UGKS_FP64);
+  // (a velocity shard exchanges the finished sums: one CTA a tile)
+  s.nsplit = s.nv == s.nv_all ? face_splits(s.ntiles, s.nvx, s.nv, p->precision != UGKS_FP64) : 1;
   for (int i = 0; i < nb; ++i) s.nmrec += macro_cells(b[i].ni, b[i].nj, s.mpad);
   return UGKS_OK;
 }
@@ -303,7 +305,7 @@ size_t carve(char *base, const Sizes &s, int nb, int fp32, int fbf, int nwork, i
   d.Tn = c.take<char>(pair * (size_t)s.nc * s.nvp);
   d.dfs = c.take<char>(pair * (size_t)s.nc * s.nvp);
   d.Dbuf = c.take<char>(pair * (size_t)s.nc * s.nvp);
-  d.fval = c.take<char>(2 * pair * (size_t)s.nf * s.nvp);
+  d.fval = c.take<char>(2 * pair * face_values(s.ntiles, s.nvp));
   d.stepc = c.take<double>(4);
   d.mpart = c.take<double>((size_t)MET_NQ * MET_BLOCKS);
   d.mout = c.take<double>(MET_NQ);
@@ -316,6 +318,7 @@ size_t carve(char *base, const Sizes &s, int nb, int fp32, int fbf, int nwork, i
   d.gradW = c.take<double>(8 * (size_t)s.nc);
   d.ghostW = c.take<double>(4 * (size_t)s.nf);
   d.fsum = c.take<double>(NFS * (size_t)s.nf);
+  d.fpart = c.take<char>(s.nsplit > 1 ? 2 * tsz * NFS * (size_t)s.nf * s.nsplit : 0);
   d.fpar = c.take<double>(NFP * (size_t)s.nf);
   d.fparT = c.take<char>(tsz * NFP * (size_t)s.nf);
   d.fflux = c.take<double>(4 * (size_t)s.nf);
@@ -618,7 +621,7 @@ int flux_prep(ugks_ctx *ctx, int level_n, bool joined = false) {
   Dev &d = ctx->d;
   cudaStream_t s = ctx->st;
   if (!joined) { Prof p(ctx, UGKS_PROF_CELL); launch_ghost_gradW(d, s); }
-  { Prof p(ctx, UGKS_PROF_FACE_REDUCE); launch_face_reduce_tile(d, s, ctx->fp32, ctx->face_tile); }
+  { Prof p(ctx, UGKS_PROF_FACE_REDUCE); launch_face_reduce(d, s, ctx->fp32); }
   int r = shard_exchange(ctx, 0);
   if (r) return r;
   if (joined) CK(cudaStreamWaitEvent(s, ctx->ev_tail, 0));
@@ -734,7 +737,7 @@ int step_body(ugks_ctx *ctx, int n_inner) {
     if (met) launch_metrics(d, s, 0, fp);
     { Prof p(ctx, UGKS_PROF_MACRO_SWEEP, ctx->side); launch_macro_sweep(d, ctx->side, ctx->max_nj, fp); }
     CK(cudaEventRecord(ctx->ev_macro, ctx->side));
-    { Prof p(ctx, UGKS_PROF_RHS); launch_flux_tile(d, s, fp, ctx->face_tile); }              // Step 3
+    { Prof p(ctx, UGKS_PROF_RHS); launch_flux(d, s, fp); }              // Step 3
     if (ctx->split_residual && !ctx->in_batch) {
       // Step 5 without the predictor's collision term while the sweep runs
       { Prof p(ctx, UGKS_PROF_RESIDUAL); launch_residual(d, s, it == 0, fp, 1); }
@@ -778,7 +781,7 @@ int step_body(ugks_ctx *ctx, int n_inner) {
 // What the captured kernels depend on beyond device memory: the device
 // struct they take by value and the launch configuration.
 std::vector<unsigned char> graph_key(const ugks_ctx *c, int n_inner) {
-  int cfg[] = {n_inner, c->fresh_pending ? 1 : 0, c->face_tile, c->sweep_vpt, c->ns_fwd, c->ns_bwd, c->sweep_nw,
+  int cfg[] = {n_inner, c->fresh_pending ? 1 : 0, c->sweep_vpt, c->ns_fwd, c->ns_bwd, c->sweep_nw,
                c->sweep_ql, c->nwork, c->nsm, c->max_nj, c->fp32, c->metrics ? 1 : 0, c->split_tail ? 1 : 0,
                c->split_residual && !c->in_batch ? 1 : 0};
   // (the step size is read from device memory; the bin count belongs to the
@@ -982,11 +985,6 @@ int ugks_init_mesh(ugks_ctx *ctx, int nblocks, const ugks_block_desc *blocks, co
   ctx->sweep_vpt = sweep_vpt_for(&ctx->p);
   ctx->sweep_nw = sweep_nw_for(nblocks, blocks);
   ctx->sweep_ql = wsweep_ql(max_nj_of(nblocks, blocks));
-  ctx->face_tile = face_tile_default();
-  if (const char *e = getenv("UGKS_FACE_TILE")) {      // tuning by hand: index of face_tile_shape
-    int v = atoi(e);
-    if (v >= 0 && v < face_tile_count()) ctx->face_tile = v;
-  }
   if (const char *e = getenv("UGKS_SWEEP_NS")) {
     int n = atoi(e);
     if (n == 2 || n == 4 || n == 6) ctx->ns_fwd = ctx->ns_bwd = n;
@@ -1029,6 +1027,7 @@ int ugks_init_mesh(ugks_ctx *ctx, int nblocks, const ugks_block_desc *blocks, co
   ctx->launches += upload_step_size(ctx);
   d.wait_polls = kWaitPolls;
   d.mpad = s.mpad;
+  d.nsplit = s.nsplit;
   d.vbox[0] = ctx->p.vx_min; d.vbox[1] = ctx->p.vx_max; d.vbox[2] = ctx->p.vy_min; d.vbox[3] = ctx->p.vy_max;
   {
     double lam = 1.0 / (2.0 * ctx->p.farfield[3]);
@@ -1375,17 +1374,6 @@ int ugks_autotune(ugks_ctx *ctx, int reps, int *items_out, int *vpt_out, int *ri
     ctx->launches += reps + 1;
     return q;
   };
-  // face kernels: reduction + flux divergence for every tile shape (FP32)
-  int bt = ctx->face_tile;
-  if (fp) {
-    float best = 1e30f;
-    for (int v = 0; v < face_tile_count() && !r; ++v) {
-      float m1, m2;
-      if ((r = timed([&] { launch_face_reduce_tile(d, s, fp, v); }, m1))) break;
-      if ((r = timed([&] { launch_flux_tile(d, s, fp, v); }, m2))) break;
-      if (m1 + m2 < best) { best = m1 + m2; bt = v; }
-    }
-  }
   // micro sweeps: velocities per lane, and per sweep the ring depth
   float best = 1e30f;
   int bv = ctx->sweep_vpt, bf = ctx->ns_fwd, bb = ctx->ns_bwd;
@@ -1413,10 +1401,8 @@ int ugks_autotune(ugks_ctx *ctx, int reps, int *items_out, int *vpt_out, int *ri
   if ((r = set_sweep_tiles(ctx, bv))) return r;
   ctx->ns_fwd = bf;
   ctx->ns_bwd = bb;
-  ctx->face_tile = bt;
   int vk, nh;
-  face_tile_shape(fp ? bt : -1, &vk, &nh);
-  if (!fp) { vk = 8; nh = 2; }
+  face_tile_shape(fp, &vk, &nh);
   if (items_out) *items_out = 32 * bv;
   if (vpt_out) *vpt_out = bv;
   if (ring_fwd_out) *ring_fwd_out = bf;

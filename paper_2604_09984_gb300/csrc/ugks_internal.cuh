@@ -101,6 +101,8 @@ struct Dev {
   double *gradW;             // nc*8
   double *ghostW;            // nf*4
   double *fsum;              // nf*NFS
+  void *fpart;               // nsplit*NFS*nf (sum, error) pairs of the face reduction's CTAs (nsplit > 1)
+  int nsplit;                // CTAs that share a tile's velocity chunks in the face kernels
   double *fpar;              // nf*NFP (double)
   void *fparT;               // nf*NFP in the arithmetic type
   double *fflux;             // nf*4 S * macro flux (L -> R / outward)
@@ -167,6 +169,42 @@ enum { SR_DBASE = 12, SR_MASK = 13, NSR = 16 };
 // per-cell parameter record (from W' or W^n)
 enum { CP_RHO = 0, CP_UX, CP_UY, CP_LAM, CP_QX, CP_QY, CP_ITAU, CP_DBASE, NCP = 8 };
 
+// float -> double on the integer pipes, from the IEEE 754 layouts (sign;
+// exponent rebiased by 1023 - 127; 23-bit fraction shifted into the 52-bit
+// one): exact for normal numbers, zero and subnormals give signed zero,
+// infinities and NaNs are kept.  The FP64 pipe of this GPU retires a warp
+// instruction in tens of cycles, so per-face and per-cell conversions go
+// through here.
+__device__ __forceinline__ double f2d_bits(float x) {
+  unsigned u = __float_as_uint(x);
+  unsigned sign = u & 0x80000000u, e = (u >> 23) & 0xffu, m = u & 0x7fffffu;
+  unsigned hi, lo;
+  if (e == 0u) { hi = sign; lo = 0u; }
+  else if (e == 0xffu) { hi = sign | 0x7ff00000u | (m >> 3); lo = (m & 7u) << 29; }
+  else { hi = sign | ((e + 896u) << 20) | (m >> 3); lo = (m & 7u) << 29; }
+  return __hiloint2double((int)hi, (int)lo);
+}
+__device__ __forceinline__ double to_double(double x) { return x; }
+__device__ __forceinline__ double to_double(float x) { return f2d_bits(x); }
+
+// error-free sum (Knuth): s + e = a + b exactly
+__device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
+  s = a + b;
+  float bb = s - a;
+  e = (a - (s - bb)) + (b - bb);
+}
+// Face sums of the velocity reduction, (sum, error) pairs on the FP32 path:
+// (h, l) += (h2, l2), and the finished value.
+__device__ __forceinline__ void face_sum_add(float &h, float &l, float h2, float l2) {
+  float s, e;
+  two_sum(h, h2, s, e);
+  h = s;
+  l = (l + e) + l2;
+}
+__device__ __forceinline__ void face_sum_add(double &h, double &, double h2, double) { h += h2; }
+__device__ __forceinline__ double face_sum_value(float h, float l) { return to_double(h) + to_double(l); }
+__device__ __forceinline__ double face_sum_value(double h, double) { return h; }
+
 // Shakhov record in the arithmetic type from a cell record (double)
 template <typename T>
 __device__ __forceinline__ void write_shrec(const Dev &d, const double *o, double vol, T *r) {
@@ -225,24 +263,6 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int N> __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;\n" ::"n"(N));
 }
-
-// float -> double on the integer pipes, from the IEEE 754 layouts (sign;
-// exponent rebiased by 1023 - 127; 23-bit fraction shifted into the 52-bit
-// one): exact for normal numbers, zero and subnormals give signed zero,
-// infinities and NaNs are kept.  The FP64 pipe of this GPU retires a warp
-// instruction in tens of cycles, so per-face and per-cell conversions go
-// through here.
-__device__ __forceinline__ double f2d_bits(float x) {
-  unsigned u = __float_as_uint(x);
-  unsigned sign = u & 0x80000000u, e = (u >> 23) & 0xffu, m = u & 0x7fffffu;
-  unsigned hi, lo;
-  if (e == 0u) { hi = sign; lo = 0u; }
-  else if (e == 0xffu) { hi = sign | 0x7ff00000u | (m >> 3); lo = (m & 7u) << 29; }
-  else { hi = sign | ((e + 896u) << 20) | (m >> 3); lo = (m & 7u) << 29; }
-  return __hiloint2double((int)hi, (int)lo);
-}
-__device__ __forceinline__ double to_double(double x) { return x; }
-__device__ __forceinline__ double to_double(float x) { return f2d_bits(x); }
 
 // mbarrier and bulk (TMA engine) copies, shared::cta addresses
 __device__ __forceinline__ unsigned smem_addr(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }

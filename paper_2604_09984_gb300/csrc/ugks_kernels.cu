@@ -322,7 +322,18 @@ template <typename T> __global__ void k_face_scalar(Dev d) {
   double W0[4], gx[4], gy[4], q0x, q0y, dts;
   double ufx = d.Uf[2 * fid], ufy = d.Uf[2 * fid + 1];
   double nx = d.nrm[2 * fid], ny = d.nrm[2 * fid + 1];
-  const double *fs = d.fsum + NFS * fid;
+  double *fs = d.fsum + NFS * fid;
+  if (d.nsplit > 1) {          // the reduction's CTAs left their parts: added here in order
+    const T *p = reinterpret_cast<const T *>(d.fpart) + 2 * (size_t)fid;
+    for (int m = 0; m < NFS; ++m) {
+      T h = T(0), l = T(0);
+      for (int s = 0; s < d.nsplit; ++s) {
+        const T *q = p + 2 * ((size_t)s * NFS + m) * d.nf;
+        face_sum_add(h, l, q[0], q[1]);
+      }
+      fs[m] = face_sum_value(h, l);
+    }
+  }
   if (wall) {
     double dx = d.xf[2 * fid] - d.xc[2 * L], dy = d.xf[2 * fid + 1] - d.xc[2 * L + 1];
     for (int m = 0; m < 4; ++m) {

@@ -10,20 +10,19 @@
 //                  LU-SGS sweep runs on another stream;
 //   k_residual     the micro residual r from D (reading R4).
 //
-// One CTA per 8x8 cell tile of a block walks all velocity chunks of VK
-// velocities.  In the reduction, per chunk, f of the tile plus a two-cell
-// halo (ghost cells hold the Maxwellian of their ghost state) is staged in
-// shared memory with asynchronous copies, double-buffered so the next chunk
-// arrives while the current one is reconstructed.  A thread owns one face
-// slot of the tile and one half of every chunk's velocities: everything that
-// does not depend on the velocity -- the face geometry, which region cells
-// are its two sides, their slope cases and inverse Jacobians, and for the
-// flux the interface record of Eq. fullSolution -- is loaded once and kept
-// in registers for the whole velocity loop.  The reduction accumulates its
-// 12 face sums in registers across all chunks (per-chunk partial sums added
-// with an error-free transformation on the FP32 path) and writes them once,
-// with no atomics: the result does not depend on scheduling.  It also stores
-// the reconstruction of every (face, velocity), so the flux pass reads one
+// A CTA takes an 8x8 cell tile of a block and a share of the velocity chunks.
+// In the reduction, per chunk, f of the tile plus a two-cell halo (ghost cells
+// hold the Maxwellian of their ghost state) is staged in shared memory with
+// asynchronous copies, double-buffered so the next chunk arrives while the
+// current one is reconstructed.  A thread owns one face slot of the tile and
+// one half of every chunk's velocities: everything that does not depend on the
+// velocity -- the face geometry, which region cells are its two sides, and for
+// the flux the interface record of Eq. fullSolution -- is loaded once and kept
+// in registers for the whole velocity loop.  The reduction accumulates its 12
+// face sums in registers across all chunks (partial sums added with an
+// error-free transformation on the FP32 path) and writes them once, with no
+// atomics: the result does not depend on scheduling.  It also stores the
+// reconstruction of every (face, velocity), so the flux pass reads one
 // 4-vector per (face, velocity) instead of re-staging f and recomputing the
 // limited gradients.
 #include "ugks_internal.cuh"
@@ -33,21 +32,12 @@ namespace ugks {
 
 constexpr int TX = 8, TY = 8, RW = TX + 4, RH = TY + 4, NR = RW * RH;
 constexpr int NSI = (TX + 1) * TY;          // i-face slots: tile row w, column x = 0..TX
-constexpr int NSLOT = NSI + TX * (TY + 1);  // + j-face slots: tile column w, row y = 0..TY
-// Tile shape of the two face kernels (the autotuner's choice): VK velocities
-// per chunk, NH threads per face slot, NT threads a CTA.  The NH threads of a
-// slot are adjacent lanes and take interleaved velocities (kk = part + NH q),
-// so the NH of them store NH consecutive reconstructions -- whole 32-byte
-// sectors for NH = 2.  Row strides (in elements) of the staged region (VKP:
-// rows of whole 16-byte copies), of the gradient rows and face-flux rows
-// (VKG) and of the staged face reconstructions (VKF), chosen so that the
-// lanes of a quarter warp -- NH velocities of 8 / NH neighbouring cells or
-// faces -- fall in different banks.
-template <typename T, int VK_, int NH_> struct FCfg {
-  static constexpr int VK = VK_, NH = NH_, NT = NSLOT * NH_, VH = VK_ / NH_;
-  static constexpr int VKP = sizeof(T) == 4 ? VK_ + 2 : VK_, VKG = VK_ + 2, VKF = VK_ + 2;
-  static_assert(NT % VK == 0 && VK % NH == 0 && NH == 2, "tile shape");
-};
+constexpr int NSLOT = NSI + TX * (TY + 1);  // + j-face slots: row y = 0..TY, tile column w
+// Two threads a face slot, adjacent lanes, take interleaved velocities of a
+// chunk (kk = half + 2 q), so they store whole 32-byte sectors of
+// reconstructions.
+constexpr int NT = 2 * NSLOT;
+static_assert(NR == NSLOT, "two threads a region cell as well");
 
 // region cell (i, j) of block b -> cell id (>= 0), ghost (-2 - face id) or
 // none (-1).  Periodic blocks wrap in i.
@@ -100,215 +90,125 @@ template <typename T> struct Vec4;
 template <> struct Vec4<float> { typedef float4 type; };
 template <> struct Vec4<double> { typedef double4 type; };
 
-// Shared memory of both kernels: the double-buffered region of f, the limited
-// Cartesian gradients of the chunk, the velocity table of both buffered
-// chunks, and per region cell its id, slope cases and inverse Jacobian (the
-// ghost Maxwellian's parameters for ghost cells).
-template <typename T, typename C> struct FaceSmem {
-  typedef typename Vec2<T>::type T2;
-  typedef typename Vec4<T>::type T4;
-  static constexpr int VK = C::VK, VKP = C::VKP, VKG = C::VKG;
-  T2 *F;         // [2][NR][VKP]
-  T4 *G;         // [NG][VKG]: (d_x h, d_x b, d_y h, d_y b)
-  T4 *vt;        // [2][VK]: vx, vy, weight, |v|^2 / 2
-  T4 *J;         // [NR]: inverse Jacobian (real cells), ghost state rho lam / pi, Vx, Vy, lam (ghosts)
-  int *gid;      // [NR]
-  int *fl;       // [NR]: slope cases, 0 for ghost / missing cells
-  __host__ __device__ static constexpr size_t bytes() {
-    return sizeof(T2) * 2 * NR * VKP + sizeof(T4) * NG * VKG + sizeof(T4) * 2 * VK + sizeof(T4) * NR +
-           sizeof(int) * 2 * NR;
-  }
-  __device__ void carve(unsigned char *p) {
-    F = reinterpret_cast<T2 *>(p);
-    p += sizeof(T2) * 2 * NR * VKP;
-    G = reinterpret_cast<T4 *>(p);
-    p += sizeof(T4) * NG * VKG;
-    vt = reinterpret_cast<T4 *>(p);
-    p += sizeof(T4) * 2 * VK;
-    J = reinterpret_cast<T4 *>(p);
-    p += sizeof(T4) * NR;
-    gid = reinterpret_cast<int *>(p);
-    p += sizeof(int) * NR;
-    fl = reinterpret_cast<int *>(p);
-  }
+// Pairs (h, b) of the arithmetic type.  FP32 pairs sit in one 64-bit register
+// pair and take the packed FP32 instructions (add, multiply, fused
+// multiply-add on both halves, each rounded as the scalar one): the face
+// kernels are bound by instruction issue, and h and b go through the same
+// arithmetic almost everywhere.
+struct alignas(8) PairF { unsigned long long v; };
+struct alignas(16) PairD { double x, y; };
+template <typename T> struct PairOf;
+template <> struct PairOf<float> { typedef PairF type; };
+template <> struct PairOf<double> { typedef PairD type; };
+__device__ __forceinline__ PairF pr_make(float a, float b) {
+  PairF r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ PairD pr_make(double a, double b) { return PairD{a, b}; }
+__device__ __forceinline__ float2 pr_get(PairF a) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a.v));
+  return r;
+}
+__device__ __forceinline__ double2 pr_get(PairD a) { return double2{a.x, a.y}; }
+__device__ __forceinline__ PairF pr_add(PairF a, PairF b) {
+  PairF r;
+  asm("add.rn.ftz.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+__device__ __forceinline__ PairF pr_sub(PairF a, PairF b) {
+  PairF r;
+  asm("sub.rn.ftz.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+__device__ __forceinline__ PairF pr_mul(PairF a, PairF b) {
+  PairF r;
+  asm("mul.rn.ftz.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+__device__ __forceinline__ PairF pr_fma(PairF a, PairF b, PairF c) {
+  PairF r;
+  asm("fma.rn.ftz.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+  return r;
+}
+__device__ __forceinline__ PairD pr_add(PairD a, PairD b) { return PairD{a.x + b.x, a.y + b.y}; }
+__device__ __forceinline__ PairD pr_sub(PairD a, PairD b) { return PairD{a.x - b.x, a.y - b.y}; }
+__device__ __forceinline__ PairD pr_mul(PairD a, PairD b) { return PairD{a.x * b.x, a.y * b.y}; }
+__device__ __forceinline__ PairD pr_fma(PairD a, PairD b, PairD c) {
+  return PairD{fma(a.x, b.x, c.x), fma(a.y, b.y, c.y)};
+}
+template <typename T> __device__ __forceinline__ typename PairOf<T>::type pr_dup(T a) { return pr_make(a, a); }
+template <typename P> struct alignas(16) Quad { P x, y; };       // two pairs: (x.h, x.b, y.h, y.b)
+
+// a b + c d with one product rounded by itself (written out where results must
+// not depend on the compiler's choice)
+__device__ __forceinline__ float mul_add2(float a, float b, float c, float d) { return __fmaf_rn(a, b, __fmul_rn(c, d)); }
+// Half of the van Leer slopes 2 a b / (a + b) (0 where a b <= 0) of a pair of
+// differences, FP32 (the factor 2 goes into the inverse Jacobian: exact).
+__device__ __forceinline__ float rcp_approx(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ float2 pr_vanleer_half(PairF a, PairF b) {
+  const PairF p = pr_mul(a, b), s = pr_add(a, b);
+  const float2 pv = pr_get(p), sv = pr_get(s);
+  const float2 q = pr_get(pr_mul(p, pr_make(rcp_approx(sv.x), rcp_approx(sv.y))));
+  return make_float2(pv.x > 0.f ? q.x : 0.f, pv.y > 0.f ? q.y : 0.f);
+}
+// FP64: both quotients from one reciprocal, 1/s_x = s_y / (s_x s_y), the
+// hardware estimate refined by Newton's iteration r <- r + r (1 - x r)
+// (quadratic: 2^-20 -> 2^-40 -> 2^-80, i.e. to rounding); a double-precision
+// division costs a dozen instructions of a pipe that retires one in tens of
+// cycles.  A product below 2^-960 counts as no common sign (slopes below 1e-144).
+__device__ __forceinline__ PairD pr_vanleer(PairD a, PairD b) {
+  const double px = a.x * b.x, py = a.y * b.y;
+  const bool ox = __double2hiint(px) >= 0x03f00000, oy = __double2hiint(py) >= 0x03f00000;
+  const double sx = ox ? a.x + b.x : 1.0, sy = oy ? a.y + b.y : 1.0;
+  const double x = sx * sy;
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  r = fma(r, fma(-x, r, 1.0), r);
+  r = fma(r, fma(-x, r, 1.0), r);
+  return PairD{ox ? 2.0 * px * (r * sy) : 0.0, oy ? 2.0 * py * (r * sx) : 0.0};
+}
+
+// Chunks of the velocity loop: every row of the velocity grid (fixed v_y) is
+// cut into `per_row` chunks of `len` <= VK velocities (the last may be
+// shorter), so that within a chunk every velocity sum is a sum of moments in
+// v_x; rows of even length get even chunks (16-byte copies of FP32 pairs).
+struct Chunks { int per_row, len, total; };
+template <int VK> __host__ __device__ __forceinline__ Chunks face_chunks(int nvx, int nv) {
+  Chunks c;
+  c.per_row = (nvx + VK - 1) / VK;
+  c.len = (nvx + c.per_row - 1) / c.per_row;
+  if (nvx % 2 == 0) c.len = (c.len + 1) / 2 * 2;
+  c.per_row = (nvx + c.len - 1) / c.len;
+  c.total = nv / nvx * c.per_row;
+  return c;
+}
+
+// Shared memory of the FP64 reduction: the double-buffered region of f, the
+// limited Cartesian gradients of the chunk, the v_x table of both buffered
+// chunks (weights times powers of v_x), and per region cell its slope cases
+// and inverse Jacobian.
+constexpr int VK64 = 8, VKP64 = VK64, VKG64 = VK64 + 2;
+struct Smem64 {
+  struct alignas(16) Tab { double w[4], vx, pad; };
+  PairD F[2][NR][VKP64];
+  Quad<PairD> G[NG][VKG64];      // (d_x h, d_x b), (d_y h, d_y b)
+  Tab tab[2][VK64];
+  double4 J[NR];
+  int fl[NR];
 };
 
-// region ids, slope cases, inverse Jacobians and ghost states (once per CTA)
-template <typename T, typename C>
-__device__ __forceinline__ void region_meta(const Dev &d, FaceSmem<T, C> &S, const int *bi, int off, int i0, int j0) {
-  typedef typename Vec4<T>::type T4;
-  for (int r = threadIdx.x; r < NR; r += blockDim.x) {
-    int rx = r % RW, ry = r / RW;
-    int g = region_gid(d, bi, off, i0 - 2 + rx, j0 - 2 + ry);
-    S.gid[r] = g;
-    T4 J = {T(0), T(0), T(0), T(0)};
-    int fl = 0;
-    if (g >= 0) {
-      fl = d.slope_flags[g];
-      if (sizeof(T) == 4) {
-        float4 j = d.jinvf[g];
-        J.x = (T)j.x; J.y = (T)j.y; J.z = (T)j.z; J.w = (T)j.w;
-      } else {
-        J.x = (T)d.jinv[4 * g]; J.y = (T)d.jinv[4 * g + 1]; J.z = (T)d.jinv[4 * g + 2]; J.w = (T)d.jinv[4 * g + 3];
-      }
-    } else if (g <= -2) {
-      Prim p = primitive(d.ghostW + 4 * (-2 - g), d.Keff);
-      J.x = (T)(p.rho * p.lam * M_1_PI); J.y = (T)p.ux; J.z = (T)p.uy; J.w = (T)p.lam;
-    }
-    S.J[r] = J;
-    S.fl[r] = fl;
-  }
-}
-
-// Issue the copies of velocity chunk `ch` into buffer `buf`: real cells by
-// asynchronous 16-byte copies (bf16 storage: load and widen), ghost cells the
-// Maxwellian of their ghost state, no cell / padding velocities zero; and the
-// chunk's velocity table.  EP velocities per copy.
-template <typename T, int FB, typename C>
-__device__ __forceinline__ void stage_chunk(const Dev &d, FaceSmem<T, C> &S, int ch, int buf) {
-  typedef typename Vec2<T>::type T2;
-  typedef typename Vec4<T>::type T4;
-  constexpr int VK = C::VK, VKP = C::VKP, EP = 16 / (int)sizeof(T2), NP = VK / EP;
-  const int kb = ch * VK;
-  T2 *Fb = S.F + (size_t)buf * NR * VKP;
-  for (int it = threadIdx.x; it < NR * NP; it += blockDim.x) {
-    int r = it / NP, kp = it - (it / NP) * NP;
-    int kk = kp * EP, k = kb + kk;
-    int g = S.gid[r];
-    T2 *dst = Fb + r * VKP + kk;
-    if (k < d.nv && g >= 0) {
-      if (FB) {
-#pragma unroll
-        for (int e = 0; e < EP; ++e) {
-          auto v = ldF<T, 1>(d, (size_t)g * d.nvp + k + e);
-          dst[e] = T2{v.x, v.y};
-        }
-      } else {
-        // k < nv <= nvp, nvp a multiple of 4 and k even: the pair stays in
-        // the cell's row (padding velocities hold zero)
-        cp_async<16>(dst, reinterpret_cast<const T2 *>(d.f) + (size_t)g * d.nvp + k);
-      }
-      continue;
-    }
-#pragma unroll
-    for (int e = 0; e < EP; ++e) {
-      T2 v = {T(0), T(0)};
-      if (k + e < d.nv && g <= -2) {
-        T4 p = S.J[r];
-        V2<T> m = maxwellian_pre<T>(p.x, p.y, p.z, p.w, (T)d.Keff / (T(2) * p.w), dvx<T>(d, k + e), dvy<T>(d, k + e));
-        v.x = m.h;
-        v.y = m.b;
-      }
-      dst[e] = v;
-    }
-  }
-  for (int kk = threadIdx.x; kk < VK; kk += blockDim.x) {
-    int k = kb + kk;
-    T vx = k < d.nv ? dvx<T>(d, k) : T(0), vy = k < d.nv ? dvy<T>(d, k) : T(0);
-    T4 t = {vx, vy, k < d.nv ? dw<T>(d, k) : T(0), T(0.5) * (vx * vx + vy * vy)};
-    S.vt[buf * VK + kk] = t;
-  }
-  cp_async_commit();
-}
-
-// limited slope of one logical direction from the backward / forward
-// differences a, b (reading R1: van Leer where both neighbours exist,
-// one-sided where one does)
-template <typename T> __device__ __forceinline__ T lim_slope(T a, T b, bool hm, bool hp) {
-  T v = vanleer<T>(a, b);
-  return hm ? (hp ? v : a) : (hp ? b : T(0));
-}
-
-// Phase A of a chunk: the limited Cartesian gradient of (h, b) of every
-// gradient cell and chunk velocity (lanes run over velocities; ghost and
-// missing cells carry none).  A thread keeps one chunk velocity and walks
-// the gradient cells with a fixed stride; cells with all four neighbours take
-// the two-sided limiter without the one-sided selections.
-template <typename T, typename C>
-__device__ __forceinline__ void chunk_gradients(FaceSmem<T, C> &S, int buf) {
-  typedef typename Vec2<T>::type T2;
-  typedef typename Vec4<T>::type T4;
-  constexpr int VK = C::VK, VKP = C::VKP, VKG = C::VKG, GS = C::NT / VK;
-  const T2 *Fb = S.F + (size_t)buf * NR * VKP;
-  const int kk = threadIdx.x % VK;
-  for (int g = threadIdx.x / VK; g < NG; g += GS) {
-    int r = region_of_g(g);
-    int fl = S.fl[r];
-    T4 G = {T(0), T(0), T(0), T(0)};
-    if (fl) {
-      T4 J = S.J[r];
-      const T2 *c = Fb + r * VKP + kk;
-      T2 fc = c[0], im = c[-VKP], ip = c[VKP], jm = c[-RW * VKP], jp = c[RW * VKP];
-      T sih, sib, sjh, sjb;
-      if (fl == 15) {
-        sih = vanleer<T>(fc.x - im.x, ip.x - fc.x);
-        sib = vanleer<T>(fc.y - im.y, ip.y - fc.y);
-        sjh = vanleer<T>(fc.x - jm.x, jp.x - fc.x);
-        sjb = vanleer<T>(fc.y - jm.y, jp.y - fc.y);
-      } else {
-        bool him = fl & 1, hip = fl & 2, hjm = fl & 4, hjp = fl & 8;
-        sih = lim_slope<T>(fc.x - im.x, ip.x - fc.x, him, hip);
-        sib = lim_slope<T>(fc.y - im.y, ip.y - fc.y, him, hip);
-        sjh = lim_slope<T>(fc.x - jm.x, jp.x - fc.x, hjm, hjp);
-        sjb = lim_slope<T>(fc.y - jm.y, jp.y - fc.y, hjm, hjp);
-      }
-      G.x = J.x * sih + J.y * sjh;
-      G.y = J.x * sib + J.y * sjb;
-      G.z = J.z * sih + J.w * sjh;
-      G.w = J.z * sib + J.w * sjb;
-    }
-    S.G[g * VKG + kk] = G;
-  }
-}
-
-// One side of a face: its region cell, its gradient cell, and the vector
-// from its centre to the face centre.
-template <typename T> struct Side {
-  int r, g;
-  T dx, dy;
-};
-
-template <typename T> __device__ __forceinline__ Side<T> make_side(int r, T dx, T dy) {
-  Side<T> s;
-  s.r = r;
-  s.g = g_of_region(r);
-  s.dx = dx;
-  s.dy = dy;
-  return s;
-}
-
-// Reconstructed face value f + dx.grad f and w.grad f of side s at chunk
-// velocity kk.
-template <typename T, typename C>
-__device__ __forceinline__ void side_value(const FaceSmem<T, C> &S, const typename Vec2<T>::type *Fb, int r, int g,
-                                           T dx, T dy, int kk, T wx, T wy, V2<T> &ff, V2<T> &wg) {
-  constexpr int VKP = C::VKP, VKG = C::VKG;
-  auto fc = Fb[r * VKP + kk];
-  auto G = S.G[g * VKG + kk];
-  ff.h = fc.x + dx * G.x + dy * G.z;
-  ff.b = fc.y + dx * G.y + dy * G.w;
-  wg.h = wx * G.x + wy * G.z;
-  wg.b = wx * G.y + wy * G.w;
-}
-
-// Upwind face value and w.grad f (walls: the interior side L only); only
-// w.S = 0 exactly averages the two sides.
-template <typename T, typename C>
-__device__ __forceinline__ void upwind(const FaceSmem<T, C> &S, const typename Vec2<T>::type *Fb, const Side<T> &L,
-                                       const Side<T> &R, bool wall, int kk, T wS, T wx, T wy, V2<T> &ff,
-                                       V2<T> &wg) {
-  if (!wall && wS == T(0)) {
-    V2<T> f1, g1, f2, g2;
-    side_value<T, C>(S, Fb, L.r, L.g, L.dx, L.dy, kk, wx, wy, f1, g1);
-    side_value<T, C>(S, Fb, R.r, R.g, R.dx, R.dy, kk, wx, wy, f2, g2);
-    ff = {T(0.5) * (f1.h + f2.h), T(0.5) * (f1.b + f2.b)};
-    wg = {T(0.5) * (g1.h + g2.h), T(0.5) * (g1.b + g2.b)};
-    return;
-  }
-  bool useR = !wall && wS < T(0);
-  side_value<T, C>(S, Fb, useR ? R.r : L.r, useR ? R.g : L.g, useR ? R.dx : L.dx, useR ? R.dy : L.dy, kk, wx, wy,
-                   ff, wg);
-}
+template <typename T> __device__ __forceinline__ T grid_vx(const Dev &d, int ix);
+template <> __device__ __forceinline__ double grid_vx<double>(const Dev &d, int ix) { return d.vx1[ix]; }
+template <> __device__ __forceinline__ float grid_vx<float>(const Dev &d, int ix) { return d.vxf[ix]; }
+template <typename T> __device__ __forceinline__ T grid_vy(const Dev &d, int iy);      // iy of the whole grid
+template <> __device__ __forceinline__ double grid_vy<double>(const Dev &d, int iy) { return d.vy1[iy]; }
+template <> __device__ __forceinline__ float grid_vy<float>(const Dev &d, int iy) { return d.vy1f[iy]; }
 
 // Slot -> (direction, tile row / column w, position x) and the region cells
 // A (lower logical side) and B of the face.
@@ -322,173 +222,517 @@ __device__ __forceinline__ void slot_geom(int slot, int &dir, int &w, int &x, in
   } else {
     int s = slot - NSI;
     dir = 1;
-    w = s / (TY + 1);
-    x = s - w * (TY + 1);
+    x = s / TX;
+    w = s - x * TX;
     A = (w + 2) + (x + 1) * RW;
     B = A + RW;
   }
 }
 
-// The stored reconstruction of one (face, velocity): (f_face h, f_face b,
-// w.grad f h, w.grad f b).
-template <typename T>
-__device__ __forceinline__ void st_fval(typename Vec4<T>::type *p, const V2<T> &ff, const V2<T> &wg) {
-  typename Vec4<T>::type v;
-  v.x = ff.h; v.y = ff.b; v.z = wg.h; v.w = wg.b;
-  *p = v;
-}
+// The stored reconstruction of (face, velocity k), a 4-vector: (f_face h,
+// f_face b, w.grad f h, w.grad f b).  Tile-major, [tile][k / 2][slot][k % 2]
+// with the face's slot in the tile that owns it, so that the threads of a CTA,
+// two a slot on interleaved velocities, store and load consecutive vectors
+// (row by row of a face, a warp's 16 faces touch 16 cache lines an access:
+// those cost the reduction a third of its shared/global data cycles).
+// fval_at: offset of (slot 0, k = 0) plus the slot's two vectors.
+__host__ __device__ constexpr size_t fval_tile(int nvp) { return (size_t)(nvp / 2) * 2 * NSLOT; }
+__device__ __forceinline__ size_t fval_at(int k, int slot) { return (size_t)(k >> 1) * (2 * NSLOT) + 2 * slot + (k & 1); }
 
-// bytes of the flux pass's face-flux rows (a multiple of 32)
-template <typename T, typename C> __host__ __device__ constexpr size_t flux_fs_bytes() {
-  return (sizeof(typename Vec2<T>::type) * NSLOT * C::VKG + 31) / 32 * 32;
+// Owner (tile, slot) of the face of slot `slot` of tile `tile` at (i0, j0) of
+// a block: the tile of the cell on its high side; a closing face belongs to
+// the block's last tile, the seam of a periodic row to its first.
+__device__ __forceinline__ void fval_owner(const int *bi, int i0, int j0, int tile, int slot, int &otile, int &oslot) {
+  const int ni = bi[0], nj = bi[1], per = bi[2], ntx = (ni + TX - 1) / TX;
+  int dir, w, x, A, B;
+  slot_geom(slot, dir, w, x, A, B);
+  int i = dir == 0 ? i0 + x : i0 + w, j = dir == 0 ? j0 + w : j0 + x;
+  if (dir == 0 && per && i == ni) i = 0;
+  int ti = i / TX, tj = j / TY;
+  if (dir == 0 && i == ni) ti = (ni - 1) / TX;
+  if (dir == 1 && j == nj) tj = (nj - 1) / TY;
+  otile = tile + (tj - j0 / TY) * ntx + (ti - i0 / TX);
+  oslot = dir == 0 ? (j - TY * tj) * (TX + 1) + (i - TX * ti) : NSI + (j - TY * tj) * TX + (i - TX * ti);
 }
-
-// error-free sum (Knuth): s + e = a + b exactly
-__device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
-  s = a + b;
-  float bb = s - a;
-  e = (a - (s - bb)) + (b - bb);
-}
+size_t face_values(int ntiles, int nvp) { return (size_t)ntiles * fval_tile(nvp); }
 
 // ------------------------------------------------------------ face reduction
 // Per owned face (the i- and j-faces on the low side of the tile's cells, and
 // the closing faces at a non-periodic block end) the 12 sums over all
 // velocities: W0 = sum V Psi f_face (interior faces), and the incident-part
 // sums sum V Psi w.S f_face and sum V Psi w.S (w.grad f) (Eq. macroscopicFlux
-// with the time integrals q1, q2 applied afterwards).  Per chunk: staging of
-// the next chunk, gradients (phase A), face sums (phase B); FP32 partial sums
-// of two chunks are folded into a (sum, error) pair by an error-free sum.
-// The reconstruction of every (face, velocity) -- the upwind face value and
-// w.grad f of Eq. fullSolution -- is stored for the flux pass, which then
-// needs neither f nor its gradients.
-template <typename T, int FB, int VKT, int NHT>
-__global__ void __launch_bounds__(NSLOT * NHT) k_face_reduce(Dev d) {
-  typedef typename Vec2<T>::type T2;
-  typedef typename Vec4<T>::type T4;
-  typedef FCfg<T, VKT, NHT> C;
-  constexpr int VK = C::VK, VKP = C::VKP, NH = C::NH, VH = VK / NH;
-  extern __shared__ __align__(16) unsigned char smraw[];
-  FaceSmem<T, C> S;
-  S.carve(smraw);
-  int tile = blockIdx.x;
-  int b = d.tiles[3 * tile], i0 = d.tiles[3 * tile + 1], j0 = d.tiles[3 * tile + 2];
-  const int *bi = d.blk_info + 8 * b;
-  int ni = bi[0], nj = bi[1], per = bi[2], off = d.cell_off[b];
-  region_meta<T, C>(d, S, bi, off, i0, j0);
-  __syncthreads();
-  const int nch = (d.nv + VK - 1) / VK;
-  stage_chunk<T, FB, C>(d, S, 0, 0);
-  // this thread's face (the NH threads of a slot are adjacent lanes)
-  int slot = threadIdx.x / NH, half = threadIdx.x % NH;
-  int dir, w, x, A, B;
-  slot_geom(slot, dir, w, x, A, B);
-  int fid = tile_face_id(d, dir, off, ni, nj, i0, j0, w, x);
-  bool act = false;
-  if (fid >= 0) {
-    int i = dir == 0 ? i0 + x : i0 + w, j = dir == 0 ? j0 + w : j0 + x;
-    bool own = dir == 0 ? ((i < ni && x < TX) || (!per && i == ni)) : ((j < nj && x < TY) || j == nj);
-    act = own && d.face_kind[fid] != BC_OVERSET;
-    if (act) {
-      int Lg = d.face_L[fid], Rg = d.face_R[fid];
-      act = d.status[Lg] == ST_FIELD || (Rg >= 0 && d.status[Rg] == ST_FIELD);
+// with the time integrals q1, q2 applied afterwards).  The reconstruction of
+// every (face, velocity) -- the upwind face value and w.grad f of Eq.
+// fullSolution -- is stored for the flux pass, which then needs neither f nor
+// its gradients.
+//
+// gridDim.y CTAs share a tile's chunks where the tiles alone leave SMs idle
+// (face_splits): each then leaves its (sum, error) pairs for the interface
+// state kernel, which adds them in order.
+
+// This thread's face of the reduction.
+struct RedFace {
+  int fid, A, B, Lr, Rr;         // region cells A (lower logical side), B; L and R
+  bool act, wall;
+};
+template <typename T> __device__ __forceinline__ RedFace red_face(const Dev &d, const int *bi, int off, int i0, int j0, int slot) {
+  RedFace f;
+  const int ni = bi[0], nj = bi[1], per = bi[2];
+  int dir, w, x;
+  slot_geom(slot, dir, w, x, f.A, f.B);
+  f.fid = tile_face_id(d, dir, off, ni, nj, i0, j0, w, x);
+  f.act = f.wall = false;
+  f.Lr = f.Rr = f.A;
+  if (f.fid >= 0) {
+    const int i = dir == 0 ? i0 + x : i0 + w, j = dir == 0 ? j0 + w : j0 + x;
+    const bool own = dir == 0 ? ((i < ni && x < TX) || (!per && i == ni)) : ((j < nj && x < TY) || j == nj);
+    f.act = own && d.face_kind[f.fid] != BC_OVERSET;
+    if (f.act) {
+      const int Lg = d.face_L[f.fid], Rg = d.face_R[f.fid];
+      f.act = d.status[Lg] == ST_FIELD || (Rg >= 0 && d.status[Rg] == ST_FIELD);
     }
   }
-  bool wall = false;
-  T snx = T(0), sny = T(0), sun = T(0), ufx = T(0), ufy = T(0);
-  Side<T> L = make_side<T>(A, T(0), T(0)), R = L;
-  if (act) {
-    wall = d.face_kind[fid] == BC_WALL;
-    __align__(16) T Gr[NFG];
-    load_rec<T, NFG>(reinterpret_cast<const T *>(d.fgeo) + (size_t)fid * NFG, Gr);
-    snx = Gr[FG_SNX]; sny = Gr[FG_SNY]; sun = Gr[FG_SUN]; ufx = Gr[FG_UFX]; ufy = Gr[FG_UFY];
-    int Lr = (S.gid[A] == d.face_L[fid]) ? A : B, Rr = (Lr == A) ? B : A;
-    L = make_side<T>(Lr, Gr[FG_DXLX], Gr[FG_DXLY]);
-    R = make_side<T>(Rr, Gr[FG_DXRX], Gr[FG_DXRY]);
+  if (f.act) {
+    f.wall = d.face_kind[f.fid] == BC_WALL;
+    const int gA = region_gid(d, bi, off, i0 - 2 + f.A % RW, j0 - 2 + f.A / RW);
+    f.Lr = (gA == d.face_L[f.fid]) ? f.A : f.B;
+    f.Rr = (f.Lr == f.A) ? f.B : f.A;
   }
-  T hi[NFS], lo[NFS], acc[NFS];
-#pragma unroll
-  for (int m = 0; m < NFS; ++m) { hi[m] = T(0); lo[m] = T(0); acc[m] = T(0); }
-  for (int ch = 0; ch < nch; ++ch) {
-    int buf = ch & 1;
-    cp_async_wait<0>();
-    __syncthreads();                       // chunk ch visible; phase B of ch-1 done everywhere
-    if (ch + 1 < nch) stage_chunk<T, FB, C>(d, S, ch + 1, buf ^ 1);
-    chunk_gradients<T, C>(S, buf);
-    __syncthreads();
-    if (act) {
-      const T2 *Fb = S.F + (size_t)buf * NR * VKP;
-      const T4 *vt = S.vt + buf * VK;
-      const int kb = ch * VK;
-      T4 *fv = reinterpret_cast<T4 *>(d.fval) + (size_t)fid * d.nvp + kb;
-#pragma unroll 4
-      for (int q = 0; q < VH; ++q) {
-        int kk = half + NH * q;
-        T4 v = vt[kk];
-        T vx = v.x, vy = v.y, v2 = v.w;
-        T wS = vx * snx + vy * sny - sun;
-        // reflected velocities of a wall carry no f (zero weight, no branch)
-        T wk = (wall && !(wS > T(0))) ? T(0) : v.z;
-        V2<T> ff, wg;
-        upwind<T, C>(S, Fb, L, R, wall, kk, wS, vx - ufx, vy - ufy, ff, wg);
-        // the flux pass reads the reconstruction from here
-        if (kb + kk < d.nv) st_fval<T>(fv + kk, ff, wg);
-        T a = wk * ff.h, bb = T(0.5) * wk * ff.b;
-        T p0 = a, p1 = vx * a, p2 = vy * a, p3 = v2 * a + bb;
-        T ga = wk * wg.h, gb = T(0.5) * wk * wg.b;
-        T g0 = ga, g1 = vx * ga, g2 = vy * ga, g3 = v2 * ga + gb;
-        acc[FS_W0 + 0] += p0; acc[FS_W0 + 1] += p1; acc[FS_W0 + 2] += p2; acc[FS_W0 + 3] += p3;
-        acc[FS_FF + 0] += wS * p0; acc[FS_FF + 1] += wS * p1; acc[FS_FF + 2] += wS * p2; acc[FS_FF + 3] += wS * p3;
-        acc[FS_WG + 0] += wS * g0; acc[FS_WG + 1] += wS * g1; acc[FS_WG + 2] += wS * g2; acc[FS_WG + 3] += wS * g3;
-      }
-      if ((ch & 1) || ch + 1 == nch) {
-        if (sizeof(T) == 4) {
-#pragma unroll
-          for (int m = 0; m < NFS; ++m) {
-            float s, e;
-            two_sum((float)hi[m], (float)acc[m], s, e);
-            hi[m] = (T)s;
-            lo[m] += (T)e;
-            acc[m] = T(0);
-          }
-        } else {
-#pragma unroll
-          for (int m = 0; m < NFS; ++m) { hi[m] += acc[m]; acc[m] = T(0); }
-        }
-      }
-    }
-  }
-  // the NH parts of a face meet in shared memory (the region buffers are
-  // free once every thread has passed the barrier), summed in part order
+  return f;
+}
+
+// The two parts of a face meet in shared memory (xs: 2 NFS NSLOT values, free
+// once every thread has passed the barrier), summed in part order.
+template <typename T>
+__device__ __forceinline__ void red_finish(const Dev &d, T *xs, const RedFace &f, int slot, int half, const T *hi, const T *lo) {
   __syncthreads();
-  T *xs = reinterpret_cast<T *>(S.F);
-  if (half > 0) {
-    T *o = xs + (size_t)(half - 1) * 2 * NFS * NSLOT;
+  if (half > 0 && slot < NSLOT) {
 #pragma unroll
-    for (int m = 0; m < NFS; ++m) { o[(2 * m) * NSLOT + slot] = hi[m]; o[(2 * m + 1) * NSLOT + slot] = lo[m]; }
+    for (int m = 0; m < NFS; ++m) { xs[(2 * m) * NSLOT + slot] = hi[m]; xs[(2 * m + 1) * NSLOT + slot] = lo[m]; }
   }
   __syncthreads();
-  if (half == 0 && act) {
-    double *out = d.fsum + (size_t)NFS * fid;
+  if (half == 0 && f.act) {
 #pragma unroll
     for (int m = 0; m < NFS; ++m) {
-      double v;
-      if (sizeof(T) == 4) {
-        float h = (float)hi[m], l = (float)lo[m];
-        for (int p = 1; p < NH; ++p) {
-          const T *o = xs + (size_t)(p - 1) * 2 * NFS * NSLOT;
-          float s, e;
-          two_sum(h, (float)o[(2 * m) * NSLOT + slot], s, e);
-          h = s;
-          l = (l + e) + (float)o[(2 * m + 1) * NSLOT + slot];
-        }
-        v = to_double(h) + to_double(l);
+      T h = hi[m], l = lo[m];
+      face_sum_add(h, l, xs[(2 * m) * NSLOT + slot], xs[(2 * m + 1) * NSLOT + slot]);
+      if (f.wall && m < FS_FF) h = l = T(0);       // walls take W0 from the interior cell
+      if (gridDim.y == 1) {
+        d.fsum[(size_t)NFS * f.fid + m] = face_sum_value(h, l);
       } else {
-        v = (double)hi[m];
-        for (int p = 1; p < NH; ++p) v += (double)xs[(size_t)(p - 1) * 2 * NFS * NSLOT + (2 * m) * NSLOT + slot];
+        T *o = reinterpret_cast<T *>(d.fpart) + 2 * (((size_t)blockIdx.y * NFS + m) * d.nf + f.fid);
+        o[0] = h;
+        o[1] = l;
       }
-      out[m] = (wall && m < FS_FF) ? 0.0 : v;     // walls take W0 from the interior cell
     }
   }
+}
+
+// FP32.  Per chunk of VK32 consecutive velocities: staging of the next chunk;
+// phase A, the limited gradients of the tile's 100 gradient cells, a thread
+// walking down five cells of a column at one velocity (the column's values
+// stay in registers: three shared loads a cell instead of five); phase B, the
+// face values and the sums.  Bound by the shared-memory data path and by
+// instruction issue together: the limiter runs on (h, b) pairs in packed FP32
+// instructions, the sums on (f_face, w.grad f) pairs, and every shared and
+// global access of a warp covers whole lines (staging 128 bytes of a cell,
+// stores 512 consecutive bytes).  Two chunks are summed plainly, then folded
+// into (sum, error) pairs by an error-free sum.
+constexpr int VK32 = 16, VKP32 = VK32 + 2, VKG32 = VK32 + 2;   // rows in distinct banks
+constexpr int NT32 = 2 * GW * VK32;                            // two threads a gradient column and velocity
+static_assert(NT32 >= NT && NT32 % 32 == 0 && TY + 2 == 10, "phase A: five of a column's ten cells a thread");
+struct Smem32 {
+  PairF F[2][NR][VKP32];
+  float4 G[NG][VKG32];     // gradients: d_x h, d_x b, d_y h, d_y b
+  float4 tab[2][VK32];     // vx, vy, weight, |v|^2 / 2
+  float4 J[NR];            // twice the inverse Jacobian (real cells), ghost state rho lam / pi, Vx, Vy, lam (ghosts)
+  int gid[NR];
+};
+
+template <int FB> __global__ void __launch_bounds__(NT32, 2) k_face_reduce32(Dev d) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  Smem32 &S = *reinterpret_cast<Smem32 *>(smraw);
+  const int tile = blockIdx.x, tid = threadIdx.x;
+  const int b = d.tiles[3 * tile], i0 = d.tiles[3 * tile + 1], j0 = d.tiles[3 * tile + 2];
+  const int *bi = d.blk_info + 8 * b;
+  const int off = d.cell_off[b];
+  for (int r = tid; r < NR; r += NT32) {
+    const int g = region_gid(d, bi, off, i0 - 2 + r % RW, j0 - 2 + r / RW);
+    float4 J = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (g >= 0) {
+      J = d.jinvf[g];
+      J = make_float4(2.f * J.x, 2.f * J.y, 2.f * J.z, 2.f * J.w);
+    } else if (g <= -2) {
+      Prim p = primitive(d.ghostW + 4 * (-2 - g), d.Keff);
+      J = make_float4((float)(p.rho * p.lam * M_1_PI), (float)p.ux, (float)p.uy, (float)p.lam);
+    }
+    S.J[r] = J;
+    S.gid[r] = g;
+  }
+  __syncthreads();
+  const int nch = (d.nv + VK32 - 1) / VK32, npair = (nch + 1) / 2;
+  const int ch0 = 2 * (int)((long)npair * blockIdx.y / gridDim.y);
+  const int ch1 = min(nch, 2 * (int)((long)npair * (blockIdx.y + 1) / gridDim.y));
+  // copies of chunk ch into buffer buf: real cells by asynchronous 16-byte
+  // copies (bf16 storage: load and widen), ghost cells the Maxwellian of their
+  // ghost state, no cell / padding velocities zero; and the velocity table
+  auto stage = [&](int ch, int buf) {
+    const int kb = ch * VK32;
+#pragma unroll
+    for (int m = 0; m < (NR * VK32 / 2 + NT32 - 1) / NT32; ++m) {
+      const int it = tid + m * NT32, r = it / (VK32 / 2), e = 2 * (it % (VK32 / 2)), k = kb + e;
+      if (it >= NR * VK32 / 2) break;
+      const int g = S.gid[r];
+      PairF *dst = &S.F[buf][r][e];
+      if (g >= 0 && k < d.nv) {
+        if (FB) {
+          for (int q = 0; q < 2; ++q) {
+            auto v = ldF<float, 1>(d, (size_t)g * d.nvp + k + q);
+            dst[q] = pr_make(v.x, v.y);
+          }
+        } else {
+          // k < nv <= nvp, nvp a multiple of 4 and k even: the pair stays in
+          // the cell's row (padding velocities hold zero)
+          cp_async<16>(dst, reinterpret_cast<const PairF *>(d.f) + (size_t)g * d.nvp + k);
+        }
+      } else {
+        for (int q = 0; q < 2; ++q) {
+          V2<float> v = {0.f, 0.f};
+          if (g <= -2 && k + q < d.nv) {
+            const float4 p = S.J[r];
+            v = maxwellian_pre<float>(p.x, p.y, p.z, p.w, (float)d.Keff / (2.f * p.w), d.vxf[k + q], d.vyf[k + q]);
+          }
+          dst[q] = pr_make(v.h, v.b);
+        }
+      }
+    }
+    if (tid < VK32) {
+      const int k = kb + tid;
+      const float vx = k < d.nv ? d.vxf[k] : 0.f, vy = k < d.nv ? d.vyf[k] : 0.f, w = k < d.nv ? d.wf[k] : 0.f;
+      S.tab[buf][tid] = make_float4(vx, vy, w, 0.5f * (vx * vx + vy * vy));
+    }
+    cp_async_commit();
+  };
+  if (ch0 < ch1) stage(ch0, 0);
+  // phase A task: column and five rows of the gradient cells, one velocity
+  const int akk = tid % VK32, acol = (tid / VK32) % GW, arow = 5 * (tid / (VK32 * GW));
+  int afl = 0;                             // slope cases of the five cells, 4 bits each
+#pragma unroll
+  for (int m = 0; m < 5; ++m) {
+    const int g = S.gid[(arow + m + 1) * RW + acol + 1];
+    if (g >= 0) afl |= d.slope_flags[g] << (4 * m);
+  }
+  auto gradients = [&](int buf) {
+    const PairF *c = &S.F[buf][(arow + 1) * RW + acol + 1][akk];
+    const float4 *J = &S.J[(arow + 1) * RW + acol + 1];
+    float4 *o = &S.G[arow * GW + acol][akk];
+    PairF jm = c[-RW * VKP32], fc = c[0];
+#pragma unroll
+    for (int m = 0; m < 5; ++m) {
+      const PairF jp = c[RW * VKP32], ia = pr_sub(fc, c[-VKP32]), ib = pr_sub(c[VKP32], fc);
+      const PairF ja = pr_sub(fc, jm), jb = pr_sub(jp, fc);
+      const float4 J2 = *J;
+      float2 si = pr_vanleer_half(ia, ib), sj = pr_vanleer_half(ja, jb);
+      if (afl != 0xfffff) {
+        // one-sided where one neighbour is missing, none without both (twice
+        // the inverse Jacobian: one-sided slopes enter by half)
+        const int fl = afl >> (4 * m);
+        const PairF h = pr_make(0.5f, 0.5f);
+        const float2 z = make_float2(0.f, 0.f);
+        if ((fl & 3) != 3) si = (fl & 1) ? pr_get(pr_mul(h, ia)) : (fl & 2) ? pr_get(pr_mul(h, ib)) : z;
+        if ((fl & 12) != 12) sj = (fl & 4) ? pr_get(pr_mul(h, ja)) : (fl & 8) ? pr_get(pr_mul(h, jb)) : z;
+      }
+      float4 G = make_float4(mul_add2(J2.x, si.x, J2.y, sj.x), mul_add2(J2.x, si.y, J2.y, sj.y),
+                             mul_add2(J2.z, si.x, J2.w, sj.x), mul_add2(J2.z, si.y, J2.w, sj.y));
+      if (afl != 0xfffff && !((afl >> (4 * m)) & 15)) G = make_float4(0.f, 0.f, 0.f, 0.f);   // (ghost: J holds its state)
+      *o = G;
+      jm = fc;
+      fc = jp;
+      c += RW * VKP32;
+      J += RW;
+      o += GW * VKG32;
+    }
+  };
+  const int slot = tid >> 1, half = tid & 1;
+  RedFace f;
+  f.act = false;
+  if (tid < NT) f = red_face<float>(d, bi, off, i0, j0, slot);
+  float snx = 0.f, sny = 0.f, sun = 0.f, ufx = 0.f, ufy = 0.f, dxl = 0.f, dyl = 0.f, dxr = 0.f, dyr = 0.f;
+  int oL = 0, oR = 0, gL = 0, gR = 0;      // region and gradient rows of the two sides
+  if (f.act) {
+    __align__(16) float Gr[NFG];
+    load_rec<float, NFG>(reinterpret_cast<const float *>(d.fgeo) + (size_t)f.fid * NFG, Gr);
+    snx = Gr[FG_SNX]; sny = Gr[FG_SNY]; sun = Gr[FG_SUN]; ufx = Gr[FG_UFX]; ufy = Gr[FG_UFY];
+    dxl = Gr[FG_DXLX]; dyl = Gr[FG_DXLY]; dxr = Gr[FG_DXRX]; dyr = Gr[FG_DXRY];
+    oL = f.Lr * VKP32; oR = f.Rr * VKP32;
+    gL = g_of_region(f.Lr) * VKG32; gR = g_of_region(f.Rr) * VKG32;
+  }
+  float hi[NFS], lo[NFS], w0[4];
+  PairF fg[4];                             // (FF, WG) sums of the fold
+#pragma unroll
+  for (int m = 0; m < NFS; ++m) { hi[m] = 0.f; lo[m] = 0.f; }
+#pragma unroll
+  for (int m = 0; m < 4; ++m) { w0[m] = 0.f; fg[m] = pr_make(0.f, 0.f); }
+  float4 *fv = reinterpret_cast<float4 *>(d.fval) + (size_t)tile * fval_tile(d.nvp) + tid;
+  for (int ch = ch0; ch < ch1; ++ch) {
+    const int buf = (ch - ch0) & 1, kb = ch * VK32;
+    cp_async_wait<0>();
+    __syncthreads();                       // chunk ch visible; phase B of ch - 1 done everywhere
+    if (ch + 1 < ch1) stage(ch + 1, buf ^ 1);
+    gradients(buf);
+    __syncthreads();
+    if (f.act) {
+      const PairF *F = S.F[buf][0];
+      const float4 *G = S.G[0];
+#pragma unroll 4
+      for (int q = 0; q < VK32 / 2; ++q) {
+        const int kk = half + 2 * q;
+        const float4 t = S.tab[buf][kk];
+        const float vx = t.x, vy = t.y;
+        const float wS = __fsub_rn(mul_add2(vx, snx, vy, sny), sun);
+        const bool r = !f.wall && wS < 0.f;
+        const float wx = vx - ufx, wy = vy - ufy;
+        V2<float> ff, wg;
+        auto side = [&](const PairF *c, const float4 *gp, float dx, float dy, V2<float> &a, V2<float> &e) {
+          const float2 fc = pr_get(*c);
+          const float4 g = *gp;
+          a.h = __fmaf_rn(dy, g.z, __fmaf_rn(dx, g.x, fc.x));
+          a.b = __fmaf_rn(dy, g.w, __fmaf_rn(dx, g.y, fc.y));
+          e.h = mul_add2(wx, g.x, wy, g.z);
+          e.b = mul_add2(wx, g.y, wy, g.w);
+        };
+        side(F + (r ? oR : oL) + kk, G + (r ? gR : gL) + kk, r ? dxr : dxl, r ? dyr : dyl, ff, wg);
+        if (wS == 0.f && !f.wall) {        // exactly along the face: the mean of both sides
+          V2<float> f2, g2;
+          side(F + oR + kk, G + gR + kk, dxr, dyr, f2, g2);
+          ff = {0.5f * (ff.h + f2.h), 0.5f * (ff.b + f2.b)};
+          wg = {0.5f * (wg.h + g2.h), 0.5f * (wg.b + g2.b)};
+        }
+        // the flux pass reads the reconstruction from here
+        if (kb + kk < d.nv) fv[(size_t)(kb / 2 + q) * NT] = make_float4(ff.h, ff.b, wg.h, wg.b);
+        // reflected velocities of a wall carry no f; p = w Psi f_face, g = w Psi (w.grad f) in pairs
+        const float w = f.wall && !(wS > 0.f) ? 0.f : t.z, hw = 0.5f * w;
+        const PairF a = pr_mul(pr_make(w, w), pr_make(ff.h, wg.h));
+        const PairF p1 = pr_mul(pr_make(vx, vx), a), p2 = pr_mul(pr_make(vy, vy), a);
+        const PairF p3 = pr_fma(pr_make(hw, hw), pr_make(ff.b, wg.b), pr_mul(pr_make(t.w, t.w), a)), ws = pr_make(wS, wS);
+        w0[0] += pr_get(a).x; w0[1] += pr_get(p1).x; w0[2] += pr_get(p2).x; w0[3] += pr_get(p3).x;
+        fg[0] = pr_fma(ws, a, fg[0]); fg[1] = pr_fma(ws, p1, fg[1]);
+        fg[2] = pr_fma(ws, p2, fg[2]); fg[3] = pr_fma(ws, p3, fg[3]);
+      }
+      if ((ch & 1) || ch + 1 == ch1) {
+#pragma unroll
+        for (int m = 0; m < NFS; ++m) {
+          const float2 p = pr_get(fg[m & 3]);
+          const float x = m < FS_FF ? w0[m & 3] : m < FS_WG ? p.x : p.y;
+          float t, e;
+          two_sum(hi[m], x, t, e);
+          hi[m] = t;
+          lo[m] += e;
+        }
+#pragma unroll
+        for (int m = 0; m < 4; ++m) { w0[m] = 0.f; fg[m] = pr_make(0.f, 0.f); }
+      }
+    }
+  }
+  static_assert(sizeof(S.F) >= sizeof(float) * 2 * NFS * NSLOT, "the parts' sums fit in the region buffers");
+  red_finish<float>(d, reinterpret_cast<float *>(S.F), f, slot, half, hi, lo);
+}
+
+// FP64.  Bound by the FP64 pipe, so the operation count decides: the limited
+// gradients of a chunk are formed once per cell (phase A) and pass through
+// shared memory, the limiter shares one reciprocal between h and b, and a
+// chunk lies in one velocity row, so phase B only adds up the moments sum w
+// v_x^n (h, b) of the face value and of w.grad f (n <= 3); the 12 sums follow
+// from them once per fold (two chunks or a row's end) with the row's v_y.
+// Which side of a face is upwind changes at most once along a row, so chunks
+// with one sign of w.n at both ends take their side once; only the chunk that
+// holds the change selects per velocity.
+__global__ void __launch_bounds__(NT, 1) k_face_reduce64(Dev d) {
+  typedef double T;
+  typedef PairD P;
+  constexpr int VK = VK64, VKP = VKP64, VKG = VKG64;
+  extern __shared__ __align__(16) unsigned char smraw[];
+  Smem64 &S = *reinterpret_cast<Smem64 *>(smraw);
+  const int tile = blockIdx.x, tid = threadIdx.x;
+  const int b = d.tiles[3 * tile], i0 = d.tiles[3 * tile + 1], j0 = d.tiles[3 * tile + 2];
+  const int *bi = d.blk_info + 8 * b;
+  const int off = d.cell_off[b];
+  // this thread's region cell and its half of the staged copies
+  const int rc = tid >> 1, half = tid & 1;
+  const int gid = region_gid(d, bi, off, i0 - 2 + rc % RW, j0 - 2 + rc / RW);
+  double4 gst = {0.0, 0.0, 0.0, 0.0};              // ghost state
+  {
+    double4 J = {0.0, 0.0, 0.0, 0.0};
+    int fl = 0;
+    if (gid >= 0) {
+      fl = d.slope_flags[gid];
+      J.x = d.jinv[4 * gid]; J.y = d.jinv[4 * gid + 1]; J.z = d.jinv[4 * gid + 2]; J.w = d.jinv[4 * gid + 3];
+    } else if (gid <= -2) {
+      Prim p = primitive(d.ghostW + 4 * (-2 - gid), d.Keff);
+      gst.x = p.rho * p.lam * M_1_PI; gst.y = p.ux; gst.z = p.uy; gst.w = p.lam;
+    } else {                                       // no cell: zero in both buffers, once
+      for (int q = half; q < VKP; q += 2) S.F[0][rc][q] = S.F[1][rc][q] = pr_dup(0.0);
+    }
+    if (half == 0) { S.J[rc] = J; S.fl[rc] = fl; }
+  }
+  const Chunks ck = face_chunks<VK>(d.nvx, d.nv);
+  const int ch0 = (int)((long)ck.total * blockIdx.y / gridDim.y), ch1 = (int)((long)ck.total * (blockIdx.y + 1) / gridDim.y);
+  // position of a chunk: its row (of this context) and first column
+  struct Pos { int iy, x0; };
+  auto advance = [&](Pos &p) {
+    p.x0 += ck.len;
+    if (p.x0 >= d.nvx) { p.x0 = 0; ++p.iy; }
+  };
+  auto count = [&](const Pos &p) { return min(ck.len, d.nvx - p.x0); };
+  auto stage = [&](const Pos &p, int buf) {
+    const int n = count(p), k0 = p.iy * d.nvx + p.x0;
+    P *dst = S.F[buf][rc];
+    if (gid >= 0) {
+      const P *src = reinterpret_cast<const P *>(d.f) + (size_t)gid * d.nvp + k0;
+      for (int e = half; e < n; e += 2) cp_async<16>(dst + e, src + e);
+    } else if (gid <= -2) {
+      for (int e = half; e < n; e += 2) {
+        V2<T> m = maxwellian_pre<T>(gst.x, gst.y, gst.z, gst.w, (T)d.Keff / (T(2) * gst.w), d.vx1[p.x0 + e],
+                                    d.vy1[d.iy0 + p.iy]);
+        dst[e] = pr_make(m.h, m.b);
+      }
+    }
+    for (int e = tid; e < n; e += NT) {
+      const T vx = d.vx1[p.x0 + e], w = d.wx1[p.x0 + e];
+      S.tab[buf][e] = Smem64::Tab{{w, w * vx, w * (vx * vx), w * (vx * vx) * vx}, vx, 0.0};
+    }
+    cp_async_commit();
+  };
+  // phase A: the limited Cartesian gradient of (h, b) of gradient cell g and
+  // chunk velocity kk (ghost and missing cells carry none)
+  auto gradient = [&](int g, int kk, int buf) {
+    const int r = region_of_g(g);
+    const int fl = S.fl[r];
+    Quad<P> out = {pr_dup(0.0), pr_dup(0.0)};
+    if (fl) {
+      const double4 J = S.J[r];
+      const P *c = &S.F[buf][r][kk];
+      const P fc = c[0];
+      const P ia = pr_sub(fc, c[-VKP]), ib = pr_sub(c[VKP], fc);
+      const P ja = pr_sub(fc, c[-RW * VKP]), jb = pr_sub(c[RW * VKP], fc);
+      P si = pr_vanleer(ia, ib), sj = pr_vanleer(ja, jb);
+      if (fl != 15) {      // one-sided where one neighbour is missing, none without both
+        const P z = pr_dup(0.0);
+        if ((fl & 3) != 3) si = (fl & 1) ? ia : (fl & 2) ? ib : z;
+        if ((fl & 12) != 12) sj = (fl & 4) ? ja : (fl & 8) ? jb : z;
+      }
+      out.x = pr_fma(pr_dup(J.x), si, pr_mul(pr_dup(J.y), sj));
+      out.y = pr_fma(pr_dup(J.z), si, pr_mul(pr_dup(J.w), sj));
+    }
+    S.G[g][kk] = out;
+  };
+  const int slot = tid >> 1;
+  const RedFace f = red_face<T>(d, bi, off, i0, j0, slot);
+  T snx = 0.0, sny = 0.0, sun = 0.0, ufx = 0.0, ufy = 0.0, dxl = 0.0, dyl = 0.0, dxr = 0.0, dyr = 0.0;
+  if (f.act) {
+    __align__(16) T Gr[NFG];
+    load_rec<T, NFG>(reinterpret_cast<const T *>(d.fgeo) + (size_t)f.fid * NFG, Gr);
+    snx = Gr[FG_SNX]; sny = Gr[FG_SNY]; sun = Gr[FG_SUN]; ufx = Gr[FG_UFX]; ufy = Gr[FG_UFY];
+    dxl = Gr[FG_DXLX]; dyl = Gr[FG_DXLY]; dxr = Gr[FG_DXRX]; dyr = Gr[FG_DXRY];
+  }
+  const int Lg = g_of_region(f.Lr), Rg = g_of_region(f.Rr);
+  T hi[NFS], lo[NFS];
+#pragma unroll
+  for (int m = 0; m < NFS; ++m) { hi[m] = 0.0; lo[m] = 0.0; }
+  P M[4], Q[4];                                    // moments of the face value and of w.grad f
+#pragma unroll
+  for (int n = 0; n < 4; ++n) { M[n] = pr_dup(0.0); Q[n] = pr_dup(0.0); }
+  Pos cur = {ch0 / ck.per_row, (ch0 % ck.per_row) * ck.len}, nxt = cur;
+  if (ch0 < ch1) stage(cur, 0);
+  advance(nxt);
+  const unsigned magic = ((1u << 20) + ck.len - 1) / ck.len;
+  for (int ch = ch0; ch < ch1; ++ch) {
+    const int buf = (ch - ch0) & 1, n = count(cur);
+    cp_async_wait<0>();
+    __syncthreads();                       // chunk ch visible; phase B of ch-1 done everywhere
+    if (ch + 1 < ch1) stage(nxt, buf ^ 1);
+    // it / len by its reciprocal (it < 2^10, len <= 8: exact)
+    for (int it = tid; it < NG * ck.len; it += NT) {
+      const int g = (int)(((unsigned)it * magic) >> 20), kk = it - g * ck.len;
+      if (kk < n) gradient(g, kk, buf);
+    }
+    __syncthreads();
+    if (f.act) {
+      const Smem64::Tab *tab = S.tab[buf];
+      const T vy = d.vy1[d.iy0 + cur.iy], cy = vy * sny - sun, wy = vy - ufy;
+      Quad<P> *fv = reinterpret_cast<Quad<P> *>(d.fval) + (size_t)tile * fval_tile(d.nvp);
+      const int k0 = cur.iy * d.nvx + cur.x0;
+      const P wyp = pr_dup(wy);
+      auto reconstruct = [&](const P *F, const Quad<P> *G, P dx, P dy, int kk, P &ff, P &wg) {
+        const Quad<P> g = G[kk];
+        ff = pr_fma(dx, g.x, pr_fma(dy, g.y, F[kk]));
+        wg = pr_fma(pr_dup(tab[kk].vx - ufx), g.x, pr_mul(wyp, g.y));
+      };
+      auto accumulate = [&](const Smem64::Tab &t, P ff, P wg) {
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+          M[m] = pr_fma(pr_dup(t.w[m]), ff, M[m]);
+          Q[m] = pr_fma(pr_dup(t.w[m]), wg, Q[m]);
+        }
+      };
+      // w.S at the chunk's ends, rounded as for each velocity: monotone in v_x
+      const T wa = tab[0].vx * snx + cy, wb = tab[n - 1].vx * snx + cy;
+      const bool allL = wa > 0.0 && wb > 0.0, allR = wa < 0.0 && wb < 0.0;
+      if (allL || (allR && !f.wall)) {
+        const P *F = S.F[buf][allL ? f.Lr : f.Rr];
+        const Quad<P> *G = S.G[allL ? Lg : Rg];
+        const P dx = pr_dup(allL ? dxl : dxr), dy = pr_dup(allL ? dyl : dyr);
+        for (int kk = half; kk < n; kk += 2) {
+          P ff, wg;
+          reconstruct(F, G, dx, dy, kk, ff, wg);
+          fv[fval_at(k0 + kk, slot)] = Quad<P>{ff, wg};                // the flux pass reads the reconstruction from here
+          accumulate(tab[kk], ff, wg);
+        }
+      } else {
+        // the upwind side changes inside the chunk (w.S = 0 exactly: the mean
+        // of both sides); a wall takes its interior side's incident part only
+        for (int kk = half; kk < n; kk += 2) {
+          const T wS = tab[kk].vx * snx + cy;
+          const bool r = !f.wall && wS < 0.0;
+          if (f.wall && !(wS > 0.0)) continue;
+          P ff, wg;
+          reconstruct(S.F[buf][r ? f.Rr : f.Lr], S.G[r ? Rg : Lg], pr_dup(r ? dxr : dxl), pr_dup(r ? dyr : dyl), kk, ff, wg);
+          if (wS == 0.0) {
+            P f2, g2;
+            reconstruct(S.F[buf][f.Rr], S.G[Rg], pr_dup(dxr), pr_dup(dyr), kk, f2, g2);
+            ff = pr_mul(pr_dup(0.5), pr_add(ff, f2));
+            wg = pr_mul(pr_dup(0.5), pr_add(wg, g2));
+          }
+          fv[fval_at(k0 + kk, slot)] = Quad<P>{ff, wg};
+          accumulate(tab[kk], ff, wg);
+        }
+      }
+      // fold after two chunks, at the end of the row and at the last chunk
+      if (((cur.x0 / ck.len) & 1) || cur.x0 + n >= d.nvx || ch + 1 == ch1) {
+        const T ww = d.wy1[d.iy0 + cur.iy], hv = 0.5 * ww, vy2 = vy * vy;
+        auto sums = [&](const P *m, T *o, bool flux) {
+          const T e0 = m[2].x + vy2 * m[0].x + m[0].y;       // sum w (|v|^2 h + b)
+          if (!flux) {
+            o[0] += ww * m[0].x; o[1] += ww * m[1].x; o[2] += ww * (vy * m[0].x); o[3] += hv * e0;
+          } else {
+            const T e1 = m[3].x + vy2 * m[1].x + m[1].y;
+            const T f0 = snx * m[1].x + cy * m[0].x;
+            o[0] += ww * f0; o[1] += ww * (snx * m[2].x + cy * m[1].x); o[2] += ww * (vy * f0);
+            o[3] += hv * (snx * e1 + cy * e0);
+          }
+        };
+        sums(M, hi + FS_W0, false);
+        sums(M, hi + FS_FF, true);
+        sums(Q, hi + FS_WG, true);
+#pragma unroll
+        for (int m = 0; m < 4; ++m) { M[m] = pr_dup(0.0); Q[m] = pr_dup(0.0); }
+      }
+    }
+    cur = nxt;
+    advance(nxt);
+  }
+  static_assert(sizeof(S.F) >= sizeof(T) * 2 * NFS * NSLOT, "the parts' sums fit in the region buffers");
+  red_finish<T>(d, &S.F[0][0][0].x, f, slot, half, hi, lo);
 }
 
 // -------------------------------------------------------- flux divergence
@@ -496,49 +740,58 @@ __global__ void __launch_bounds__(NSLOT * NHT) k_face_reduce(Dev d) {
 // evaluated by both) computes S F_hat per velocity into shared memory from
 // the reconstruction the reduction pass stored; then each (tile cell,
 // velocity) sums its four faces with the cell's orientation signs and stores
-// D.  A streaming pass: the reconstructions of a chunk arrive in shared
-// memory as one bulk copy per face row (VK 4-vectors, issued by the face's
-// own thread, completing on the buffer's mbarrier; double-buffered), each
-// (face, velocity) adds the equilibrium part from the face's cubics, and each
-// (cell, velocity) makes one store.  ROW: the chunk lies in one row of the
-// velocity grid (VK divides N_vx), so c_y is fixed over it: the cubics
-// become cubics in c_x with coefficients formed once per chunk, and the
-// c_y factor of the Maxwellian is one exponential per chunk.
-template <typename T, typename C> __host__ __device__ constexpr size_t flux_fv_bytes() {
-  return sizeof(typename Vec4<T>::type) * 2 * NSLOT * C::VKF;
+// D.  A chunk is at most VK velocities of one velocity row, and the rows are
+// walked for a fixed range of columns; the interface cubics become cubics in
+// c_x whose coefficients a row shares.  SEP: the Maxwellian as the product of
+// a v_x factor, one exponential per column and range, and a v_y factor, one
+// per row; FP64 always (an exponential costs some thirty instructions of its
+// pipe), FP32 where N_v_x is a multiple of 16, else one exponential an item
+// (the hardware's takes two instructions; each form keeps its own rounding).
+//
+// A thread's own (face, velocity) items come through a ring of FS stages with
+// per-thread asynchronous copies: nobody else reads them, so a chunk needs one
+// barrier (the face fluxes, double-buffered) and FS - 1 chunks are in flight.
+// (One bulk copy per face row instead, completing on an mbarrier: its operands
+// are uniform, so lanes with different addresses issue one by one, some 1,400
+// warp instructions a chunk against 36.)  gridDim.y CTAs share a tile's rows.
+// Streaming: 16 bytes in per (face, velocity), 8 out per (cell, velocity) in
+// FP32; FP64 is bound by its pipe.
+template <typename T> struct FluxCfg;
+template <> struct FluxCfg<float> { static constexpr int VK = 8, FS = 4, CTAS = 2; };
+template <> struct FluxCfg<double> { static constexpr int VK = 8, FS = 3, CTAS = 1; };
+template <typename T> static constexpr size_t flux_smem() {
+  typedef typename PairOf<T>::type P;
+  typedef FluxCfg<T> C;
+  return sizeof(Quad<P>) * C::FS * C::VK / 2 * NT + sizeof(P) * 2 * NSLOT * (C::VK + 2);
 }
 
-template <typename T, int VKT, int NHT, bool ROW> __global__ void __launch_bounds__(NSLOT * NHT) k_flux(Dev d) {
-  typedef typename Vec2<T>::type T2;
-  typedef typename Vec4<T>::type T4;
-  typedef FCfg<T, VKT, NHT> C;
-  constexpr int VK = C::VK, VKG = C::VKG, VKF = C::VKF, NH = C::NH, VH = C::VH;
+template <typename T, bool SEP> __global__ void __launch_bounds__(NT, FluxCfg<T>::CTAS) k_flux(Dev d) {
+  typedef typename PairOf<T>::type P;
+  constexpr int VK = FluxCfg<T>::VK, FS = FluxCfg<T>::FS, VH = VK / 2, VKG = VK + 2;
   extern __shared__ __align__(16) unsigned char smraw[];
-  T4 *FV = reinterpret_cast<T4 *>(smraw);                                    // [2][NSLOT][VKF]
-  T2 *Fs = reinterpret_cast<T2 *>(smraw + flux_fv_bytes<T, C>());            // [NSLOT][VKG]
-  T4 *sgn = reinterpret_cast<T4 *>(smraw + flux_fv_bytes<T, C>() + flux_fs_bytes<T, C>());  // [TX*TY]
-  T2 *vt = reinterpret_cast<T2 *>(sgn + TX * TY);                           // [2][VK]: vx, vy
-  unsigned long long *mb = reinterpret_cast<unsigned long long *>(vt + 2 * VK);  // [2]
-  int *cinf = reinterpret_cast<int *>(mb + 2);                              // [TX*TY]: cell id or -1
-  int tile = blockIdx.x;
-  int b = d.tiles[3 * tile], i0 = d.tiles[3 * tile + 1], j0 = d.tiles[3 * tile + 2];
+  Quad<P> *FV = reinterpret_cast<Quad<P> *>(smraw);                         // [FS][VH][NT]
+  P *Fs = reinterpret_cast<P *>(smraw + sizeof(Quad<P>) * FS * VH * NT);    // [2][NSLOT][VKG]
+  const int tile = blockIdx.x, tid = threadIdx.x;
+  const int b = d.tiles[3 * tile], i0 = d.tiles[3 * tile + 1], j0 = d.tiles[3 * tile + 2];
   const int *bi = d.blk_info + 8 * b;
-  int ni = bi[0], nj = bi[1], off = d.cell_off[b];
-  if (threadIdx.x == 0) {
-    mbar_init(&mb[0], 1);
-    mbar_init(&mb[1], 1);
-    mbar_fence_init();
+  const int ni = bi[0], nj = bi[1], off = d.cell_off[b];
+  // this thread's cell of the sums (four threads a cell)
+  int g = -1;
+  P sg[4];
+  const P *fa = Fs, *fc = Fs;
+  {
+    const int c = tid >> 2, tx = c % TX, ty = c / TX, i = i0 + tx, j = j0 + ty;
+    if (tid < 4 * TX * TY && i < ni && j < nj) {
+      g = off + j * ni + i;
+      if (d.status[g] != ST_FIELD) g = -1;
+    }
+    const char4 sc = g >= 0 ? reinterpret_cast<const char4 *>(d.cell_sgn)[g] : make_char4(0, 0, 0, 0);
+    sg[0] = pr_dup((T)sc.x); sg[1] = pr_dup((T)sc.y); sg[2] = pr_dup((T)sc.z); sg[3] = pr_dup((T)sc.w);
+    fa += (ty * (TX + 1) + tx) * VKG;
+    fc += (NSI + ty * TX + tx) * VKG;
   }
-  for (int c = threadIdx.x; c < TX * TY; c += blockDim.x) {
-    int tx = c % TX, ty = c / TX, i = i0 + tx, j = j0 + ty;
-    int g = (i < ni && j < nj) ? off + j * ni + i : -1;
-    if (g >= 0 && d.status[g] != ST_FIELD) g = -1;
-    cinf[c] = g;
-    char4 sc = g >= 0 ? reinterpret_cast<const char4 *>(d.cell_sgn)[g] : make_char4(0, 0, 0, 0);
-    sgn[c] = T4{(T)sc.x, (T)sc.y, (T)sc.z, (T)sc.w};
-  }
-  const int nv = d.nv, nch = (nv + VK - 1) / VK;
-  int slot = threadIdx.x / NH, half = threadIdx.x % NH;
+  // this thread's face
+  const int slot = tid >> 1, half = tid & 1;
   bool act = false;
   int fid;
   {
@@ -550,135 +803,134 @@ template <typename T, int VKT, int NHT, bool ROW> __global__ void __launch_bound
       act = d.status[Lg] == ST_FIELD || (Rg >= 0 && d.status[Rg] == ST_FIELD);
     }
   }
-  const T4 *frow = reinterpret_cast<const T4 *>(d.fval) + (size_t)(act ? fid : 0) * d.nvp;
-  // velocity table of chunk ch into buffer ch & 1
-  auto stage_v = [&](int ch) {
-    for (int kk = threadIdx.x; kk < VK; kk += blockDim.x) {
-      int k = ch * VK + kk;
-      T2 t = {T(0), T(0)};
-      if (k < nv) { t.x = dvx<T>(d, k); t.y = dvy<T>(d, k); }
-      vt[(ch & 1) * VK + kk] = t;
-    }
-  };
-  // this face's row of chunk ch into buffer ch & 1 (the slot's first thread)
-  auto stage_row = [&](int ch) {
-    if (act && half == 0) {
-      int kb = ch * VK;
-      unsigned bytes = (unsigned)(sizeof(T4) * (nv - kb < VK ? nv - kb : VK));
-      unsigned long long *m = &mb[ch & 1];
-      mbar_expect_tx(m, bytes);
-      bulk_g2s(FV + ((ch & 1) * NSLOT + slot) * VKF, frow + kb, bytes, m);
-    }
-  };
-  bool wall = false;
-  __align__(16) T P[NFP];
+  if (!act)
+    for (int e = half; e < 2 * VKG; e += 2) Fs[((e >= VKG) * NSLOT + slot) * VKG + e % VKG] = pr_dup(T(0));
+  const bool wall = act && d.face_kind[fid] == BC_WALL;
+  __align__(16) T P_[NFP];
   if (act) {
-    wall = d.face_kind[fid] == BC_WALL;
-    load_rec<T, NFP>(reinterpret_cast<const T *>(d.fparT) + (size_t)fid * NFP, P);
+    load_rec<T, NFP>(reinterpret_cast<const T *>(d.fparT) + (size_t)fid * NFP, P_);
   } else {
 #pragma unroll
-    for (int m = 0; m < NFP; ++m) P[m] = T(0);
+    for (int m = 0; m < NFP; ++m) P_[m] = T(0);
   }
-  stage_v(0);
-  __syncthreads();                 // mbarriers initialised; cinf, sgn, vt of chunk 0 visible
-  stage_row(0);
-  __syncthreads();                 // every expectation of chunk 0 registered
-  if (threadIdx.x == 0) mbar_arrive(&mb[0]);
-  const T Keff = (T)d.Keff;
-  for (int ch = 0; ch < nch; ++ch) {
-    const int buf = ch & 1, kb = ch * VK;
-    // one warp polls the chunk's mbarrier (bounded; after a timeout, flagged,
-    // a second wait drains the copies), the others wait at the barrier
-    // without taking issue slots
-    if (threadIdx.x < 32)
-      if (!mbar_wait(&mb[buf], (ch >> 1) & 1, d.err)) mbar_wait(&mb[buf], (ch >> 1) & 1, d.err);
-    __syncthreads();               // chunk ch visible; the face fluxes of ch-1 consumed
-    if (ch + 1 < nch) {            // buffer buf ^ 1 was last read before the previous combine
-      stage_row(ch + 1);
-      stage_v(ch + 1);
+  const Chunks ck = face_chunks<VK>(d.nvx, d.nv);
+  const int rows = d.nv / d.nvx;
+  const int r0 = (int)((long)rows * blockIdx.y / gridDim.y), r1 = (int)((long)rows * (blockIdx.y + 1) / gridDim.y);
+  const int nch = ck.per_row * (r1 - r0);
+  struct Pos { int x0, iy; };
+  auto advance = [&](Pos &p) {
+    if (++p.iy == r1) { p.iy = r0; p.x0 += ck.len; }
+  };
+  int otile = tile, oslot = slot;
+  if (act) fval_owner(bi, i0, j0, tile, slot, otile, oslot);
+  const Quad<P> *fown = reinterpret_cast<const Quad<P> *>(d.fval) + (size_t)otile * fval_tile(d.nvp);
+  Quad<P> *ring = FV + tid;
+  auto stage = [&](const Pos &p, int st) {
+    if (act && p.x0 < d.nvx) {
+      const int n = min(ck.len, d.nvx - p.x0) - half;
+      const int k0 = p.iy * d.nvx + p.x0 + half;
+      const Quad<P> *src = fown + fval_at(k0, oslot);      // k0 + 2 q: NT vectors further each
+#pragma unroll
+      for (int q = 0; q < VH; ++q)
+        if (2 * q < n) {
+          char *dst = reinterpret_cast<char *>(ring + (st * VH + q) * NT);
+#pragma unroll
+          for (int e = 0; e < (int)sizeof(Quad<P>) / 16; ++e)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem_addr(dst + 16 * e)),
+                         "l"(reinterpret_cast<const char *>(src + q * NT) + 16 * e) : "memory");
+        }
     }
-    const T4 *fvb = FV + (buf * NSLOT + slot) * VKF;
-    const T2 *vtb = vt + buf * VK;
-    T2 *fso = Fs + slot * VKG;
-    // the loops below are uniform per thread: walls (reflected part for
-    // w.n <= 0), interior faces of a chunk inside one velocity row (ROW, no
-    // ragged tail: N_v is a multiple of VK), other interior faces
-    if (act && !wall && ROW) {
-      // per-chunk factors: the c_y parts of the cubics and of the Maxwellian
-      const T vy = vtb[0].y, cy = vy - P[FP_UY];
-      const T *ch3 = P + FP_IH, *cb3 = P + FP_IB;
-      const T ah0 = ch3[0] + cy * (ch3[2] + cy * (ch3[5] + cy * ch3[9]));
-      const T ah1 = ch3[1] + cy * (ch3[4] + cy * ch3[8]);
-      const T ah2 = ch3[3] + cy * ch3[7], ah3 = ch3[6];
-      const T ab0 = cb3[0] + cy * (cb3[2] + cy * (cb3[5] + cy * cb3[9]));
-      const T ab1 = cb3[1] + cy * (cb3[4] + cy * cb3[8]);
-      const T ab2 = cb3[3] + cy * cb3[7], ab3 = cb3[6];
-      const T ey = P[FP_HPRE] * r_exp<T>(-P[FP_LAM] * (cy * cy));
-      const T wsy = vy * P[FP_SNY] - P[FP_SUN];
-      const T snx = P[FP_SNX], ux = P[FP_UX], nlam = -P[FP_LAM], q1 = P[FP_Q1], q2 = P[FP_Q2];
+    cp_async_commit();
+  };
+  Pos cur = {0, r0}, nxt = cur;
+  if (r0 == r1) nxt.x0 = d.nvx;
+#pragma unroll
+  for (int s = 0; s < FS - 1; ++s) { stage(nxt, s); advance(nxt); }
+  const T Keff = (T)d.Keff;
+  const P snx2 = pr_dup(P_[FP_SNX]), nux2 = pr_dup(-P_[FP_UX]), q12 = pr_dup(P_[FP_Q1]), q22 = pr_dup(P_[FP_Q2]);
+  P cub[10];
+#pragma unroll
+  for (int m = 0; m < 10; ++m) cub[m] = pr_make(P_[FP_IH + m], P_[FP_IB + m]);
+  P vx2[VH];
+  T ex[VH];                                            // SEP: the columns' factors of the Maxwellian
+  int xcur = -1, st = 0, sn = FS - 1;                  // ring stages: this chunk's, the next copy's
+  for (int ch = 0; ch < nch; ++ch) {
+    const int n = min(ck.len, d.nvx - cur.x0);
+    if (cur.x0 != xcur) {                              // another range of columns
+      xcur = cur.x0;
 #pragma unroll
       for (int q = 0; q < VH; ++q) {
-        const int kk = half + NH * q;
-        const T4 fv = fvb[kk];
-        const T vx = vtb[kk].x;
-        // Eq. fullSolution averaged over dt_s: q1 f + q2 w.grad f + H ih(c)
-        // (and b), the equilibrium factors as per-face cubics in c = v - U0
-        const T wS = vx * snx + wsy, cx = vx - ux;
-        const T H = ey * r_exp<T>(nlam * (cx * cx));
-        const T ph = ah0 + cx * (ah1 + cx * (ah2 + cx * ah3));
-        const T pb = ab0 + cx * (ab1 + cx * (ab2 + cx * ab3));
-        T2 Fo;
-        Fo.x = wS * (q1 * fv.x + q2 * fv.z + H * ph);
-        Fo.y = wS * (q1 * fv.y + q2 * fv.w + H * pb);
-        fso[kk] = Fo;
+        const int kk = half + 2 * q;
+        const T vx = kk < n ? grid_vx<T>(d, xcur + kk) : T(0), cx = vx - P_[FP_UX];
+        vx2[q] = pr_dup(vx);
+        ex[q] = SEP ? r_exp<T>(-P_[FP_LAM] * (cx * cx)) : T(0);
       }
-    } else if (act) {
-#pragma unroll 4
+    }
+    const T vy = grid_vy<T>(d, d.iy0 + cur.iy);
+    cp_async_wait<FS - 2>();
+    P *fso = Fs + ((ch & 1) * NSLOT + slot) * VKG + half;
+    const Quad<P> *fvb = ring + st * VH * NT;
+    if (act) {
+      // per-row factors: the c_y parts of the cubics and of the Maxwellian
+      const T cy = vy - P_[FP_UY];
+      const P cy2 = pr_dup(cy);
+      const P a0 = pr_fma(cy2, pr_fma(cy2, pr_fma(cy2, cub[9], cub[5]), cub[2]), cub[0]);
+      const P a1 = pr_fma(cy2, pr_fma(cy2, cub[8], cub[4]), cub[1]);
+      const P a2 = pr_fma(cy2, cub[7], cub[3]), a3 = cub[6];
+      const T ey = SEP ? P_[FP_HPRE] * r_exp<T>(-P_[FP_LAM] * (cy * cy)) : T(0);
+      const P wsy2 = pr_dup(vy * P_[FP_SNY] - P_[FP_SUN]);
+#pragma unroll
       for (int q = 0; q < VH; ++q) {
-        const int kk = half + NH * q, k = kb + kk;
-        T2 Fo = {T(0), T(0)};
-        if (k < nv) {
-          const T4 fv = fvb[kk];
-          const T2 v = vtb[kk];
-          const T vx = v.x, vy = v.y;
-          const T wS = vx * P[FP_SNX] + vy * P[FP_SNY] - P[FP_SUN];
-          if (wall && !(wS > T(0))) {
-            // reflected part: wall Maxwellian at the face velocity (Eq. maxWalldes)
-            T wx = vx - P[FP_UFX], wy = vy - P[FP_UFY];
-            T lw = P[FP_LAMW];
-            T Hw = P[FP_RHOW] * (lw * T(M_1_PI)) * r_exp<T>(-lw * (wx * wx + wy * wy));
-            Fo.x = wS * Hw;
-            Fo.y = wS * Keff / (T(2) * lw) * Hw;
+        if (half + 2 * q < n) {
+          // Eq. fullSolution averaged over dt_s: q1 f + q2 w.grad f + H ih(c)
+          // (and b), the equilibrium factors as per-face cubics in c = v - U0
+          const Quad<P> fv = fvb[q * NT];
+          const P cx = pr_add(vx2[q], nux2);
+          const P ph = pr_fma(cx, pr_fma(cx, pr_fma(cx, a3, a2), a1), a0);
+          P I = pr_fma(q12, fv.x, pr_mul(q22, fv.y)), wS;
+          T H;
+          if (SEP && !wall) {
+            wS = pr_fma(vx2[q], snx2, wsy2);
+            H = ey * ex[q];
           } else {
-            T cx = vx - P[FP_UX], cy = vy - P[FP_UY];
-            T H = P[FP_HPRE] * r_exp<T>(-P[FP_LAM] * (cx * cx + cy * cy));
-            T Ih = P[FP_Q1] * fv.x + P[FP_Q2] * fv.z + H * poly3_at<T>(P + FP_IH, cx, cy);
-            T Ib = P[FP_Q1] * fv.y + P[FP_Q2] * fv.w + H * poly3_at<T>(P + FP_IB, cx, cy);
-            Fo.x = wS * Ih;
-            Fo.y = wS * Ib;
+            wS = pr_add(pr_fma(vx2[q], snx2, pr_dup(vy * P_[FP_SNY])), pr_dup(-P_[FP_SUN]));
+            H = P_[FP_HPRE] * r_exp<T>(-P_[FP_LAM] * (pr_get(cx).x * pr_get(cx).x + cy * cy));
           }
+          I = pr_fma(pr_dup(H), ph, I);
+          P out = pr_mul(wS, I);
+          if (wall && !(pr_get(wS).x > T(0))) {
+            // reflected part: wall Maxwellian at the face velocity (Eq. maxWalldes)
+            const T w = pr_get(wS).x, wx = pr_get(vx2[q]).x - P_[FP_UFX], wy = vy - P_[FP_UFY], lw = P_[FP_LAMW];
+            const T Hw = P_[FP_RHOW] * (lw * T(M_1_PI)) * r_exp<T>(-lw * (wx * wx + wy * wy));
+            out = pr_make(w * Hw, w * Keff / (T(2) * lw) * Hw);
+          }
+          fso[2 * q] = out;
         }
-        fso[kk] = Fo;
       }
-    } else {
-#pragma unroll 4
-      for (int q = 0; q < VH; ++q) fso[half + NH * q] = T2{T(0), T(0)};
     }
-    __syncthreads();               // face fluxes complete; expectations of chunk ch + 1 registered
-    if (threadIdx.x == 0 && ch + 1 < nch) mbar_arrive(&mb[buf ^ 1]);
-    for (int it = threadIdx.x; it < TX * TY * VK; it += blockDim.x) {
-      int c = it / VK, kk = it - (it / VK) * VK;
-      int g = cinf[c];
-      if (g < 0 || kb + kk >= nv) continue;
-      int tx = c % TX, ty = c / TX;
-      T4 sg = sgn[c];
-      T2 a = Fs[(ty * (TX + 1) + tx) * VKG + kk], bq = Fs[(ty * (TX + 1) + tx + 1) * VKG + kk];
-      T2 cq = Fs[(NSI + tx * (TY + 1) + ty) * VKG + kk], dq = Fs[(NSI + tx * (TY + 1) + ty + 1) * VKG + kk];
-      T Dh = sg.x * a.x + sg.y * bq.x + sg.z * cq.x + sg.w * dq.x;
-      T Db = sg.x * a.y + sg.y * bq.y + sg.z * cq.y + sg.w * dq.y;
-      stf<T>(d.Dbuf, (size_t)g * d.nvp + kb + kk, Dh, Db);
+    stage(nxt, sn);                                    // into the stage read one chunk ago
+    advance(nxt);
+    __syncthreads();                                   // face fluxes complete
+    if (g >= 0) {
+      const int o = (ch & 1) * NSLOT * VKG;
+      P *out = reinterpret_cast<P *>(d.Dbuf) + (size_t)g * d.nvp + cur.iy * d.nvx + cur.x0;
+#pragma unroll
+      for (int m = 0; m < VK / 4; ++m) {
+        const int kk = (tid & 3) + 4 * m;
+        if (kk < n) {
+          P D = pr_mul(sg[0], fa[o + kk]);
+          D = pr_fma(sg[1], fa[o + VKG + kk], D);
+          D = pr_fma(sg[2], fc[o + kk], D);
+          D = pr_fma(sg[3], fc[o + TX * VKG + kk], D);
+          out[kk] = D;
+        }
+      }
     }
+    advance(cur);
+    st = st + 1 == FS ? 0 : st + 1;
+    sn = sn + 1 == FS ? 0 : sn + 1;
   }
+  cp_async_wait<0>();
 }
 
 // Micro residual (Steps 3, 5; reading R4), elementwise over (cell, velocity):
@@ -789,45 +1041,38 @@ template <typename T, int FB> __global__ void k_residual_post(Dev d) {
   }
 }
 
-template <typename T, typename C> static size_t flux_smem() {
-  return flux_fv_bytes<T, C>() + flux_fs_bytes<T, C>() + sizeof(typename Vec4<T>::type) * TX * TY +
-         sizeof(typename Vec2<T>::type) * 2 * C::VK + 2 * sizeof(unsigned long long) + sizeof(int) * TX * TY;
-}
-template <typename T, typename C> static size_t reduce_smem() {
-  size_t a = FaceSmem<T, C>::bytes(), b = sizeof(T) * 2 * NFS * NSLOT * (C::NH > 1 ? C::NH - 1 : 1);
-  return a > b ? a : b;
-}
-
-// Candidate tile shapes of the FP32 face kernels (velocities per chunk,
-// threads per face slot); the FP64 path keeps (8, 2).
-constexpr int kFaceVK[] = {8, 16, 32};
-constexpr int kFaceNH[] = {2, 2, 2};
-constexpr int kFaceDefault = 1;     // (16, 2)
-int face_tile_count() { return 3; }
-void face_tile_shape(int v, int *vk, int *nh) {
-  if (v < 0 || v >= face_tile_count()) v = kFaceDefault;
-  *vk = kFaceVK[v];
-  *nh = kFaceNH[v];
-}
-int face_tile_default() { return kFaceDefault; }
-
-template <typename T, int FB, int VK, int NH> static void face_attr() {
-  typedef FCfg<T, VK, NH> C;
-  cudaFuncSetAttribute(k_flux<T, VK, NH, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)flux_smem<T, C>());
-  cudaFuncSetAttribute(k_flux<T, VK, NH, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)flux_smem<T, C>());
-  cudaFuncSetAttribute(k_face_reduce<T, FB, VK, NH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)reduce_smem<T, C>());
-}
-template <int FB> static void face_attr_f32() {
-  face_attr<float, FB, 8, 2>();
-  face_attr<float, FB, 16, 2>();
-  face_attr<float, FB, 32, 2>();
+// CTAs that share a tile's velocity chunks: the share that ends a pass soonest
+// on 152 SMs with two resident CTAs each (FP64: one), with ~4 us of set-up and
+// finish a CTA against ~7 us a pair of chunks (FP32, the fold's unit) or ~22 us
+// a chunk (FP64).  8 tiles at 16 x 16 velocities (32 x 16 cells): 8 CTAs a tile,
+// reduction 62 -> 14 us; 88 tiles in FP64 (96 x 48 + 64 x 16 cells, 32 x 32
+// velocities): 4.2 -> 1.7 ms; from about 600 tiles on a tile keeps its CTA.
+int face_splits(int ntiles, int nvx, int nv, int fp32) {
+  const int chunks = fp32 ? (nv + 2 * VK32 - 1) / (2 * VK32) : face_chunks<VK64>(nvx, nv).total;
+  const int slots = fp32 ? 304 : 152;
+  const double setup = 4.0, per = fp32 ? 7.0 : 22.0;
+  int best = 1;
+  double tb = 1e300;
+  for (int n = 1; n <= chunks && n <= 32; ++n) {
+    const double t = ((long)ntiles * n + slots - 1) / slots * (setup + per * ((chunks + n - 1) / n));
+    if (t < 0.97 * tb) { tb = t; best = n; }
+  }
+  return best;
 }
 
+void face_tile_shape(int fp32, int *vk, int *nh) {
+  *vk = fp32 ? VK32 : VK64;
+  *nh = 2;
+}
+
+template <typename T, bool SEP> static void flux_attr() {
+  cudaFuncSetAttribute(k_flux<T, SEP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)flux_smem<T>());
+}
 void tile_setup() {
-  face_attr_f32<0>();
-  face_attr_f32<1>();
-  face_attr<double, 0, 8, 2>();
+  cudaFuncSetAttribute(k_face_reduce32<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Smem32));
+  cudaFuncSetAttribute(k_face_reduce32<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Smem32));
+  cudaFuncSetAttribute(k_face_reduce64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Smem64));
+  flux_attr<float, true>(); flux_attr<float, false>(); flux_attr<double, true>();
 }
 
 int tile_count(int ni, int nj) { return ((ni + TX - 1) / TX) * ((nj + TY - 1) / TY); }
@@ -837,28 +1082,17 @@ void tile_origins(int ni, int nj, int *out) {   // (i0, j0) pairs
     for (int ti = 0; ti < (ni + TX - 1) / TX; ++ti) { out[q++] = ti * TX; out[q++] = tj * TY; }
 }
 
-template <typename T, int FB, int VK, int NH> static void face_launch(const Dev &d, cudaStream_t s, int which) {
-  typedef FCfg<T, VK, NH> C;
-  if (which == 0) k_face_reduce<T, FB, VK, NH><<<d.ntiles, C::NT, reduce_smem<T, C>(), s>>>(d);
-  else if (d.nvx % VK == 0) k_flux<T, VK, NH, true><<<d.ntiles, C::NT, flux_smem<T, C>(), s>>>(d);
-  else k_flux<T, VK, NH, false><<<d.ntiles, C::NT, flux_smem<T, C>(), s>>>(d);
+void launch_face_reduce(const Dev &d, cudaStream_t s, int fp32) {
+  const dim3 grid(d.ntiles, d.nsplit);
+  if (!fp32) k_face_reduce64<<<grid, NT, sizeof(Smem64), s>>>(d);
+  else if (d.fbf) k_face_reduce32<1><<<grid, NT32, sizeof(Smem32), s>>>(d);
+  else k_face_reduce32<0><<<grid, NT32, sizeof(Smem32), s>>>(d);
 }
-template <int FB> static void face_launch_f32(const Dev &d, cudaStream_t s, int which, int v) {
-  switch (v) {
-    case 0: face_launch<float, FB, 8, 2>(d, s, which); break;
-    case 2: face_launch<float, FB, 32, 2>(d, s, which); break;
-    default: face_launch<float, FB, 16, 2>(d, s, which); break;
-  }
-}
-static void face_dispatch(const Dev &d, cudaStream_t s, int which, int fp32, int v) {
-  if (!fp32) face_launch<double, 0, 8, 2>(d, s, which);
-  else if (d.fbf) face_launch_f32<1>(d, s, which, v);
-  else face_launch_f32<0>(d, s, which, v);
-}
-
-void launch_flux_tile(const Dev &d, cudaStream_t s, int fp32, int tile) { face_dispatch(d, s, 1, fp32, tile); }
-void launch_face_reduce_tile(const Dev &d, cudaStream_t s, int fp32, int tile) {
-  face_dispatch(d, s, 0, fp32, tile);
+void launch_flux(const Dev &d, cudaStream_t s, int fp32) {
+  const dim3 grid(d.ntiles, d.nsplit);
+  if (!fp32) k_flux<double, true><<<grid, NT, flux_smem<double>(), s>>>(d);
+  else if (d.nvx % 16 == 0) k_flux<float, true><<<grid, NT, flux_smem<float>(), s>>>(d);
+  else k_flux<float, false><<<grid, NT, flux_smem<float>(), s>>>(d);
 }
 void launch_residual(const Dev &d, cudaStream_t s, int first_iter, int fp32, int part) {
   int pairs = (d.nv + 1) / 2;
