@@ -51,9 +51,9 @@ struct ugks_ctx {
   std::vector<ugks_block_desc> blocks;
   std::vector<int> cell_off, node_off;
   int max_nj = 0;
-  int sweep_nw = 1, sweep_ql = 4, nwork = 0, nsm = 0;  // micro sweeps: warps per CTA, lanes per row, CTAs
+  int sweep_nw = 1, nwork = 0, nsm = 0;  // micro sweeps: warps per CTA, CTAs
   int nwork_cap = 0;                  // work-list capacity (largest tuning candidate)
-  int sweep_vpt = 2;                  // micro sweeps: velocities per lane
+  int sweep_rg = 4;                   // micro sweeps: rows per group
   int ns_fwd = 4, ns_bwd = 4;         // prefetch ring depths (steps) of the two sweeps
   ugks_exchange_fn xfn = nullptr;     // velocity sharding: the caller's exchange
   void *xuser = nullptr;
@@ -191,37 +191,30 @@ struct Carver {
   }
 };
 // Micro sweeps (skewed wavefront, ugks_sweep.cu): a warp takes a band of
-// 32 / QL rows of a block and QL * VPT consecutive velocities (QL lanes a row,
-// VPT velocities a lane); a CTA holds, for one block, a warp per band for each
-// of its velocity groups; every CTA has nw warps, nw = the largest band count
-// of the blocks, so a smaller block takes several groups per CTA.
-int max_nj_of(int nb, const ugks_block_desc *b) {
+// wsweep_rows(rg) rows of a block and wsweep_vw consecutive velocities; a CTA
+// holds, for one block, a warp per band for each of its velocity groups; every
+// CTA has nw warps, nw = the largest band count of the blocks, so a smaller
+// block takes several groups per CTA.
+int bands_of(int nj, int rg) { return (nj + wsweep_rows(rg) - 1) / wsweep_rows(rg); }
+int sweep_nw_for(int nb, const ugks_block_desc *b, int rg) {
   int m = 1;
-  for (int i = 0; i < nb; ++i) m = std::max(m, b[i].nj);
+  for (int i = 0; i < nb; ++i) m = std::max(m, bands_of(b[i].nj, rg));
   return m;
 }
-int bands_of(int nj, int ql) { int rows = 32 / ql; return (nj + rows - 1) / rows; }
-int sweep_nw_for(int nb, const ugks_block_desc *b) {
-  int ql = wsweep_ql(max_nj_of(nb, b)), m = 1;
-  for (int i = 0; i < nb; ++i) m = std::max(m, bands_of(b[i].nj, ql));
-  return m;
+int sweep_rg_for(const ugks_params *p, int nb, const ugks_block_desc *b) {
+  int nj = 1;
+  for (int i = 0; i < nb; ++i) nj = std::max(nj, b[i].nj);
+  return wsweep_rg(nj, p->precision != UGKS_FP64);
 }
 
-// Velocities per lane: 2 (UGKS_SWEEP_VPT=4 selects four on the FP32 paths).
-int sweep_vpt_for(const ugks_params *p) {
-  if (p->precision != UGKS_FP64)
-    if (const char *e = getenv("UGKS_SWEEP_VPT"))
-      if (atoi(e) == 4) return 4;
-  return 2;
-}
-
-// Work list (block, first velocity, velocity groups in the CTA) per CTA.
-std::vector<int> ws_work(int nb, const ugks_block_desc *b, int nvp, int vpt, int nw) {
+// Work list (block, first velocity, velocity groups in the CTA) per CTA (nvp:
+// the context's padded velocity count).
+std::vector<int> ws_work(const ugks_params *p, int nb, const ugks_block_desc *b, int nvp, int rg) {
   std::vector<int> work;
-  int ql = wsweep_ql(max_nj_of(nb, b)), vw = ql * vpt;
+  int vw = wsweep_vw(p->precision != UGKS_FP64), nw = sweep_nw_for(nb, b, rg);
   int groups = (nvp + vw - 1) / vw;
   for (int i = 0; i < nb; ++i) {
-    int gpc = std::max(1, nw / bands_of(b[i].nj, ql));
+    int gpc = std::max(1, nw / bands_of(b[i].nj, rg));
     for (int g0 = 0; g0 < groups; g0 += gpc) {
       work.push_back(i);
       work.push_back(g0 * vw);
@@ -231,23 +224,14 @@ std::vector<int> ws_work(int nb, const ugks_block_desc *b, int nvp, int vpt, int
   return work;
 }
 
-// CTAs of the sweeps (nvp: the context's padded velocity count)
-int nwork_for(int nvp, int nb, const ugks_block_desc *b, int vpt) {
-  return (int)ws_work(nb, b, nvp, vpt, sweep_nw_for(nb, b)).size() / 3;
-}
-
-// Candidates of the sweep autotuner: velocities per lane (FP32 paths; FP64
-// keeps 2) and prefetch ring depths (steps).
-constexpr int kTuneVpt[] = {2, 4};
+// Candidates of the sweep autotuner: prefetch ring depths (steps).
 constexpr int kTuneRing[] = {2, 4, 6};
 
-// Work-list capacity: the most CTAs any candidate needs (sized for the
-// whole velocity grid, which covers any shard of it).
+// Work-list capacity (sized for the whole velocity grid, which covers any
+// shard of it).
 int nwork_cap_for(const ugks_params *p, int nb, const ugks_block_desc *b) {
   int nvp = (p->nvx * p->nvy + 3) / 4 * 4;
-  int n = nwork_for(nvp, nb, b, sweep_vpt_for(p));
-  for (int v : kTuneVpt) n = std::max(n, nwork_for(nvp, nb, b, v));
-  return n;
+  return (int)ws_work(p, nb, b, nvp, sweep_rg_for(p, nb, b)).size() / 3;
 }
 
 // Lay out every device array of the context in the workspace (base may be
@@ -517,18 +501,6 @@ int check_err_flag(ugks_ctx *ctx) {
 
 int launch_status(ugks_ctx *ctx) { return cuda_check(ctx, cudaPeekAtLastError(), "kernel launch"); }
 
-// Switch the micro sweeps to another number of velocities per lane
-// (uploads the work list).
-int set_sweep_tiles(ugks_ctx *ctx, int vpt) {
-  std::vector<int> work = ws_work(ctx->nblocks, ctx->blocks.data(), ctx->d.nvp, vpt, ctx->sweep_nw);
-  if ((int)work.size() / 3 > ctx->nwork_cap) return fail(ctx, UGKS_ERR_WORKSPACE, "sweep work list");
-  CK(cudaMemcpyAsync(ctx->work, work.data(), sizeof(int) * work.size(), cudaMemcpyHostToDevice, ctx->st));
-  CK(cudaStreamSynchronize(ctx->st));
-  ctx->nwork = (int)work.size() / 3;
-  ctx->sweep_vpt = vpt;
-  return UGKS_OK;
-}
-
 // Event pair around one launch of a kernel group (only while profiling).
 // With UGKS_DEBUG_SYNC=1 in the environment at context creation, every
 // launch group is followed by a stream synchronisation and an error check, and
@@ -749,8 +721,8 @@ int step_body(ugks_ctx *ctx, int n_inner) {
       { Prof p(ctx, UGKS_PROF_RESIDUAL); launch_residual(d, s, it == 0, fp); }               // Step 5
     }
     if (met) launch_metrics(d, s, 1, fp);
-    { Prof p(ctx, UGKS_PROF_MICRO_FWD); launch_wsweep(d, s, 0, ctx->work, ctx->nwork, ctx->sweep_nw, ctx->ns_fwd, ctx->sweep_vpt, fp, ctx->sweep_ql); }  // Step 6
-    { Prof p(ctx, UGKS_PROF_MICRO_BWD); launch_wsweep(d, s, 1, ctx->work, ctx->nwork, ctx->sweep_nw, ctx->ns_bwd, ctx->sweep_vpt, fp, ctx->sweep_ql); }
+    { Prof p(ctx, UGKS_PROF_MICRO_FWD); launch_wsweep(d, s, 0, ctx->work, ctx->nwork, ctx->sweep_nw, ctx->ns_fwd, ctx->sweep_rg, fp); }  // Step 6
+    { Prof p(ctx, UGKS_PROF_MICRO_BWD); launch_wsweep(d, s, 1, ctx->work, ctx->nwork, ctx->sweep_nw, ctx->ns_bwd, ctx->sweep_rg, fp); }
     if (split && it + 1 < n_inner) {
       // Step 7, the receptors' W and q and the W gradients of the next
       // iteration on the tail stream, beside its velocity reduction
@@ -781,8 +753,8 @@ int step_body(ugks_ctx *ctx, int n_inner) {
 // What the captured kernels depend on beyond device memory: the device
 // struct they take by value and the launch configuration.
 std::vector<unsigned char> graph_key(const ugks_ctx *c, int n_inner) {
-  int cfg[] = {n_inner, c->fresh_pending ? 1 : 0, c->sweep_vpt, c->ns_fwd, c->ns_bwd, c->sweep_nw,
-               c->sweep_ql, c->nwork, c->nsm, c->max_nj, c->fp32, c->metrics ? 1 : 0, c->split_tail ? 1 : 0,
+  int cfg[] = {n_inner, c->fresh_pending ? 1 : 0, c->sweep_rg, c->ns_fwd, c->ns_bwd, c->sweep_nw,
+               c->nwork, c->nsm, c->max_nj, c->fp32, c->metrics ? 1 : 0, c->split_tail ? 1 : 0,
                c->split_residual && !c->in_batch ? 1 : 0};
   // (the step size is read from device memory; the bin count belongs to the
   // assembly, which is not part of the step)
@@ -982,9 +954,8 @@ int ugks_init_mesh(ugks_ctx *ctx, int nblocks, const ugks_block_desc *blocks, co
   ctx->nblocks = nblocks;
   ctx->blocks.assign(blocks, blocks + nblocks);
   ctx->max_nj = s.max_nj;
-  ctx->sweep_vpt = sweep_vpt_for(&ctx->p);
-  ctx->sweep_nw = sweep_nw_for(nblocks, blocks);
-  ctx->sweep_ql = wsweep_ql(max_nj_of(nblocks, blocks));
+  ctx->sweep_rg = sweep_rg_for(&ctx->p, nblocks, blocks);
+  ctx->sweep_nw = sweep_nw_for(nblocks, blocks, ctx->sweep_rg);
   if (const char *e = getenv("UGKS_SWEEP_NS")) {
     int n = atoi(e);
     if (n == 2 || n == 4 || n == 6) ctx->ns_fwd = ctx->ns_bwd = n;
@@ -996,8 +967,7 @@ int ugks_init_mesh(ugks_ctx *ctx, int nblocks, const ugks_block_desc *blocks, co
       ctx->nsm = nsm;
     cudaGetLastError();
   }
-  ctx->nwork = nwork_for(s.nvp, nblocks, blocks, ctx->sweep_vpt);
-  if (!wsweep_fits(ctx->fp32, ctx->fbf, ctx->sweep_vpt, ctx->sweep_nw, 1, ctx->sweep_ql))
+  if (!wsweep_fits(ctx->fp32, ctx->fbf, ctx->sweep_rg, ctx->sweep_nw, 1))
     return fail(ctx, UGKS_ERR_ARG, "micro-sweep CTA of the tallest block exceeds shared memory");
   ctx->nwork_cap = nwork_cap_for(&ctx->p, nblocks, blocks);
   ctx->cap_interp = cap_interp_for(s, nblocks);
@@ -1087,9 +1057,9 @@ int ugks_init_mesh(ugks_ctx *ctx, int nblocks, const ugks_block_desc *blocks, co
       if (blocks[order[b]].priority > blocks[order[a]].priority ||
           (blocks[order[b]].priority == blocks[order[a]].priority && order[b] < order[a]))
         std::swap(order[a], order[b]);
-  std::vector<int> work = ws_work(nblocks, blocks, s.nvp, ctx->sweep_vpt, ctx->sweep_nw);
-  if ((int)work.size() / 3 != ctx->nwork || ctx->nwork > ctx->nwork_cap)
-    return fail(ctx, UGKS_ERR_WORKSPACE, "sweep work list");
+  std::vector<int> work = ws_work(&ctx->p, nblocks, blocks, s.nvp, ctx->sweep_rg);
+  ctx->nwork = (int)work.size() / 3;
+  if (ctx->nwork > ctx->nwork_cap) return fail(ctx, UGKS_ERR_WORKSPACE, "sweep work list");
   std::vector<int> tiles;
   for (int b = 0; b < nblocks; ++b) {
     std::vector<int> org(2 * (size_t)tile_count(blocks[b].ni, blocks[b].nj));
@@ -1374,37 +1344,28 @@ int ugks_autotune(ugks_ctx *ctx, int reps, int *items_out, int *vpt_out, int *ri
     ctx->launches += reps + 1;
     return q;
   };
-  // micro sweeps: velocities per lane, and per sweep the ring depth
-  float best = 1e30f;
-  int bv = ctx->sweep_vpt, bf = ctx->ns_fwd, bb = ctx->ns_bwd;
-  for (int vpt : kTuneVpt) {
+  // micro sweeps: per sweep the ring depth
+  int bf = ctx->ns_fwd, bb = ctx->ns_bwd;
+  float tf = 1e30f, tb = 1e30f;
+  for (int ns : kTuneRing) {
     if (r) break;
-    if (!fp && vpt != 2) continue;
-    if ((r = set_sweep_tiles(ctx, vpt))) break;
-    float tf = 1e30f, tb = 1e30f;
-    int nf = 0, nb = 0;
-    for (int ns : kTuneRing) {
-      if (!wsweep_fits(fp, ctx->fbf, vpt, ctx->sweep_nw, ns, ctx->sweep_ql)) continue;
-      float ms;
-      if ((r = timed([&] { launch_wsweep(d, s, 0, ctx->work, ctx->nwork, ctx->sweep_nw, ns, vpt, fp, ctx->sweep_ql); }, ms))) break;
-      if (ms < tf) { tf = ms; nf = ns; }
-      if ((r = timed([&] { launch_wsweep(d, s, 1, ctx->work, ctx->nwork, ctx->sweep_nw, ns, vpt, fp, ctx->sweep_ql); }, ms))) break;
-      if (ms < tb) { tb = ms; nb = ns; }
-    }
-    if (r) break;
-    if (nf && nb && tf + tb < best) { best = tf + tb; bv = vpt; bf = nf; bb = nb; }
+    if (!wsweep_fits(fp, ctx->fbf, ctx->sweep_rg, ctx->sweep_nw, ns)) continue;
+    float ms;
+    if ((r = timed([&] { launch_wsweep(d, s, 0, ctx->work, ctx->nwork, ctx->sweep_nw, ns, ctx->sweep_rg, fp); }, ms))) break;
+    if (ms < tf) { tf = ms; bf = ns; }
+    if ((r = timed([&] { launch_wsweep(d, s, 1, ctx->work, ctx->nwork, ctx->sweep_nw, ns, ctx->sweep_rg, fp); }, ms))) break;
+    if (ms < tb) { tb = ms; bb = ns; }
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   if (r) return r;
   CK(cudaMemcpyAsync(d.f, d.Tn, fbytes, cudaMemcpyDeviceToDevice, s));
-  if ((r = set_sweep_tiles(ctx, bv))) return r;
   ctx->ns_fwd = bf;
   ctx->ns_bwd = bb;
   int vk, nh;
   face_tile_shape(fp, &vk, &nh);
-  if (items_out) *items_out = 32 * bv;
-  if (vpt_out) *vpt_out = bv;
+  if (items_out) *items_out = 64;      // no longer varied
+  if (vpt_out) *vpt_out = 2;
   if (ring_fwd_out) *ring_fwd_out = bf;
   if (ring_bwd_out) *ring_bwd_out = bb;
   if (face_vk_out) *face_vk_out = vk;

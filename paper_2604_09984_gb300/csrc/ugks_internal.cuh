@@ -161,10 +161,12 @@ constexpr int kWaitPolls = 1 << 21;
 
 // face geometry record / per-cell sweep record
 enum { FG_SNX = 0, FG_SNY, FG_SUN, FG_UFX, FG_UFY, FG_DXLX, FG_DXLY, FG_DXRX, FG_DXRY, NFG = 12 };
-// sweep record: per face slot s, outward (S n_x, S n_y, S U.n) at 3 s; the
-// micro-sweep diagonal base at SR_DBASE and the neighbour mask (int bits) at
-// SR_MASK; 16 values so a record is a whole number of 16-byte chunks
-enum { SR_DBASE = 12, SR_MASK = 13, NSR = 16 };
+// sweep record: half the outward S n_x, S n_y, S U.n of the four face slots,
+// the i and the j faces in pairs ((n_x i-low, i-high), (n_y ..), (U.n ..), then j),
+// and the micro-sweep diagonal base at SR_DBASE, zero for a cell that is not
+// solved; 16 values so a record is a whole number of 16-byte chunks
+enum { SR_DBASE = 12, NSR = 16 };
+__host__ __device__ constexpr int sr_at(int comp, int slot) { return 6 * (slot >> 1) + 2 * comp + (slot & 1); }
 
 // per-cell parameter record (from W' or W^n)
 enum { CP_RHO = 0, CP_UX, CP_UY, CP_LAM, CP_QX, CP_QY, CP_ITAU, CP_DBASE, NCP = 8 };
@@ -231,6 +233,64 @@ __device__ __forceinline__ void stf(void *base, size_t idx, T h, T b) {
   v.x = h;
   v.y = b;
   reinterpret_cast<typename Vec2<T>::type *>(base)[idx] = v;
+}
+
+// Pairs (h, b) of the arithmetic type.  FP32 pairs sit in one 64-bit register
+// pair and take the packed FP32 instructions (add, multiply, fused
+// multiply-add on both halves, each rounded as the scalar one): the velocity
+// loops are bound by instruction issue, and h and b go through the same
+// arithmetic almost everywhere.
+struct alignas(8) PairF { unsigned long long v; };
+struct alignas(16) PairD { double x, y; };
+template <typename T> struct PairOf;
+template <> struct PairOf<float> { typedef PairF type; };
+template <> struct PairOf<double> { typedef PairD type; };
+__device__ __forceinline__ PairF pr_make(float a, float b) {
+  PairF r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ PairD pr_make(double a, double b) { return PairD{a, b}; }
+__device__ __forceinline__ float2 pr_get(PairF a) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a.v));
+  return r;
+}
+__device__ __forceinline__ double2 pr_get(PairD a) { return double2{a.x, a.y}; }
+__device__ __forceinline__ PairF pr_add(PairF a, PairF b) {
+  PairF r;
+  asm("add.rn.ftz.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+__device__ __forceinline__ PairF pr_sub(PairF a, PairF b) {
+  PairF r;
+  asm("sub.rn.ftz.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+__device__ __forceinline__ PairF pr_mul(PairF a, PairF b) {
+  PairF r;
+  asm("mul.rn.ftz.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+__device__ __forceinline__ PairF pr_fma(PairF a, PairF b, PairF c) {
+  PairF r;
+  asm("fma.rn.ftz.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+  return r;
+}
+__device__ __forceinline__ PairD pr_add(PairD a, PairD b) { return PairD{a.x + b.x, a.y + b.y}; }
+__device__ __forceinline__ PairD pr_sub(PairD a, PairD b) { return PairD{a.x - b.x, a.y - b.y}; }
+__device__ __forceinline__ PairD pr_mul(PairD a, PairD b) { return PairD{a.x * b.x, a.y * b.y}; }
+__device__ __forceinline__ PairD pr_fma(PairD a, PairD b, PairD c) {
+  return PairD{fma(a.x, b.x, c.x), fma(a.y, b.y, c.y)};
+}
+template <typename T> __device__ __forceinline__ typename PairOf<T>::type pr_dup(T a) { return pr_make(a, a); }
+template <typename P> struct alignas(16) Quad { P x, y; };       // two pairs: (x.h, x.b, y.h, y.b)
+
+// the hardware's reciprocal (the factor of the fast approximate quotient)
+__device__ __forceinline__ float rcp_approx(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
 }
 
 // The distribution f in its storage type: the arithmetic type's pair, or on

@@ -176,9 +176,9 @@ template <typename T> __global__ void k_geo_records(Dev d) {
     for (int s = 0; s < 4; ++s) {
       int f = d.cell_faces[4 * c + s];
       double sg = (double)d.cell_sgn[4 * c + s];
-      r[3 * s] = (T)(0.5 * sg * d.Sn[2 * f]);
-      r[3 * s + 1] = (T)(0.5 * sg * d.Sn[2 * f + 1]);
-      r[3 * s + 2] = (T)(0.5 * sg * d.SUn[f]);
+      r[sr_at(0, s)] = (T)(0.5 * sg * d.Sn[2 * f]);
+      r[sr_at(1, s)] = (T)(0.5 * sg * d.Sn[2 * f + 1]);
+      r[sr_at(2, s)] = (T)(0.5 * sg * d.SUn[f]);
     }
   }
 }

@@ -524,10 +524,9 @@ template <typename T> __global__ void k_macro_post(Dev d) {
   int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= d.nc) return;
   T *sr = reinterpret_cast<T *>(d.srec) + (size_t)NSR * c;
-  int mask = d.cmask[c];
-  *reinterpret_cast<int *>(sr + SR_MASK) = mask;
-  if (!(mask & 1)) {
+  if (!(d.cmask[c] & 1)) {
     for (int m = 0; m < 4; ++m) d.Wp[4 * c + m] = d.W[4 * c + m];
+    sr[SR_DBASE] = T(0);
     return;
   }
   int njp;

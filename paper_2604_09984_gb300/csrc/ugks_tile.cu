@@ -90,67 +90,11 @@ template <typename T> struct Vec4;
 template <> struct Vec4<float> { typedef float4 type; };
 template <> struct Vec4<double> { typedef double4 type; };
 
-// Pairs (h, b) of the arithmetic type.  FP32 pairs sit in one 64-bit register
-// pair and take the packed FP32 instructions (add, multiply, fused
-// multiply-add on both halves, each rounded as the scalar one): the face
-// kernels are bound by instruction issue, and h and b go through the same
-// arithmetic almost everywhere.
-struct alignas(8) PairF { unsigned long long v; };
-struct alignas(16) PairD { double x, y; };
-template <typename T> struct PairOf;
-template <> struct PairOf<float> { typedef PairF type; };
-template <> struct PairOf<double> { typedef PairD type; };
-__device__ __forceinline__ PairF pr_make(float a, float b) {
-  PairF r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(a), "f"(b));
-  return r;
-}
-__device__ __forceinline__ PairD pr_make(double a, double b) { return PairD{a, b}; }
-__device__ __forceinline__ float2 pr_get(PairF a) {
-  float2 r;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a.v));
-  return r;
-}
-__device__ __forceinline__ double2 pr_get(PairD a) { return double2{a.x, a.y}; }
-__device__ __forceinline__ PairF pr_add(PairF a, PairF b) {
-  PairF r;
-  asm("add.rn.ftz.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
-  return r;
-}
-__device__ __forceinline__ PairF pr_sub(PairF a, PairF b) {
-  PairF r;
-  asm("sub.rn.ftz.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
-  return r;
-}
-__device__ __forceinline__ PairF pr_mul(PairF a, PairF b) {
-  PairF r;
-  asm("mul.rn.ftz.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
-  return r;
-}
-__device__ __forceinline__ PairF pr_fma(PairF a, PairF b, PairF c) {
-  PairF r;
-  asm("fma.rn.ftz.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
-  return r;
-}
-__device__ __forceinline__ PairD pr_add(PairD a, PairD b) { return PairD{a.x + b.x, a.y + b.y}; }
-__device__ __forceinline__ PairD pr_sub(PairD a, PairD b) { return PairD{a.x - b.x, a.y - b.y}; }
-__device__ __forceinline__ PairD pr_mul(PairD a, PairD b) { return PairD{a.x * b.x, a.y * b.y}; }
-__device__ __forceinline__ PairD pr_fma(PairD a, PairD b, PairD c) {
-  return PairD{fma(a.x, b.x, c.x), fma(a.y, b.y, c.y)};
-}
-template <typename T> __device__ __forceinline__ typename PairOf<T>::type pr_dup(T a) { return pr_make(a, a); }
-template <typename P> struct alignas(16) Quad { P x, y; };       // two pairs: (x.h, x.b, y.h, y.b)
-
 // a b + c d with one product rounded by itself (written out where results must
 // not depend on the compiler's choice)
 __device__ __forceinline__ float mul_add2(float a, float b, float c, float d) { return __fmaf_rn(a, b, __fmul_rn(c, d)); }
 // Half of the van Leer slopes 2 a b / (a + b) (0 where a b <= 0) of a pair of
 // differences, FP32 (the factor 2 goes into the inverse Jacobian: exact).
-__device__ __forceinline__ float rcp_approx(float x) {
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return r;
-}
 __device__ __forceinline__ float2 pr_vanleer_half(PairF a, PairF b) {
   const PairF p = pr_mul(a, b), s = pr_add(a, b);
   const float2 pv = pr_get(p), sv = pr_get(s);
