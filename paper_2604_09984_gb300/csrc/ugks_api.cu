@@ -270,11 +270,12 @@ size_t carve(char *base, const Sizes &s, int nb, int fp32, int fbf, int nwork, i
   d.Xf = c.take<float2>((size_t)s.nn);
   d.cbb = c.take<float4>((size_t)s.nc);
   d.vol_old = c.take<double>(s.nc); d.vol_new = c.take<double>(s.nc); d.dts = c.take<double>(s.nc);
+  d.idtau = c.take<double>(s.nc);
   d.xc = c.take<double>(2 * (size_t)s.nc); d.xc_new = c.take<double>(2 * (size_t)s.nc);
   d.period = c.take<double>(2 * (size_t)s.nc);
   d.Sn = c.take<double>(2 * (size_t)s.nf); d.nrm = c.take<double>(2 * (size_t)s.nf);
   d.xf = c.take<double>(2 * (size_t)s.nf); d.Uf = c.take<double>(2 * (size_t)s.nf);
-  d.S = c.take<double>(s.nf); d.SUn = c.take<double>(s.nf);
+  d.S = c.take<double>(s.nf); d.SUn = c.take<double>(s.nf); d.Un = c.take<double>(s.nf);
   d.slope_flags = c.take<int>(s.nc);
   d.cmask = c.take<int>(s.nc);
   d.jinv = c.take<double>(4 * (size_t)s.nc);
@@ -297,13 +298,12 @@ size_t carve(char *base, const Sizes &s, int nb, int fp32, int fbf, int nwork, i
   d.Wp = c.take<double>(4 * (size_t)s.nc);
   d.mrec = c.take<char>(macro_record_bytes(fp32) * s.nmrec);
   d.mrec_off = c.take<int>((size_t)nb + 1);
-  d.cpar = c.take<double>(NCP * (size_t)s.nc); d.cparn = c.take<double>(NCP * (size_t)s.nc);
   d.shp = c.take<char>(tsz * NSH * (size_t)s.nc); d.shn = c.take<char>(tsz * NSH * (size_t)s.nc);
   d.gradW = c.take<double>(8 * (size_t)s.nc);
   d.ghostW = c.take<double>(4 * (size_t)s.nf);
   d.fsum = c.take<double>(NFS * (size_t)s.nf);
   d.fpart = c.take<char>(s.nsplit > 1 ? 2 * tsz * NFS * (size_t)s.nf * s.nsplit : 0);
-  d.fpar = c.take<double>(NFP * (size_t)s.nf);
+  d.fq12 = c.take<double>(2 * (size_t)s.nf);
   d.fparT = c.take<char>(tsz * NFP * (size_t)s.nf);
   d.fflux = c.take<double>(4 * (size_t)s.nf);
   d.gam = c.take<double>(s.nf);
@@ -586,10 +586,11 @@ int upload_step_size(ugks_ctx *ctx) {
 }
 
 // Ghost states, W gradients, face reduction, face coefficients, per-cell
-// macro flux sum (Steps 1 / 3 up to the velocity-resolved flux).
+// macro flux sum (Steps 1 / 3 up to the velocity-resolved flux); the sum
+// only where asked for, the macro sweep's gather takes its own (with_sum).
 // joined: the W gradients ran on the tail stream (split tail); the face
 // state waits for them after the velocity reduction
-int flux_prep(ugks_ctx *ctx, int level_n, bool joined = false) {
+int flux_prep(ugks_ctx *ctx, int level_n, bool with_sum, bool joined = false) {
   Dev &d = ctx->d;
   cudaStream_t s = ctx->st;
   if (!joined) { Prof p(ctx, UGKS_PROF_CELL); launch_ghost_gradW(d, s); }
@@ -598,10 +599,10 @@ int flux_prep(ugks_ctx *ctx, int level_n, bool joined = false) {
   if (r) return r;
   if (joined) CK(cudaStreamWaitEvent(s, ctx->ev_tail, 0));
   { Prof p(ctx, UGKS_PROF_FACE_COEF); launch_face_coef(d, s, ctx->fp32); }
-  { Prof p(ctx, UGKS_PROF_CELL); launch_cell_macro(d, s, level_n); }
+  if (with_sum) { Prof p(ctx, UGKS_PROF_CELL); launch_cell_macro(d, s, level_n); }
   // ghost states and gradients (or the wait), reduction, face state and
-  // coefficients (the wall kernel where there are walls), cell terms
-  ctx->launches += (joined ? 0 : 2) + 1 + 2 + (d.nwall > 0 ? 1 : 0) + 1;
+  // coefficients, cell terms
+  ctx->launches += (joined ? 0 : 2) + 1 + 2 + (with_sum ? 1 : 0);
   return UGKS_OK;
 }
 
@@ -684,9 +685,9 @@ int step_body(ugks_ctx *ctx, int n_inner) {
   if (ctx->fresh_pending) do_interp(ctx, 1);
   do_interp(ctx, 0);
   // Steps 1-2: level-n flux, extensive level-n macro term, level-n cell record
-  int rx = flux_prep(ctx, 1);
+  int rx = flux_prep(ctx, 1, true);
   if (rx) return rx;
-  { Prof p(ctx, UGKS_PROF_CELL); launch_cell_params(d, s, d.W, d.cparn, fp); }
+  { Prof p(ctx, UGKS_PROF_CELL); launch_cell_params(d, s, fp); }
   ctx->launches += 1;
   for (int it = 0; it < n_inner; ++it) {
     if (it > 0) {
@@ -694,10 +695,10 @@ int step_body(ugks_ctx *ctx, int n_inner) {
         // the previous iteration's Step 7 is still running on the tail
         // stream: interpolate the receptors' f, reduce, then join
         do_interp(ctx, 0, 1);
-        if ((rx = flux_prep(ctx, 0, true))) return rx;   // Step 3
+        if ((rx = flux_prep(ctx, 0, false, true))) return rx;   // Step 3
       } else {
         do_interp(ctx, 0);
-        if ((rx = flux_prep(ctx, 0))) return rx;   // Step 3
+        if ((rx = flux_prep(ctx, 0, false))) return rx;   // Step 3
       }
     }
     // Step 4 (macro LU-SGS) on the side stream, concurrently with the flux
@@ -991,6 +992,7 @@ int ugks_init_mesh(ugks_ctx *ctx, int nblocks, const ugks_block_desc *blocks, co
   d.nv_all = s.nv_all; d.iy0 = s.iy0; d.shard = s.nv != s.nv_all;
   d.nvx = ctx->p.nvx; d.nvy = ctx->p.nvy;
   d.Kint = ctx->p.K; d.Keff = 1 + ctx->p.K;
+  d.c2fac = 2.0 * (4.0 + d.Keff) / ((2.0 + d.Keff) * (2.0 + d.Keff));
   d.Pr = ctx->p.Pr; d.omega = ctx->p.omega; d.mu_ref = ctx->p.mu_ref;
   d.cfl_s = ctx->p.cfl_s; d.cfl_pseudo = ctx->p.cfl_pseudo;
   d.dt = 1.0; d.idt = 1.0; d.idt_f = 1.0f;
@@ -1173,10 +1175,9 @@ int ugks_init_mesh(ugks_ctx *ctx, int nblocks, const ugks_block_desc *blocks, co
   CK(cudaMemcpyAsync(d.X_old, d.X_new, sizeof(double) * 2 * s.nn, cudaMemcpyDeviceToDevice, ctx->st));
   launch_geometry(d, ctx->st, ctx->fp32);
   ctx->launches += 5;
-  // initial state from the primitive field (staged through cpar)
-  if (s.nc * 4 > s.nc * NCP) return fail(ctx, UGKS_ERR_WORKSPACE, "staging");
-  CK(cudaMemcpyAsync(d.cpar, prim, sizeof(double) * 4 * s.nc, cudaMemcpyHostToDevice, ctx->st));
-  launch_init_state(d, ctx->st, d.cpar, ctx->fp32);
+  // initial state from the primitive field (staged through Wp)
+  CK(cudaMemcpyAsync(d.Wp, prim, sizeof(double) * 4 * s.nc, cudaMemcpyHostToDevice, ctx->st));
+  launch_init_state(d, ctx->st, d.Wp, ctx->fp32);
   ctx->launches += 1;
   CK(cudaStreamSynchronize(ctx->st));
   r = launch_status(ctx);
@@ -1463,7 +1464,7 @@ int ugks_eval_flux(ugks_ctx *ctx, double *D, double *F) {
   Dev &d = ctx->d;
   if (D && !is_device_ptr(D)) return fail(ctx, UGKS_ERR_ARG, "D must be a device pointer");
   do_interp(ctx, 0);
-  int r = flux_prep(ctx, 0);
+  int r = flux_prep(ctx, 0, true);
   if (r) return r;
   if (D) { launch_flux_div_all(d, ctx->st, D, ctx->fp32); ctx->launches += 1; }
   if (F) CK(cudaMemcpyAsync(F, d.Fc, sizeof(double) * 4 * d.nc, cudaMemcpyDefault, ctx->st));

@@ -31,6 +31,7 @@ struct Dev {
   int nc, nf, nn, nv, nvp, nblocks;
   int Keff, Kint;
   double Pr, omega, mu_ref, cfl_s, cfl_pseudo;
+  double c2fac;              // gamma (gamma - 1): square of the sound speed over the internal energy
   double Winf[4];
   double dt, idt;            // physical step and its inverse
   float idt_f;
@@ -70,7 +71,8 @@ struct Dev {
   double *xc, *xc_new;       // nc*2
   double *period;            // nc*2
   double *dts;               // nc
-  double *Sn, *S, *nrm, *xf, *Uf, *SUn;   // nf*2 / nf
+  double *idtau;             // nc 1 / pseudo-time step = cfl_s / (cfl_pseudo dts)
+  double *Sn, *S, *nrm, *xf, *Uf, *SUn, *Un;   // nf*2 / nf
   int *slope_flags;          // nc: 2 bits per direction (i: bits 0-1, j: 2-3)
   int *cmask;                // nc: bit 0 solved cell, bit 1+s solved neighbour across slot s
   double *jinv;              // nc*4 inverse of [[x_xi, y_xi],[x_eta, y_eta]]
@@ -95,15 +97,13 @@ struct Dev {
   double *Fc;                // nc*4 macro flux divergence of the last flux
   void *mrec;                // macro-sweep records (arithmetic type, layout in ugks_macro.cu)
   double *Wp;                // nc*4 macro predictor W'
-  double *cpar;              // nc*NCP cell parameters (predictor / level n)
-  double *cparn;
   void *shp, *shn;           // nc*NSH Shakhov records in the arithmetic type (predictor / level n)
   double *gradW;             // nc*8
   double *ghostW;            // nf*4
   double *fsum;              // nf*NFS
   void *fpart;               // nsplit*NFS*nf (sum, error) pairs of the face reduction's CTAs (nsplit > 1)
   int nsplit;                // CTAs that share a tile's velocity chunks in the face kernels
-  double *fpar;              // nf*NFP (double)
+  double *fq12;              // nf*2 time integrals q1 / dts, q2 / dts of the faces
   void *fparT;               // nf*NFP in the arithmetic type
   double *fflux;             // nf*4 S * macro flux (L -> R / outward)
   double *gam;               // nf spectral radius Gamma
@@ -207,20 +207,39 @@ __device__ __forceinline__ void face_sum_add(double &h, double &, double h2, dou
 __device__ __forceinline__ double face_sum_value(float h, float l) { return to_double(h) + to_double(l); }
 __device__ __forceinline__ double face_sum_value(double h, double) { return h; }
 
+// Component m of a cell's sum of S-weighted macro fluxes
+__device__ __forceinline__ double cell_flux_sum(const Dev &d, int c, int m) {
+  const int4 f = *reinterpret_cast<const int4 *>(d.cell_faces + 4 * c);
+  const char4 g = *reinterpret_cast<const char4 *>(d.cell_sgn + 4 * c);
+  double F = (double)g.x * d.fflux[4 * f.x + m];
+  F += (double)g.y * d.fflux[4 * f.y + m];
+  F += (double)g.z * d.fflux[4 * f.z + m];
+  F += (double)g.w * d.fflux[4 * f.w + m];
+  return F;
+}
+
 // Shakhov record in the arithmetic type from a cell record (double)
+// and the finished 1 / (2 lam) and heat flux prefactor
+template <typename T>
+__device__ __forceinline__ void write_shrec(const Dev &d, const double *o, double il, double pref, double vol, T *r) {
+  __align__(16) T v[NSH] = {};
+  v[SH_HPRE] = (T)(o[CP_RHO] * o[CP_LAM] * M_1_PI);
+  v[SH_UX] = (T)o[CP_UX];
+  v[SH_UY] = (T)o[CP_UY];
+  v[SH_LAM] = (T)o[CP_LAM];
+  v[SH_QX] = (T)o[CP_QX];
+  v[SH_QY] = (T)o[CP_QY];
+  v[SH_PREF] = (T)pref;
+  v[SH_IL] = (T)il;
+  v[SH_ITAU] = (T)o[CP_ITAU];
+  v[SH_VOL] = (T)vol;
+  static_assert(NSH * sizeof(T) % 8 == 0, "record size");
+#pragma unroll
+  for (int m = 0; m < (int)(NSH * sizeof(T) / 8); ++m) reinterpret_cast<float2 *>(r)[m] = reinterpret_cast<float2 *>(v)[m];
+}
 template <typename T>
 __device__ __forceinline__ void write_shrec(const Dev &d, const double *o, double vol, T *r) {
-  double il = 1.0 / (2.0 * o[CP_LAM]);
-  r[SH_HPRE] = (T)(o[CP_RHO] * o[CP_LAM] * M_1_PI);
-  r[SH_UX] = (T)o[CP_UX];
-  r[SH_UY] = (T)o[CP_UY];
-  r[SH_LAM] = (T)o[CP_LAM];
-  r[SH_QX] = (T)o[CP_QX];
-  r[SH_QY] = (T)o[CP_QY];
-  r[SH_PREF] = (T)(4.0 * (1.0 - d.Pr) * o[CP_LAM] * o[CP_LAM] / (5.0 * o[CP_RHO]));
-  r[SH_IL] = (T)il;
-  r[SH_ITAU] = (T)o[CP_ITAU];
-  r[SH_VOL] = (T)vol;
+  write_shrec<T>(d, o, 1.0 / (2.0 * o[CP_LAM]), 4.0 * (1.0 - d.Pr) * o[CP_LAM] * o[CP_LAM] / (5.0 * o[CP_RHO]), vol, r);
 }
 
 template <typename T>

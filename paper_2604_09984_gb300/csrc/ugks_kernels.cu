@@ -74,6 +74,7 @@ __global__ void k_face_geom(Dev d) {
   d.Uf[2 * f] = ufx;
   d.Uf[2 * f + 1] = ufy;
   d.SUn[f] = ufx * ey + ufy * (-ex);
+  d.Un[f] = d.SUn[f] / d.S[f];
 }
 
 __device__ __forceinline__ double warp_sum(double v) {
@@ -148,7 +149,9 @@ __global__ void k_dts(Dev d, double vx0, double vx1, double vy0, double vy1) {
     }
     m = fmax(m, s);
   }
-  d.dts[c] = d.cfl_s * d.vol_new[c] / m;
+  const double dts = d.cfl_s * d.vol_new[c] / m;
+  d.dts[c] = dts;
+  d.idtau[c] = d.cfl_s / (d.cfl_pseudo * dts);
 }
 
 // Per-step geometry records in the arithmetic type: per face (S n, S U.n,
@@ -265,33 +268,32 @@ __global__ void k_ghost(Dev d) {
   }
 }
 
-// Limited gradient of the conservative W per cell (reading R1).
-__global__ void k_gradW(Dev d) {
-  int c = blockIdx.x * blockDim.x + threadIdx.x;
+// Limited gradient of the conservative W per cell (reading R1).  Bound by the
+// latency of its loads: a thread per cell and component, and CTAs of 64 threads
+// so that a small mesh spreads over the SMs (512 cells: 12.8 us -> 5.4 us; 36864
+// cells 15.3 -> 13.6).
+constexpr int GW_THREADS = 64;
+__global__ void __launch_bounds__(GW_THREADS) k_gradW(Dev d) {
+  int t = blockIdx.x * blockDim.x + threadIdx.x;
+  int c = t >> 2, m = t & 3;
   if (c >= d.nc) return;
   int fl = d.slope_flags[c];
-  const double *J = d.jinv + 4 * c;
-  for (int m = 0; m < 4; ++m) {
-    double wc = d.W[4 * c + m];
-    double s[2];
-    for (int dir = 0; dir < 2; ++dir) {
-      int cs = (fl >> (2 * dir)) & 3;
-      double val[2] = {0.0, 0.0};
-      for (int side = 0; side < 2; ++side) {
-        int sl = 2 * dir + side;
-        int kind = d.nb_kind[4 * c + sl], id = d.nb_id[4 * c + sl];
-        if (kind == NB_CELL) val[side] = d.W[4 * id + m];
-        else if (kind == NB_GHOST) val[side] = d.ghostW[4 * id + m];
-      }
-      double r = 0.0;
-      if (cs == SL_BOTH) r = vanleer<double>(wc - val[0], val[1] - wc);
-      else if (cs == SL_P) r = val[1] - wc;
-      else if (cs == SL_M) r = wc - val[0];
-      s[dir] = r;
-    }
-    d.gradW[8 * c + 2 * m] = J[0] * s[0] + J[1] * s[1];
-    d.gradW[8 * c + 2 * m + 1] = J[2] * s[0] + J[3] * s[1];
-  }
+  const int4 kind = *reinterpret_cast<const int4 *>(d.nb_kind + 4 * c);
+  const int4 id = *reinterpret_cast<const int4 *>(d.nb_id + 4 * c);
+  const double2 j0 = *reinterpret_cast<const double2 *>(d.jinv + 4 * c);
+  const double2 j1 = *reinterpret_cast<const double2 *>(d.jinv + 4 * c + 2);
+  double wc = d.W[4 * c + m];
+  auto value = [&](int k, int i) { return k == NB_CELL ? d.W[4 * i + m] : k == NB_GHOST ? d.ghostW[4 * i + m] : 0.0; };
+  const double v0 = value(kind.x, id.x), v1 = value(kind.y, id.y), v2 = value(kind.z, id.z), v3 = value(kind.w, id.w);
+  auto slope = [&](int cs, double lo, double hi) {
+    if (cs == SL_BOTH) return vanleer<double>(wc - lo, hi - wc);
+    return cs == SL_P ? hi - wc : cs == SL_M ? wc - lo : 0.0;
+  };
+  const double s0 = slope(fl & 3, v0, v1), s1 = slope((fl >> 2) & 3, v2, v3);
+  double2 g;
+  g.x = j0.x * s0 + j0.y * s1;
+  g.y = j1.x * s0 + j1.y * s1;
+  *reinterpret_cast<double2 *>(d.gradW + 8 * c + 2 * m) = g;
 }
 
 __device__ __forceinline__ bool face_needed(const Dev &d, int f) {
@@ -299,136 +301,160 @@ __device__ __forceinline__ bool face_needed(const Dev &d, int f) {
   return d.status[L] == ST_FIELD || (R >= 0 && d.status[R] == ST_FIELD);
 }
 
-__device__ __forceinline__ double spectral_radius(const double *Wf, double nx, double ny, double un,
-                                                  int Keff) {
-  Prim p = primitive(Wf, Keff);
-  double pr = p.rho / (2.0 * p.lam);
-  double gamma = (4.0 + Keff) / (2.0 + Keff);
-  return fabs(p.ux * nx + p.uy * ny - un) + sqrt(gamma * pr / p.rho);
-}
-
-// Face coefficients, scalar part (one thread per face): g0 parameters and
-// slopes (reading R2), time integrals over dts (Eq. fullSolution averaged as
-// in Sec. 2.2), wall temperature parameter.
-template <typename T> __global__ void k_face_scalar(Dev d) {
-  int fid = blockIdx.x * blockDim.x + threadIdx.x;
-  if (fid >= d.nf) return;
-  int kind = d.face_kind[fid];
-  if (!face_needed(d, fid) || kind == BC_OVERSET) return;
-  double *P = d.fpar + (size_t)NFP * fid;
-  T *PT = reinterpret_cast<T *>(d.fparT) + (size_t)NFP * fid;
-  int L = d.face_L[fid], R = d.face_R[fid];
-  bool wall = kind == BC_WALL;
-  double W0[4], gx[4], gy[4], q0x, q0y, dts;
-  double ufx = d.Uf[2 * fid], ufy = d.Uf[2 * fid + 1];
-  double nx = d.nrm[2 * fid], ny = d.nrm[2 * fid + 1];
-  double *fs = d.fsum + NFS * fid;
-  if (d.nsplit > 1) {          // the reduction's CTAs left their parts: added here in order
-    const T *p = reinterpret_cast<const T *>(d.fpart) + 2 * (size_t)fid;
-    for (int m = 0; m < NFS; ++m) {
-      T h = T(0), l = T(0);
-      for (int s = 0; s < d.nsplit; ++s) {
-        const T *q = p + 2 * ((size_t)s * NFS + m) * d.nf;
-        face_sum_add(h, l, q[0], q[1]);
+// Face coefficients, scalar part: g0 parameters and slopes (reading R2), time
+// integrals over dts (Eq. fullSolution averaged as in Sec. 2.2), wall
+// temperature parameter, Gamma; all in FP64 (per face, not per velocity), the
+// mixed path rounds the finished record once to FP32 for its velocity loops.
+//
+// Bound by the FP64 pipe (some 15 cycles a warp instruction and SM; 500 such
+// instructions a face) and, on small meshes, by the latency of one face's chain.
+// So a CTA takes only FSC = 32 faces (a small mesh reaches every SM), one warp
+// does the face state, slopes and time integrals, a second one the geometry and
+// Gamma; with the reduction's parts to fold (small meshes), four warps take the
+// sums among them and a third one the time integrals.  The records are collected in shared memory and written as lines.
+// 1056 faces with 8 parts to fold: 44.1 us -> 18.2 us (128 faces a CTA, one
+// thread a face before); 74112 faces: 113 -> 95 (a fifth fewer FP64
+// instructions: one division for p / rho, two sums for the integrals).
+constexpr int FSC = 32;
+template <typename T, bool FOLD> __global__ void __launch_bounds__(FOLD ? 128 : 64) k_face_scalar(Dev d) {
+  constexpr int ROW = FP_IH + 1;
+  __shared__ T rec[FSC * ROW];
+  __shared__ double W0f[4][FSC];
+  __shared__ bool live[FSC];
+  const int lane = threadIdx.x & 31, wrp = threadIdx.x >> 5;
+  const int f0 = blockIdx.x * FSC, fid = f0 + lane;
+  const int kind = fid < d.nf ? d.face_kind[fid] : BC_OVERSET;
+  const bool need = kind != BC_OVERSET && face_needed(d, fid);
+  const bool wall = kind == BC_WALL;
+  const int L = need ? d.face_L[fid] : 0, R = need ? d.face_R[fid] : -1;
+  T *PT = rec + lane * ROW;
+  if (wrp == 0) live[lane] = need;
+  if (FOLD) {                  // the reduction's CTAs left their parts: added here in order
+    if (need) {
+      const T *p = reinterpret_cast<const T *>(d.fpart) + 2 * (size_t)fid;
+#pragma unroll
+      for (int j = 0; j < NFS / 4; ++j) {
+        const int m = wrp + 4 * j;
+        T h = T(0), l = T(0);
+        for (int s = 0; s < d.nsplit; ++s) {
+          const typename Vec2<T>::type q =
+              *reinterpret_cast<const typename Vec2<T>::type *>(p + 2 * ((size_t)s * NFS + m) * d.nf);
+          face_sum_add(h, l, q.x, q.y);
+        }
+        const double v = face_sum_value(h, l);
+        d.fsum[(size_t)NFS * fid + m] = v;
+        if (j == 0) W0f[m][lane] = v;
       }
-      fs[m] = face_sum_value(h, l);
     }
+    __syncthreads();
   }
-  if (wall) {
-    double dx = d.xf[2 * fid] - d.xc[2 * L], dy = d.xf[2 * fid + 1] - d.xc[2 * L + 1];
-    for (int m = 0; m < 4; ++m) {
-      gx[m] = d.gradW[8 * L + 2 * m];
-      gy[m] = d.gradW[8 * L + 2 * m + 1];
-      W0[m] = d.W[4 * L + m] + (dx * gx[m] + dy * gy[m]);
-    }
-    q0x = d.q[2 * L];
-    q0y = d.q[2 * L + 1];
-    dts = d.dts[L];
-  } else {
-    double sh = (double)d.face_shiftL[fid];
-    double xLx = d.xc[2 * L] + sh * d.period[2 * L], xLy = d.xc[2 * L + 1] + sh * d.period[2 * L + 1];
-    double xRx, xRy, WL[4], WR[4], dL[8], dR[8];
-    for (int m = 0; m < 4; ++m) WL[m] = d.W[4 * L + m];
-    for (int m = 0; m < 8; ++m) dL[m] = d.gradW[8 * L + m];
-    if (R >= 0) {
-      xRx = d.xc[2 * R];
-      xRy = d.xc[2 * R + 1];
-      for (int m = 0; m < 4; ++m) WR[m] = d.W[4 * R + m];
-      for (int m = 0; m < 8; ++m) dR[m] = d.gradW[8 * R + m];
-      q0x = 0.5 * (d.q[2 * L] + d.q[2 * R]);
-      q0y = 0.5 * (d.q[2 * L + 1] + d.q[2 * R + 1]);
-      dts = fmin(d.dts[L], d.dts[R]);
+  static_assert(FS_W0 == 0 && NFS == 12, "the first sums are the face state");
+  // face state: of a wall extrapolated from its cell
+  auto face_state = [&](double *W0) {
+    if (wall) {
+      double dx = d.xf[2 * fid] - d.xc[2 * L], dy = d.xf[2 * fid + 1] - d.xc[2 * L + 1];
+      for (int m = 0; m < 4; ++m) W0[m] = d.W[4 * L + m] + (dx * d.gradW[8 * L + 2 * m] + dy * d.gradW[8 * L + 2 * m + 1]);
     } else {
-      double dd = (d.xf[2 * fid] - xLx) * nx + (d.xf[2 * fid + 1] - xLy) * ny;
-      xRx = xLx + 2.0 * dd * nx;
-      xRy = xLy + 2.0 * dd * ny;
-      for (int m = 0; m < 4; ++m) WR[m] = d.ghostW[4 * fid + m];
-      for (int m = 0; m < 8; ++m) dR[m] = 0.0;
-      q0x = 0.5 * d.q[2 * L];
-      q0y = 0.5 * d.q[2 * L + 1];
-      dts = d.dts[L];
+      for (int m = 0; m < 4; ++m) W0[m] = FOLD ? W0f[m][lane] : d.fsum[(size_t)NFS * fid + m];
     }
-    double tx = xRx - xLx, ty = xRy - xLy, it2 = 1.0 / (tx * tx + ty * ty);
-    double ex = tx * it2, ey = ty * it2;
-    for (int m = 0; m < 4; ++m) {
-      W0[m] = fs[FS_W0 + m];
-      double avx = 0.5 * (dL[2 * m] + dR[2 * m]), avy = 0.5 * (dL[2 * m + 1] + dR[2 * m + 1]);
-      double jump = (WR[m] - WL[m]) - (avx * tx + avy * ty);
-      gx[m] = avx + jump * ex;
-      gy[m] = avy + jump * ey;
+  };
+  auto integrals = [&](const Prim &p0) {
+    double qi[5];
+    const double dts = R >= 0 ? fmin(d.dts[L], d.dts[R]) : d.dts[L];
+    time_integrals(dts, collision_time(p0.rho, p0.lam, d.mu_ref, d.omega), qi);
+    const double idts = 1.0 / dts;
+    for (int m = 0; m < 5; ++m) PT[FP_Q1 + m] = (T)(qi[m] * idts);
+    *reinterpret_cast<double2 *>(d.fq12 + 2 * (size_t)fid) = make_double2(qi[0] * idts, qi[1] * idts);
+  };
+  if (need && wrp == 0) {
+    double W0[4], gx[4], gy[4];
+    const double ufx = d.Uf[2 * fid], ufy = d.Uf[2 * fid + 1];
+    face_state(W0);
+    if (wall) {
+      for (int m = 0; m < 4; ++m) {
+        gx[m] = d.gradW[8 * L + 2 * m];
+        gy[m] = d.gradW[8 * L + 2 * m + 1];
+      }
+    } else {
+      double sh = (double)d.face_shiftL[fid];
+      double xLx = d.xc[2 * L] + sh * d.period[2 * L], xLy = d.xc[2 * L + 1] + sh * d.period[2 * L + 1];
+      double xRx, xRy, WL[4], WR[4], dL[8], dR[8];
+      for (int m = 0; m < 4; ++m) WL[m] = d.W[4 * L + m];
+      for (int m = 0; m < 8; ++m) dL[m] = d.gradW[8 * L + m];
+      if (R >= 0) {
+        xRx = d.xc[2 * R];
+        xRy = d.xc[2 * R + 1];
+        for (int m = 0; m < 4; ++m) WR[m] = d.W[4 * R + m];
+        for (int m = 0; m < 8; ++m) dR[m] = d.gradW[8 * R + m];
+      } else {
+        double nx = d.nrm[2 * fid], ny = d.nrm[2 * fid + 1];
+        double dd = (d.xf[2 * fid] - xLx) * nx + (d.xf[2 * fid + 1] - xLy) * ny;
+        xRx = xLx + 2.0 * dd * nx;
+        xRy = xLy + 2.0 * dd * ny;
+        for (int m = 0; m < 4; ++m) WR[m] = d.ghostW[4 * fid + m];
+        for (int m = 0; m < 8; ++m) dR[m] = 0.0;
+      }
+      double tx = xRx - xLx, ty = xRy - xLy, it2 = 1.0 / (tx * tx + ty * ty);
+      double ex = tx * it2, ey = ty * it2;
+      for (int m = 0; m < 4; ++m) {
+        double avx = 0.5 * (dL[2 * m] + dR[2 * m]), avy = 0.5 * (dL[2 * m + 1] + dR[2 * m + 1]);
+        double jump = (WR[m] - WL[m]) - (avx * tx + avy * ty);
+        gx[m] = avx + jump * ex;
+        gy[m] = avy + jump * ey;
+      }
     }
+    Prim p0 = primitive(W0, d.Keff);
+    const SlopeInv<double> inv = slope_inv<double>(p0, d.Keff);
+    double ax[4], ay[4], At[4];
+    micro_slope_r<double>(p0, d.Keff, inv, gx, ax);
+    micro_slope_r<double>(p0, d.Keff, inv, gy, ay);
+    time_slope_r<double>(p0, d.Keff, inv, ax, ay, gx, gy, ufx, ufy, At);
+    PT[FP_RHO] = (T)p0.rho; PT[FP_UX] = (T)p0.ux; PT[FP_UY] = (T)p0.uy; PT[FP_LAM] = (T)p0.lam;
+    for (int m = 0; m < 4; ++m) { PT[FP_AX + m] = (T)ax[m]; PT[FP_AY + m] = (T)ay[m]; PT[FP_AT + m] = (T)At[m]; }
+    PT[FP_PREF] = (T)(0.8 * (1.0 - d.Pr) * p0.lam * p0.lam * inv.irho);
+    PT[FP_HPRE] = (T)(p0.rho * p0.lam * M_1_PI);
+    PT[FP_IL] = (T)inv.il;
+    PT[FP_EH] = (T)(0.5 * d.Keff * inv.il);
+    PT[FP_EB] = (T)(0.5 * (d.Keff + 2.0) * inv.il);
+    if (!FOLD) integrals(p0);
   }
-  // face state, slopes, collision time and time integrals in FP64 on every
-  // path (per face, not per velocity); the mixed path rounds the finished
-  // record once to FP32 for its velocity loops
-  typedef double RT;
-  RT W0r[4], gxr[4], gyr[4];
-  for (int m = 0; m < 4; ++m) { W0r[m] = (RT)W0[m]; gxr[m] = (RT)gx[m]; gyr[m] = (RT)gy[m]; }
-  PrimR<RT> p0 = primitive_r<RT>(W0r, d.Keff);
-  const SlopeInv<RT> inv = slope_inv<RT>(p0, d.Keff);
-  RT ax[4], ay[4], At[4];
-  micro_slope_r<RT>(p0, d.Keff, inv, gxr, ax);
-  micro_slope_r<RT>(p0, d.Keff, inv, gyr, ay);
-  time_slope_r<RT>(p0, d.Keff, inv, ax, ay, gxr, gyr, (RT)ufx, (RT)ufy, At);
-  RT tau = collision_time_r<RT>(p0.rho, p0.lam, (RT)d.mu_ref, (RT)d.omega);
-  RT dtsr = (RT)dts;
-  RT qi[5];
-  time_integrals_r<RT>(dtsr, tau, qi);
-  RT par[NFP];
-  for (int m = 0; m < NFP; ++m) par[m] = RT(0);
-  par[FP_RHO] = p0.rho; par[FP_UX] = p0.ux; par[FP_UY] = p0.uy; par[FP_LAM] = p0.lam;
-  par[FP_QX] = (RT)q0x; par[FP_QY] = (RT)q0y;
-  for (int m = 0; m < 4; ++m) { par[FP_AX + m] = ax[m]; par[FP_AY + m] = ay[m]; par[FP_AT + m] = At[m]; }
-  const RT idts = RT(1) / dtsr;
-  for (int m = 0; m < 5; ++m) par[FP_Q1 + m] = qi[m] * idts;
-  par[FP_UFX] = (RT)ufx; par[FP_UFY] = (RT)ufy;
-  par[FP_PREF] = RT(0.8) * (RT(1) - (RT)d.Pr) * p0.lam * p0.lam * inv.irho;
-  par[FP_HPRE] = p0.rho * p0.lam * RT(M_1_PI);
-  par[FP_IL] = inv.il;
-  par[FP_EH] = RT(0.5) * RT(d.Keff) * par[FP_IL];
-  par[FP_EB] = RT(0.5) * (RT(d.Keff) + RT(2)) * par[FP_IL];
-  par[FP_LAMW] = wall ? (RT)(1.0 / (2.0 * d.face_Tw[fid])) : RT(0);
-  par[FP_RHOW] = RT(0);
-  par[FP_SNX] = (RT)d.Sn[2 * fid];
-  par[FP_SNY] = (RT)d.Sn[2 * fid + 1];
-  par[FP_SUN] = (RT)d.SUn[fid];
-  {
-    double sh = (double)d.face_shiftL[fid];
-    par[FP_DXLX] = (RT)(d.xf[2 * fid] - (d.xc[2 * L] + sh * d.period[2 * L]));
-    par[FP_DXLY] = (RT)(d.xf[2 * fid + 1] - (d.xc[2 * L + 1] + sh * d.period[2 * L + 1]));
-    par[FP_DXRX] = (R >= 0) ? (RT)(d.xf[2 * fid] - d.xc[2 * R]) : RT(0);
-    par[FP_DXRY] = (R >= 0) ? (RT)(d.xf[2 * fid + 1] - d.xc[2 * R + 1]) : RT(0);
+  if (FOLD && need && wrp == 2) {
+    double W0[4];
+    face_state(W0);
+    integrals(primitive(W0, d.Keff));
   }
-  for (int m = 0; m < NFP; ++m) { P[m] = par[m]; PT[m] = (T)par[m]; }
-  // Gamma from the mean of the two cells' W (boundary: the cell)
-  RT Wf[4];
-  for (int m = 0; m < 4; ++m)
-    Wf[m] = (R >= 0) ? RT(0.5) * ((RT)d.W[4 * L + m] + (RT)d.W[4 * R + m]) : (RT)d.W[4 * L + m];
-  PrimR<RT> pf = primitive_r<RT>(Wf, d.Keff);
-  RT pr = pf.rho / (RT(2) * pf.lam);
-  RT gamma = (RT(4) + RT(d.Keff)) / (RT(2) + RT(d.Keff));
-  RT un = (RT)d.SUn[fid] / (RT)d.S[fid];
-  d.gam[fid] = fabs(pf.ux * nx + pf.uy * ny - un) + sqrt(gamma * pr / pf.rho);
+  if (need && wrp == 1) {
+    const double nx = d.nrm[2 * fid], ny = d.nrm[2 * fid + 1], sun = d.SUn[fid];
+    const double fx = d.xf[2 * fid], fy = d.xf[2 * fid + 1], sh = (double)d.face_shiftL[fid];
+    const double half = wall ? 1.0 : 0.5;
+    PT[FP_QX] = (T)(R >= 0 ? 0.5 * (d.q[2 * L] + d.q[2 * R]) : half * d.q[2 * L]);
+    PT[FP_QY] = (T)(R >= 0 ? 0.5 * (d.q[2 * L + 1] + d.q[2 * R + 1]) : half * d.q[2 * L + 1]);
+    PT[FP_UFX] = (T)d.Uf[2 * fid]; PT[FP_UFY] = (T)d.Uf[2 * fid + 1];
+    PT[FP_LAMW] = wall ? (T)(1.0 / (2.0 * d.face_Tw[fid])) : T(0);
+    PT[FP_RHOW] = T(0);
+    PT[FP_SNX] = (T)d.Sn[2 * fid];
+    PT[FP_SNY] = (T)d.Sn[2 * fid + 1];
+    PT[FP_SUN] = (T)sun;
+    PT[FP_DXLX] = (T)(fx - (d.xc[2 * L] + sh * d.period[2 * L]));
+    PT[FP_DXLY] = (T)(fy - (d.xc[2 * L + 1] + sh * d.period[2 * L + 1]));
+    PT[FP_DXRX] = (R >= 0) ? (T)(fx - d.xc[2 * R]) : T(0);
+    PT[FP_DXRY] = (R >= 0) ? (T)(fy - d.xc[2 * R + 1]) : T(0);
+    PT[FP_EB + 1] = T(0);
+    // Gamma from the mean of the two cells' W (boundary: the cell):
+    // |u.n - U.n| + sqrt(gamma p / rho), p / rho = (gamma - 1) e
+    double W[4];
+    for (int m = 0; m < 4; ++m) W[m] = (R >= 0) ? 0.5 * (d.W[4 * L + m] + d.W[4 * R + m]) : d.W[4 * L + m];
+    const double ir = 1.0 / W[0], ux = W[1] * ir, uy = W[2] * ir;
+    const double e = W[3] * ir - 0.5 * (ux * ux + uy * uy);
+    d.gam[fid] = fabs(ux * nx + uy * ny - d.Un[fid]) + sqrt(d.c2fac * e);
+  }
+  __syncthreads();
+  // rows of the record up to the coefficients of the pass below
+  T *out = reinterpret_cast<T *>(d.fparT) + (size_t)f0 * NFP;
+  for (int t = threadIdx.x; t < FSC * FP_IH; t += blockDim.x) {
+    const int r = t / FP_IH, m = t - r * FP_IH;
+    if (live[r]) out[(size_t)r * NFP + m] = rec[r * ROW + m];
+  }
 }
 
 // Face coefficients, velocity part (one warp per face): the g-part of the
@@ -502,18 +528,21 @@ __device__ __forceinline__ void face_eq_flux_separable(const Dev &d, const R *P,
   out[3] = hpre * p2_sum(p2_mul(ws, e3), mx, my);
 }
 
-// Velocity-loop face coefficients for the faces of `list` (all faces when
-// null): FCW warps per face split the velocities, their warp totals meet in
-// shared memory (summed in warp order).  The FP32 path runs it over the wall
-// faces only.
-constexpr int FCW = 4;
-template <typename T> __global__ void __launch_bounds__(256, 2) k_face_coef(Dev d, const int *list, int n) {
-  __shared__ double part[256 / 32][9];
+// Face coefficients, velocity part, in one launch: its first CTAs take the
+// walls (a longer job per face), the others every other face (two launches one
+// after the other: 16.7 us, one: 9.1, 1056 faces, 64 of them walls; 74112
+// faces: 63 -> 55).
+//
+// Wall faces (`list`, n of them): FCW warps per face split the velocities,
+// their warp totals meet in shared memory (summed in warp order).
+constexpr int FCW = 4, FC_THREADS = 256;
+template <typename T> __device__ __forceinline__ void wall_coef(const Dev &d, const int *list, int n) {
+  __shared__ double part[FC_THREADS / 32][9];
   int wg = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   int w = wg / FCW, sub = wg - (wg / FCW) * FCW;
   int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
   bool in = w < n;
-  int fid = in ? (list ? list[w] : w) : 0;
+  int fid = in ? list[w] : 0;
   int kind = in ? d.face_kind[fid] : BC_OVERSET;
   bool act = in && kind != BC_OVERSET && face_needed(d, fid);
   if (in && !act && sub == 0) {
@@ -564,15 +593,14 @@ template <typename T> __global__ void __launch_bounds__(256, 2) k_face_coef(Dev 
       acc[m] = part[wl][m];
       for (int j = 1; j < FCW; ++j) acc[m] += part[wl + j][m];
     }
-    double *P = d.fpar + (size_t)NFP * fid;
+    const double *P = d.fq12 + 2 * (size_t)fid;
     T *PT = reinterpret_cast<T *>(d.fparT) + (size_t)NFP * fid;
     const double *fs = d.fsum + NFS * fid;
     double F[4];
     for (int m = 0; m < 4; ++m)
-      F[m] = P[FP_Q1] * fs[FS_FF + m] + P[FP_Q2] * fs[FS_WG + m] + acc[m];
+      F[m] = P[0] * fs[FS_FF + m] + P[1] * fs[FS_WG + m] + acc[m];
     if (wall) {
       double rhow = -F[0] / acc[8];
-      P[FP_RHOW] = rhow;
       PT[FP_RHOW] = (T)rhow;
       for (int m = 0; m < 4; ++m) F[m] += rhow * acc[4 + m];
     }
@@ -587,13 +615,12 @@ template <typename T> __global__ void __launch_bounds__(256, 2) k_face_coef(Dev 
   }
 }
 
-// Face coefficients of the non-wall faces: FCG lanes per face, the
-// equilibrium part of the macro flux from 1D velocity moments (exact
-// separable rewrite of the tensor-grid sum); faces outside the field get
-// zero flux.
+// The non-wall faces: FCG lanes per face, the equilibrium part of the macro
+// flux from 1D velocity moments (exact separable rewrite of the tensor-grid
+// sum); faces outside the field get zero flux.  block: index among their CTAs.
 constexpr int FCG = 8;
-template <typename T> __global__ void __launch_bounds__(256) k_face_coef_sep(Dev d) {
-  int t = blockIdx.x * blockDim.x + threadIdx.x;
+template <typename T> __device__ __forceinline__ void sep_coef(const Dev &d, int block) {
+  int t = block * blockDim.x + threadIdx.x;
   int fid = t / FCG, sub = t % FCG;
   bool in = fid < d.nf;
   int kind = in ? d.face_kind[fid] : BC_OVERSET;
@@ -624,41 +651,40 @@ template <typename T> __global__ void __launch_bounds__(256) k_face_coef_sep(Dev
       if (m % FCG == sub) PT[FP_IH + m] = m < 10 ? ih.c[m] : ib.c[m - 10];
   }
   if (act && sub < 4) {                           // lane m of the group: component m
-    const double *P = d.fpar + (size_t)NFP * fid;
+    const double *P = d.fq12 + 2 * (size_t)fid;
     const double *fs = d.fsum + NFS * fid;
     T om = sub == 0 ? o[0] : sub == 1 ? o[1] : sub == 2 ? o[2] : o[3];
-    d.fflux[4 * fid + sub] = P[FP_Q1] * fs[FS_FF + sub] + P[FP_Q2] * fs[FS_WG + sub] + to_double(om);
+    d.fflux[4 * fid + sub] = P[0] * fs[FS_FF + sub] + P[1] * fs[FS_WG + sub] + to_double(om);
   }
+}
+
+template <typename T> __global__ void __launch_bounds__(FC_THREADS, sizeof(T) == 4 ? 2 : 1) k_face_coef(Dev d, int wall_blocks) {
+  if ((int)blockIdx.x < wall_blocks) wall_coef<T>(d, d.wall_faces, d.nwall);
+  else sep_coef<T>(d, (int)blockIdx.x - wall_blocks);
 }
 
 // Per-cell sum of the S-weighted macro fluxes (Eq. macroscopicFlux summed
 // over the faces); with level_n also the extensive level-n macro term
-// TW = Omega^n W^n / dt - F^n / 2 (reading R4).
+// TW = Omega^n W^n / dt - F^n / 2 (reading R4).  (The inner iterations sum it
+// while they gather the macro sweep's records.)
 __global__ void k_cell_macro(Dev d, int level_n) {
-  int c = blockIdx.x * blockDim.x + threadIdx.x;
+  int t = blockIdx.x * blockDim.x + threadIdx.x;
+  int c = t >> 2, m = t & 3;
   if (c >= d.nc) return;
-  double F[4] = {0, 0, 0, 0};
-  for (int s = 0; s < 4; ++s) {
-    int f = d.cell_faces[4 * c + s];
-    double sg = (double)d.cell_sgn[4 * c + s];
-    for (int m = 0; m < 4; ++m) F[m] += sg * d.fflux[4 * f + m];
-  }
-  for (int m = 0; m < 4; ++m) d.Fc[4 * c + m] = F[m];
-  if (level_n)
-    for (int m = 0; m < 4; ++m) d.TW[4 * c + m] = d.vol_old[c] / d.stepc[0] * d.W[4 * c + m] - 0.5 * F[m];
+  const double F = cell_flux_sum(d, c, m);
+  d.Fc[t] = F;
+  if (level_n) d.TW[t] = d.vol_old[c] / d.stepc[0] * d.W[t] - 0.5 * F;
 }
 
-// Cell parameter record (prim, q, 1/tau) from W and q, and its Shakhov
-// record in the arithmetic type (level n).
-template <typename T> __global__ void k_cell_params(Dev d, const double *Wsrc, double *out) {
+// Shakhov record in the arithmetic type from W and q (level n).
+template <typename T> __global__ void k_cell_params(Dev d) {
   int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= d.nc) return;
-  Prim p = primitive(Wsrc + 4 * c, d.Keff);
-  double *o = out + NCP * c;
+  Prim p = primitive(d.W + 4 * c, d.Keff);
+  double o[NCP];
   o[CP_RHO] = p.rho; o[CP_UX] = p.ux; o[CP_UY] = p.uy; o[CP_LAM] = p.lam;
   o[CP_QX] = d.q[2 * c]; o[CP_QY] = d.q[2 * c + 1];
   o[CP_ITAU] = 1.0 / collision_time(p.rho, p.lam, d.mu_ref, d.omega);
-  o[CP_DBASE] = 0.0;
   write_shrec<T>(d, o, d.vol_old[c], reinterpret_cast<T *>(d.shn) + (size_t)NSH * c);
 }
 
@@ -980,28 +1006,27 @@ void launch_slope_geo(const Dev &d, cudaStream_t s) { k_slope_geo<<<nblk(d.nc, 2
 
 void launch_ghost_gradW(const Dev &d, cudaStream_t s) {
   k_ghost<<<nblk(d.nf, 256), 256, 0, s>>>(d);
-  k_gradW<<<nblk(d.nc, 256), 256, 0, s>>>(d);
+  launch_gradW(d, s);
 }
-void launch_gradW(const Dev &d, cudaStream_t s) { k_gradW<<<nblk(d.nc, 256), 256, 0, s>>>(d); }
+void launch_gradW(const Dev &d, cudaStream_t s) {
+  k_gradW<<<nblk(4 * (size_t)d.nc, GW_THREADS), GW_THREADS, 0, s>>>(d);
+}
+template <typename T> static void face_coef(const Dev &d, cudaStream_t s) {
+  if (d.nsplit > 1) k_face_scalar<T, true><<<nblk(d.nf, FSC), 128, 0, s>>>(d);
+  else k_face_scalar<T, false><<<nblk(d.nf, FSC), 64, 0, s>>>(d);
+  const int walls = nblk((size_t)d.nwall * 32 * FCW, FC_THREADS);
+  k_face_coef<T><<<walls + nblk((size_t)d.nf * FCG, FC_THREADS), FC_THREADS, 0, s>>>(d, walls);
+}
 void launch_face_coef(const Dev &d, cudaStream_t s, int fp32) {
-  if (fp32) {
-    k_face_scalar<float><<<nblk(d.nf, 128), 128, 0, s>>>(d);
-    k_face_coef_sep<float><<<nblk((size_t)d.nf * FCG, 256), 256, 0, s>>>(d);
-    if (d.nwall > 0)
-      k_face_coef<float><<<nblk((size_t)d.nwall * 32 * FCW, 256), 256, 0, s>>>(d, d.wall_faces, d.nwall);
-  } else {
-    k_face_scalar<double><<<nblk(d.nf, 128), 128, 0, s>>>(d);
-    k_face_coef_sep<double><<<nblk((size_t)d.nf * FCG, 256), 256, 0, s>>>(d);
-    if (d.nwall > 0)
-      k_face_coef<double><<<nblk((size_t)d.nwall * 32 * FCW, 256), 256, 0, s>>>(d, d.wall_faces, d.nwall);
-  }
+  if (fp32) face_coef<float>(d, s);
+  else face_coef<double>(d, s);
 }
 void launch_cell_macro(const Dev &d, cudaStream_t s, int level_n) {
-  k_cell_macro<<<nblk(d.nc, 256), 256, 0, s>>>(d, level_n);
+  k_cell_macro<<<nblk(4 * (size_t)d.nc, 128), 128, 0, s>>>(d, level_n);
 }
-void launch_cell_params(const Dev &d, cudaStream_t s, const double *W, double *out, int fp32) {
-  if (fp32) k_cell_params<float><<<nblk(d.nc, 256), 256, 0, s>>>(d, W, out);
-  else k_cell_params<double><<<nblk(d.nc, 256), 256, 0, s>>>(d, W, out);
+void launch_cell_params(const Dev &d, cudaStream_t s, int fp32) {
+  if (fp32) k_cell_params<float><<<nblk(d.nc, 32), 32, 0, s>>>(d);
+  else k_cell_params<double><<<nblk(d.nc, 32), 32, 0, s>>>(d);
 }
 void launch_moments_finish(const Dev &d, cudaStream_t s) { k_moments_finish<<<nblk(d.nc, 256), 256, 0, s>>>(d); }
 // Two cells (warps) a CTA: small CTAs fit beside the velocity reduction's

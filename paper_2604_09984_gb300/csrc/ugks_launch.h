@@ -12,7 +12,7 @@ void launch_ghost_gradW(const Dev &d, cudaStream_t s);                      // 2
 void launch_gradW(const Dev &d, cudaStream_t s);                            // the gradients alone
 void launch_face_coef(const Dev &d, cudaStream_t s, int fp32);
 void launch_cell_macro(const Dev &d, cudaStream_t s, int level_n);
-void launch_cell_params(const Dev &d, cudaStream_t s, const double *W, double *out, int fp32);
+void launch_cell_params(const Dev &d, cudaStream_t s, int fp32);
 // macro LU-SGS (ugks_macro.cu); rows: of the tallest block
 int macro_pad(int rows, int fp32);                     // padding diagonals of the records
 size_t macro_cells(int ni, int nj, int pad);           // records of a block

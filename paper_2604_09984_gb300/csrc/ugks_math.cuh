@@ -145,31 +145,26 @@ template <typename R> UG_HD void time_integrals_r(R dts, R tau, R q[5]) {
     q[4] = R(0.5) * dts * dts - tau * dts + tau * tau * em;
     return;
   }
-  // q1/dts = sum_{m>=1} (-1)^{m+1} x^{m-1}/m!
-  // q2/dts^2 = sum_{m>=2} (-1)^{m+1} (m-1) x^{m-2}/m!
-  // q4/dts^2 = sum_{m>=3} (-1)^{m+1} (2-m) x^{m-2}/m!
-  // q5/dts^2 = sum_{m>=3} (-1)^{m+1} x^{m-2}/m!
-  R s1 = 0, s2 = 0, s4 = 0, s5 = 0;
-  R xp = 1;       // x^{m-1}
-  R xm2 = 0;      // x^{m-2}
-  R ifac = 1;     // 1/m!
+  // q4/dts^2 = s4 = sum_{m>=3} (-1)^{m+1} (2-m) x^{m-2}/m!
+  // q5/dts^2 = s5 = sum_{m>=3} (-1)^{m+1} x^{m-2}/m!
+  // q1/dts   = sum_{m>=1} (-1)^{m+1} x^{m-1}/m! = 1 - x/2 + x s5
+  // q2/dts^2 = sum_{m>=2} (-1)^{m+1} (m-1) x^{m-2}/m! = -1/2 + s5 - s4
+  constexpr int N = SeriesTerms<R>::N;
+  double c[N + 1];                // (-1)^{m+1} / m!, folded by the compiler
+  c[0] = -1.0;
 #pragma unroll
-  for (int m = 1; m <= SeriesTerms<R>::N; ++m) {
-    ifac *= R(1) / R(m);
-    R tm = ((m & 1) ? R(1) : R(-1)) * ifac;
-    s1 += tm * xp;
-    if (m >= 2) {
-      s2 += tm * R(m - 1) * xm2;
-      if (m >= 3) {
-        s4 += tm * R(2 - m) * xm2;
-        s5 += tm * xm2;
-      }
-    }
-    xm2 = xp;
-    xp *= x;
+  for (int m = 1; m <= N; ++m) c[m] = -c[m - 1] / m;
+  R s4 = 0, s5 = 0;
+#pragma unroll
+  for (int m = N; m >= 3; --m) {
+    s4 = s4 * x + (R)(c[m] * (2 - m));
+    s5 = s5 * x + (R)c[m];
   }
+  s4 *= x;
+  s5 *= x;
+  const R s1 = R(1) - R(0.5) * x + x * s5;
   q[0] = dts * s1;
-  q[1] = dts * dts * s2;
+  q[1] = dts * dts * (s5 - s4 - R(0.5));
   q[2] = dts - dts * s1;
   q[3] = dts * dts * s4;
   q[4] = dts * dts * s5;
