@@ -1466,7 +1466,7 @@ int ugks_eval_flux(ugks_ctx *ctx, double *D, double *F) {
   do_interp(ctx, 0);
   int r = flux_prep(ctx, 0, true);
   if (r) return r;
-  if (D) { launch_flux_div_all(d, ctx->st, D, ctx->fp32); ctx->launches += 1; }
+  if (D) { launch_flux_eval(d, ctx->st, D, ctx->fp32); ctx->launches += 1; }
   if (F) CK(cudaMemcpyAsync(F, d.Fc, sizeof(double) * 4 * d.nc, cudaMemcpyDefault, ctx->st));
   CK(cudaStreamSynchronize(ctx->st));
   return launch_status(ctx);

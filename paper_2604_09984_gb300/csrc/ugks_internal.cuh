@@ -416,57 +416,6 @@ template <typename T> __device__ __forceinline__ T dwa(const Dev &d, int k);
 template <> __device__ __forceinline__ double dwa<double>(const Dev &d, int k) { return d.wa[k]; }
 template <> __device__ __forceinline__ float dwa<float>(const Dev &d, int k) { return d.waf[k]; }
 
-// value of the cell field f at velocity k for neighbour slot `s` of cell c
-// (cell neighbour or ghost Maxwellian of the ghost state)
-template <typename T>
-__device__ __forceinline__ V2<T> nb_value(const Dev &d, int c, int s, int k) {
-  int kind = d.nb_kind[c * 4 + s];
-  int id = d.nb_id[c * 4 + s];
-  if (kind == NB_CELL) {
-    auto v = ldF<T>(d, (size_t)id * d.nvp + k);
-    return {v.x, v.y};
-  }
-  const double *g = d.ghostW + 4 * id;
-  Prim p = primitive(g, d.Keff);
-  return maxwellian<T>((T)p.rho, (T)p.ux, (T)p.uy, (T)p.lam, dvx<T>(d, k), dvy<T>(d, k),
-                       (T)d.Keff);
-}
-
-// Limited Cartesian gradient of (h, b) of cell c at velocity k (reading R1:
-// van Leer on both-sided centre differences, one-sided where a side has no
-// neighbour, mapped with the inverse Jacobian of the centre differences).
-template <typename T>
-__device__ __forceinline__ void grad_f(const Dev &d, int c, int k, V2<T> fc, V2<T> &gx,
-                                       V2<T> &gy) {
-  int fl = d.slope_flags[c];
-  V2<T> s[2];
-#pragma unroll
-  for (int dir = 0; dir < 2; ++dir) {
-    int cs = (fl >> (2 * dir)) & 3;
-    V2<T> r = {T(0), T(0)};
-    if (cs == SL_BOTH) {
-      V2<T> m = nb_value<T>(d, c, 2 * dir, k), p = nb_value<T>(d, c, 2 * dir + 1, k);
-      r.h = vanleer<T>(fc.h - m.h, p.h - fc.h);
-      r.b = vanleer<T>(fc.b - m.b, p.b - fc.b);
-    } else if (cs == SL_P) {
-      V2<T> p = nb_value<T>(d, c, 2 * dir + 1, k);
-      r.h = p.h - fc.h;
-      r.b = p.b - fc.b;
-    } else if (cs == SL_M) {
-      V2<T> m = nb_value<T>(d, c, 2 * dir, k);
-      r.h = fc.h - m.h;
-      r.b = fc.b - m.b;
-    }
-    s[dir] = r;
-  }
-  const double *J = d.jinv + 4 * c;
-  T i11 = (T)J[0], i12 = (T)J[1], i21 = (T)J[2], i22 = (T)J[3];
-  gx.h = i11 * s[0].h + i12 * s[1].h;
-  gx.b = i11 * s[0].b + i12 * s[1].b;
-  gy.h = i21 * s[0].h + i22 * s[1].h;
-  gy.b = i21 * s[0].b + i22 * s[1].b;
-}
-
 // Copy a record of N values (N * sizeof(T) a multiple of 16, 16-byte aligned)
 // into registers with 128-bit loads.
 template <typename T, int N> __device__ __forceinline__ void load_rec(const T *src, T *dst) {
@@ -475,10 +424,6 @@ template <typename T, int N> __device__ __forceinline__ void load_rec(const T *s
   float4 *o = reinterpret_cast<float4 *>(dst);
 #pragma unroll
   for (int q = 0; q < (int)(N * sizeof(T) / 16); ++q) o[q] = __ldg(s + q);
-}
-
-template <typename T> __device__ __forceinline__ const T *fparT(const Dev &d, int f) {
-  return reinterpret_cast<const T *>(d.fparT) + (size_t)f * NFP;
 }
 
 // Bivariate polynomials sum_{a+b<=D} c_ab cx^a cy^b, coefficients stored
@@ -596,87 +541,6 @@ __device__ __forceinline__ void interface_polys(const R *P, R Keff, R Kint, Poly
 template <typename R> __device__ __forceinline__ void store_polys(R *P, const Poly2<3, R> &ih, const Poly2<3, R> &ib) {
 #pragma unroll
   for (int m = 0; m < 10; ++m) { P[FP_IH + m] = ih.c[m]; P[FP_IB + m] = ib.c[m]; }
-}
-
-// S * time-averaged interface flux of velocity k through face fid, oriented
-// along the face normal (L -> R, outward for boundary faces).
-template <typename T> __device__ V2<T> face_flux(const Dev &d, int fid, int k) {
-  T vx = dvx<T>(d, k), vy = dvy<T>(d, k);
-  T wS = vx * (T)d.Sn[2 * fid] + vy * (T)d.Sn[2 * fid + 1] - (T)d.SUn[fid];
-  const T *P = fparT<T>(d, fid);
-  int kind = d.face_kind[fid];
-  int L = d.face_L[fid];
-  T ufx = P[FP_UFX], ufy = P[FP_UFY];
-  T wx = vx - ufx, wy = vy - ufy;
-  V2<T> ff, wgf;
-  if (kind == BC_WALL) {
-    if (!(wS > T(0))) {
-      // reflected part: wall Maxwellian at the face velocity (Eq. maxWalldes)
-      T lw = P[FP_LAMW];
-      T Hw = P[FP_RHOW] * (lw * T(M_1_PI)) * r_exp<T>(-lw * (wx * wx + wy * wy));
-      return {wS * Hw, wS * (T)d.Keff / (T(2) * lw) * Hw};
-    }
-    auto fv = ldF<T>(d, (size_t)L * d.nvp + k);
-    V2<T> fc = {fv.x, fv.y}, gx, gy;
-    grad_f<T>(d, L, k, fc, gx, gy);
-    T dx = (T)(d.xf[2 * fid] - d.xc[2 * L]), dy = (T)(d.xf[2 * fid + 1] - d.xc[2 * L + 1]);
-    ff = {fc.h + dx * gx.h + dy * gy.h, fc.b + dx * gx.b + dy * gy.b};
-    wgf = {wx * gx.h + wy * gy.h, wx * gx.b + wy * gy.b};
-  } else {
-    int R = d.face_R[fid];
-    bool useL = wS > T(0), useR = wS < T(0);
-    V2<T> fL = {0, 0}, fR = {0, 0}, gL = {0, 0}, gR = {0, 0};
-    if (!useR) {
-      auto fv = ldF<T>(d, (size_t)L * d.nvp + k);
-      V2<T> fc = {fv.x, fv.y}, gx, gy;
-      grad_f<T>(d, L, k, fc, gx, gy);
-      double sh = (double)d.face_shiftL[fid];
-      T dx = (T)(d.xf[2 * fid] - (d.xc[2 * L] + sh * d.period[2 * L]));
-      T dy = (T)(d.xf[2 * fid + 1] - (d.xc[2 * L + 1] + sh * d.period[2 * L + 1]));
-      fL = {fc.h + dx * gx.h + dy * gy.h, fc.b + dx * gx.b + dy * gy.b};
-      gL = {wx * gx.h + wy * gy.h, wx * gx.b + wy * gy.b};
-    }
-    if (!useL) {
-      if (R >= 0) {
-        auto fv = ldF<T>(d, (size_t)R * d.nvp + k);
-        V2<T> fc = {fv.x, fv.y}, gx, gy;
-        grad_f<T>(d, R, k, fc, gx, gy);
-        T dx = (T)(d.xf[2 * fid] - d.xc[2 * R]), dy = (T)(d.xf[2 * fid + 1] - d.xc[2 * R + 1]);
-        fR = {fc.h + dx * gx.h + dy * gy.h, fc.b + dx * gx.b + dy * gy.b};
-        gR = {wx * gx.h + wy * gy.h, wx * gx.b + wy * gy.b};
-      } else {
-        const double *g = d.ghostW + 4 * fid;
-        Prim p = primitive(g, d.Keff);
-        fR = maxwellian<T>((T)p.rho, (T)p.ux, (T)p.uy, (T)p.lam, vx, vy, (T)d.Keff);
-      }
-    }
-    if (useL) {
-      ff = fL; wgf = gL;
-    } else if (useR) {
-      ff = fR; wgf = gR;
-    } else {
-      ff = {T(0.5) * (fL.h + fR.h), T(0.5) * (fL.b + fR.b)};
-      wgf = {T(0.5) * (gL.h + gR.h), T(0.5) * (gL.b + gR.b)};
-    }
-  }
-  V2<T> I = interface_integral<T>(P, vx, vy, ff, wgf, (T)d.Keff, (T)d.Kint, (T)d.Pr);
-  return {wS * I.h, wS * I.b};
-}
-
-// D_ik = sum over the faces of cell c of S F_hat (outward positive).
-template <typename T> __device__ V2<T> flux_div(const Dev &d, int c, int k) {
-  V2<T> acc = {T(0), T(0)};
-#pragma unroll
-  for (int s = 0; s < 4; ++s) {
-    int fid = d.cell_faces[c * 4 + s];
-    int kind = d.face_kind[fid];
-    if (kind == BC_OVERSET) continue;   // outer edge of a component grid: receptors only
-    V2<T> F = face_flux<T>(d, fid, k);
-    T sg = (T)d.cell_sgn[c * 4 + s];
-    acc.h += sg * F.h;
-    acc.b += sg * F.b;
-  }
-  return acc;
 }
 
 }  // namespace ugks

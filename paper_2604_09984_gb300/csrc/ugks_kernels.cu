@@ -809,18 +809,6 @@ template <typename T> __global__ void k_init_state(Dev d, const double *prim) {
   }
 }
 
-// Diagnostic: D_ik for every (cell, velocity), written as FP64.
-template <typename T> __global__ void k_flux_div_all(Dev d, double *D) {
-  size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  size_t n = (size_t)d.nc * d.nv;
-  if (t >= n) return;
-  int c = (int)(t / d.nv), k = (int)(t % d.nv);
-  V2<T> r = {0, 0};
-  if (d.status[c] == ST_FIELD) r = flux_div<T>(d, c, k);
-  D[2 * t] = (double)r.h;
-  D[2 * t + 1] = (double)r.b;
-}
-
 // Sum of S * wall macro flux per block: one CTA per block, a strided partial
 // sum per thread and a fixed-shape tree, so the order (and the result) is
 // the same on every call.
@@ -1041,11 +1029,6 @@ void launch_moments(const Dev &d, cudaStream_t s, int fp32) {
 void launch_init_state(const Dev &d, cudaStream_t s, const double *prim, int fp32) {
   if (fp32) k_init_state<float><<<nblk((size_t)d.nc * 32, 256), 256, 0, s>>>(d, prim);
   else k_init_state<double><<<nblk((size_t)d.nc * 32, 256), 256, 0, s>>>(d, prim);
-}
-void launch_flux_div_all(const Dev &d, cudaStream_t s, double *D, int fp32) {
-  size_t n = (size_t)d.nc * d.nv;
-  if (fp32) k_flux_div_all<float><<<nblk(n, 256), 256, 0, s>>>(d, D);
-  else k_flux_div_all<double><<<nblk(n, 256), 256, 0, s>>>(d, D);
 }
 void launch_wall_loads(const Dev &d, cudaStream_t s) { k_wall_loads<<<d.nblocks, WL_THREADS, 0, s>>>(d); }
 void launch_wall_torque(const Dev &d, cudaStream_t s, const double *ctr, double *out) {

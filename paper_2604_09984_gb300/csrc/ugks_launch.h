@@ -35,7 +35,7 @@ void launch_moments_finish(const Dev &d, cudaStream_t s);   // sharded step, aft
 // (|r|^2), 2 after the moments (|W - W'|^2, totals; 2 kernels)
 void launch_metrics(const Dev &d, cudaStream_t s, int stage, int fp32);
 void launch_init_state(const Dev &d, cudaStream_t s, const double *prim, int fp32);
-void launch_flux_div_all(const Dev &d, cudaStream_t s, double *D, int fp32);
+void launch_flux_eval(const Dev &d, cudaStream_t s, double *D, int fp32);   // the flux sums to the caller's D
 void launch_wall_loads(const Dev &d, cudaStream_t s);
 void launch_wall_torque(const Dev &d, cudaStream_t s, const double *ctr, double *out);
 void launch_f_convert(const Dev &d, cudaStream_t s, double *out, const double *in, int fp32);
