@@ -16,12 +16,6 @@
 
 using namespace ugks;
 
-// (cell, velocity) items per diagonal step of the longest macro sweep below
-// which the flux pass plus the residual's first pass end within the sweep,
-// from the rates measured on GB300: ~1.0e-11 s and ~4.8e-12 s per item for
-// the two, ~0.8 us per diagonal step of the sweep
-constexpr double kResidualWindow = 5.3e4;
-
 struct ugks_ctx {
   ugks_params p;
   cudaStream_t st = nullptr;
@@ -35,11 +29,8 @@ struct ugks_ctx {
   // (which reads none of them); not where an outflow ghost state follows W
   // or on a velocity shard (whose Step 7 waits for the host exchange)
   bool split_tail = false;
-  // FP32 path: the residual's predictor-free part beside the macro sweep,
-  // where the flux pass and that part end within the sweep (not on the FP64
-  // path, where the flux pass alone outlasts it, nor for velocity grids large
-  // against the sweep's length); not within a batch of several instances,
-  // whose other steps fill the SMs the sweep leaves
+  // the residual in two passes (residual_split); not within a batch of several
+  // instances, whose other steps fill the SMs the sweep leaves
   bool split_residual = false;
   bool in_batch = false;
   char *ws = nullptr;
@@ -581,7 +572,8 @@ int shard_exchange(ugks_ctx *ctx, int which) {
 // The step size where the step's kernels read it (stream-ordered upload).
 int upload_step_size(ugks_ctx *ctx) {
   const Dev &d = ctx->d;
-  double v[4] = {d.dt, d.idt, (double)d.idt_f, 0.0};
+  double v[4] = {d.dt, d.idt, 0.0, 0.0};
+  memcpy(&v[2], &d.idt_f, sizeof(float));
   return launch_upload(const_cast<double *>(d.stepc), v, sizeof(v), ctx->st);
 }
 
@@ -711,16 +703,11 @@ int step_body(ugks_ctx *ctx, int n_inner) {
     { Prof p(ctx, UGKS_PROF_MACRO_SWEEP, ctx->side); launch_macro_sweep(d, ctx->side, ctx->max_nj, fp); }
     CK(cudaEventRecord(ctx->ev_macro, ctx->side));
     { Prof p(ctx, UGKS_PROF_RHS); launch_flux(d, s, fp); }              // Step 3
-    if (ctx->split_residual && !ctx->in_batch) {
-      // Step 5 without the predictor's collision term while the sweep runs
-      { Prof p(ctx, UGKS_PROF_RESIDUAL); launch_residual(d, s, it == 0, fp, 1); }
-      CK(cudaStreamWaitEvent(s, ctx->ev_macro, 0));
-      { Prof p(ctx, UGKS_PROF_RESIDUAL); launch_residual(d, s, it == 0, fp, 2); }
-      ctx->launches += 1;
-    } else {
-      CK(cudaStreamWaitEvent(s, ctx->ev_macro, 0));
-      { Prof p(ctx, UGKS_PROF_RESIDUAL); launch_residual(d, s, it == 0, fp); }               // Step 5
-    }
+    const bool two = ctx->split_residual && !ctx->in_batch;            // Step 5
+    if (two) { Prof p(ctx, UGKS_PROF_RESIDUAL); launch_residual(d, s, it == 0, fp, 1); }
+    CK(cudaStreamWaitEvent(s, ctx->ev_macro, 0));
+    { Prof p(ctx, UGKS_PROF_RESIDUAL); launch_residual(d, s, it == 0, fp, two ? 2 : 0); }
+    if (two) ctx->launches += 1;
     if (met) launch_metrics(d, s, 1, fp);
     { Prof p(ctx, UGKS_PROF_MICRO_FWD); launch_wsweep(d, s, 0, ctx->work, ctx->nwork, ctx->sweep_nw, ctx->ns_fwd, ctx->sweep_rg, fp); }  // Step 6
     { Prof p(ctx, UGKS_PROF_MICRO_BWD); launch_wsweep(d, s, 1, ctx->work, ctx->nwork, ctx->sweep_nw, ctx->ns_bwd, ctx->sweep_rg, fp); }
@@ -1126,11 +1113,9 @@ int ugks_init_mesh(ugks_ctx *ctx, int nblocks, const ugks_block_desc *blocks, co
     for (int f = 0; f < s.nf; ++f) outflow = outflow || T.face_kind[f] == BC_OUTFLOW;
     const char *e = getenv("UGKS_SERIAL_TAIL");      // 1: Step 7 and the gradients in line
     ctx->split_tail = !outflow && !d.shard && !(e && atoi(e) != 0);
-    const char *e1 = getenv("UGKS_RESIDUAL_ONE_PASS");   // 1: the residual in one pass
-    long steps = 0;                                       // diagonal steps of the longest macro sweep
+    long steps = 0;                                  // diagonals of the longest macro sweep
     for (int b = 0; b < nblocks; ++b) steps = std::max(steps, 2L * (blocks[b].ni + blocks[b].nj - 1));
-    double items = (double)s.nc * s.nv;
-    ctx->split_residual = ctx->fp32 && !(e1 && atoi(e1) != 0) && items < kResidualWindow * (double)steps;
+    ctx->split_residual = residual_split((long)s.nc * s.nv, steps, ctx->fp32);
   }
   {
     std::vector<int> wf;

@@ -690,6 +690,14 @@ template <typename T> __global__ void k_cell_params(Dev d) {
 
 // Step 7 (one warp per cell): W^{s+1} = W' + sum V Psi (f^{s+1} - g(W')),
 // heat flux about V' (reading R7); flags non-physical states.
+//
+// FP32: streaming f.  FP64: its pipe (some 15 cycles a warp instruction and
+// SM), so the exponential of g (thirty of them) splits into a factor per column
+// and one per row, tabulated first by the warp, and the sums share their
+// products (40 -> 21 a velocity; 96x48 + 64x16 cells, 1024 velocities: 454 -> 272
+// us).  A velocity grid of more than MOM_TAB columns and rows keeps one
+// exponential a velocity.
+constexpr int MOM_THREADS = 64, MOM_TAB = 256;
 template <typename T, int FB> __global__ void k_moments(Dev d) {
   int c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   int lane = threadIdx.x & 31;
@@ -701,7 +709,47 @@ template <typename T, int FB> __global__ void k_moments(Dev d) {
   Acc<T> a[6];
   typedef typename Vec2<T>::type T2;
   constexpr int NB = 4;                     // loads of a lane in flight per batch
-  for (int kb = lane; kb < d.nv; kb += 32 * NB) {
+  constexpr bool SEP = sizeof(T) == 8;
+  __shared__ T tab[SEP ? MOM_THREADS / 32 : 1][SEP ? MOM_TAB : 1];
+  const int rows = SEP ? d.nv / d.nvx : 0;
+  const bool sep = SEP && d.nvx + rows <= MOM_TAB;
+  if (sep) {
+    T *ex = tab[(threadIdx.x >> 5) % (SEP ? MOM_THREADS / 32 : 1)], *ey = ex + d.nvx;
+    for (int i = lane; i < d.nvx + rows; i += 32) {
+      const T u = i < d.nvx ? dvx<T>(d, i) - ux : dvy<T>(d, (i - d.nvx) * d.nvx) - uy;
+      ex[i] = (i < d.nvx ? hpre : T(1)) * r_exp<T>(-lam * u * u);
+    }
+    __syncwarp();
+    for (int kb = lane; kb < d.nv; kb += 32 * NB) {
+      T2 fb[NB];
+#pragma unroll
+      for (int u = 0; u < NB; ++u) {
+        int k = kb + 32 * u;
+        fb[u] = k < d.nv ? ldF<T, FB>(d, (size_t)c * d.nvp + k) : T2{T(0), T(0)};
+      }
+      T p[6] = {T(0), T(0), T(0), T(0), T(0), T(0)};
+#pragma unroll
+      for (int u = 0; u < NB; ++u) {
+        const int k = kb + 32 * u;
+        if (k >= d.nv) break;
+        const int iy = k / d.nvx, ix = k - iy * d.nvx;
+        const T vx = dvx<T>(d, k), vy = dvy<T>(d, k), w = dw<T>(d, k), hw = T(0.5) * w;
+        const T h = fb[u].x, b = fb[u].y, H = ex[ix] * ey[iy];
+        const T wd = w * (h - H);
+        p[0] += wd;
+        p[1] += vx * wd;
+        p[2] += vy * wd;
+        p[3] += T(0.5) * (vx * vx + vy * vy) * wd + hw * (b - bfac * H);
+        const T cx = vx - ux, cy = vy - uy;
+        const T e = hw * ((cx * cx + cy * cy) * h + b);
+        p[4] += cx * e;
+        p[5] += cy * e;
+      }
+#pragma unroll
+      for (int m = 0; m < 6; ++m) a[m].add(p[m]);
+    }
+  }
+  for (int kb = sep ? d.nv : lane; kb < d.nv; kb += 32 * NB) {
     T2 fb[NB];
 #pragma unroll
     for (int u = 0; u < NB; ++u) {
@@ -1019,7 +1067,6 @@ void launch_cell_params(const Dev &d, cudaStream_t s, int fp32) {
 void launch_moments_finish(const Dev &d, cudaStream_t s) { k_moments_finish<<<nblk(d.nc, 256), 256, 0, s>>>(d); }
 // Two cells (warps) a CTA: small CTAs fit beside the velocity reduction's
 // two CTAs an SM, with which this Step 7 runs concurrently.
-constexpr int MOM_THREADS = 64;
 void launch_moments(const Dev &d, cudaStream_t s, int fp32) {
   int g = nblk((size_t)d.nc * 32, MOM_THREADS);
   if (fp32 && d.fbf) k_moments<float, 1><<<g, MOM_THREADS, 0, s>>>(d);

@@ -52,7 +52,8 @@ void tile_origins(int ni, int nj, int *out);
 void launch_flux(const Dev &d, cudaStream_t s, int fp32);
 // part 0: the residual in one pass; 1: its part without the predictor W'
 // (beside the macro sweep); 2: the collision term at W' added (after it)
-void launch_residual(const Dev &d, cudaStream_t s, int first_iter, int fp32, int part = 0);
+void launch_residual(const Dev &d, cudaStream_t s, int first_iter, int fp32, int part);
+bool residual_split(long items, long steps, int fp32);
 void launch_face_reduce(const Dev &d, cudaStream_t s, int fp32);
 int face_splits(int ntiles, int nvx, int nv, int fp32);   // CTAs that share a tile's velocities
 size_t face_values(int ntiles, int nvp);                  // 4-vectors of the stored reconstruction

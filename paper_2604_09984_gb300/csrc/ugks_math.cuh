@@ -289,16 +289,30 @@ UG_HD V2<R> interface_integral(const R *P, R vx, R vy, V2<R> ff, V2<R> wgf, R Ke
 // Per-cell record of the Shakhov equilibrium (Sec. 2.1) with the constants
 // of the velocity loop precomputed: f+ of one velocity without divisions.
 enum { SH_HPRE = 0, SH_UX, SH_UY, SH_LAM, SH_QX, SH_QY, SH_PREF, SH_IL, SH_ITAU, SH_VOL, NSH = 10 };
+// H: the Maxwellian of the record at (vx, vy)
 template <typename R>
-UG_HD V2<R> shakhov_rec(const R *c, R vx, R vy, R Keff, R Kint) {
+UG_HD V2<R> shakhov_exp(const R *c, R vx, R vy, R H, R Keff, R Kint) {
   R cx = vx - c[SH_UX], cy = vy - c[SH_UY];
   R c2 = cx * cx + cy * cy;
   R lam = c[SH_LAM], il = c[SH_IL];
-  R H = c[SH_HPRE] * r_exp<R>(-lam * c2);
   R pref = c[SH_PREF] * (cx * c[SH_QX] + cy * c[SH_QY]);
   R Hp = pref * (R(2) * lam * c2 - R(4)) * H;
   R Bp = pref * ((R(2) * lam * c2 - R(2)) * Keff - R(2) * Kint) * H * il;
   return {H + Hp, Keff * il * H + Bp};
+}
+// the same with its constants gathered: p = pref c.q, t = 2 lam c^2
+template <typename R>
+UG_HD V2<R> shakhov_short(const R *c, R vx, R vy, R H, R Keff, R Kint) {
+  const R a = c[SH_PREF] * c[SH_QX], b = c[SH_PREF] * c[SH_QY], l2 = R(2) * c[SH_LAM];
+  const R k1 = Keff * c[SH_IL], k2 = R(2) * (Keff + Kint) * c[SH_IL];
+  const R cx = vx - c[SH_UX], cy = vy - c[SH_UY];
+  const R p = a * cx + b * cy, t = l2 * (cx * cx + cy * cy);
+  return {H + p * (t - R(4)) * H, H * (k1 + p * (k1 * t - k2))};
+}
+template <typename R>
+UG_HD V2<R> shakhov_rec(const R *c, R vx, R vy, R Keff, R Kint) {
+  R cx = vx - c[SH_UX], cy = vy - c[SH_UY];
+  return shakhov_exp<R>(c, vx, vy, c[SH_HPRE] * r_exp<R>(-c[SH_LAM] * (cx * cx + cy * cy)), Keff, Kint);
 }
 
 // Shakhov equilibrium f+ = g + g+ of a cell (Sec. 2.1), one velocity.

@@ -896,107 +896,103 @@ __global__ void __launch_bounds__(NT, FluxCfg<T>::CTAS) k_flux(Dev d, double *ev
 //   r = T - Omega^{n+1} f / dt + (Omega^{n+1} (f+(W') - f)/tau' - D) / 2,
 // with the level-n term T = Omega^n f^n / dt + (Omega^n (f+(W^n) - f^n)/tau^n
 // - D^n) / 2 formed on the first inner iteration.  r goes to the sweep buffer.
-template <typename T, int FB> __global__ void k_residual(Dev d, int first_iter) {
-  typedef typename Vec2<T>::type T2;
-  // grid: cells x velocity chunks; a thread takes two adjacent velocities
-  // (nvp is a multiple of 4, so the pair stays inside the cell's row)
-  int c = blockIdx.x, k0 = 2 * (blockIdx.y * blockDim.x + threadIdx.x);
-  if (k0 >= d.nv || !(d.cmask[c] & 1)) return;
-  const T *cp = reinterpret_cast<const T *>(d.shp) + (size_t)NSH * c;
-  T itau = cp[SH_ITAU];
-  T vol1 = cp[SH_VOL];
-  T idt = sizeof(T) == 4 ? (T)(float)d.stepc[2] : (T)d.stepc[1];
-  const T *cn = reinterpret_cast<const T *>(d.shn) + (size_t)NSH * c;
-  T2 fv[2], D[2], tn[2];
-#pragma unroll
-  for (int u = 0; u < 2; ++u) {
-    size_t t = (size_t)c * d.nvp + k0 + u;
-    fv[u] = ldF<T, FB>(d, t);
-    D[u] = ldf<T>(d.Dbuf, t);
-    if (!first_iter) tn[u] = ldf<T>(d.Tn, t);
+//
+// FP32: streaming (f, D, T in, r out; 6.4 TB/s).  Where the macro sweep, whose
+// W' it needs, outlasts the flux pass that runs beside it (small velocity grids
+// against the sweep's length: residual_split), a first pass (PART 1) forms the
+// part without W', P = T_n - Omega^{n+1} f / dt - D / 2, within the sweep, and a
+// second one (PART 2) adds the collision term; else one pass (PART 0), with the
+// same roundings (256x128 + 128x32 cells, 1024 velocities: two passes 190 + 158
+// us, one 203).  FP64: its pipe; the exponential of f+ (some
+// thirty of its instructions) splits into a factor per column and one per row of
+// the CTA's velocities, tabulated first, and f+ is written with the fewest
+// operations (96x48 + 64x16 cells, 1024 velocities: 524 -> 334 us).
+constexpr int RES_NT = 256;                      // most threads of a CTA
+// pairs of adjacent velocities a thread takes (FP64: the tables and the
+// constants of a cell serve two)
+template <typename T> struct ResPairs { static constexpr int N = sizeof(T) == 8 ? 2 : 1; };
+template <typename T> struct ResTable {          // exponentials per column and row of a CTA's velocities
+  T ex[2 * RES_NT * ResPairs<T>::N], ey[2 * RES_NT * ResPairs<T>::N];
+};
+template <typename T>
+__device__ __forceinline__ void res_table(const Dev &d, const T *rec, int k0, int n, ResTable<T> &tb) {
+  // n consecutive velocities from k0: at most min(n, nvx) columns (from k0's
+  // on) and the rows iy0 .. iy1
+  const int iy0 = k0 / d.nvx, iy1 = (k0 + n - 1) / d.nvx;
+  for (int i = threadIdx.x; i < min(n, d.nvx); i += blockDim.x) {
+    const int k = k0 + i;                        // (columns of the first n velocities: all of them)
+    const T cx = dvx<T>(d, k) - rec[SH_UX];
+    tb.ex[i] = r_exp<T>(-rec[SH_LAM] * cx * cx);
   }
-#pragma unroll
-  for (int u = 0; u < 2; ++u) {
-    int k = k0 + u;
-    if (k >= d.nv) break;
-    size_t t = (size_t)c * d.nvp + k;
-    T vx = dvx<T>(d, k), vy = dvy<T>(d, k);
-    V2<T> fp = shakhov_rec<T>(cp, vx, vy, (T)d.Keff, (T)d.Kint);
-    if (first_iter) {
-      T itn = cn[SH_ITAU];
-      V2<T> fn = shakhov_rec<T>(cn, vx, vy, (T)d.Keff, (T)d.Kint);
-      T vol0 = cn[SH_VOL];
-      tn[u].x = vol0 * idt * fv[u].x + T(0.5) * (vol0 * (fn.h - fv[u].x) * itn - D[u].x);
-      tn[u].y = vol0 * idt * fv[u].y + T(0.5) * (vol0 * (fn.b - fv[u].y) * itn - D[u].y);
-      stf<T>(d.Tn, t, tn[u].x, tn[u].y);
-    }
-    T rh = tn[u].x - vol1 * idt * fv[u].x + T(0.5) * (vol1 * (fp.h - fv[u].x) * itau - D[u].x);
-    T rb = tn[u].y - vol1 * idt * fv[u].y + T(0.5) * (vol1 * (fp.b - fv[u].y) * itau - D[u].y);
-    stf<T>(d.dfs, t, rh, rb);
+  for (int i = threadIdx.x; i <= iy1 - iy0; i += blockDim.x) {
+    const T cy = dvy<T>(d, (iy0 + i) * d.nvx) - rec[SH_UY];
+    tb.ey[i] = rec[SH_HPRE] * r_exp<T>(-rec[SH_LAM] * cy * cy);
   }
 }
-
-// The residual in two passes (FP32 path): the part without the predictor W'
-// of Step 4, P = T_n - Omega^{n+1} f / dt - D / 2, runs right after the flux
-// divergence, beside the macro LU-SGS (the level-n term T_n is formed and
-// stored on the first inner iteration); after the macro sweep the second
-// pass adds the collision term at W': r = P + Omega^{n+1} (f+(W') - f) / (2 tau').
-template <typename T, int FB> __global__ void k_residual_pre(Dev d, int first_iter) {
+template <typename T, int FB, int PART> __global__ void __launch_bounds__(RES_NT) k_residual(Dev d, int first_iter) {
   typedef typename Vec2<T>::type T2;
-  int c = blockIdx.x, k0 = 2 * (blockIdx.y * blockDim.x + threadIdx.x);
-  if (k0 >= d.nv || !(d.cmask[c] & 1)) return;
-  T vol1 = (T)d.vol_new[c];                 // the value the cell record holds
-  T idt = sizeof(T) == 4 ? (T)(float)d.stepc[2] : (T)d.stepc[1];
+  constexpr bool SEP = sizeof(T) == 8;
+  __shared__ ResTable<T> tp, tn0;
+  // grid: cells x velocity chunks; a thread takes pairs of adjacent velocities
+  // (nvp is a multiple of 4, so a pair stays inside the cell's row)
+  constexpr int NP = ResPairs<T>::N;
+  const int c = blockIdx.x, kc = 2 * NP * blockIdx.y * blockDim.x;
+  if (!(d.cmask[c] & 1)) return;
+  const T *cp = reinterpret_cast<const T *>(d.shp) + (size_t)NSH * c;
   const T *cn = reinterpret_cast<const T *>(d.shn) + (size_t)NSH * c;
-  T2 fv[2], D[2], tn[2];
-#pragma unroll
-  for (int u = 0; u < 2; ++u) {
-    size_t t = (size_t)c * d.nvp + k0 + u;
-    fv[u] = ldF<T, FB>(d, t);
-    D[u] = ldf<T>(d.Dbuf, t);
-    if (!first_iter) tn[u] = ldf<T>(d.Tn, t);
+  if (SEP) {
+    const int n = min(2 * NP * (int)blockDim.x, d.nv - kc);
+    res_table<T>(d, cp, kc, n, tp);
+    if (first_iter) res_table<T>(d, cn, kc, n, tn0);
+    __syncthreads();
   }
+  // (PART 1 runs before the cell record of W' is there; the record holds this volume)
+  const T itau = PART == 1 ? T(0) : cp[SH_ITAU], vol1 = PART == 1 ? (T)d.vol_new[c] : cp[SH_VOL];
+  const T hv = T(0.5) * vol1, hi = hv * itau;
+  const T idt = sizeof(T) == 4 ? (T)reinterpret_cast<const float *>(d.stepc)[4] : (T)d.stepc[1];
 #pragma unroll
-  for (int u = 0; u < 2; ++u) {
-    int k = k0 + u;
-    if (k >= d.nv) break;
-    size_t t = (size_t)c * d.nvp + k;
-    if (first_iter) {
+  for (int m = 0; m < NP; ++m) {
+    const int k0 = kc + 2 * (threadIdx.x + m * blockDim.x);
+    if (k0 >= d.nv) return;
+    T2 fv[2], D[2], tn[2];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      size_t t = (size_t)c * d.nvp + k0 + u;
+      fv[u] = ldF<T, FB>(d, t);
+      if (PART == 2) {
+        tn[u] = ldf<T>(d.dfs, t);                // P
+      } else {
+        D[u] = ldf<T>(d.Dbuf, t);
+        if (!first_iter) tn[u] = ldf<T>(d.Tn, t);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      int k = k0 + u;
+      if (k >= d.nv) break;
+      size_t t = (size_t)c * d.nvp + k;
       T vx = dvx<T>(d, k), vy = dvy<T>(d, k);
-      T itn = cn[SH_ITAU];
-      V2<T> fn = shakhov_rec<T>(cn, vx, vy, (T)d.Keff, (T)d.Kint);
-      T vol0 = cn[SH_VOL];
-      tn[u].x = vol0 * idt * fv[u].x + T(0.5) * (vol0 * (fn.h - fv[u].x) * itn - D[u].x);
-      tn[u].y = vol0 * idt * fv[u].y + T(0.5) * (vol0 * (fn.b - fv[u].y) * itn - D[u].y);
-      stf<T>(d.Tn, t, tn[u].x, tn[u].y);
+      auto equilibrium = [&](const T *rec, const ResTable<T> &tb) {
+        if (!SEP) return shakhov_rec<T>(rec, vx, vy, (T)d.Keff, (T)d.Kint);
+        const int i = k - kc, row = k / d.nvx - kc / d.nvx;
+        return shakhov_short<T>(rec, vx, vy, tb.ex[i % d.nvx] * tb.ey[row], (T)d.Keff, (T)d.Kint);
+      };
+      V2<T> fp = {T(0), T(0)};
+      if (PART != 1) fp = equilibrium(cp, tp);
+      if (PART != 2 && first_iter) {
+        T itn = cn[SH_ITAU];
+        V2<T> fn = equilibrium(cn, tn0);
+        T vol0 = cn[SH_VOL];
+        tn[u].x = vol0 * idt * fv[u].x + T(0.5) * (vol0 * (fn.h - fv[u].x) * itn - D[u].x);
+        tn[u].y = vol0 * idt * fv[u].y + T(0.5) * (vol0 * (fn.b - fv[u].y) * itn - D[u].y);
+        stf<T>(d.Tn, t, tn[u].x, tn[u].y);
+      }
+      const T ph = PART == 2 ? tn[u].x : tn[u].x - vol1 * idt * fv[u].x - T(0.5) * D[u].x;
+      const T pb = PART == 2 ? tn[u].y : tn[u].y - vol1 * idt * fv[u].y - T(0.5) * D[u].y;
+      if (PART == 1) stf<T>(d.dfs, t, ph, pb);
+      else if (SEP) stf<T>(d.dfs, t, ph + hi * (fp.h - fv[u].x), pb + hi * (fp.b - fv[u].y));
+      else stf<T>(d.dfs, t, ph + hv * (fp.h - fv[u].x) * itau, pb + hv * (fp.b - fv[u].y) * itau);
     }
-    stf<T>(d.dfs, t, tn[u].x - vol1 * idt * fv[u].x - T(0.5) * D[u].x,
-           tn[u].y - vol1 * idt * fv[u].y - T(0.5) * D[u].y);
-  }
-}
-
-template <typename T, int FB> __global__ void k_residual_post(Dev d) {
-  typedef typename Vec2<T>::type T2;
-  int c = blockIdx.x, k0 = 2 * (blockIdx.y * blockDim.x + threadIdx.x);
-  if (k0 >= d.nv || !(d.cmask[c] & 1)) return;
-  const T *cp = reinterpret_cast<const T *>(d.shp) + (size_t)NSH * c;
-  T itau = cp[SH_ITAU];
-  T hv = T(0.5) * cp[SH_VOL];
-  T2 fv[2], P[2];
-#pragma unroll
-  for (int u = 0; u < 2; ++u) {
-    size_t t = (size_t)c * d.nvp + k0 + u;
-    fv[u] = ldF<T, FB>(d, t);
-    P[u] = ldf<T>(d.dfs, t);
-  }
-#pragma unroll
-  for (int u = 0; u < 2; ++u) {
-    int k = k0 + u;
-    if (k >= d.nv) break;
-    T vx = dvx<T>(d, k), vy = dvy<T>(d, k);
-    V2<T> fp = shakhov_rec<T>(cp, vx, vy, (T)d.Keff, (T)d.Kint);
-    stf<T>(d.dfs, (size_t)c * d.nvp + k, P[u].x + hv * (fp.h - fv[u].x) * itau,
-           P[u].y + hv * (fp.b - fv[u].y) * itau);
   }
 }
 
@@ -1056,21 +1052,27 @@ template <bool EVAL> static void flux(const Dev &d, cudaStream_t s, int fp32, do
 }
 void launch_flux(const Dev &d, cudaStream_t s, int fp32) { flux<false>(d, s, fp32, nullptr); }
 void launch_flux_eval(const Dev &d, cudaStream_t s, double *D, int fp32) { flux<true>(d, s, fp32, D); }
+// Whether the macro sweep (steps: diagonals of its two passes, some 0.25 us each)
+// outlasts the flux pass and the residual's first pass (8.4 + 5.0 ps an item, a
+// cell and velocity).  128x64 + 64x16 cells, 576 velocities (1.4e4 items a
+// diagonal): a step of 10 iterations 5.03 ms in two passes, 5.13 in one;
+// 256x128 + 128x32 cells, 1024 velocities (4.9e4): 20.79 ms and 19.01.
+bool residual_split(long items, long steps, int fp32) { return fp32 && (double)items < 1.9e4 * (double)steps; }
+
+template <typename T, int FB, int PART> static void residual(const Dev &d, cudaStream_t s, int first_iter) {
+  const int n = (d.nv + 2 * ResPairs<T>::N - 1) / (2 * ResPairs<T>::N);      // threads a cell
+  const int bt = n >= RES_NT ? RES_NT : ((n + 31) / 32) * 32;
+  k_residual<T, FB, PART><<<dim3(d.nc, (n + bt - 1) / bt), bt, 0, s>>>(d, first_iter);
+}
+template <int FB> static void residual32(const Dev &d, cudaStream_t s, int first_iter, int part) {
+  if (part == 1) residual<float, FB, 1>(d, s, first_iter);
+  else if (part == 2) residual<float, FB, 2>(d, s, first_iter);
+  else residual<float, FB, 0>(d, s, first_iter);
+}
 void launch_residual(const Dev &d, cudaStream_t s, int first_iter, int fp32, int part) {
-  int pairs = (d.nv + 1) / 2;
-  int bt = pairs >= 256 ? 256 : ((pairs + 31) / 32) * 32;
-  dim3 grid(d.nc, (pairs + bt - 1) / bt);
-  if (part == 1) {
-    if (fp32 && d.fbf) k_residual_pre<float, 1><<<grid, bt, 0, s>>>(d, first_iter);
-    else if (fp32) k_residual_pre<float, 0><<<grid, bt, 0, s>>>(d, first_iter);
-    else k_residual_pre<double, 0><<<grid, bt, 0, s>>>(d, first_iter);
-  } else if (part == 2) {
-    if (fp32 && d.fbf) k_residual_post<float, 1><<<grid, bt, 0, s>>>(d);
-    else if (fp32) k_residual_post<float, 0><<<grid, bt, 0, s>>>(d);
-    else k_residual_post<double, 0><<<grid, bt, 0, s>>>(d);
-  } else if (fp32 && d.fbf) k_residual<float, 1><<<grid, bt, 0, s>>>(d, first_iter);
-  else if (fp32) k_residual<float, 0><<<grid, bt, 0, s>>>(d, first_iter);
-  else k_residual<double, 0><<<grid, bt, 0, s>>>(d, first_iter);
+  if (!fp32) residual<double, 0, 0>(d, s, first_iter);
+  else if (d.fbf) residual32<1>(d, s, first_iter, part);
+  else residual32<0>(d, s, first_iter, part);
 }
 
 }  // namespace ugks
