@@ -457,17 +457,16 @@ template <typename T, bool FOLD> __global__ void __launch_bounds__(FOLD ? 128 : 
   }
 }
 
-// Face coefficients, velocity part (one warp per face): the g-part of the
-// macro flux by a sum over the discrete velocities, the wall density rho_w
-// (Eq. maxWalldes) and the total S-weighted macro flux (Eq. macroscopicFlux).
-// Equilibrium part of the macro flux of an interior face (the velocity sum
+// Face coefficients, velocity part: the g-part of the macro flux by a sum over
+// the discrete velocities, the wall density rho_w (Eq. maxWalldes) and the
+// total S-weighted macro flux (Eq. macroscopicFlux).  Equilibrium part of the macro flux of an interior face (the velocity sum
 // of w wS Psi (q3 (g + g+) + q4 g (a.w Psi) + q5 g (A Psi)) in reduced form,
 // Eqs. fullSolution / macroscopicFlux) through the tensor structure of the
 // velocity grid: every term is g = HPRE Ex(cx) Ey(cy) (c = v - U0) times a
 // polynomial of degree <= 6 in (cx, cy), so the 2D sum is exactly (up to
 // rounding) sum_ab coef_ab Mx_a My_b with the 1D moments
 // Mx_a = sum_ix wx cx^a Ex(cx), My_b likewise: O(nvx + nvy) work per face
-// instead of O(nvx nvy).  One warp per face; out (all lanes): 4 sums.
+// instead of O(nvx nvy).
 // 1D grids of the separable sums in the arithmetic type
 template <typename R> struct Grid1;
 template <> struct Grid1<float> {
@@ -485,14 +484,11 @@ template <> struct Grid1<double> {
   __device__ static double ex(double x) { return exp(x); }
 };
 
+// 1D moments: lane = index in the face's GS-lane group, a = 0..6 (mx) and b =
+// 0..6 (my); every lane of the warp takes part in the shuffles
 template <typename R, int GS>
-__device__ __forceinline__ void face_eq_flux_separable(const Dev &d, const R *P, R snx, R sny, R sun, int lane,
-                                                       R out[4]) {
+__device__ __forceinline__ void face_moments(const Dev &d, R ux, R uy, R lam, int lane, R *mx, R *my) {
   typedef Grid1<R> G;
-  R ux = P[FP_UX], uy = P[FP_UY], lam = P[FP_LAM];
-  // 1D moments: lane of the face's GS-lane group = grid index, a = 0..6 (x)
-  // and b = 0..6 (y); every lane of the warp takes part in the shuffles
-  R mx[7], my[7];
 #pragma unroll
   for (int a = 0; a < 7; ++a) { mx[a] = R(0); my[a] = R(0); }
   for (int ix = lane; ix < d.nvx; ix += GS) {
@@ -514,8 +510,13 @@ __device__ __forceinline__ void face_eq_flux_separable(const Dev &d, const R *P,
       mx[a] += __shfl_xor_sync(0xffffffffu, mx[a], o);
       my[a] += __shfl_xor_sync(0xffffffffu, my[a], o);
     }
-  Poly2<3, R> ih, ib;
-  interface_polys<R>(P, (R)d.Keff, (R)d.Kint, ih, ib);
+}
+
+// the four sums from the moments and the interface cubics
+template <typename R>
+__device__ __forceinline__ void face_eq_flux(const R *P, const Poly2<3, R> &ih, const Poly2<3, R> &ib, const R *mx,
+                                             const R *my, R out[4]) {
+  R ux = P[FP_UX], uy = P[FP_UY], snx = P[FP_SNX], sny = P[FP_SNY], sun = P[FP_SUN];
   Poly2<1, R> vxp = p2_lin<R>(ux, R(1), R(0)), vyp = p2_lin<R>(uy, R(0), R(1));
   Poly2<2, R> v2 = p2_axpby(R(1), p2_mul(vxp, vxp), R(1), p2_mul(vyp, vyp));
   Poly2<1, R> ws = p2_lin<R>(snx * ux + sny * uy - sun, snx, sny);
@@ -615,47 +616,69 @@ template <typename T> __device__ __forceinline__ void wall_coef(const Dev &d, co
   }
 }
 
-// The non-wall faces: FCG lanes per face, the equilibrium part of the macro
-// flux from 1D velocity moments (exact separable rewrite of the tensor-grid
-// sum); faces outside the field get zero flux.  block: index among their CTAs.
+// The non-wall faces: the equilibrium part of the macro flux from 1D velocity
+// moments (exact separable rewrite of the tensor-grid sum), the cubics of the
+// interface distribution for the flux pass; faces outside the field get zero
+// flux.  FCG lanes a face take the moments, then one warp a face per lane: the
+// products of polynomials are the larger part, and eight lanes that each made
+// them for their face spent eight times the instructions (FP64 96x48 + 64x16
+// cells: 243 us -> 178 with the walls; FP32 256x128 + 128x32: 55 -> 49).
+// block: index among their CTAs.
 constexpr int FCG = 8;
 template <typename T> __device__ __forceinline__ void sep_coef(const Dev &d, int block) {
-  int t = block * blockDim.x + threadIdx.x;
-  int fid = t / FCG, sub = t % FCG;
-  bool in = fid < d.nf;
-  int kind = in ? d.face_kind[fid] : BC_OVERSET;
-  bool need = in && kind != BC_OVERSET && face_needed(d, fid);
-  if (in && !need) {
-    if (sub < 4) d.fflux[4 * fid + sub] = 0.0;
-    if (sub == 0) d.gam[fid] = 0.0;
-  }
-  bool act = need && kind != BC_WALL;
-  if (!__any_sync(0xffffffffu, act)) return;      // warp-uniform
-  __align__(16) T parT[NFP];
-  if (act) {
-    load_rec<T, NFP>(reinterpret_cast<const T *>(d.fparT) + (size_t)NFP * fid, parT);
-  } else {
+  constexpr int FPB = FC_THREADS / FCG;          // faces of a CTA, the lanes of a warp
+  static_assert(FPB == 32, "one warp finishes the CTA's faces");
+  __shared__ T mom[FPB][15];
+  const int f0 = block * FPB;
+  {
+    const int r = threadIdx.x / FCG, sub = threadIdx.x % FCG, fid = f0 + r;
+    const bool in = fid < d.nf;
+    const int kind = in ? d.face_kind[fid] : BC_OVERSET;
+    const bool act = in && kind != BC_OVERSET && kind != BC_WALL && face_needed(d, fid);
+    T mx[7], my[7], ux = T(0), uy = T(0), lam = T(0);
+    if (act) {
+      const T *P = reinterpret_cast<const T *>(d.fparT) + (size_t)NFP * fid;
+      ux = P[FP_UX]; uy = P[FP_UY]; lam = P[FP_LAM];
+    }
+    if (__any_sync(0xffffffffu, act)) {
+      face_moments<T, FCG>(d, ux, uy, lam, sub, mx, my);
+      if (sub == 0)
 #pragma unroll
-    for (int q = 0; q < NFP; ++q) parT[q] = T(0);
+        for (int a = 0; a < 7; ++a) { mom[r][a] = mx[a]; mom[r][7 + a] = my[a]; }
+    }
   }
+  __syncthreads();
+  if (threadIdx.x >= 32) return;
+  const int fid = f0 + threadIdx.x;
+  if (fid >= d.nf) return;
+  const int kind = d.face_kind[fid];
+  double2 *F = reinterpret_cast<double2 *>(d.fflux + 4 * (size_t)fid);
+  if (kind == BC_OVERSET || !face_needed(d, fid)) {
+    F[0] = F[1] = make_double2(0.0, 0.0);
+    d.gam[fid] = 0.0;
+    return;
+  }
+  if (kind == BC_WALL) return;
+  T *PT = reinterpret_cast<T *>(d.fparT) + (size_t)NFP * fid;
+  __align__(16) T P[FP_IH];
+  load_rec<T, FP_IH>(PT, P);
+  Poly2<3, T> ih, ib;
+  interface_polys<T>(P, (T)d.Keff, (T)d.Kint, ih, ib);
   T o[4];
-  face_eq_flux_separable<T, FCG>(d, parT, parT[FP_SNX], parT[FP_SNY], parT[FP_SUN], sub, o);
-  if (act) {
-    // the cubics of the interface distribution for the flux pass (lane sub
-    // of the face's group writes coefficients sub, sub + FCG, ...)
-    Poly2<3, T> ih, ib;
-    interface_polys<T>(parT, (T)d.Keff, (T)d.Kint, ih, ib);
-    T *PT = reinterpret_cast<T *>(d.fparT) + (size_t)NFP * fid;
+  face_eq_flux<T>(P, ih, ib, mom[threadIdx.x], mom[threadIdx.x] + 7, o);
+  __align__(16) T poly[20];
 #pragma unroll
-    for (int m = 0; m < 20; ++m)
-      if (m % FCG == sub) PT[FP_IH + m] = m < 10 ? ih.c[m] : ib.c[m - 10];
-  }
-  if (act && sub < 4) {                           // lane m of the group: component m
-    const double *P = d.fq12 + 2 * (size_t)fid;
-    const double *fs = d.fsum + NFS * fid;
-    T om = sub == 0 ? o[0] : sub == 1 ? o[1] : sub == 2 ? o[2] : o[3];
-    d.fflux[4 * fid + sub] = P[0] * fs[FS_FF + sub] + P[1] * fs[FS_WG + sub] + to_double(om);
-  }
+  for (int m = 0; m < 10; ++m) { poly[m] = ih.c[m]; poly[10 + m] = ib.c[m]; }
+#pragma unroll
+  for (int m = 0; m < 20 * (int)sizeof(T) / 16; ++m)
+    reinterpret_cast<float4 *>(PT + FP_IH)[m] = reinterpret_cast<const float4 *>(poly)[m];
+  const double2 q = *reinterpret_cast<const double2 *>(d.fq12 + 2 * (size_t)fid);
+  const double *fs = d.fsum + NFS * (size_t)fid;
+  double v[4];
+#pragma unroll
+  for (int m = 0; m < 4; ++m) v[m] = q.x * fs[FS_FF + m] + q.y * fs[FS_WG + m] + to_double(o[m]);
+  F[0] = make_double2(v[0], v[1]);
+  F[1] = make_double2(v[2], v[3]);
 }
 
 template <typename T> __global__ void __launch_bounds__(FC_THREADS, sizeof(T) == 4 ? 2 : 1) k_face_coef(Dev d, int wall_blocks) {
