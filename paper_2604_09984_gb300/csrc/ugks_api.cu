@@ -319,6 +319,7 @@ size_t carve(char *base, const Sizes &s, int nb, int fp32, int fbf, int nwork, i
   d.body_ring = c.take<int>((size_t)s.nring + 1);
   d.body_ring_off = c.take<int>(nb + 1);
   d.body_bb = c.take<float4>(nb);
+  d.bin_bb = c.take<float4>(nb);
   d.cell_off = c.take<int>(nb + 1);
   d.node_off = c.take<int>(nb + 1);
   d.blk_info = c.take<int>(8 * (size_t)nb);
@@ -327,6 +328,9 @@ size_t carve(char *base, const Sizes &s, int nb, int fp32, int fbf, int nwork, i
   d.bin_cnt = c.take<int>((size_t)s.nc + nb + 1);
   d.bin_start = c.take<int>((size_t)s.nc + nb + 2);
   d.bin_items = c.take<int>(bin_capacity(s));
+  d.bin_rng = c.take<int2>((size_t)s.nc);
+  d.node_todo = c.take<int>((size_t)s.nn + 1);
+  d.node_todo_n = d.node_todo + s.nn;
   d.tiles = c.take<int>(3 * (size_t)s.ntiles);
   d.err = c.take<int>(4);
   (void)nwork;
@@ -649,7 +653,7 @@ int do_connect(ugks_ctx *ctx, ugks_connect_stats *stats, bool initial, bool sync
     launch_lists(d, ctx->st, ctx->prev_status, ctx->n_orphan);
   }
   launch_slope_geo(d, ctx->st);     // holes changed
-  ctx->launches += 12;
+  ctx->launches += 13;
   ctx->fresh_pending = !initial;
   int r = launch_status(ctx);
   if (r || !sync) return r;

@@ -131,6 +131,7 @@ struct Dev {
   int *body_ring;            // body polygon node ids, grouped per block
   int *body_ring_off;        // nblocks+1
   float4 *body_bb;           // nblocks: outward-rounded float box of the body polygon
+  float4 *bin_bb;            // per block: box of its bins, rounded outward
   const int *cell_off;       // nblocks+1 (device copy)
   const int *node_off;       // nblocks+1
   const int *blk_info;       // nblocks*8: ni, nj, periodic, priority, n_fringe, n_gap, bc-overset mask, body?
@@ -139,6 +140,9 @@ struct Dev {
   int *bin_dim;              // nblocks*3: nbx, nby, first bin
   int *bin_cnt, *bin_start;  // nbins, nbins+1
   int *bin_items;            // bin_cap
+  int2 *bin_rng;             // nc: a cell's first and last bin, x | y << 16
+  int *node_todo;            // nn: nodes of the second classification pass
+  int *node_todo_n;          // their count
   int nbins, bin_cap;
   const int *tiles;          // ntiles*3: block, i0, j0 of the 8x8 cell tiles
   int ntiles;

@@ -48,76 +48,83 @@ __device__ __forceinline__ double seg_dist2(const Dev &d, int s, double x, doubl
   return ad(ml(dx, dx), ml(dy, dy));
 }
 
-// Minimum squared distance to the zone's wall segments (+inf without).
-// A float pass picks a near segment, whose exact distance bounds the
-// minimum; then only segments whose float lower bound (distance to their
-// bounding box, shrunk by the float rounding of the coordinates and
-// scaled down) does not exceed that bound are evaluated exactly.  The
-// skipped ones are farther than the minimum, so the result is the exact
-// minimum over all segments.
+// Wall distances and the body test of a node run over a group of NLANES lanes
+// (each takes every NLANES-th segment; all of them get the result).
+constexpr int NLANES = 8;
+struct Group {
+  unsigned mask;
+  int lane;
+  __device__ Group() : mask(0xffu << (threadIdx.x & 24)), lane(threadIdx.x & (NLANES - 1)) {}
+  template <typename V> __device__ V down(V v, int o) const { return __shfl_xor_sync(mask, v, o); }
+};
+static_assert(NLANES == 8, "the group's lane mask");
+
+// Segment nearest to (x, y) in float, and a bracket [lo, hi] of the squared
+// distance to the nearest one in floats that allow for all roundings: lo from
+// the distances to the segments' bounding boxes, shrunk, hi from the point
+// found on the near segment (any point on it bounds), widened by 1e-6 of the
+// coordinates (some 16 float roundings of 6e-8).
 // `seg` holds the float endpoints (A.x, A.y, B.x, B.y) of every segment
 // (shared memory, or the global copy when they do not fit there).
-__device__ double wall_dist2(const Dev &d, const float4 *seg, int blk, double x, double y) {
-  double best = __longlong_as_double(0x7ff0000000000000LL);   // +inf
-  int s0 = d.wall_seg_off[blk], s1 = d.wall_seg_off[blk + 1];
-  if (s1 <= s0) return best;
-  float xf = __double2float_rn(x), yf = __double2float_rn(y);
+__device__ __forceinline__ float seg_size(float4 AB, float xf, float yf) {
+  return fabsf(xf) + fabsf(yf) + fabsf(AB.x) + fabsf(AB.y) + fabsf(AB.z) + fabsf(AB.w);
+}
+__device__ __forceinline__ float seg_bound(float4 AB, float xf, float yf) {
+  float lx = fminf(AB.x, AB.z), hx = fmaxf(AB.x, AB.z), ly = fminf(AB.y, AB.w), hy = fmaxf(AB.y, AB.w);
+  float tol = 2.4e-7f * seg_size(AB, xf, yf);
+  float gx = fmaxf(fmaxf(lx - xf, xf - hx) - tol, 0.f);
+  float gy = fmaxf(fmaxf(ly - yf, yf - hy) - tol, 0.f);
+  return (gx * gx + gy * gy) * 0.99999f;
+}
+__device__ int near_segment(const Group &g, const float4 *seg, int s0, int s1, float xf, float yf, float &lo, float &hi) {
   int sg = s0;
   float gbest = __int_as_float(0x7f800000);
-  for (int s = s0; s < s1; ++s) {
-    float4 AB = seg[s];
-    float2 A = make_float2(AB.x, AB.y), B = make_float2(AB.z, AB.w);
-    float ex = B.x - A.x, ey = B.y - A.y, px = xf - A.x, py = yf - A.y;
-    float ee = ex * ex + ey * ey;
-    float t = ee > 0.f ? fminf(fmaxf((px * ex + py * ey) / ee, 0.f), 1.f) : 0.f;
-    float dx = px - t * ex, dy = py - t * ey, g = dx * dx + dy * dy;
-    if (g < gbest) { gbest = g; sg = s; }
-  }
-  best = seg_dist2(d, sg, x, y);
-  float bestf = __double2float_ru(best);
-  for (int s = s0; s < s1; ++s) {
-    if (s == sg) continue;
-    float4 AB = seg[s];
-    float2 A = make_float2(AB.x, AB.y), B = make_float2(AB.z, AB.w);
-    float lx = fminf(A.x, B.x), hx = fmaxf(A.x, B.x), ly = fminf(A.y, B.y), hy = fmaxf(A.y, B.y);
-    float tol = 2.4e-7f * (fabsf(xf) + fabsf(yf) + fabsf(lx) + fabsf(hx) + fabsf(ly) + fabsf(hy));
-    float gx = fmaxf(fmaxf(lx - xf, xf - hx) - tol, 0.f);
-    float gy = fmaxf(fmaxf(ly - yf, yf - hy) - tol, 0.f);
-    float lb = (gx * gx + gy * gy) * 0.99999f;
-    if (lb > bestf) continue;
-    double d2 = seg_dist2(d, s, x, y);
-    if (d2 < best) { best = d2; bestf = __double2float_ru(best); }
-  }
-  return best;
-}
-
-// Bracket of the same minimum without its exact evaluation over every
-// candidate: hi = the exact distance of the float-nearest segment (an upper
-// bound), lo = the smallest float lower bound over all segments (rounded
-// so that lo <= every exact segment distance).  Both +inf without walls.
-__device__ void wall_dist2_bounds(const Dev &d, const float4 *seg, int blk, double x, double y,
-                                  double &lo, double &hi) {
-  lo = hi = __longlong_as_double(0x7ff0000000000000LL);
-  int s0 = d.wall_seg_off[blk], s1 = d.wall_seg_off[blk + 1];
-  if (s1 <= s0) return;
-  float xf = __double2float_rn(x), yf = __double2float_rn(y);
-  int sg = s0;
-  float gbest = __int_as_float(0x7f800000), lbmin = __int_as_float(0x7f800000);
-  for (int s = s0; s < s1; ++s) {
+  lo = hi = gbest;
+  for (int s = s0 + g.lane; s < s1; s += NLANES) {
     float4 AB = seg[s];
     float ex = AB.z - AB.x, ey = AB.w - AB.y, px = xf - AB.x, py = yf - AB.y;
     float ee = ex * ex + ey * ey;
-    float t = ee > 0.f ? fminf(fmaxf((px * ex + py * ey) / ee, 0.f), 1.f) : 0.f;
-    float dx = px - t * ex, dy = py - t * ey, g = dx * dx + dy * dy;
-    if (g < gbest) { gbest = g; sg = s; }
-    float lx = fminf(AB.x, AB.z), hx = fmaxf(AB.x, AB.z), ly = fminf(AB.y, AB.w), hy = fmaxf(AB.y, AB.w);
-    float tol = 2.4e-7f * (fabsf(xf) + fabsf(yf) + fabsf(lx) + fabsf(hx) + fabsf(ly) + fabsf(hy));
-    float gx = fmaxf(fmaxf(lx - xf, xf - hx) - tol, 0.f);
-    float gy = fmaxf(fmaxf(ly - yf, yf - hy) - tol, 0.f);
-    lbmin = fminf(lbmin, (gx * gx + gy * gy) * 0.99999f);
+    float t = ee > 0.f ? fminf(fmaxf(__fdividef(px * ex + py * ey, ee), 0.f), 1.f) : 0.f;
+    float dx = fabsf(px - t * ex), dy = fabsf(py - t * ey), d2 = dx * dx + dy * dy;
+    if (d2 < gbest) {
+      gbest = d2;
+      sg = s;
+      const float tol = 1e-6f * seg_size(AB, xf, yf);
+      hi = ((dx + tol) * (dx + tol) + (dy + tol) * (dy + tol)) * 1.00001f;
+    }
+    lo = fminf(lo, seg_bound(AB, xf, yf));
   }
-  hi = seg_dist2(d, sg, x, y);
-  lo = (double)lbmin;
+#pragma unroll
+  for (int o = NLANES / 2; o > 0; o >>= 1) {
+    const float ob = g.down(gbest, o), oh = g.down(hi, o), ol = g.down(lo, o);
+    const int os = g.down(sg, o);
+    if (ob < gbest || (ob == gbest && os < sg)) { gbest = ob; sg = os; }
+    hi = fminf(hi, oh);
+    lo = fminf(lo, ol);
+  }
+  return sg;
+}
+
+// Minimum squared distance to the zone's wall segments exactly (+inf without):
+// the near segment's exact distance bounds it; then only segments whose float
+// lower bound does not exceed that bound are evaluated exactly.  The skipped
+// ones are farther than the minimum.
+__device__ double wall_dist2(const Group &g, const Dev &d, const float4 *seg, int blk, double x, double y) {
+  double best = __longlong_as_double(0x7ff0000000000000LL);   // +inf
+  int s0 = d.wall_seg_off[blk], s1 = d.wall_seg_off[blk + 1];
+  if (s1 <= s0) return best;
+  float xf = __double2float_rn(x), yf = __double2float_rn(y), lo, hi;
+  int sg = near_segment(g, seg, s0, s1, xf, yf, lo, hi);
+  best = seg_dist2(d, sg, x, y);
+  float bestf = __double2float_ru(best);
+  for (int s = s0 + g.lane; s < s1; s += NLANES) {
+    if (s == sg || seg_bound(seg[s], xf, yf) > bestf) continue;
+    double d2 = seg_dist2(d, s, x, y);
+    if (d2 < best) { best = d2; bestf = __double2float_ru(best); }
+  }
+#pragma unroll
+  for (int o = NLANES / 2; o > 0; o >>= 1) best = fmin(best, g.down(best, o));
+  return best;
 }
 
 __device__ bool inside_quad(const Dev &d, int c, double x, double y) {
@@ -133,8 +140,10 @@ __device__ bool inside_quad(const Dev &d, int c, double x, double y) {
   return true;
 }
 
-// Float box of each block's body polygon, rounded outward (one warp per
-// block): a point outside it is outside the polygon.
+// Float boxes of each block's body polygon and of its bins, rounded outward (one
+// warp per block): a point outside the first is outside the polygon, outside
+// the second in no bin.  (A coordinate rounded to float keeps its side of a
+// float bound, so the tests against them need no FP64.)
 __global__ void k_body_box(Dev d) {
   int b = blockIdx.x, lane = threadIdx.x;
   int r0 = d.body_ring_off[b], r1 = d.body_ring_off[b + 1];
@@ -153,16 +162,28 @@ __global__ void k_body_box(Dev d) {
   if (lane == 0)
     d.body_bb[b] = make_float4(__double2float_rd(xl), __double2float_rd(yl), __double2float_ru(xh),
                                __double2float_ru(yh));
+  if (lane == 0) {      // the bins' box, widened past the roundings of bin_of
+    const double *g = d.bin_geo + 4 * b;
+    const double w = d.bin_dim[3 * b] / g[2], h = d.bin_dim[3 * b + 1] / g[3];
+    const double px = 1e-12 * (fabs(g[0]) + w), py = 1e-12 * (fabs(g[1]) + h);
+    d.bin_bb[b] = make_float4(__double2float_rd(g[0] - px), __double2float_rd(g[1] - py),
+                              __double2float_ru(g[0] + w + px), __double2float_ru(g[1] + h + py));
+  }
 }
 
-__device__ bool inside_body(const Dev &d, int blk, double x, double y) {
-  float4 bb = d.body_bb[blk];
-  if (x < (double)bb.x || x > (double)bb.z || y < (double)bb.y || y > (double)bb.w) return false;
-  int r0 = d.body_ring_off[blk], r1 = d.body_ring_off[blk + 1];
-  int M = r1 - r0;
-  bool in = false;
+__device__ __forceinline__ bool in_box(float4 bb, float x, float y) {
+  return !(x < bb.x || x > bb.z || y < bb.y || y > bb.w);
+}
+__device__ __forceinline__ bool in_body_box(const Dev &d, int blk, float x, float y) {
+  return d.body_ring_off[blk + 1] > d.body_ring_off[blk] && in_box(d.body_bb[blk], x, y);
+}
+
+__device__ bool inside_body(const Group &g, const Dev &d, int blk, double x, double y) {
   float yf = __double2float_rn(y);
-  for (int i = 0; i < M; ++i) {
+  if (!in_body_box(d, blk, __double2float_rn(x), yf)) return false;
+  int r0 = d.body_ring_off[blk], r1 = d.body_ring_off[blk + 1];
+  int M = r1 - r0, in = 0;
+  for (int i = g.lane; i < M; i += NLANES) {
     int a = d.body_ring[r0 + i], b = d.body_ring[r0 + (i + 1 < M ? i + 1 : 0)];
     // side of y for each end from the floats where they differ, else exactly
     float af = d.Xf[a].y, bf = d.Xf[b].y;
@@ -173,10 +194,12 @@ __device__ bool inside_body(const Dev &d, int blk, double x, double y) {
     bool crosses = (ay > y) != (by > y);
     if (crosses) {
       double xint = ad(ax, dv(ml(sb(y, ay), sb(bx, ax)), sb(by, ay)));
-      if (x < xint) in = !in;
+      if (x < xint) in ^= 1;
     }
   }
-  return in;
+#pragma unroll
+  for (int o = NLANES / 2; o > 0; o >>= 1) in ^= g.down(in, o);
+  return in != 0;
 }
 
 __device__ __forceinline__ bool in_layer(const int *bi, int i, int j, int L) {
@@ -215,6 +238,7 @@ __device__ __forceinline__ int bin_of(const Dev &d, int b, double x, double y) {
 
 __global__ void k_node_f(Dev d) {
   int n = blockIdx.x * blockDim.x + threadIdx.x;
+  if (n == 0) *d.node_todo_n = 0;
   if (n < d.nn)
     d.Xf[n] = make_float2(__double2float_rn(d.X_new[2 * n]), __double2float_rn(d.X_new[2 * n + 1]));
   if (n < d.nseg) {      // float endpoints of wall segment n, one record each
@@ -224,146 +248,198 @@ __global__ void k_node_f(Dev d) {
   }
 }
 
+// bounding box and bin range of every cell (at most 2048 bins an axis)
 __global__ void k_bin_count(Dev d) {
   int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= d.nc) return;
   int b = d.cell_block[c];
-  const int *nd = d.cell_nodes + 4 * c;
-  double xl = d.X_new[2 * nd[0]], xh = xl, yl = d.X_new[2 * nd[0] + 1], yh = yl;
-  for (int v = 1; v < 4; ++v) {
-    double x = d.X_new[2 * nd[v]], y = d.X_new[2 * nd[v] + 1];
-    xl = fmin(xl, x); xh = fmax(xh, x); yl = fmin(yl, y); yh = fmax(yh, y);
-  }
+  const int4 n4 = *reinterpret_cast<const int4 *>(d.cell_nodes + 4 * c);
+  const double2 *X = reinterpret_cast<const double2 *>(d.X_new);
+  const double2 p0 = X[n4.x], p1 = X[n4.y], p2 = X[n4.z], p3 = X[n4.w];
+  const double xl = fmin(fmin(fmin(p0.x, p1.x), p2.x), p3.x), xh = fmax(fmax(fmax(p0.x, p1.x), p2.x), p3.x);
+  const double yl = fmin(fmin(fmin(p0.y, p1.y), p2.y), p3.y), yh = fmax(fmax(fmax(p0.y, p1.y), p2.y), p3.y);
   d.cbb[c] = make_float4(__double2float_rd(xl), __double2float_rd(yl), __double2float_ru(xh),
                          __double2float_ru(yh));
   int ix0, ix1, iy0, iy1;
   bin_range(d, b, xl, xh, 0, ix0, ix1);
   bin_range(d, b, yl, yh, 1, iy0, iy1);
+  d.bin_rng[c] = make_int2(ix0 | iy0 << 16, ix1 | iy1 << 16);
   int nx = d.bin_dim[3 * b], base = d.bin_dim[3 * b + 2];
   for (int iy = iy0; iy <= iy1; ++iy)
     for (int ix = ix0; ix <= ix1; ++ix) atomicAdd(&d.bin_cnt[base + iy * nx + ix], 1);
 }
 
-// exclusive scan of the bin counts (one CTA), cursor = start
-__global__ void k_bin_scan(Dev d) {
-  __shared__ int part[1024];
-  int n = d.nbins;
-  int per = (n + blockDim.x - 1) / blockDim.x;
-  int lo = threadIdx.x * per, hi = min(n, lo + per);
-  int s = 0;
-  for (int i = lo; i < hi; ++i) s += d.bin_cnt[i];
-  part[threadIdx.x] = s;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int run = 0;
-    for (int t = 0; t < (int)blockDim.x; ++t) { int v = part[t]; part[t] = run; run += v; }
-    d.bin_start[n] = run;
-    if (run > d.bin_cap) atomicOr(d.err, EF_BINS);
+// Exclusive scan of the bin counts.  Each CTA adds the counts before its
+// chunk itself (75,000 bins: at most 73 loads of 16 bytes a thread, from L2),
+// so the CTAs need no order among them: 110 us with one CTA, 11 so.
+constexpr int SCAN_THREADS = 256, SCAN_CHUNK = 4 * SCAN_THREADS;
+__global__ void __launch_bounds__(SCAN_THREADS) k_bin_scan(Dev d) {
+  __shared__ int wsum[2][SCAN_THREADS / 32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, n = d.nbins;
+  const int4 *cnt = reinterpret_cast<const int4 *>(d.bin_cnt);
+  int before = 0;
+#pragma unroll 8
+  for (int q = threadIdx.x; q < (int)blockIdx.x * SCAN_THREADS; q += SCAN_THREADS) {
+    const int4 v = cnt[q];
+    before += v.x + v.y + v.z + v.w;
   }
+  const int i0 = blockIdx.x * SCAN_CHUNK + 4 * threadIdx.x;
+  int v[4];
+#pragma unroll
+  for (int m = 0; m < 4; ++m) v[m] = i0 + m < n ? d.bin_cnt[i0 + m] : 0;
+  const int mine = v[0] + v[1] + v[2] + v[3];
+  int incl = mine;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int t = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += t;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
+  if (lane == 31) { wsum[0][w] = before; wsum[1][w] = incl; }
   __syncthreads();
-  int run = part[threadIdx.x];
-  for (int i = lo; i < hi; ++i) {
-    int v = d.bin_cnt[i];
-    d.bin_start[i] = run;
-    d.bin_cnt[i] = run;            // reused as the fill cursor
-    run += v;
+  int run = incl - mine;
+#pragma unroll
+  for (int q = 0; q < SCAN_THREADS / 32; ++q) {
+    run += wsum[0][q];
+    if (q < w) run += wsum[1][q];
+  }
+#pragma unroll
+  for (int m = 0; m < 4; ++m) {
+    if (i0 + m < n) d.bin_start[i0 + m] = run;
+    run += v[m];
+    if (i0 + m == n - 1) {
+      d.bin_start[n] = run;
+      if (run > d.bin_cap) atomicOr(d.err, EF_BINS);
+    }
   }
 }
 
+// (the counts run down as the bins fill)
 __global__ void k_bin_fill(Dev d) {
   int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= d.nc) return;
-  int b = d.cell_block[c];
-  const int *nd = d.cell_nodes + 4 * c;
-  double xl = d.X_new[2 * nd[0]], xh = xl, yl = d.X_new[2 * nd[0] + 1], yh = yl;
-  for (int v = 1; v < 4; ++v) {
-    double x = d.X_new[2 * nd[v]], y = d.X_new[2 * nd[v] + 1];
-    xl = fmin(xl, x); xh = fmax(xh, x); yl = fmin(yl, y); yh = fmax(yh, y);
-  }
-  int ix0, ix1, iy0, iy1;
-  bin_range(d, b, xl, xh, 0, ix0, ix1);
-  bin_range(d, b, yl, yh, 1, iy0, iy1);
-  int nx = d.bin_dim[3 * b], base = d.bin_dim[3 * b + 2];
-  for (int iy = iy0; iy <= iy1; ++iy)
-    for (int ix = ix0; ix <= ix1; ++ix) {
-      int pos = atomicAdd(&d.bin_cnt[base + iy * nx + ix], 1);
+  const int2 rng = d.bin_rng[c];
+  const int b = d.cell_block[c], nx = d.bin_dim[3 * b], base = d.bin_dim[3 * b + 2];
+  for (int iy = rng.x >> 16; iy <= rng.y >> 16; ++iy)
+    for (int ix = rng.x & 0xffff; ix <= (rng.y & 0xffff); ++ix) {
+      const int bin = base + iy * nx + ix;
+      const int pos = d.bin_start[bin] + atomicSub(&d.bin_cnt[bin], 1) - 1;
       if (pos < d.bin_cap) d.bin_items[pos] = c;
     }
 }
 
 // lowest-index cell of block b containing (x, y) among the cells accepted by
-// `ok` (bins guarantee the same answer as a scan of the block)
+// `ok` (bins guarantee the same answer as a scan of the block); the group's
+// lanes share the bin's candidates (a bin at a stretched wall holds a hundred)
 template <typename Pred>
-__device__ int first_containing(const Dev &d, int b, double x, double y, Pred ok) {
+__device__ int first_containing(const Group &g, const Dev &d, int b, double x, double y, Pred ok) {
+  const float xf = __double2float_rn(x), yf = __double2float_rn(y);
+  if (!in_box(d.bin_bb[b], xf, yf)) return -1;
   int bin = bin_of(d, b, x, y);
   if (bin < 0) return -1;
   int best = 0x7fffffff;
-  float xf = __double2float_rn(x), yf = __double2float_rn(y);
   int q1 = min(d.bin_start[bin + 1], d.bin_cap);
-  for (int q = d.bin_start[bin]; q < q1; ++q) {
+  for (int q = d.bin_start[bin] + g.lane; q < q1; q += NLANES) {
     int c = d.bin_items[q];
     if (c >= best) continue;
-    float4 bb = d.cbb[c];                       // the cell lies inside its box
-    if (xf < bb.x || xf > bb.z || yf < bb.y || yf > bb.w) continue;
+    if (!in_box(d.cbb[c], xf, yf)) continue;     // the cell lies inside its box
     if (ok(c) && inside_quad(d, c, x, y)) best = c;
   }
+#pragma unroll
+  for (int o = NLANES / 2; o > 0; o >>= 1) best = min(best, g.down(best, o));
   return best == 0x7fffffff ? -1 : best;
 }
 
-// node classification (one thread per node); the wall segments' float
-// records are staged in shared memory when they fit (STAGE)
-template <bool STAGE> __global__ void k_node_classify(Dev d) {
+// Whether a cell of block b outside its outer layers contains (x, y)
+__device__ bool in_core(const Group &g, const Dev &d, int b, double x, double y) {
+  const int *bi = d.blk_info + 8 * b;
+  const int ni = bi[0], L = bi[4] + bi[5], c0 = d.cell_off[b];
+  return first_containing(g, d, b, x, y, [&](int c) {
+    int loc = c - c0;
+    return !in_layer(bi, loc % ni, loc / ni, L);
+  }) >= 0;
+}
+
+// Node classification.  Most nodes lie in no other zone's bins and no body's
+// box: one thread a node finds them active from float boxes.  The others go to
+// a list, whose nodes take a group of lanes each in a second launch: their
+// loops over a bin's candidates, wall segments and body edges (some 20,000
+// instructions a node for three blocks with 192 segments) belong to
+// neighbouring nodes, so that one thread a node left them to few warps (150784
+// nodes: 128 us, 6 + 64 in two launches).
+__global__ void __launch_bounds__(128) k_node_classify(Dev d) {
+  const int n = blockIdx.x * blockDim.x + threadIdx.x;
+  bool todo = false;
+  if (n < d.nn) {
+    const int z = d.node_block[n];
+    const float2 X = d.Xf[n];
+    for (int b = 0; b < d.nblocks && !todo; ++b)
+      todo = b != z && (in_box(d.bin_bb[b], X.x, X.y) || in_body_box(d, b, X.x, X.y));
+    d.node_active[n] = 1;
+  }
+  const unsigned all = __ballot_sync(0xffffffffu, todo);
+  if (!all) return;
+  const int lane = threadIdx.x & 31;
+  int at = 0;
+  if (lane == 0) at = atomicAdd(d.node_todo_n, __popc(all));
+  at = __shfl_sync(0xffffffffu, at, 0);
+  if (todo) d.node_todo[at + __popc(all & ((1u << lane) - 1u))] = n;
+}
+
+// the wall segments' float records are staged in shared memory when they fit
+// (STAGE)
+template <bool STAGE> __global__ void __launch_bounds__(256) k_node_todo(Dev d) {
   extern __shared__ float4 seg_s[];
+  const int count = *d.node_todo_n;
+  if ((int)(blockIdx.x * blockDim.x / NLANES) >= count) return;
   if (STAGE) {
     for (int q = threadIdx.x; q < d.nseg; q += blockDim.x) seg_s[q] = d.segf[q];
     __syncthreads();
   }
   const float4 *seg = STAGE ? seg_s : d.segf;
-  int n = blockIdx.x * blockDim.x + threadIdx.x;
-  if (n >= d.nn) return;
-  int z = d.node_block[n];
-  double x = d.X_new[2 * n], y = d.X_new[2 * n + 1];
-  // the node's own wall distance is needed only where another zone's core
-  // contains it (most background nodes lie in no other zone), and exactly
-  // only where the brackets of the two distances overlap: elsewhere the
-  // brackets already decide db < dz (or db > dz) as the exact values would
-  double dz = 0.0, zlo = 0.0, zhi = 0.0;
-  bool have_z = false, have_dz = false;
-  bool inact = false;
-  for (int b = 0; b < d.nblocks && !inact; ++b) {
-    if (b == z) continue;
-    if (d.body_ring_off[b + 1] > d.body_ring_off[b] && inside_body(d, b, x, y)) {
-      inact = true;
-      break;
-    }
-    const int *bi = d.blk_info + 8 * b;
-    int ni = bi[0], L = bi[4] + bi[5];
-    int c0 = d.cell_off[b];
-    bool hit = first_containing(d, b, x, y, [&](int c) {
-      int loc = c - c0;
-      return !in_layer(bi, loc % ni, loc / ni, L);
-    }) >= 0;
-    if (hit) {
+  const Group g;
+  const float inf = __int_as_float(0x7f800000);
+  for (int t = (blockIdx.x * blockDim.x + threadIdx.x) / NLANES; t < count; t += gridDim.x * blockDim.x / NLANES) {
+    const int n = d.node_todo[t], z = d.node_block[n];
+    const double x = d.X_new[2 * n], y = d.X_new[2 * n + 1];
+    const float xf = __double2float_rn(x), yf = __double2float_rn(y);
+    auto bracket = [&](int b, float &lo, float &hi) {        // of the distance to b's walls; both +inf without
+      lo = hi = inf;
+      const int s0 = d.wall_seg_off[b], s1 = d.wall_seg_off[b + 1];
+      if (s1 > s0) near_segment(g, seg, s0, s1, xf, yf, lo, hi);
+    };
+    // the exact distances are needed only where their brackets overlap:
+    // elsewhere the brackets decide db < dz (or db > dz) as they would
+    double dz = 0.0;
+    float zlo = 0.f, zhi = 0.f;
+    bool have_z = false, have_dz = false, inact = false;
+    for (int b = 0; b < d.nblocks && !inact; ++b) {
+      if (b == z) continue;
+      if (inside_body(g, d, b, x, y)) {
+        inact = true;
+        break;
+      }
+      if (!in_core(g, d, b, x, y)) continue;
       if (!have_z) {
-        wall_dist2_bounds(d, seg, z, x, y, zlo, zhi);
+        bracket(z, zlo, zhi);
         have_z = true;
       }
-      double blo, bhi;
-      wall_dist2_bounds(d, seg, b, x, y, blo, bhi);
+      float blo, bhi;
+      bracket(b, blo, bhi);
       if (bhi < zlo) {                  // db <= bhi < zlo <= dz
         inact = true;
       } else if (!(blo > zhi)) {        // brackets overlap: exact values
         if (!have_dz) {
-          dz = wall_dist2(d, seg, z, x, y);
+          dz = wall_dist2(g, d, seg, z, x, y);
           have_dz = true;
         }
-        double db = wall_dist2(d, seg, b, x, y);
-        const int *bz = d.blk_info + 8 * z;
-        if (db < dz || (db == dz && bi[3] > bz[3])) inact = true;
+        double db = wall_dist2(g, d, seg, b, x, y);
+        if (db < dz || (db == dz && d.blk_info[8 * b + 3] > d.blk_info[8 * z + 3])) inact = true;
       }                                 // else db >= blo > zhi >= dz: stays active
     }
+    if (inact && g.lane == 0) d.node_active[n] = 0;
   }
-  d.node_active[n] = inact ? 0 : 1;
 }
 
 __global__ void k_cell_classify(Dev d) {
@@ -405,52 +481,66 @@ __global__ void k_cell_buffer(Dev d, int *prev_status) {
   d.status[c] = st;
 }
 
-// donor search and IDW weights for receptor / fresh cells
-__global__ void k_donor(Dev d, const int *fresh_flag, const int *blk_order, int *n_orphan) {
-  int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= d.nc) return;
-  int st = d.status[c];
-  for (int m = 0; m < 5; ++m) { d.donors[5 * c + m] = -1; d.dwgt[5 * c + m] = 0.0; }
-  if (st != ST_RECEPTOR && !fresh_flag[c]) return;
-  double x = d.xc_new[2 * c], y = d.xc_new[2 * c + 1];
-  int own = d.cell_block[c];
-  int found = -1;
-  for (int cls = ST_FIELD; cls <= ST_RECEPTOR && found < 0; ++cls) {
-    for (int o = 0; o < d.nblocks && found < 0; ++o) {
-      int b = blk_order[o];
-      if (b == own) continue;
-      int e = first_containing(d, b, x, y, [&](int q) { return d.status[q] == cls; });
-      if (e >= 0) found = e;
+// Donor search and IDW weights of receptor and fresh cells; all other rows are
+// cleared.  A CTA lists the searching ones of its 32 cells and gives each a group of lanes
+// (bins' candidates, then a lane per donor); one thread a cell left the search,
+// a chain of dependent loads, to a few lanes of a warp (149504 cells: 43 us,
+// 22 so).
+constexpr int DONOR_CELLS = 32, DONOR_THREADS = DONOR_CELLS * NLANES;
+__global__ void __launch_bounds__(DONOR_THREADS) k_donor(Dev d, const int *fresh_flag, const int *blk_order,
+                                                         int *n_orphan) {
+  __shared__ int list[DONOR_CELLS], count;
+  if (threadIdx.x == 0) count = 0;
+  __syncthreads();
+  const int c0 = blockIdx.x * DONOR_CELLS, cells = min(DONOR_CELLS, d.nc - c0), here = c0 + threadIdx.x;
+  if ((int)threadIdx.x < cells && (d.status[here] == ST_RECEPTOR || fresh_flag[here])) list[atomicAdd(&count, 1)] = here;
+  for (int t = threadIdx.x; t < 5 * cells; t += DONOR_THREADS) {
+    d.donors[5 * (size_t)c0 + t] = -1;
+    d.dwgt[5 * (size_t)c0 + t] = 0.0;
+  }
+  __syncthreads();
+  const Group g;
+  const int t = threadIdx.x / NLANES;
+  if (t < count) {
+    const int c = list[t], own = d.cell_block[c];
+    const double x = d.xc_new[2 * c], y = d.xc_new[2 * c + 1];
+    int found = -1;
+    for (int cls = ST_FIELD; cls <= ST_RECEPTOR && found < 0; ++cls)
+      for (int o = 0; o < d.nblocks && found < 0; ++o) {
+        int b = blk_order[o];
+        if (b != own) found = first_containing(g, d, b, x, y, [&](int q) { return d.status[q] == cls; });
+      }
+    if (found < 0) {
+      if (g.lane == 0) atomicAdd(n_orphan, 1);
+      return;
+    }
+    // lane 0: the found cell, lanes 1 to 4 its neighbours that are no holes
+    int e = g.lane == 0 ? found : -1;
+    if (g.lane >= 1 && g.lane < 5 && d.nb_kind[4 * found + g.lane - 1] == NB_CELL) {
+      e = d.nb_id[4 * found + g.lane - 1];
+      if (d.status[e] == ST_HOLE) e = -1;
+    }
+    double d2 = 1.0;
+    if (e >= 0) {
+      const double ex = sb(x, d.xc_new[2 * e]), ey = sb(y, d.xc_new[2 * e + 1]);
+      d2 = ad(ml(ex, ex), ml(ey, ey));
+    }
+    const int shift = threadIdx.x & 24;
+    const unsigned valid = __ballot_sync(g.mask, e >= 0) >> shift & 0xffu;
+    const unsigned zero = __ballot_sync(g.mask, e >= 0 && d2 == 0.0) >> shift & 0xffu;
+    const int m = __popc(valid & ((1u << g.lane) - 1u));          // the lane's place in the row
+    const double inv = dv(1.0, d2);
+    double tot = 0.0;
+#pragma unroll
+    for (int l = 0; l < 5; ++l) {                                 // in the row's order
+      const double v = __shfl_sync(g.mask, inv, l, NLANES);
+      if (valid >> l & 1u) tot = ad(tot, v);
+    }
+    if (e >= 0) {
+      d.donors[5 * (size_t)c + m] = e;
+      d.dwgt[5 * (size_t)c + m] = zero ? (g.lane == __ffs(zero) - 1 ? 1.0 : 0.0) : dv(inv, tot);
     }
   }
-  if (found < 0) {
-    atomicAdd(n_orphan, 1);
-    return;
-  }
-  int stn[5];
-  int ns = 0;
-  stn[ns++] = found;
-  for (int s = 0; s < 4; ++s) {
-    if (d.nb_kind[4 * found + s] != NB_CELL) continue;
-    int e = d.nb_id[4 * found + s];
-    if (d.status[e] != ST_HOLE) stn[ns++] = e;
-  }
-  double d2[5];
-  int zero = -1;
-  for (int m = 0; m < ns; ++m) {
-    double ex = sb(x, d.xc_new[2 * stn[m]]), ey = sb(y, d.xc_new[2 * stn[m] + 1]);
-    d2[m] = ad(ml(ex, ex), ml(ey, ey));
-    if (d2[m] == 0.0 && zero < 0) zero = m;
-  }
-  for (int m = 0; m < ns; ++m) d.donors[5 * c + m] = stn[m];
-  if (zero >= 0) {
-    d.dwgt[5 * c + zero] = 1.0;
-    return;
-  }
-  double inv[5], tot = 0.0;
-  for (int m = 0; m < ns; ++m) inv[m] = dv(1.0, d2[m]);
-  for (int m = 0; m < ns; ++m) tot = ad(tot, inv[m]);
-  for (int m = 0; m < ns; ++m) d.dwgt[5 * c + m] = dv(inv[m], tot);
 }
 
 // Receptor and fresh-cell lists, compacted on the device in ascending cell
@@ -587,14 +677,16 @@ void launch_connect(const Dev &d, cudaStream_t s, int *prev_status, const int *b
   k_node_f<<<nblk(d.nn > d.nseg ? d.nn : d.nseg, 256), 256, 0, s>>>(d);
   k_body_box<<<d.nblocks, 32, 0, s>>>(d);
   k_bin_count<<<nblk(d.nc, 256), 256, 0, s>>>(d);
-  k_bin_scan<<<1, 1024, 0, s>>>(d);
+  k_bin_scan<<<nblk(d.nbins, SCAN_CHUNK), SCAN_THREADS, 0, s>>>(d);
   k_bin_fill<<<nblk(d.nc, 256), 256, 0, s>>>(d);
+  k_node_classify<<<nblk(d.nn, 128), 128, 0, s>>>(d);
+  const int todo = std::min(nblk((size_t)d.nn * NLANES, 256), 152 * 8);      // CTAs, strided over the list
   size_t segb = sizeof(float4) * (size_t)d.nseg;
-  if (segb <= 48 * 1024) k_node_classify<true><<<nblk(d.nn, 128), 128, segb, s>>>(d);
-  else k_node_classify<false><<<nblk(d.nn, 128), 128, 0, s>>>(d);
+  if (segb <= 48 * 1024) k_node_todo<true><<<todo, 256, segb, s>>>(d);
+  else k_node_todo<false><<<todo, 256, 0, s>>>(d);
   k_cell_classify<<<nblk(d.nc, 256), 256, 0, s>>>(d);
   k_cell_buffer<<<nblk(d.nc, 256), 256, 0, s>>>(d, prev_status);
-  k_donor<<<nblk(d.nc, 128), 128, 0, s>>>(d, prev_status, blk_order, n_orphan);
+  k_donor<<<nblk(d.nc, DONOR_CELLS), DONOR_THREADS, 0, s>>>(d, prev_status, blk_order, n_orphan);
 }
 
 void launch_lists(const Dev &d, cudaStream_t s, const int *fresh_flag, const int *n_orphan) {
