@@ -29,6 +29,7 @@ struct ugks_ctx {
   // (which reads none of them); not where an outflow ghost state follows W
   // or on a velocity shard (whose Step 7 waits for the host exchange)
   bool split_tail = false;
+  bool slope_stale = false;           // moved, the slope cases not yet set (no assembly so far)
   // the residual in two passes (residual_split); not within a batch of several
   // instances, whose other steps fill the SMs the sweep leaves
   bool split_residual = false;
@@ -581,6 +582,14 @@ int upload_step_size(ugks_ctx *ctx) {
   return launch_upload(const_cast<double *>(d.stepc), v, sizeof(v), ctx->st);
 }
 
+// The slope cases of a move that no assembly followed.
+void fresh_slopes(ugks_ctx *ctx) {
+  if (!ctx->slope_stale) return;
+  launch_slope_geo(ctx->d, ctx->st);
+  ctx->launches += 1;
+  ctx->slope_stale = false;
+}
+
 // Ghost states, W gradients, face reduction, face coefficients, per-cell
 // macro flux sum (Steps 1 / 3 up to the velocity-resolved flux); the sum
 // only where asked for, the macro sweep's gather takes its own (with_sum).
@@ -653,6 +662,7 @@ int do_connect(ugks_ctx *ctx, ugks_connect_stats *stats, bool initial, bool sync
     launch_lists(d, ctx->st, ctx->prev_status, ctx->n_orphan);
   }
   launch_slope_geo(d, ctx->st);     // holes changed
+  ctx->slope_stale = false;
   ctx->launches += 13;
   ctx->fresh_pending = !initial;
   int r = launch_status(ctx);
@@ -1163,7 +1173,7 @@ int ugks_init_mesh(ugks_ctx *ctx, int nblocks, const ugks_block_desc *blocks, co
   launch_move_nodes(d, ctx->st);
   CK(cudaMemcpyAsync(d.X_old, d.X_new, sizeof(double) * 2 * s.nn, cudaMemcpyDeviceToDevice, ctx->st));
   launch_geometry(d, ctx->st, ctx->fp32);
-  ctx->launches += 5;
+  ctx->launches += 3;
   // initial state from the primitive field (staged through Wp)
   CK(cudaMemcpyAsync(d.Wp, prim, sizeof(double) * 4 * s.nc, cudaMemcpyHostToDevice, ctx->st));
   launch_init_state(d, ctx->st, d.Wp, ctx->fp32);
@@ -1202,9 +1212,11 @@ int ugks_move_mesh(ugks_ctx *ctx, double t_new, const double *affine) {
     Prof p(ctx, UGKS_PROF_GEOMETRY);
     launch_move_nodes(d, ctx->st);
     launch_geometry(d, ctx->st, ctx->fp32);
-    launch_slope_geo(d, ctx->st);
+    // with several blocks the assembly that follows sets the slope cases anew
+    ctx->slope_stale = ctx->nblocks > 1;
+    if (!ctx->slope_stale) launch_slope_geo(d, ctx->st);
   }
-  ctx->launches += 6;
+  ctx->launches += ctx->slope_stale ? 3 : 4;
   ctx->moved = true;
   return launch_status(ctx);
 }
@@ -1225,6 +1237,7 @@ int ugks_step(ugks_ctx *ctx, double dt, int n_inner) {
   if (fabs(dt - d.dt) > 1e-12 * fabs(d.dt)) return fail(ctx, UGKS_ERR_ARG, "dt differs from the move's step");
   // graphs need a step free of host work: not while profiling or checking
   // each launch, and not on a velocity shard (its exchange runs on the host)
+  fresh_slopes(ctx);
   bool graph = ctx->graphs && !ctx->prof_on && !ctx->debug_sync && !d.shard;
   int rx = graph ? step_graph(ctx, n_inner) : step_body(ctx, n_inner);
   if (rx) return rx;
@@ -1452,6 +1465,7 @@ int ugks_eval_flux(ugks_ctx *ctx, double *D, double *F) {
   if (!ctx->moved) return fail(ctx, UGKS_ERR_ORDER, "ugks_eval_flux needs a preceding ugks_move_mesh");
   Dev &d = ctx->d;
   if (D && !is_device_ptr(D)) return fail(ctx, UGKS_ERR_ARG, "D must be a device pointer");
+  fresh_slopes(ctx);
   do_interp(ctx, 0);
   int r = flux_prep(ctx, 0, true);
   if (r) return r;

@@ -29,9 +29,7 @@ __device__ __forceinline__ double shoelace(const double *X, const int *nd) {
 
 // Cell volumes at both levels (shoelace), mid-time and new vertex centres,
 // period vector of the cell's row.
-__global__ void k_cell_geom(Dev d) {
-  int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= d.nc) return;
+__device__ __forceinline__ void cell_geom(const Dev &d, int c) {
   const int *nd = d.cell_nodes + 4 * c;
   double vo = shoelace(d.X_old, nd), vn = shoelace(d.X_new, nd);
   d.vol_old[c] = vo;
@@ -54,27 +52,46 @@ __global__ void k_cell_geom(Dev d) {
 
 // Mid-time face vector S n (L -> R / outward), centre, face velocity (mean
 // node velocity) and S U.n.
-__global__ void k_face_geom(Dev d) {
-  int f = blockIdx.x * blockDim.x + threadIdx.x;
-  if (f >= d.nf) return;
+template <typename T> __device__ __forceinline__ void face_geom(const Dev &d, int f) {
   int a = d.face_a[f], b = d.face_b[f];
   double ax = 0.5 * (d.X_old[2 * a] + d.X_new[2 * a]), ay = 0.5 * (d.X_old[2 * a + 1] + d.X_new[2 * a + 1]);
   double bx = 0.5 * (d.X_old[2 * b] + d.X_new[2 * b]), by = 0.5 * (d.X_old[2 * b + 1] + d.X_new[2 * b + 1]);
   double ex = bx - ax, ey = by - ay;
-  double S = sqrt(ex * ex + ey * ey);
+  const double S = sqrt(ex * ex + ey * ey), iS = 1.0 / S, idt = 1.0 / d.dt;
   d.Sn[2 * f] = ey;
   d.Sn[2 * f + 1] = -ex;
   d.S[f] = S;
-  d.nrm[2 * f] = ey / S;
-  d.nrm[2 * f + 1] = -ex / S;
+  d.nrm[2 * f] = ey * iS;
+  d.nrm[2 * f + 1] = -ex * iS;
   d.xf[2 * f] = 0.5 * (ax + bx);
   d.xf[2 * f + 1] = 0.5 * (ay + by);
-  double ufx = 0.5 * ((d.X_new[2 * a] - d.X_old[2 * a]) + (d.X_new[2 * b] - d.X_old[2 * b])) / d.dt;
-  double ufy = 0.5 * ((d.X_new[2 * a + 1] - d.X_old[2 * a + 1]) + (d.X_new[2 * b + 1] - d.X_old[2 * b + 1])) / d.dt;
+  double ufx = 0.5 * ((d.X_new[2 * a] - d.X_old[2 * a]) + (d.X_new[2 * b] - d.X_old[2 * b])) * idt;
+  double ufy = 0.5 * ((d.X_new[2 * a + 1] - d.X_old[2 * a + 1]) + (d.X_new[2 * b + 1] - d.X_old[2 * b + 1])) * idt;
   d.Uf[2 * f] = ufx;
   d.Uf[2 * f + 1] = ufy;
-  d.SUn[f] = ufx * ey + ufy * (-ex);
-  d.Un[f] = d.SUn[f] / d.S[f];
+  const double sun = ufx * ey + ufy * (-ex);
+  d.SUn[f] = sun;
+  d.Un[f] = sun * iS;
+  T *g = reinterpret_cast<T *>(d.fgeo) + (size_t)NFG * f;
+  g[FG_SNX] = (T)ey;
+  g[FG_SNY] = (T)(-ex);
+  g[FG_SUN] = (T)sun;
+  g[FG_UFX] = (T)ufx;
+  g[FG_UFY] = (T)ufy;
+}
+
+// Both in one launch (they share nothing): the first CTAs take the faces.  The
+// FP64 pipe bounds them (one division and a square root a face), on small
+// meshes the launches.
+constexpr int GEO_THREADS = 128;
+template <typename T> __global__ void __launch_bounds__(GEO_THREADS) k_geom(Dev d, int face_blocks) {
+  if ((int)blockIdx.x < face_blocks) {
+    const int f = blockIdx.x * GEO_THREADS + threadIdx.x;
+    if (f < d.nf) face_geom<T>(d, f);
+  } else {
+    const int c = ((int)blockIdx.x - face_blocks) * GEO_THREADS + threadIdx.x;
+    if (c < d.nc) cell_geom(d, c);
+  }
 }
 
 __device__ __forceinline__ double warp_sum(double v) {
@@ -135,20 +152,24 @@ __device__ __forceinline__ float warp_total(const Acc<float> &a) {
 // The sum is a convex piecewise-linear function of v, so over the tensor
 // velocity grid its maximum is attained at one of the four corners of the
 // velocity box (which are grid points): only those are evaluated.
-__global__ void k_dts(Dev d, double vx0, double vx1, double vy0, double vy1) {
-  int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= d.nc) return;
-  double m = 0.0;
-  for (int corner = 0; corner < 4; ++corner) {
-    double vx = (corner & 1) ? vx1 : vx0, vy = (corner & 2) ? vy1 : vy0;
-    double s = 0.0;
-    for (int q = 0; q < 4; ++q) {
-      int f = d.cell_faces[4 * c + q];
-      double wS = vx * d.Sn[2 * f] + vy * d.Sn[2 * f + 1] - d.SUn[f];
-      s += fmax(d.cell_sgn[4 * c + q] * wS, 0.0);
-    }
-    m = fmax(m, s);
+__device__ __forceinline__ void cell_dts(const Dev &d, int c) {
+  const double vx0 = d.vbox[0], vx1 = d.vbox[1], vy0 = d.vbox[2], vy1 = d.vbox[3];
+  // (positive parts by the sign bit, off the FP64 pipe)
+  auto pos = [](double x) { return __double2hiint(x) >= 0 ? x : 0.0; };
+  double s00 = 0.0, s01 = 0.0, s10 = 0.0, s11 = 0.0;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int f = d.cell_faces[4 * c + q];
+    const bool in = d.cell_sgn[4 * c + q] < 0;
+    const double2 n = *reinterpret_cast<const double2 *>(d.Sn + 2 * (size_t)f);
+    const double u = d.SUn[f], nx = in ? -n.x : n.x, ny = in ? -n.y : n.y, un = in ? -u : u;
+    const double x0 = vx0 * nx, x1 = vx1 * nx, y0 = vy0 * ny - un, y1 = vy1 * ny - un;
+    s00 += pos(x0 + y0);
+    s01 += pos(x0 + y1);
+    s10 += pos(x1 + y0);
+    s11 += pos(x1 + y1);
   }
+  const double m = fmax(fmax(s00, s01), fmax(s10, s11));
   const double dts = d.cfl_s * d.vol_new[c] / m;
   d.dts[c] = dts;
   d.idtau[c] = d.cfl_s / (d.cfl_pseudo * dts);
@@ -156,33 +177,40 @@ __global__ void k_dts(Dev d, double vx0, double vx1, double vy0, double vy1) {
 
 // Per-step geometry records in the arithmetic type: per face (S n, S U.n,
 // U_f, vectors from the L image / R centres to the face centre), per cell
-// the outward (S n, S U.n) of its four faces for the sweeps.
-template <typename T> __global__ void k_geo_records(Dev d) {
-  int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t < d.nf) {
-    int f = t, L = d.face_L[f], R = d.face_R[f];
-    T *g = reinterpret_cast<T *>(d.fgeo) + (size_t)NFG * f;
-    double sh = (double)d.face_shiftL[f];
-    g[FG_SNX] = (T)d.Sn[2 * f];
-    g[FG_SNY] = (T)d.Sn[2 * f + 1];
-    g[FG_SUN] = (T)d.SUn[f];
-    g[FG_UFX] = (T)d.Uf[2 * f];
-    g[FG_UFY] = (T)d.Uf[2 * f + 1];
-    g[FG_DXLX] = (T)(d.xf[2 * f] - (d.xc[2 * L] + sh * d.period[2 * L]));
-    g[FG_DXLY] = (T)(d.xf[2 * f + 1] - (d.xc[2 * L + 1] + sh * d.period[2 * L + 1]));
-    g[FG_DXRX] = R >= 0 ? (T)(d.xf[2 * f] - d.xc[2 * R]) : T(0);
-    g[FG_DXRY] = R >= 0 ? (T)(d.xf[2 * f + 1] - d.xc[2 * R + 1]) : T(0);
+// half the outward (S n, S U.n) of its four faces for the sweeps.
+// The face's part without cell centres comes from the face geometry, so that a
+// cell takes it in the arithmetic type (conversions pass the FP64 pipe; a half
+// and a sign commute with the rounding).
+template <typename T> __device__ __forceinline__ void face_record(const Dev &d, int f) {
+  int L = d.face_L[f], R = d.face_R[f];
+  T *g = reinterpret_cast<T *>(d.fgeo) + (size_t)NFG * f;
+  double sh = (double)d.face_shiftL[f];
+  g[FG_DXLX] = (T)(d.xf[2 * f] - (d.xc[2 * L] + sh * d.period[2 * L]));
+  g[FG_DXLY] = (T)(d.xf[2 * f + 1] - (d.xc[2 * L + 1] + sh * d.period[2 * L + 1]));
+  g[FG_DXRX] = R >= 0 ? (T)(d.xf[2 * f] - d.xc[2 * R]) : T(0);
+  g[FG_DXRY] = R >= 0 ? (T)(d.xf[2 * f + 1] - d.xc[2 * R + 1]) : T(0);
+}
+template <typename T> __device__ __forceinline__ void cell_record(const Dev &d, int c) {
+  T *r = reinterpret_cast<T *>(d.srec) + (size_t)NSR * c;
+#pragma unroll
+  for (int s = 0; s < 4; ++s) {
+    const T *g = reinterpret_cast<const T *>(d.fgeo) + (size_t)NFG * d.cell_faces[4 * c + s];
+    const T h = d.cell_sgn[4 * c + s] < 0 ? T(-0.5) : T(0.5);
+    r[sr_at(0, s)] = h * g[FG_SNX];
+    r[sr_at(1, s)] = h * g[FG_SNY];
+    r[sr_at(2, s)] = h * g[FG_SUN];
   }
-  if (t < d.nc) {
-    int c = t;
-    T *r = reinterpret_cast<T *>(d.srec) + (size_t)NSR * c;
-    for (int s = 0; s < 4; ++s) {
-      int f = d.cell_faces[4 * c + s];
-      double sg = (double)d.cell_sgn[4 * c + s];
-      r[sr_at(0, s)] = (T)(0.5 * sg * d.Sn[2 * f]);
-      r[sr_at(1, s)] = (T)(0.5 * sg * d.Sn[2 * f + 1]);
-      r[sr_at(2, s)] = (T)(0.5 * sg * d.SUn[f]);
-    }
+}
+// the records and the time steps of the cells in one launch
+template <typename T> __global__ void __launch_bounds__(GEO_THREADS) k_geo_records(Dev d, int face_blocks) {
+  if ((int)blockIdx.x < face_blocks) {
+    const int f = blockIdx.x * GEO_THREADS + threadIdx.x;
+    if (f < d.nf) face_record<T>(d, f);
+  } else {
+    const int c = ((int)blockIdx.x - face_blocks) * GEO_THREADS + threadIdx.x;
+    if (c >= d.nc) return;
+    cell_dts(d, c);
+    cell_record<T>(d, c);
   }
 }
 
@@ -237,7 +265,7 @@ __global__ void k_slope_geo(Dev d) {
     flags |= cs << (2 * dir);
   }
   double a11 = g[0][0], a12 = g[0][1], a21 = g[1][0], a22 = g[1][1];
-  double det = a11 * a22 - a12 * a21;
+  const double idet = 1.0 / (a11 * a22 - a12 * a21);
   d.slope_flags[c] = flags;
   // sweep mask: bit 0 solved cell, bit 1+s: neighbour across face slot s is solved
   int mask = d.status[c] == ST_FIELD ? 1 : 0;
@@ -247,12 +275,10 @@ __global__ void k_slope_geo(Dev d) {
     if (nb >= 0 && d.status[nb] == ST_FIELD) mask |= 2 << s;
   }
   d.cmask[c] = mask;
-  d.jinv[4 * c + 0] = a22 / det;
-  d.jinv[4 * c + 1] = -a12 / det;
-  d.jinv[4 * c + 2] = -a21 / det;
-  d.jinv[4 * c + 3] = a11 / det;
-  d.jinvf[c] = make_float4((float)d.jinv[4 * c + 0], (float)d.jinv[4 * c + 1], (float)d.jinv[4 * c + 2],
-                           (float)d.jinv[4 * c + 3]);
+  const double j0 = a22 * idet, j1 = -a12 * idet, j2 = -a21 * idet, j3 = a11 * idet;
+  reinterpret_cast<double2 *>(d.jinv + 4 * c)[0] = make_double2(j0, j1);
+  reinterpret_cast<double2 *>(d.jinv + 4 * c)[1] = make_double2(j2, j3);
+  d.jinvf[c] = make_float4((float)j0, (float)j1, (float)j2, (float)j3);
 }
 
 // Ghost states of far-field / outflow faces (reading R6).
@@ -1054,14 +1080,13 @@ int launch_upload(void *dst, const void *src, size_t n, cudaStream_t s) {
   return launches;
 }
 void launch_geometry(const Dev &d, cudaStream_t s, int fp32) {
-  k_cell_geom<<<nblk(d.nc, 256), 256, 0, s>>>(d);
-  k_face_geom<<<nblk(d.nf, 256), 256, 0, s>>>(d);
-  k_dts<<<nblk(d.nc, 256), 256, 0, s>>>(d, d.vbox[0], d.vbox[1], d.vbox[2], d.vbox[3]);
-  int n = d.nf > d.nc ? d.nf : d.nc;
-  if (fp32) k_geo_records<float><<<nblk(n, 256), 256, 0, s>>>(d);
-  else k_geo_records<double><<<nblk(n, 256), 256, 0, s>>>(d);
+  const int faces = nblk(d.nf, GEO_THREADS), grid = faces + nblk(d.nc, GEO_THREADS);
+  if (fp32) k_geom<float><<<grid, GEO_THREADS, 0, s>>>(d, faces);
+  else k_geom<double><<<grid, GEO_THREADS, 0, s>>>(d, faces);
+  if (fp32) k_geo_records<float><<<grid, GEO_THREADS, 0, s>>>(d, faces);
+  else k_geo_records<double><<<grid, GEO_THREADS, 0, s>>>(d, faces);
 }
-void launch_slope_geo(const Dev &d, cudaStream_t s) { k_slope_geo<<<nblk(d.nc, 256), 256, 0, s>>>(d); }
+void launch_slope_geo(const Dev &d, cudaStream_t s) { k_slope_geo<<<nblk(d.nc, 128), 128, 0, s>>>(d); }
 
 void launch_ghost_gradW(const Dev &d, cudaStream_t s) {
   k_ghost<<<nblk(d.nf, 256), 256, 0, s>>>(d);
