@@ -43,9 +43,9 @@ struct ugks_ctx {
   std::vector<ugks_block_desc> blocks;
   std::vector<int> cell_off, node_off;
   int max_nj = 0;
-  int sweep_nw = 1, nwork = 0, nsm = 0;  // micro sweeps: warps per CTA, CTAs
-  int nwork_cap = 0;                  // work-list capacity (largest tuning candidate)
-  int sweep_rg = 4;                   // micro sweeps: rows per group
+  // micro sweeps (forward, backward): shape, warps per CTA, first CTA in the work list, CTAs
+  struct Sweep { int shape = 0, nw = 1, first = 0, n = 0; } sweep[2];
+  int nwork_cap = 0, nsm = 0;         // work-list capacity
   int ns_fwd = 4, ns_bwd = 4;         // prefetch ring depths (steps) of the two sweeps
   ugks_exchange_fn xfn = nullptr;     // velocity sharding: the caller's exchange
   void *xuser = nullptr;
@@ -107,6 +107,9 @@ int cuda_check(ugks_ctx *c, cudaError_t e, const char *what) {
     if (_r) return _r;                                             \
   } while (0)
 
+// Velocities between cells: a cell's (h, b) pairs start on a line of 128 bytes.
+int velocity_stride(int nv) { return (nv + 15) / 16 * 16; }
+
 struct Sizes {
   int nc = 0, nf = 0, nn = 0, nv = 0, nvp = 0, nseg = 0, nring = 0, max_nj = 0, ntiles = 0;
   int nvx = 0, nvy = 0;
@@ -138,9 +141,9 @@ int validate(const ugks_params *p, int nb, const ugks_block_desc *b, Sizes &s, s
   }
   s.iy0 = iy0;
   s.nv = p->nvx * (iy1 - iy0);
-  s.nvp = (s.nv + 3) / 4 * 4;
+  s.nvp = velocity_stride(s.nv);
   s.nv_all = p->nvx * p->nvy;
-  s.nvp_all = (s.nv_all + 3) / 4 * 4;
+  s.nvp_all = velocity_stride(s.nv_all);
   s.nvx = p->nvx;
   s.nvy = p->nvy;
   for (int i = 0; i < nb; ++i) {
@@ -183,37 +186,42 @@ struct Carver {
   }
 };
 // Micro sweeps (skewed wavefront, ugks_sweep.cu): a warp takes a band of
-// wsweep_rows(rg) rows of a block and wsweep_vw consecutive velocities; a CTA
+// wsweep_rows rows of a block and wsweep_vw consecutive velocities; a CTA
 // holds, for one block, a warp per band for each of its velocity groups; every
 // CTA has nw warps, nw = the largest band count of the blocks, so a smaller
-// block takes several groups per CTA.
-int bands_of(int nj, int rg) { return (nj + wsweep_rows(rg) - 1) / wsweep_rows(rg); }
-int sweep_nw_for(int nb, const ugks_block_desc *b, int rg) {
+// block takes several groups per CTA.  The shape of a sweep follows from the
+// whole velocity grid (the same on every shard of it).
+int bands_of(int nj, int shape) { return (nj + wsweep_rows(shape) - 1) / wsweep_rows(shape); }
+int sweep_nw_for(int nb, const ugks_block_desc *b, int shape) {
   int m = 1;
-  for (int i = 0; i < nb; ++i) m = std::max(m, bands_of(b[i].nj, rg));
+  for (int i = 0; i < nb; ++i) m = std::max(m, bands_of(b[i].nj, shape));
   return m;
 }
-int sweep_rg_for(const ugks_params *p, int nb, const ugks_block_desc *b) {
+int sweep_shape(const ugks_params *p, int nb, const ugks_block_desc *b, int pass) {
   int nj = 1;
-  for (int i = 0; i < nb; ++i) nj = std::max(nj, b[i].nj);
-  return wsweep_rg(nj, p->precision != UGKS_FP64);
+  double cells = 0.0;
+  for (int i = 0; i < nb; ++i) {
+    nj = std::max(nj, b[i].nj);
+    cells += (double)b[i].ni * b[i].nj;
+  }
+  const char *e = getenv("UGKS_SWEEP_SHAPE");      // one of the FP32 shapes (all give the same bits)
+  return wsweep_shape(p->precision != UGKS_FP64, pass, nj, 8.0 * cells * p->nvx * p->nvy, e ? atoi(e) : -1);
 }
 
 // Work list (block, first velocity, velocity groups in the CTA) per CTA (nvp:
-// the context's padded velocity count).
-std::vector<int> ws_work(const ugks_params *p, int nb, const ugks_block_desc *b, int nvp, int rg) {
-  std::vector<int> work;
-  int vw = wsweep_vw(p->precision != UGKS_FP64), nw = sweep_nw_for(nb, b, rg);
+// the context's padded velocity count), appended to `work`; returns the CTAs.
+int ws_work(int nb, const ugks_block_desc *b, int nvp, int shape, std::vector<int> &work) {
+  int vw = wsweep_vw(shape), nw = sweep_nw_for(nb, b, shape), n = 0;
   int groups = (nvp + vw - 1) / vw;
   for (int i = 0; i < nb; ++i) {
-    int gpc = std::max(1, nw / bands_of(b[i].nj, rg));
-    for (int g0 = 0; g0 < groups; g0 += gpc) {
+    int gpc = std::max(1, nw / bands_of(b[i].nj, shape));
+    for (int g0 = 0; g0 < groups; g0 += gpc, ++n) {
       work.push_back(i);
       work.push_back(g0 * vw);
       work.push_back(std::min(gpc, groups - g0));
     }
   }
-  return work;
+  return n;
 }
 
 // Candidates of the sweep autotuner: prefetch ring depths (steps).
@@ -222,8 +230,9 @@ constexpr int kTuneRing[] = {2, 4, 6};
 // Work-list capacity (sized for the whole velocity grid, which covers any
 // shard of it).
 int nwork_cap_for(const ugks_params *p, int nb, const ugks_block_desc *b) {
-  int nvp = (p->nvx * p->nvy + 3) / 4 * 4;
-  return (int)ws_work(p, nb, b, nvp, sweep_rg_for(p, nb, b)).size() / 3;
+  int nvp = velocity_stride(p->nvx * p->nvy);
+  std::vector<int> work;
+  return ws_work(nb, b, nvp, sweep_shape(p, nb, b, 0), work) + ws_work(nb, b, nvp, sweep_shape(p, nb, b, 1), work);
 }
 
 // Lay out every device array of the context in the workspace (base may be
@@ -582,6 +591,12 @@ int upload_step_size(ugks_ctx *ctx) {
   return launch_upload(const_cast<double *>(d.stepc), v, sizeof(v), ctx->st);
 }
 
+// Micro sweep (pass 0 forward, 1 backward) with ring depth ns.
+void launch_sweep(const ugks_ctx *ctx, int pass, int ns) {
+  const auto &w = ctx->sweep[pass];
+  launch_wsweep(ctx->d, ctx->st, pass, ctx->work + 3 * w.first, w.n, w.nw, ns, w.shape);
+}
+
 // The slope cases of a move that no assembly followed.
 void fresh_slopes(ugks_ctx *ctx) {
   if (!ctx->slope_stale) return;
@@ -723,8 +738,8 @@ int step_body(ugks_ctx *ctx, int n_inner) {
     { Prof p(ctx, UGKS_PROF_RESIDUAL); launch_residual(d, s, it == 0, fp, two ? 2 : 0); }
     if (two) ctx->launches += 1;
     if (met) launch_metrics(d, s, 1, fp);
-    { Prof p(ctx, UGKS_PROF_MICRO_FWD); launch_wsweep(d, s, 0, ctx->work, ctx->nwork, ctx->sweep_nw, ctx->ns_fwd, ctx->sweep_rg, fp); }  // Step 6
-    { Prof p(ctx, UGKS_PROF_MICRO_BWD); launch_wsweep(d, s, 1, ctx->work, ctx->nwork, ctx->sweep_nw, ctx->ns_bwd, ctx->sweep_rg, fp); }
+    { Prof p(ctx, UGKS_PROF_MICRO_FWD); launch_sweep(ctx, 0, ctx->ns_fwd); }  // Step 6
+    { Prof p(ctx, UGKS_PROF_MICRO_BWD); launch_sweep(ctx, 1, ctx->ns_bwd); }
     if (split && it + 1 < n_inner) {
       // Step 7, the receptors' W and q and the W gradients of the next
       // iteration on the tail stream, beside its velocity reduction
@@ -755,8 +770,8 @@ int step_body(ugks_ctx *ctx, int n_inner) {
 // What the captured kernels depend on beyond device memory: the device
 // struct they take by value and the launch configuration.
 std::vector<unsigned char> graph_key(const ugks_ctx *c, int n_inner) {
-  int cfg[] = {n_inner, c->fresh_pending ? 1 : 0, c->sweep_rg, c->ns_fwd, c->ns_bwd, c->sweep_nw,
-               c->nwork, c->nsm, c->max_nj, c->fp32, c->metrics ? 1 : 0, c->split_tail ? 1 : 0,
+  int cfg[] = {n_inner, c->fresh_pending ? 1 : 0, c->ns_fwd, c->ns_bwd, c->sweep[0].shape, c->sweep[0].n,
+               c->sweep[1].shape, c->sweep[1].n, c->nsm, c->max_nj, c->fp32, c->metrics ? 1 : 0, c->split_tail ? 1 : 0,
                c->split_residual && !c->in_batch ? 1 : 0};
   // (the step size is read from device memory; the bin count belongs to the
   // assembly, which is not part of the step)
@@ -956,8 +971,10 @@ int ugks_init_mesh(ugks_ctx *ctx, int nblocks, const ugks_block_desc *blocks, co
   ctx->nblocks = nblocks;
   ctx->blocks.assign(blocks, blocks + nblocks);
   ctx->max_nj = s.max_nj;
-  ctx->sweep_rg = sweep_rg_for(&ctx->p, nblocks, blocks);
-  ctx->sweep_nw = sweep_nw_for(nblocks, blocks, ctx->sweep_rg);
+  for (int pass = 0; pass < 2; ++pass) {
+    ctx->sweep[pass].shape = sweep_shape(&ctx->p, nblocks, blocks, pass);
+    ctx->sweep[pass].nw = sweep_nw_for(nblocks, blocks, ctx->sweep[pass].shape);
+  }
   if (const char *e = getenv("UGKS_SWEEP_NS")) {
     int n = atoi(e);
     if (n == 2 || n == 4 || n == 6) ctx->ns_fwd = ctx->ns_bwd = n;
@@ -969,7 +986,8 @@ int ugks_init_mesh(ugks_ctx *ctx, int nblocks, const ugks_block_desc *blocks, co
       ctx->nsm = nsm;
     cudaGetLastError();
   }
-  if (!wsweep_fits(ctx->fp32, ctx->fbf, ctx->sweep_rg, ctx->sweep_nw, 1))
+  if (!wsweep_fits(ctx->sweep[0].shape, ctx->fbf, ctx->sweep[0].nw, 1) ||
+      !wsweep_fits(ctx->sweep[1].shape, ctx->fbf, ctx->sweep[1].nw, 1))
     return fail(ctx, UGKS_ERR_ARG, "micro-sweep CTA of the tallest block exceeds shared memory");
   ctx->nwork_cap = nwork_cap_for(&ctx->p, nblocks, blocks);
   ctx->cap_interp = cap_interp_for(s, nblocks);
@@ -1060,9 +1078,12 @@ int ugks_init_mesh(ugks_ctx *ctx, int nblocks, const ugks_block_desc *blocks, co
       if (blocks[order[b]].priority > blocks[order[a]].priority ||
           (blocks[order[b]].priority == blocks[order[a]].priority && order[b] < order[a]))
         std::swap(order[a], order[b]);
-  std::vector<int> work = ws_work(&ctx->p, nblocks, blocks, s.nvp, ctx->sweep_rg);
-  ctx->nwork = (int)work.size() / 3;
-  if (ctx->nwork > ctx->nwork_cap) return fail(ctx, UGKS_ERR_WORKSPACE, "sweep work list");
+  std::vector<int> work;
+  for (auto &w : ctx->sweep) {
+    w.first = (int)work.size() / 3;
+    w.n = ws_work(nblocks, blocks, s.nvp, w.shape, work);
+  }
+  if ((int)work.size() / 3 > ctx->nwork_cap) return fail(ctx, UGKS_ERR_WORKSPACE, "sweep work list");
   std::vector<int> tiles;
   for (int b = 0; b < nblocks; ++b) {
     std::vector<int> org(2 * (size_t)tile_count(blocks[b].ni, blocks[b].nj));
@@ -1352,12 +1373,12 @@ int ugks_autotune(ugks_ctx *ctx, int reps, int *items_out, int *vpt_out, int *ri
   float tf = 1e30f, tb = 1e30f;
   for (int ns : kTuneRing) {
     if (r) break;
-    if (!wsweep_fits(fp, ctx->fbf, ctx->sweep_rg, ctx->sweep_nw, ns)) continue;
-    float ms;
-    if ((r = timed([&] { launch_wsweep(d, s, 0, ctx->work, ctx->nwork, ctx->sweep_nw, ns, ctx->sweep_rg, fp); }, ms))) break;
-    if (ms < tf) { tf = ms; bf = ns; }
-    if ((r = timed([&] { launch_wsweep(d, s, 1, ctx->work, ctx->nwork, ctx->sweep_nw, ns, ctx->sweep_rg, fp); }, ms))) break;
-    if (ms < tb) { tb = ms; bb = ns; }
+    for (int pass = 0; pass < 2 && !r; ++pass) {
+      if (!wsweep_fits(ctx->sweep[pass].shape, ctx->fbf, ctx->sweep[pass].nw, ns)) continue;
+      float ms, &best = pass ? tb : tf;
+      if ((r = timed([&] { launch_sweep(ctx, pass, ns); }, ms))) break;
+      if (ms < best) { best = ms; (pass ? bb : bf) = ns; }
+    }
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);

@@ -22,13 +22,13 @@ void launch_macro_pad(const Dev &d, cudaStream_t s, int fp32);              // o
 void launch_macro_prep(const Dev &d, cudaStream_t s, int fp32);
 void launch_macro_sweep(const Dev &d, cudaStream_t s, int rows, int fp32);   // sweep + post (after launch_macro_prep)
 // micro LU-SGS sweeps (ugks_sweep.cu): pass 0 forward, 1 backward; nw warps
-// per CTA, ns prefetch steps (1, 2, 4 or 6), rg rows per group (1, 2 or 4)
-void launch_wsweep(const Dev &d, cudaStream_t s, int pass, const int *work, int nwork, int nw, int ns, int rg, int fp32);
+// per CTA, ns prefetch steps (1, 2, 4 or 6), shape from wsweep_shape
+void launch_wsweep(const Dev &d, cudaStream_t s, int pass, const int *work, int nwork, int nw, int ns, int shape);
 void wsweep_setup();
-int wsweep_vw(int fp32);                  // velocities of a warp
-int wsweep_rows(int rg);                  // rows of a warp's band
-int wsweep_rg(int max_nj, int fp32);      // rows per group
-int wsweep_fits(int fp32, int fbf, int rg, int nw, int ns);
+int wsweep_shape(int fp32, int pass, int max_nj, double bytes, int forced);   // bytes of a (cell, velocity) array
+int wsweep_vw(int shape);                 // velocities of a warp
+int wsweep_rows(int shape);               // rows of a warp's band
+int wsweep_fits(int shape, int fbf, int nw, int ns);
 void launch_moments(const Dev &d, cudaStream_t s, int fp32);
 void launch_moments_finish(const Dev &d, cudaStream_t s);   // sharded step, after the exchange
 // step metrics: stage 0 after the macro prep (|R|^2), 1 after the residual

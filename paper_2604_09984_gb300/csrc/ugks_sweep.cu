@@ -4,70 +4,70 @@
 // / D, f += d, over every block in lexicographic order (i fastest), for
 // every discrete velocity independently.
 //
-// The sweep runs as a skewed wavefront.  A warp owns a band of 8 RG rows of a
-// block: 8 groups of QL = 4 lanes, RG rows a group, two velocities a lane (one
-// in FP64).  At step s, group g takes column i = s - g of its RG
-// rows one after the other: the lower neighbour along a row is the lane's own
-// result of the step before, the one across rows the row just computed, and
-// for the group's first row the last row of the group before, of its step
-// before, one warp shuffle away: no barrier inside a band.  Bands of one block
-// (warps of one CTA) pass the last row's values to the next band through a
-// ring in shared memory with progress counters (bounded waits).  Cells of
-// lower (upper) neighbours always come from earlier steps or rows, so the
-// result is the lexicographic Gauss-Seidel exactly.
+// The sweep runs as a skewed wavefront.  A warp owns a band of rows of a block:
+// 32 / QL groups of QL lanes, RG rows a group, VP velocities a lane.  At step s,
+// group g takes column i = s - g of its RG rows one after the other: the lower
+// neighbour along a row is the lane's own result of the step before, the one
+// across rows the row just computed, and for the group's first row the last row
+// of the group before, of its step before, one warp shuffle away: no barrier
+// inside a band.  Bands of one block (warps of one CTA) pass the last row's
+// values to the next band through a ring in shared memory with progress
+// counters (bounded waits).  Cells of lower (upper) neighbours always come from
+// earlier steps or rows, so the result is the lexicographic Gauss-Seidel exactly,
+// and the same to the bit for every shape.
 //
-// What bounds it: the latency of a step.  A step is some hundred instructions
-// of one warp, and a mesh has only one to four warps for a scheduler (issue
-// slots used: 31 %).  So the only chain between steps is the shuffle and four
-// operations a row; the rows of a lane share the step's overhead (copies, link,
-// shuffle); (h, b) go through packed FP32 instructions, and so do the two faces
-// of a direction in the coefficients; no copy is predicated, and the seam of a
-// periodic row has a body of its own.  A lane's inputs (residual / forward
-// result, f) and the cells' records come through the warp's ring of
-// asynchronous copies.  FP64 is bound by its pipe (some 15 cycles a warp
-// instruction and SM): one velocity a lane and few rows a group spread the work
-// over the SMs, and a step reads and prepares the next one's coefficients
-// behind its own results (FP32: in order, which holds fewer registers).
-// Forward / backward, us, before (one row a group of 2 or 4 lanes, one warp
-// shuffle and link a row) and after:
-//   FP32  32x16 cells, 256 velocities            26.5 / 28.5   22.5 / 19.0
-//   FP32  128x64 + 64x16 cells, 576 velocities    115 / 126      86 / 74
-//   FP32  256x128 + 128x32 cells, 1024            284 / 400     223 / 328
-//   FP32  512x256 + 192x48 cells, 4096           4602 / 5988   3570 / 5534
+// What bounds it: while the arrays stay in the L2, the latency of a step (some
+// hundred instructions of one warp, one to four warps a scheduler), beyond it
+// the lines touched (shapes below).  So the only chain between steps is the
+// shuffle and four operations a row; the rows of a lane share the step's
+// overhead (copies, link, shuffle); (h, b) go through packed FP32 instructions,
+// and so do the two faces of a direction in the coefficients; no copy is
+// predicated, and the seam of a periodic row has a body of its own.  A lane's
+// inputs (residual / forward result, f) and the cells' records come through the
+// warp's ring of asynchronous copies.  FP64 is bound by its pipe (some 15 cycles
+// a warp instruction and SM): one velocity a lane and few rows a group spread
+// the work over the SMs, and a step reads and prepares the next one's
+// coefficients behind its own results (FP32: in order, which holds fewer
+// registers).
+// Forward / backward, us, before (one row a group of 2 or 4 lanes, a warp
+// shuffle and link a row, 64 bytes of a cell a warp) and after:
+//   FP32  32x16 cells, 256 velocities            26.5 / 28.5   18.1 / 16.5
+//   FP32  128x64 + 64x16 cells, 576 velocities    115 / 126      70 / 76
+//   FP32  256x128 + 128x32 cells, 1024            284 / 400     190 / 236
+//   FP32  512x256 + 2 x 192x48 cells, 4096       4602 / 5988   1713 / 2862
 //   FP64  64x32 cells, 576                        445 / 405     135 / 141
 //   FP64  96x48 + 64x16 cells, 1024               927 / 713     414 / 361
-// (the largest one moves 9 / 14 GB: 2.7 / 2.6 TB/s)
+// (the largest one moves 9.8 / 14.7 GB: 5.7 / 5.1 TB/s)
 #include <type_traits>
 #include "ugks_internal.cuh"
 #include "ugks_launch.h"
 
 namespace ugks {
 
-constexpr int QL = 4, NGRP = 32 / QL;            // lanes a group, groups a warp
-template <typename T> struct WsVpt { static constexpr int N = sizeof(T) == 4 ? 2 : 1; };   // velocities a lane
 constexpr int WS_LR = 64;            // most ring entries between two bands (columns): the next band
                                      // trails by NGRP steps, the rest of the ring is slack; fewer
                                      // (a power of two >= 2) where shared memory is short
 
-// Shared memory of a warp and ring step, in 16-byte chunks: per row and lane
-// the lane's values (XC chunks; backward also f), per group its rows' records
-// (one chunk of padding: groups in distinct banks).
-template <typename T, int PASS, int RG, int FB> struct WsCfg {
+// Shared memory of a warp and ring step: per row and lane the lane's values
+// (XB bytes; backward also f), per group its rows' records (16 bytes of padding:
+// groups in distinct banks).
+template <typename T, int PASS, int FB, int QL, int RG, int VP> struct WsCfg {
   typedef typename Vec2<T>::type T2;
-  static constexpr int VPT = WsVpt<T>::N;
+  static constexpr int VPT = VP, NGRP = 32 / QL;                    // velocities a lane, groups a warp
   static constexpr bool BF = PASS == 1 && FB == 1;                  // bf16 f in the backward pass
-  static constexpr int XC = VPT * (int)sizeof(T2) / 16;
-  static constexpr int FBYTES = PASS == 1 ? (BF ? VPT * 4 : VPT * (int)sizeof(T2)) : 0;   // f of a lane and row
-  static constexpr int FC = (FBYTES + 15) / 16;
+  static constexpr int XB = VPT * (int)sizeof(T2);                  // bytes of a lane's values: 8 or 16
+  static_assert(XB == 8 || XB == 16, "one access a lane and row");
+  typedef typename std::conditional<XB == 16, float4, float2>::type XV;
+  static constexpr int FB_ = PASS == 1 ? (BF ? VPT * 4 : XB) : 0;   // bytes of f of a lane and row
   static constexpr int RC = NSR * (int)sizeof(T) / 16, RGS = RG * RC + 1;   // chunks of a record, of a group's records
-  static constexpr int OF = RG * XC * 32, OR = OF + RG * FC * 32, STEP = OR + NGRP * RGS;
+  static constexpr int OF = RG * XB * 32, OR = OF + RG * FB_ * 32, STEP = OR + NGRP * RGS * 16;   // bytes
 };
 
 // Shared memory of a sweep CTA with nw warps and ring depth ns.
-template <typename T, int PASS, int RG, int FB>
+template <typename T, int PASS, int FB, int QL, int RG, int VP>
 __host__ __device__ constexpr size_t ws_smem(int nw, int ns, int lr = WS_LR) {
-  typedef WsCfg<T, PASS, RG, FB> C;
-  return (size_t)nw * ns * C::STEP * 16 + (size_t)nw * lr * QL * C::VPT * sizeof(typename Vec2<T>::type) +
+  typedef WsCfg<T, PASS, FB, QL, RG, VP> C;
+  return (size_t)nw * ns * C::STEP + (size_t)nw * lr * QL * C::VPT * sizeof(typename Vec2<T>::type) +
          (size_t)nw * 2 * QL * sizeof(int);
 }
 
@@ -97,14 +97,14 @@ template <int BYTES> __device__ __forceinline__ void ws_copy(void *dst, const vo
 }
 
 // work item: block, first velocity, velocity groups in this CTA
-template <typename T, int PASS, int NS, int RG, int FB>
+template <typename T, int PASS, int FB, int NS, int QL, int RG, int VP>
 __global__ void __launch_bounds__(512) k_wsweep(Dev d, const int *work, int lr) {
   typedef typename Vec2<T>::type T2;
   typedef typename PairOf<T>::type P;
-  typedef WsCfg<T, PASS, RG, FB> C;
+  typedef WsCfg<T, PASS, FB, QL, RG, VP> C;
+  typedef typename C::XV XV;
   constexpr bool PIPE = sizeof(T) == 8;
-  constexpr int WROWS = NGRP * RG, VPT = C::VPT, VW = QL * VPT;
-  struct alignas(16) Chunk { unsigned char b[16]; };
+  constexpr int NGRP = C::NGRP, WROWS = NGRP * RG, VPT = C::VPT, VW = QL * VPT;
   extern __shared__ __align__(16) unsigned char smraw[];
   const int nw = blockDim.x >> 5, w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int grp = lane / QL, q = lane - grp * QL;
@@ -114,8 +114,8 @@ __global__ void __launch_bounds__(512) k_wsweep(Dev d, const int *work, int lr) 
   const bool per = bi[2] != 0;
   const int nb = (nj + WROWS - 1) / WROWS;        // bands of the block
   const int gw = w / nb, band = w - gw * nb;     // velocity group, band
-  Chunk *ring = reinterpret_cast<Chunk *>(smraw) + (size_t)w * NS * C::STEP;
-  P *links = reinterpret_cast<P *>(smraw + (size_t)nw * NS * C::STEP * 16);
+  unsigned char *ring = smraw + (size_t)w * NS * C::STEP;
+  P *links = reinterpret_cast<P *>(smraw + (size_t)nw * NS * C::STEP);
   volatile int *prog = reinterpret_cast<volatile int *>(links + (size_t)nw * lr * VW);
   volatile int *cons = prog + nw * QL;
   if (lane < QL) prog[w * QL + lane] = cons[w * QL + lane] = 0;
@@ -152,22 +152,14 @@ __global__ void __launch_bounds__(512) k_wsweep(Dev d, const int *work, int lr) 
   }
   // copies of step st into ring slot sl
   auto issue = [&](int st, int sl) {
-    Chunk *dst = ring + sl * C::STEP;
+    unsigned char *dst = ring + sl * C::STEP;
 #pragma unroll
     for (int r = 0; r < RG; ++r) {
+      ws_copy<C::XB>(dst + (r * 32 + lane) * C::XB, xp[r]);
+      if (PASS == 1) ws_copy<C::FB_>(dst + C::OF + (r * 32 + lane) * C::FB_, fp[r]);
 #pragma unroll
-      for (int m = 0; m < C::XC; ++m) ws_copy<16>(dst + (r * C::XC + m) * 32 + lane, xp[r] + 16 * m);
-      if (PASS == 1) {
-        if (C::BF) {
-          ws_copy<VPT * 4>(dst + C::OF + r * 32 + lane, fp[r]);
-        } else {
-#pragma unroll
-          for (int m = 0; m < C::FC; ++m) ws_copy<16>(dst + C::OF + (r * C::FC + m) * 32 + lane, fp[r] + 16 * m);
-        }
-      }
-#pragma unroll
-      for (int m = 0; m < C::RC / QL; ++m)
-        ws_copy<16>(dst + C::OR + grp * C::RGS + r * C::RC + q + QL * m, rp[r] + 16 * QL * m);
+      for (int m = 0; m < (C::RC + QL - 1) / QL; ++m)
+        if (C::RC % QL == 0 || q + QL * m < C::RC) ws_copy<16>(dst + C::OR + (grp * C::RGS + r * C::RC + q + QL * m) * 16, rp[r] + 16 * QL * m);
     }
     const int il = st - grp;
     const bool on = il >= 0 && il < ni - 1;      // the next step's column is another one
@@ -196,7 +188,7 @@ __global__ void __launch_bounds__(512) k_wsweep(Dev d, const int *work, int lr) 
   struct Item { T cr, cc, idg; P in, f; };
   Item nx[RG][VPT];
   unsigned non = 0;                              // solved cells, bit r
-  auto prepare = [&](int il, const Chunk *st) {
+  auto prepare = [&](int il, const unsigned char *st) {
     const bool act = il >= 0 && il < ni;
     non = 0;
 #pragma unroll
@@ -204,23 +196,20 @@ __global__ void __launch_bounds__(512) k_wsweep(Dev d, const int *work, int lr) 
       __align__(16) T rec[NSR];
 #pragma unroll
       for (int m = 0; m < C::RC; ++m)
-        reinterpret_cast<float4 *>(rec)[m] = reinterpret_cast<const float4 *>(st + C::OR + grp * C::RGS + r * C::RC)[m];
+        reinterpret_cast<float4 *>(rec)[m] =
+            reinterpret_cast<const float4 *>(st + C::OR)[grp * C::RGS + r * C::RC + m];
       __align__(16) P in[VPT], fv[VPT];
-#pragma unroll
-      for (int m = 0; m < C::XC; ++m)
-        reinterpret_cast<float4 *>(in)[m] = *reinterpret_cast<const float4 *>(st + (r * C::XC + m) * 32 + lane);
+      *reinterpret_cast<XV *>(in) = reinterpret_cast<const XV *>(st)[r * 32 + lane];
       if (PASS == 1) {
         if (C::BF) {
-          const __nv_bfloat162 *p = reinterpret_cast<const __nv_bfloat162 *>(st + C::OF + r * 32 + lane);
+          const __nv_bfloat162 *p = reinterpret_cast<const __nv_bfloat162 *>(st + C::OF) + (r * 32 + lane) * VPT;
 #pragma unroll
           for (int u = 0; u < VPT; ++u) {
             const float2 x = __bfloat1622float2(p[u]);
             fv[u] = pr_make((T)x.x, (T)x.y);
           }
         } else {
-#pragma unroll
-          for (int m = 0; m < C::FC; ++m)
-            reinterpret_cast<float4 *>(fv)[m] = *reinterpret_cast<const float4 *>(st + C::OF + (r * C::FC + m) * 32 + lane);
+          *reinterpret_cast<XV *>(fv) = reinterpret_cast<const XV *>(st + C::OF)[r * 32 + lane];
         }
       }
       const T dbase = rec[SR_DBASE];
@@ -276,10 +265,7 @@ __global__ void __launch_bounds__(512) k_wsweep(Dev d, const int *work, int lr) 
         }
       } else {
         P *o = reinterpret_cast<P *>(PASS == 0 ? d.dfs : d.f) + xo[r];
-        if (on && whole) {
-#pragma unroll
-          for (int m = 0; m < C::XC; ++m) reinterpret_cast<float4 *>(o)[m] = reinterpret_cast<const float4 *>(out)[m];
-        }
+        if (on && whole) *reinterpret_cast<XV *>(o) = *reinterpret_cast<const XV *>(out);
         if (VPT > 1 && on && some && !whole) o[0] = out[0];
       }
       xo[r] += il >= 0 ? cs : 0;
@@ -381,78 +367,110 @@ __global__ void __launch_bounds__(512) k_wsweep(Dev d, const int *work, int lr) 
 // ring depths: one step only where 16 bands of four rows leave no room for two
 template <int RG> constexpr int ws_depth(int n) { return n == 1 && RG < 4 ? 2 : n; }
 
-template <typename T, int PASS, int RG, int FB>
+template <typename T, int PASS, int FB, int QL, int RG, int VP>
 static void ws_launch(const Dev &d, cudaStream_t s, const int *work, int nwork, int nw, int ns) {
   size_t lim = 227 * 1024;
   // deepest ring that fits (6, 4, 2 or 1 steps; 1 = no prefetch), no deeper
   // than asked; then the longest link ring that fits
   int n = ns >= 6 ? 6 : (ns >= 4 ? 4 : (ns >= 2 ? 2 : 1));
-  while (n > ws_depth<RG>(1) && ws_smem<T, PASS, RG, FB>(nw, n) > lim) n = n == 2 ? 1 : n - 2;
+  while (n > ws_depth<RG>(1) && ws_smem<T, PASS, FB, QL, RG, VP>(nw, n) > lim) n = n == 2 ? 1 : n - 2;
   int lr = WS_LR;
-  while (lr > 2 && ws_smem<T, PASS, RG, FB>(nw, n, lr) > lim) lr >>= 1;
-  size_t sm = ws_smem<T, PASS, RG, FB>(nw, n, lr);
+  while (lr > 2 && ws_smem<T, PASS, FB, QL, RG, VP>(nw, n, lr) > lim) lr >>= 1;
+  size_t sm = ws_smem<T, PASS, FB, QL, RG, VP>(nw, n, lr);
   int th = 32 * nw;
-  if (n == 6) k_wsweep<T, PASS, 6, RG, FB><<<nwork, th, sm, s>>>(d, work, lr);
-  else if (n == 4) k_wsweep<T, PASS, 4, RG, FB><<<nwork, th, sm, s>>>(d, work, lr);
-  else if (n == 2) k_wsweep<T, PASS, 2, RG, FB><<<nwork, th, sm, s>>>(d, work, lr);
-  else k_wsweep<T, PASS, ws_depth<RG>(1), RG, FB><<<nwork, th, sm, s>>>(d, work, lr);
+  if (n == 6) k_wsweep<T, PASS, FB, 6, QL, RG, VP><<<nwork, th, sm, s>>>(d, work, lr);
+  else if (n == 4) k_wsweep<T, PASS, FB, 4, QL, RG, VP><<<nwork, th, sm, s>>>(d, work, lr);
+  else if (n == 2) k_wsweep<T, PASS, FB, 2, QL, RG, VP><<<nwork, th, sm, s>>>(d, work, lr);
+  else k_wsweep<T, PASS, FB, ws_depth<RG>(1), QL, RG, VP><<<nwork, th, sm, s>>>(d, work, lr);
 }
-
-template <typename T, int PASS, int RG, int FB> static void ws_attr() {
+template <typename T, int PASS, int FB, int QL, int RG, int VP> static void ws_attr_pass() {
   int lim = 227 * 1024;
-  cudaFuncSetAttribute(k_wsweep<T, PASS, ws_depth<RG>(1), RG, FB>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-  cudaFuncSetAttribute(k_wsweep<T, PASS, 2, RG, FB>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-  cudaFuncSetAttribute(k_wsweep<T, PASS, 4, RG, FB>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-  cudaFuncSetAttribute(k_wsweep<T, PASS, 6, RG, FB>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-}
-template <int RG> static void ws_attr_all() {
-  if (RG > 1) { ws_attr<float, 0, RG, 0>(); ws_attr<float, 1, RG, 0>(); ws_attr<float, 1, RG, 1>(); }
-  ws_attr<double, 0, RG, 0>(); ws_attr<double, 1, RG, 0>();
-}
-void wsweep_setup() {
-  ws_attr_all<1>();
-  ws_attr_all<2>();
-  ws_attr_all<4>();
+  cudaFuncSetAttribute(k_wsweep<T, PASS, FB, ws_depth<RG>(1), QL, RG, VP>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+  cudaFuncSetAttribute(k_wsweep<T, PASS, FB, 2, QL, RG, VP>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+  cudaFuncSetAttribute(k_wsweep<T, PASS, FB, 4, QL, RG, VP>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+  cudaFuncSetAttribute(k_wsweep<T, PASS, FB, 6, QL, RG, VP>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
 }
 
-int wsweep_vw(int fp32) { return QL * (fp32 ? WsVpt<float>::N : WsVpt<double>::N); }
-int wsweep_rows(int rg) { return NGRP * rg; }
-// Rows a group: as few as give at most 16 bands (warps of a CTA).  FP64: more
-// warps share its pipe (64x32 cells, 576 velocities: 1 row 134 / 140 us, 2
-// rows 191 / 195, 4 rows 311 / 334).  FP32: not below 2, where the lag of the
-// bands outgrows the shorter step (256x128 + 128x32 cells, 1024 velocities: 1 row
-// 246 / 392 us, 2 rows 223 / 329, 4 rows 238 / 352).
-int wsweep_rg(int max_nj, int fp32) { return max_nj <= 128 && !fp32 ? 1 : max_nj <= 256 ? 2 : 4; }
-
-// shared memory of the backward sweep (the larger one) with ring depth ns
-// and the longest link ring for ns > 1, the shortest for ns = 1
-template <int RG> static size_t ws_need(int fp32, int fbf, int nw, int ns) {
-  int lr = ns > 1 ? WS_LR : 2;
-  ns = ns == 1 ? ws_depth<RG>(1) : ns;
-  if (!fp32) return ws_smem<double, 1, RG, 0>(nw, ns, lr);
-  return fbf ? ws_smem<float, 1, RG, 1>(nw, ns, lr) : ws_smem<float, 1, RG, 0>(nw, ns, lr);
-}
-int wsweep_fits(int fp32, int fbf, int rg, int nw, int ns) {
-  size_t need = rg == 4 ? ws_need<4>(fp32, fbf, nw, ns) : rg == 2 ? ws_need<2>(fp32, fbf, nw, ns) : ws_need<1>(fp32, fbf, nw, ns);
-  return nw <= 16 && need <= 227 * 1024;
-}
-
-template <int RG>
-static void ws_dispatch(const Dev &d, cudaStream_t s, int pass, const int *work, int nwork, int nw, int ns, int fp32) {
-  if (!fp32) {
-    if (pass == 0) ws_launch<double, 0, RG, 0>(d, s, work, nwork, nw, ns);
-    else ws_launch<double, 1, RG, 0>(d, s, work, nwork, nw, ns);
-    return;
+// what the host does with a shape: set up, shared memory of the backward sweep
+// (the larger one) with ring depth ns and the longest link ring for ns > 1, the
+// shortest for ns = 1, and launch
+template <typename T, int QL, int RG, int VP> struct WsOps {
+  static void attr() {
+    ws_attr_pass<T, 0, 0, QL, RG, VP>();
+    ws_attr_pass<T, 1, 0, QL, RG, VP>();
+    if (sizeof(T) == 4) ws_attr_pass<T, 1, sizeof(T) == 4, QL, RG, VP>();
   }
-  constexpr int RF = RG > 1 ? RG : 2;
-  if (pass == 0) ws_launch<float, 0, RF, 0>(d, s, work, nwork, nw, ns);
-  else if (d.fbf) ws_launch<float, 1, RF, 1>(d, s, work, nwork, nw, ns);
-  else ws_launch<float, 1, RF, 0>(d, s, work, nwork, nw, ns);
+  static size_t need(int fbf, int nw, int ns) {
+    const int lr = ns > 1 ? WS_LR : 2, n = ns == 1 ? ws_depth<RG>(1) : ns;
+    return fbf ? ws_smem<T, 1, sizeof(T) == 4, QL, RG, VP>(nw, n, lr) : ws_smem<T, 1, 0, QL, RG, VP>(nw, n, lr);
+  }
+  static void launch(const Dev &d, cudaStream_t s, int pass, const int *work, int nwork, int nw, int ns) {
+    if (pass == 0) ws_launch<T, 0, 0, QL, RG, VP>(d, s, work, nwork, nw, ns);
+    else if (sizeof(T) == 4 && d.fbf) ws_launch<T, 1, sizeof(T) == 4, QL, RG, VP>(d, s, work, nwork, nw, ns);
+    else ws_launch<T, 1, 0, QL, RG, VP>(d, s, work, nwork, nw, ns);
+  }
+};
+struct WsEntry {
+  int ql, rg, vp;
+  void (*attr)();
+  size_t (*need)(int, int, int);
+  void (*launch)(const Dev &, cudaStream_t, int, const int *, int, int, int);
+};
+template <typename T, int QL, int RG, int VP> constexpr WsEntry ws_entry() {
+  typedef WsOps<T, QL, RG, VP> O;
+  return {QL, RG, VP, O::attr, O::need, O::launch};
 }
-void launch_wsweep(const Dev &d, cudaStream_t s, int pass, const int *work, int nwork, int nw, int ns, int rg, int fp32) {
-  if (rg == 4) ws_dispatch<4>(d, s, pass, work, nwork, nw, ns, fp32);
-  else if (rg == 2) ws_dispatch<2>(d, s, pass, work, nwork, nw, ns, fp32);
-  else ws_dispatch<1>(d, s, pass, work, nwork, nw, ns, fp32);
+// Shapes: lanes a group, rows a group, velocities a lane; rows a band and the
+// bytes of a cell that a warp touches.  FP32 forward / backward, us (bytes of one
+// (cell, velocity) array; rows of the tallest block):
+//                              4,2,1    4,2,2    8,2,1    8,2,2    8,4,2
+//                              16 32 B  16 64 B  8 64 B   8 128 B  16 128 B
+//   1 MB, 16 rows              18/17    22/20    20/21    27/23    31/35
+//   14 MB, 32                  32/31    40/37    37/40    47/44    55/68
+//   22 MB, 51 (21 x 21 vel.)   68/79    75/64    59/64    84/76    104/121
+//   42 MB, 64                  70/72    84/76    76/82    98/93    113/137
+//   75 MB, 64                  89/130   90/81    84/93    100/94   116/138
+//   96 MB, 96                  124/131  136/123  125/138  164/156  187/239
+//   170 MB, 96                 195/312  146/188  156/157  165/156  187/238
+//   302 MB, 128                299/620  231/338  190/338  248/236  263/406
+//   524 MB, 128                446/884  296/537  373/506  250/307  264/412
+//   445 MB, 150                391/911  326/469  -        -        364/454
+//   1188 MB, 200               1318/2231 903/1485 -       -        547/1020
+//   4899 MB, 256               6700/10660 3488/5437 -     -        1713/2862
+// While the arrays stay in the L2 a sweep is bound by the latency of its steps:
+// few velocities a lane make them short.  Beyond it lines touched in parts are
+// the bound, more so for the backward sweep (two arrays in, one out): a warp
+// then takes whole lines, in bands of 8 rows where 16 bands reach (a step of
+// two rows is the shorter one), else of 16.
+enum { WS32_4_2_1, WS32_4_2_2, WS32_8_2_1, WS32_8_2_2, WS32_8_4_2, WS32_4_4_2, WS64_4_1, WS64_4_2, WS64_4_4 };
+static const WsEntry kWs[] = {
+    ws_entry<float, 4, 2, 1>(), ws_entry<float, 4, 2, 2>(), ws_entry<float, 8, 2, 1>(), ws_entry<float, 8, 2, 2>(),
+    ws_entry<float, 8, 4, 2>(), ws_entry<float, 4, 4, 2>(), ws_entry<double, 4, 1, 1>(), ws_entry<double, 4, 2, 1>(),
+    ws_entry<double, 4, 4, 1>()};
+
+void wsweep_setup() {
+  for (const WsEntry &e : kWs) e.attr();
+}
+int wsweep_vw(int shape) { return kWs[shape].ql * kWs[shape].vp; }
+int wsweep_rows(int shape) { return 32 / kWs[shape].ql * kWs[shape].rg; }
+// By the table above.  FP64: as few rows as give at most 16 bands, more warps
+// share its pipe (64x32 cells, 576 velocities: 1 row 134 / 140 us, 2 rows 191 /
+// 195, 4 rows 311 / 334).  `forced` (>= 0): that FP32 shape where the block's
+// bands fit.
+int wsweep_shape(int fp32, int pass, int max_nj, double bytes, int forced) {
+  if (!fp32) return max_nj <= 128 ? WS64_4_1 : max_nj <= 256 ? WS64_4_2 : WS64_4_4;
+  if (forced >= WS32_4_2_1 && forced <= WS32_4_4_2 && max_nj <= 16 * wsweep_rows(forced)) return forced;
+  if (max_nj > 256) return WS32_4_4_2;
+  if (bytes <= (pass ? 16e6 : 60e6)) return WS32_4_2_1;
+  if (max_nj > 128) return bytes > (pass ? 400e6 : 600e6) ? WS32_8_4_2 : WS32_4_2_2;
+  if (pass == 0) return bytes <= 400e6 ? WS32_8_2_1 : WS32_8_2_2;
+  return bytes <= 120e6 ? WS32_4_2_2 : WS32_8_2_2;
+}
+int wsweep_fits(int shape, int fbf, int nw, int ns) {
+  return nw <= 16 && kWs[shape].need(fbf, nw, ns) <= 227 * 1024;
+}
+void launch_wsweep(const Dev &d, cudaStream_t s, int pass, const int *work, int nwork, int nw, int ns, int shape) {
+  kWs[shape].launch(d, s, pass, work, nwork, nw, ns);
 }
 
 }  // namespace ugks
