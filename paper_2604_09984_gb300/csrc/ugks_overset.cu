@@ -613,58 +613,81 @@ __global__ void __launch_bounds__(LCHUNK) k_list_write(Dev d, const int *fresh_f
 // strides over it.
 // parts: bit 0 the distributions, bit 1 W and q (the two may run apart: the
 // distributions right after the micro sweep, W and q after Step 7)
-template <typename T> __global__ void k_interp_gather(Dev d, const int *list, const int *cnt, int parts) {
-  int n = min(*cnt, d.cap_interp);
-  size_t nk = (parts & 1) ? (size_t)d.nvp : 1;
-  size_t tot = (size_t)n * nk;
-  for (size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x; t < tot; t += (size_t)gridDim.x * blockDim.x) {
-    int r = (int)(t / nk), k = (int)(t % nk);
-    int c = list[r];
+//
+// A CTA takes one receptor and up to INTERP_CHUNK velocities at a time, so that
+// list, donors and weights are read (and the weights converted, which passes
+// the FP64 pipe) once a warp and not once a velocity; the first warp's lanes
+// take the components of W and q.  Both parts, gather and scatter: 256x128 +
+// 128x32 cells, 1024 velocities 33 us -> 21; 512x256 + 2 x 192x48, 4096: 305 ->
+// 121.
+constexpr int INTERP_THREADS = 256, INTERP_CHUNK = 2 * INTERP_THREADS;
+template <typename T> __global__ void __launch_bounds__(INTERP_THREADS) k_interp_gather(Dev d, const int *list,
+                                                                                       const int *cnt, int parts) {
+  const int n = min(*cnt, d.cap_interp), lane = threadIdx.x & 31;
+  const int nch = (parts & 1) ? (d.nvp + INTERP_CHUNK - 1) / INTERP_CHUNK : 1;
+  for (int u = blockIdx.x; u < n * nch; u += gridDim.x) {
+    const int r = u / nch, ch = u - r * nch, c = list[r];
+    const int e0 = lane < 5 ? d.donors[5 * c + lane] : -1;
+    const double w0 = lane < 5 ? d.dwgt[5 * c + lane] : 0.0;
+    const T t0 = (T)w0;
+    int e[5];
+#pragma unroll
+    for (int m = 0; m < 5; ++m) e[m] = __shfl_sync(0xffffffffu, e0, m);
     if (parts & 1) {
       // f in the arithmetic type (its storage type): FP32 weights and sums on
       // the mixed path keep the FP64 pipe out of the per-velocity loop
-      T ah = T(0), ab = T(0);
-      for (int m = 0; m < 5; ++m) {
-        int e = d.donors[5 * c + m];
-        if (e < 0) continue;
-        T w = (T)d.dwgt[5 * c + m];
-        auto v = ldF<T>(d, (size_t)e * d.nvp + k);
-        ah = ah + w * v.x;
-        ab = ab + w * v.y;
+      T w[5];
+#pragma unroll
+      for (int m = 0; m < 5; ++m) w[m] = __shfl_sync(0xffffffffu, t0, m);
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        const int k = ch * INTERP_CHUNK + j * INTERP_THREADS + threadIdx.x;
+        if (k >= d.nvp) continue;
+        T ah = T(0), ab = T(0);
+#pragma unroll
+        for (int m = 0; m < 5; ++m) {
+          if (e[m] < 0) continue;
+          auto v = ldF<T>(d, (size_t)e[m] * d.nvp + k);
+          ah = ah + w[m] * v.x;
+          ab = ab + w[m] * v.y;
+        }
+        stf<T>(d.itmp, (size_t)r * d.nvp + k, ah, ab);
       }
-      stf<T>(d.itmp, (size_t)r * d.nvp + k, ah, ab);
     }
-    if ((parts & 2) && k == 0) {
-      double acc[6] = {0, 0, 0, 0, 0, 0};
+    if ((parts & 2) && ch == 0 && threadIdx.x < 32) {
+      double acc = 0.0;
+#pragma unroll
       for (int m = 0; m < 5; ++m) {
-        int e = d.donors[5 * c + m];
-        if (e < 0) continue;
-        double w = d.dwgt[5 * c + m];
-        for (int q = 0; q < 4; ++q) acc[q] = acc[q] + w * d.W[4 * e + q];
-        acc[4] = acc[4] + w * d.q[2 * e];
-        acc[5] = acc[5] + w * d.q[2 * e + 1];
+        const double w = __shfl_sync(0xffffffffu, w0, m);
+        if (e[m] < 0 || lane >= 6) continue;
+        acc = acc + w * (lane < 4 ? d.W[4 * e[m] + lane] : d.q[2 * e[m] + lane - 4]);
       }
-      for (int q = 0; q < 6; ++q) d.itmpW[6 * r + q] = acc[q];
+      if (lane < 6) d.itmpW[6 * r + lane] = acc;
     }
   }
 }
 
-template <typename T> __global__ void k_interp_scatter(Dev d, const int *list, const int *cnt, int parts) {
-  int n = min(*cnt, d.cap_interp);
-  size_t nk = (parts & 1) ? (size_t)d.nvp : 1;
-  size_t tot = (size_t)n * nk;
-  for (size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x; t < tot; t += (size_t)gridDim.x * blockDim.x) {
-    int r = (int)(t / nk), k = (int)(t % nk);
-    int c = list[r];
+template <typename T> __global__ void __launch_bounds__(INTERP_THREADS) k_interp_scatter(Dev d, const int *list,
+                                                                                        const int *cnt, int parts) {
+  const int n = min(*cnt, d.cap_interp);
+  const int nch = (parts & 1) ? (d.nvp + INTERP_CHUNK - 1) / INTERP_CHUNK : 1;
+  for (int u = blockIdx.x; u < n * nch; u += gridDim.x) {
+    const int r = u / nch, ch = u - r * nch, c = list[r];
     if (d.donors[5 * c] < 0) continue;          // orphan: keep its values
     if (parts & 1) {
-      auto v = ldf<T>(d.itmp, (size_t)r * d.nvp + k);
-      stF<T>(d, (size_t)c * d.nvp + k, v.x, v.y);
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        const int k = ch * INTERP_CHUNK + j * INTERP_THREADS + threadIdx.x;
+        if (k >= d.nvp) continue;
+        auto v = ldf<T>(d.itmp, (size_t)r * d.nvp + k);
+        stF<T>(d, (size_t)c * d.nvp + k, v.x, v.y);
+      }
     }
-    if ((parts & 2) && k == 0) {
-      for (int q = 0; q < 4; ++q) d.W[4 * c + q] = d.itmpW[6 * r + q];
-      d.q[2 * c] = d.itmpW[6 * r + 4];
-      d.q[2 * c + 1] = d.itmpW[6 * r + 5];
+    if ((parts & 2) && ch == 0 && threadIdx.x < 6) {
+      const int m = threadIdx.x;
+      const double v = d.itmpW[6 * r + m];
+      if (m < 4) d.W[4 * c + m] = v;
+      else d.q[2 * c + m - 4] = v;
     }
   }
 }
@@ -696,14 +719,16 @@ void launch_lists(const Dev &d, cudaStream_t s, const int *fresh_flag, const int
 }
 
 void launch_interp(const Dev &d, cudaStream_t s, const int *list, const int *cnt, int nsm, int fp32, int parts) {
-  size_t tot = (size_t)d.cap_interp * ((parts & 1) ? d.nvp : 1);
-  int grid = std::max(1, std::min(nblk(tot, 256), 8 * std::max(nsm, 1)));
+  // W and q alone take one warp a receptor
+  const int th = (parts & 1) ? INTERP_THREADS : 32;
+  const size_t units = (size_t)d.cap_interp * ((parts & 1) ? nblk(d.nvp, INTERP_CHUNK) : 1);
+  const int grid = (int)std::max<size_t>(1, std::min<size_t>(units, (size_t)(2048 / th) * std::max(nsm, 1)));
   if (fp32) {
-    k_interp_gather<float><<<grid, 256, 0, s>>>(d, list, cnt, parts);
-    k_interp_scatter<float><<<grid, 256, 0, s>>>(d, list, cnt, parts);
+    k_interp_gather<float><<<grid, th, 0, s>>>(d, list, cnt, parts);
+    k_interp_scatter<float><<<grid, th, 0, s>>>(d, list, cnt, parts);
   } else {
-    k_interp_gather<double><<<grid, 256, 0, s>>>(d, list, cnt, parts);
-    k_interp_scatter<double><<<grid, 256, 0, s>>>(d, list, cnt, parts);
+    k_interp_gather<double><<<grid, th, 0, s>>>(d, list, cnt, parts);
+    k_interp_scatter<double><<<grid, th, 0, s>>>(d, list, cnt, parts);
   }
 }
 
