@@ -714,7 +714,12 @@ template <typename T> static constexpr size_t flux_smem() {
 // that gathered the gradients and fluxes of its four faces from the cells:
 // 5.1 ms for 192 x 96 + 96 x 24 cells and 1024 velocities, 6.03 ms the call;
 // from the face values that the reduction leaves, 0.83 ms the call.)
-template <typename T, bool SEP, bool EVAL>
+// PAIR (FP32 joint form, arrays beyond the L2): two ranges of columns in turn, row
+// by row, so that a cell's sums of both are stored close together (300x150 + 2 x
+// 120x30 cells, 33x33 velocities: 728 -> 649 us; within the L2 and in the separable
+// form the longer registers cost more: 128x64 + 64x16, 24x24: 56 -> 61,
+// 256x128 + 128x32, 32x32: 313 -> 431).
+template <typename T, bool SEP, bool PAIR, bool EVAL>
 __global__ void __launch_bounds__(NT, FluxCfg<T>::CTAS) k_flux(Dev d, double *eval) {
   typedef typename PairOf<T>::type P;
   constexpr int VK = FluxCfg<T>::VK, FS = FluxCfg<T>::FS, VH = VK / 2, VKG = VK + 2;
@@ -769,9 +774,18 @@ __global__ void __launch_bounds__(NT, FluxCfg<T>::CTAS) k_flux(Dev d, double *ev
   const int rows = d.nv / d.nvx;
   const int r0 = (int)((long)rows * blockIdx.y / gridDim.y), r1 = (int)((long)rows * (blockIdx.y + 1) / gridDim.y);
   const int nch = ck.per_row * (r1 - r0);
-  struct Pos { int x0, iy; };
+  struct Pos { int x0, iy, odd; };
   auto advance = [&](Pos &p) {
-    if (++p.iy == r1) { p.iy = r0; p.x0 += ck.len; }
+    if (PAIR && !p.odd && p.x0 + ck.len < d.nvx) {
+      p.odd = 1;
+      p.x0 += ck.len;
+      return;
+    }
+    if (PAIR && p.odd) {
+      p.odd = 0;
+      p.x0 -= ck.len;
+    }
+    if (++p.iy == r1) { p.iy = r0; p.x0 += (PAIR ? 2 : 1) * ck.len; }
   };
   int otile = tile, oslot = slot;
   if (act) fval_owner(bi, i0, j0, tile, slot, otile, oslot);
@@ -794,7 +808,7 @@ __global__ void __launch_bounds__(NT, FluxCfg<T>::CTAS) k_flux(Dev d, double *ev
     }
     cp_async_commit();
   };
-  Pos cur = {0, r0}, nxt = cur;
+  Pos cur = {0, r0, 0}, nxt = cur;
   if (r0 == r1) nxt.x0 = d.nvx;
 #pragma unroll
   for (int s = 0; s < FS - 1; ++s) { stage(nxt, s); advance(nxt); }
@@ -805,10 +819,27 @@ __global__ void __launch_bounds__(NT, FluxCfg<T>::CTAS) k_flux(Dev d, double *ev
   for (int m = 0; m < 10; ++m) cub[m] = pr_make(P_[FP_IH + m], P_[FP_IB + m]);
   P vx2[VH];
   T ex[VH];                                            // SEP: the columns' factors of the Maxwellian
+  T vxr[PAIR ? 2 : 1][VH];                             // PAIR: the columns of both ranges
   int xcur = -1, st = 0, sn = FS - 1;                  // ring stages: this chunk's, the next copy's
   for (int ch = 0; ch < nch; ++ch) {
     const int n = min(ck.len, d.nvx - cur.x0);
-    if (cur.x0 != xcur) {                              // another range of columns
+    if (PAIR) {
+      if (!cur.odd && cur.x0 != xcur) {                // another pair of ranges
+        xcur = cur.x0;
+#pragma unroll
+        for (int h = 0; h < (PAIR ? 2 : 1); ++h)
+#pragma unroll
+          for (int q = 0; q < VH; ++q) {
+            const int x = xcur + h * ck.len + half + 2 * q;
+            vxr[h][q] = x < d.nvx ? grid_vx<T>(d, x) : T(0);
+          }
+      }
+#pragma unroll
+      for (int q = 0; q < VH; ++q) {
+        vx2[q] = pr_dup(cur.odd ? vxr[PAIR ? 1 : 0][q] : vxr[0][q]);
+        ex[q] = T(0);
+      }
+    } else if (cur.x0 != xcur) {                       // another range of columns
       xcur = cur.x0;
 #pragma unroll
       for (int q = 0; q < VH; ++q) {
@@ -1021,8 +1052,9 @@ void face_tile_shape(int fp32, int *vk, int *nh) {
 }
 
 template <typename T, bool SEP> static void flux_attr() {
-  cudaFuncSetAttribute(k_flux<T, SEP, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)flux_smem<T>());
-  cudaFuncSetAttribute(k_flux<T, SEP, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)flux_smem<T>());
+  cudaFuncSetAttribute(k_flux<T, SEP, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)flux_smem<T>());
+  cudaFuncSetAttribute(k_flux<T, SEP, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)flux_smem<T>());
+  if (!SEP) cudaFuncSetAttribute(k_flux<T, SEP, !SEP, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)flux_smem<T>());
 }
 void tile_setup() {
   cudaFuncSetAttribute(k_face_reduce32<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Smem32));
@@ -1046,9 +1078,11 @@ void launch_face_reduce(const Dev &d, cudaStream_t s, int fp32) {
 }
 template <bool EVAL> static void flux(const Dev &d, cudaStream_t s, int fp32, double *eval) {
   const dim3 grid(d.ntiles, d.nsplit);
-  if (!fp32) k_flux<double, true, EVAL><<<grid, NT, flux_smem<double>(), s>>>(d, eval);
-  else if (d.nvx % 16 == 0) k_flux<float, true, EVAL><<<grid, NT, flux_smem<float>(), s>>>(d, eval);
-  else k_flux<float, false, EVAL><<<grid, NT, flux_smem<float>(), s>>>(d, eval);
+  const bool pair = !EVAL && (double)d.nc * d.nvp * 8.0 > 120e6;         // beyond the L2
+  if (!fp32) k_flux<double, true, false, EVAL><<<grid, NT, flux_smem<double>(), s>>>(d, eval);
+  else if (d.nvx % 16 == 0) k_flux<float, true, false, EVAL><<<grid, NT, flux_smem<float>(), s>>>(d, eval);
+  else if (pair) k_flux<float, false, true, false><<<grid, NT, flux_smem<float>(), s>>>(d, nullptr);
+  else k_flux<float, false, false, EVAL><<<grid, NT, flux_smem<float>(), s>>>(d, eval);
 }
 void launch_flux(const Dev &d, cudaStream_t s, int fp32) { flux<false>(d, s, fp32, nullptr); }
 void launch_flux_eval(const Dev &d, cudaStream_t s, double *D, int fp32) { flux<true>(d, s, fp32, D); }
