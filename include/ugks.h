@@ -245,7 +245,7 @@ int ugks_graph_stats(const ugks_ctx *ctx, int64_t *captures, int64_t *replays);
  * there, so instances created on distinct streams run concurrently on the
  * GPU while the host returns at once.  Each instance computes what a
  * separate ugks_move_mesh / ugks_overset_connect / ugks_step sequence
- * computes (the face sums' atomic additions may land in another order).
+ * computes.
  * Orphans, staging overflow and non-physical states are reported by the
  * next synchronising call on the instance (ugks_moments).  `failed` (HOST,
  * may be NULL) receives the index of the instance whose call failed, or -1.
@@ -262,24 +262,17 @@ int ugks_advance_batch(ugks_ctx *const *ctx, int n, const double *t_new,
  * Synchronises the stream.  Errors: UGKS_ERR_ORDER, UGKS_ERR_ARG. */
 int ugks_wall_torque(ugks_ctx *ctx, const double *center, double *torque);
 
-/* Tile autotuner, on the context's own state (`reps` timed passes after one
- * warm-up of each candidate, CUDA events on the stream), keeping the fastest:
- *  - the face kernels (velocity reduction and flux divergence, FP32 paths):
- *    their tile of 8x8 cells walks the velocities in chunks of `face_vk` in
- *    {8, 16, 32} with `face_nh` = 2 threads per face slot (each takes
- *    face_vk / face_nh velocities of a chunk); the FP64 path keeps (8, 2);
- *  - the micro LU-SGS sweeps, skewed wavefronts (a warp takes a band of 8
- *    rows, 4 lanes a row; 16 rows, 2 lanes a row when a block is taller than
- *    256 cells): velocities per lane `vpt` in {2, 4} (FP32 paths; 2 in FP64)
- *    and, per sweep, the prefetch ring depth in {2, 4, 6} steps (shallower
- *    where shared memory is short).
- * The candidates differ only in the grouping of the FP32 face sums over the
- * velocities (partial sums per thread and chunk, folded error-free), i.e. in
- * rounding; the sweeps take each velocity in the same lexicographic order.  f is saved before the trials and restored after them.  Needs
- * a preceding ugks_step (the kernels read records the step writes).  `items`
- * (the (cell, velocity) items of one sweep warp step, 32 x vpt), `vpt`,
- * `ring_fwd`, `ring_bwd`, `face_vk`, `face_nh` (HOST, each may be NULL)
- * receive the choice.  Synchronises the stream.  Errors: UGKS_ERR_ORDER,
+/* Tuner, on the context's own state (`reps` timed passes after one warm-up of
+ * each candidate, CUDA events on the stream), keeping the fastest: per micro
+ * LU-SGS sweep the depth of its prefetch ring in {2, 4, 6} steps (shallower
+ * where shared memory is short), which changes no result.  What else the sweeps
+ * and the face kernels choose (rows and velocities of a warp, CTAs that share a
+ * tile) follows from the sizes by fixed rules.  f is saved before the trials and
+ * restored after them.  Needs a preceding ugks_step (the kernels read records
+ * the step writes).  `ring_fwd`, `ring_bwd` (HOST, each may be NULL) receive the
+ * choice; `items` and `vpt` receive 64 and 2, `face_vk` and `face_nh` the chunk of
+ * velocities and the threads per face slot of the velocity reduction (16 and 2,
+ * FP64 8 and 2).  Synchronises the stream.  Errors: UGKS_ERR_ORDER,
  * UGKS_ERR_CUDA. */
 int ugks_autotune(ugks_ctx *ctx, int reps, int *items, int *vpt, int *ring_fwd, int *ring_bwd, int *face_vk,
                   int *face_nh);
@@ -380,13 +373,11 @@ int ugks_shard_buffers(const ugks_ctx *ctx, size_t *face_off, size_t *face_count
 int64_t ugks_launch_count(const ugks_ctx *ctx);
 
 /* Bounded waits.  The only device-side waits of a step are those of the
- * wavefront sweeps: the macro LU-SGS CTA waits (mbarrier) for the bulk copy of
- * the next diagonal's records, the bands of a micro-sweep CTA wait for the
- * band before them (shared-memory progress counters, Sec. 2.2 sweep order).
- * Each wait polls at most `polls` times (0 restores the default, 2^21); a wait
- * that runs out sets a flag, the CTA stops its sweep at the end of the
- * current step, waits (default bound) for every copy it issued, and exits;
- * the step's results are then invalid and the next synchronising call
+ * micro sweeps: a band of a CTA waits for the band before it, and for room in
+ * the ring to the band after it (shared-memory progress counters, Sec. 2.2 sweep
+ * order).  Each wait polls at most `polls` times (0 restores the default, 2^21);
+ * a wait that runs out sets a flag, the band stops its sweep at the end of the
+ * current step, waits for every copy it issued, and exits; the step's results are then invalid and the next synchronising call
  * returns UGKS_ERR_TIMEOUT (and clears the flag, leaving the context usable:
  * set a valid state with ugks_set_state before stepping again).  Takes effect
  * for work issued after the call.  Errors: UGKS_ERR_ARG (polls < 0). */

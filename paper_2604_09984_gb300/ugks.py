@@ -288,10 +288,9 @@ class Solver:
         self.step(dt, n_inner)
 
     def autotune(self, reps=3):
-        """Pick the fastest tiles on this context's own state (ugks_autotune);
-        returns (sweep items per warp step, sweep velocities per lane, forward
-        ring depth, backward ring depth, face-kernel velocities per chunk,
-        face-kernel threads per face slot)."""
+        """Pick the fastest ring depths of the micro sweeps on this context's own
+        state (ugks_autotune); returns (64, 2, forward ring depth, backward ring
+        depth, velocity chunk of the reduction, its threads per face slot)."""
         v = [c_int() for _ in range(6)]
         self._check(self.lib.ugks_autotune(self.ctx, int(reps), *[ctypes.byref(x) for x in v]))
         self.tiles = tuple(x.value for x in v)
