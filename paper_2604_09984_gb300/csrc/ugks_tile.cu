@@ -93,6 +93,16 @@ template <> struct Vec4<double> { typedef double4 type; };
 // a b + c d with one product rounded by itself (written out where results must
 // not depend on the compiler's choice)
 __device__ __forceinline__ float mul_add2(float a, float b, float c, float d) { return __fmaf_rn(a, b, __fmul_rn(c, d)); }
+// S w.n of a face at one velocity.  At a wall its sign splits the velocities into
+// incident and reflected ones, and the reduction and the flux pass have to split
+// alike (along a wall that slides in its own plane w.n is zero up to its rounding):
+// both take these forms, every rounding written out.  FP64: from the row's part,
+// vy S n_y - S U.n.
+__device__ __forceinline__ float face_ws(float vx, float vy, float snx, float sny, float sun) {
+  return __fsub_rn(mul_add2(vx, snx, vy, sny), sun);
+}
+__device__ __forceinline__ double face_ws_row(double vy, double sny, double sun) { return __fma_rn(vy, sny, -sun); }
+__device__ __forceinline__ double face_ws(double vx, double snx, double row) { return __fma_rn(vx, snx, row); }
 // Half of the van Leer slopes 2 a b / (a + b) (0 where a b <= 0) of a pair of
 // differences, FP32 (the factor 2 goes into the inverse Jacobian: exact).
 __device__ __forceinline__ float2 pr_vanleer_half(PairF a, PairF b) {
@@ -433,7 +443,7 @@ template <int FB> __global__ void __launch_bounds__(NT32, 2) k_face_reduce32(Dev
         const int kk = half + 2 * q;
         const float4 t = S.tab[buf][kk];
         const float vx = t.x, vy = t.y;
-        const float wS = __fsub_rn(mul_add2(vx, snx, vy, sny), sun);
+        const float wS = face_ws(vx, vy, snx, sny, sun);
         const bool r = !f.wall && wS < 0.f;
         const float wx = vx - ufx, wy = vy - ufy;
         V2<float> ff, wg;
@@ -603,7 +613,7 @@ __global__ void __launch_bounds__(NT, 1) k_face_reduce64(Dev d) {
     __syncthreads();
     if (f.act) {
       const Smem64::Tab *tab = S.tab[buf];
-      const T vy = d.vy1[d.iy0 + cur.iy], cy = vy * sny - sun, wy = vy - ufy;
+      const T vy = d.vy1[d.iy0 + cur.iy], cy = face_ws_row(vy, sny, sun), wy = vy - ufy;
       Quad<P> *fv = reinterpret_cast<Quad<P> *>(d.fval) + (size_t)tile * fval_tile(d.nvp);
       const int k0 = cur.iy * d.nvx + cur.x0;
       const P wyp = pr_dup(wy);
@@ -620,7 +630,7 @@ __global__ void __launch_bounds__(NT, 1) k_face_reduce64(Dev d) {
         }
       };
       // w.S at the chunk's ends, rounded as for each velocity: monotone in v_x
-      const T wa = tab[0].vx * snx + cy, wb = tab[n - 1].vx * snx + cy;
+      const T wa = face_ws(tab[0].vx, snx, cy), wb = face_ws(tab[n - 1].vx, snx, cy);
       const bool allL = wa > 0.0 && wb > 0.0, allR = wa < 0.0 && wb < 0.0;
       if (allL || (allR && !f.wall)) {
         const P *F = S.F[buf][allL ? f.Lr : f.Rr];
@@ -634,21 +644,21 @@ __global__ void __launch_bounds__(NT, 1) k_face_reduce64(Dev d) {
         }
       } else {
         // the upwind side changes inside the chunk (w.S = 0 exactly: the mean
-        // of both sides); a wall takes its interior side's incident part only
+        // of both sides); a wall takes its interior side, summed over the
+        // incident part
         for (int kk = half; kk < n; kk += 2) {
-          const T wS = tab[kk].vx * snx + cy;
+          const T wS = face_ws(tab[kk].vx, snx, cy);
           const bool r = !f.wall && wS < 0.0;
-          if (f.wall && !(wS > 0.0)) continue;
           P ff, wg;
           reconstruct(S.F[buf][r ? f.Rr : f.Lr], S.G[r ? Rg : Lg], pr_dup(r ? dxr : dxl), pr_dup(r ? dyr : dyl), kk, ff, wg);
-          if (wS == 0.0) {
+          if (wS == 0.0 && !f.wall) {
             P f2, g2;
             reconstruct(S.F[buf][f.Rr], S.G[Rg], pr_dup(dxr), pr_dup(dyr), kk, f2, g2);
             ff = pr_mul(pr_dup(0.5), pr_add(ff, f2));
             wg = pr_mul(pr_dup(0.5), pr_add(wg, g2));
           }
           fv[fval_at(k0 + kk, slot)] = Quad<P>{ff, wg};
-          accumulate(tab[kk], ff, wg);
+          if (!f.wall || wS > 0.0) accumulate(tab[kk], ff, wg);
         }
       }
       // fold after two chunks, at the end of the row and at the last chunk
@@ -861,7 +871,9 @@ __global__ void __launch_bounds__(NT, FluxCfg<T>::CTAS) k_flux(Dev d, double *ev
       const P a1 = pr_fma(cy2, pr_fma(cy2, cub[8], cub[4]), cub[1]);
       const P a2 = pr_fma(cy2, cub[7], cub[3]), a3 = cub[6];
       const T ey = SEP ? P_[FP_HPRE] * r_exp<T>(-P_[FP_LAM] * (cy * cy)) : T(0);
-      const P wsy2 = pr_dup(vy * P_[FP_SNY] - P_[FP_SUN]);
+      P wsy2;
+      if constexpr (sizeof(T) == 8) wsy2 = pr_dup(face_ws_row(vy, P_[FP_SNY], P_[FP_SUN]));
+      else wsy2 = pr_dup(vy * P_[FP_SNY] - P_[FP_SUN]);
 #pragma unroll
       for (int q = 0; q < VH; ++q) {
         if (half + 2 * q < n) {
@@ -872,11 +884,12 @@ __global__ void __launch_bounds__(NT, FluxCfg<T>::CTAS) k_flux(Dev d, double *ev
           const P ph = pr_fma(cx, pr_fma(cx, pr_fma(cx, a3, a2), a1), a0);
           P I = pr_fma(q12, fv.x, pr_mul(q22, fv.y)), wS;
           T H;
+          // (pr_fma and the sum of the joint form round as face_ws)
+          if (SEP && (!wall || sizeof(T) == 8)) wS = pr_fma(vx2[q], snx2, wsy2);
+          else wS = pr_add(pr_fma(vx2[q], snx2, pr_dup(vy * P_[FP_SNY])), pr_dup(-P_[FP_SUN]));
           if (SEP && !wall) {
-            wS = pr_fma(vx2[q], snx2, wsy2);
             H = ey * ex[q];
           } else {
-            wS = pr_add(pr_fma(vx2[q], snx2, pr_dup(vy * P_[FP_SNY])), pr_dup(-P_[FP_SUN]));
             H = P_[FP_HPRE] * r_exp<T>(-P_[FP_LAM] * (pr_get(cx).x * pr_get(cx).x + cy * cy));
           }
           I = pr_fma(pr_dup(H), ph, I);
