@@ -745,6 +745,7 @@ __global__ void __launch_bounds__(NT, FluxCfg<T>::CTAS) k_flux(Dev d, double *ev
   bool field = false;
   P sg[4];
   const P *fa = Fs, *fc = Fs;
+  const bool wide = !EVAL || (reinterpret_cast<uintptr_t>(eval) & 15) == 0;    // the caller's array: 8-byte aligned at least
   {
     const int c = tid >> 2, tx = c % TX, ty = c / TX, i = i0 + tx, j = j0 + ty;
     if (tid < 4 * TX * TY && i < ni && j < nj) {
@@ -921,8 +922,14 @@ __global__ void __launch_bounds__(NT, FluxCfg<T>::CTAS) k_flux(Dev d, double *ev
           D = pr_fma(sg[3], fc[o + TX * VKG + kk], D);
           if (EVAL) {
             const auto v = pr_get(D);
-            reinterpret_cast<double2 *>(eval)[(size_t)g * d.nv + k0 + kk] =
-                field ? make_double2((double)v.x, (double)v.y) : make_double2(0.0, 0.0);
+            double *o2 = eval + 2 * ((size_t)g * d.nv + k0 + kk);
+            const double2 w = field ? make_double2((double)v.x, (double)v.y) : make_double2(0.0, 0.0);
+            if (wide) {
+              *reinterpret_cast<double2 *>(o2) = w;
+            } else {
+              o2[0] = w.x;
+              o2[1] = w.y;
+            }
           } else {
             out[kk] = D;
           }
