@@ -454,9 +454,8 @@ int ugks_probe_fp64(double *out, int kind, int nblocks, int nthreads, int iters,
  * that first call before any stream capture.  All calls on a device share
  * the one scratch array, which keeps the last call's contents: calls that
  * overlap on the GPU (different streams, no ordering between them) race.
- * (Where the receptors fit in a CTA's shared memory -- up to 384, or 512 below
- * 512 velocities -- the call takes one pass without the scratch; the limits above
- * are the same.) */
+ * (With at most 512 receptors and 8192 velocities the call takes one pass without
+ * the scratch; the limits above are the same.) */
 #define UGKS_STATIC_SCRATCH_DOUBLES (1 << 19)
 int ugks_idw_interpolate_static(double *f, double *W, double *q, int ncells, int nv,
                                 const int32_t *receptors, int nrec,

@@ -164,7 +164,7 @@ __global__ void k_idw_scatter_static(const double *scratch, double *f, double *W
 // registers: 16.4 us), and weights, their sum and a division of the FP64 pipe
 // are formed once a receptor in shared memory (280 receptors, 576 velocities:
 // 14.4 us a call in two passes, 8.5 in one; with 256 threads 10.2).
-constexpr int ITHREADS = 512;
+constexpr int ITHREADS = 512, ONE_PASS_NV = 8192;
 struct IdwRow { double w[5]; int e[5], target; };      // e: valid donors, else -1
 template <int CH, typename V>
 __global__ void __launch_bounds__(ITHREADS) k_idw_one_pass(double *f, double *W, double *q, int ncells, int nv, int nrec,
@@ -253,9 +253,15 @@ extern "C" int ugks_idw_interpolate_static(double *f, double *W, double *q, int 
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   // One pass where a CTA's shared memory (48 KB) holds every receptor: four pairs
   // (a line of 64 bytes) a CTA, two where four would leave SMs idle.  Else two
-  // passes through the scratch.
+  // passes through the scratch; so too beyond ONE_PASS_NV velocities, which leave
+  // few receptors (the scratch bounds their product) and a CTA with four pairs of
+  // each mostly idle threads, CTA after CTA (one pass / two, us a call back to
+  // back: 4096 velocities, 1 and 63 receptors 6.3 / 10.4 and 10.4 / 18.5; 8192, 1
+  // and 31 receptors 10.3 / 10.3 and 12.4 / 18.4; 16000, 1 and 16 receptors
+  // 14.5 / 10.3 and 16.5 / 18.5, with cold caches 21.1 / 15.0 and 25.2 / 21.2;
+  // 262000, 1 receptor 172 / 18).
   const bool four = nv >= 4 * 128 && one_pass_smem<4>(nrec) <= 48 * 1024;
-  if (four || one_pass_smem<2>(nrec) <= 48 * 1024) {
+  if (nv <= ONE_PASS_NV && (four || one_pass_smem<2>(nrec) <= 48 * 1024)) {
     if (four) one_pass<4>(f, W, q, ncells, nv, nrec, receptors, donors, weights, s);
     else one_pass<2>(f, W, q, ncells, nv, nrec, receptors, donors, weights, s);
     if (cudaPeekAtLastError() != cudaSuccess) {
