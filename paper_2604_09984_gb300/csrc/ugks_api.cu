@@ -1150,7 +1150,8 @@ int ugks_init_mesh(ugks_ctx *ctx, int nblocks, const ugks_block_desc *blocks, co
     ctx->split_tail = !outflow && !d.shard && !(e && atoi(e) != 0);
     long steps = 0;                                  // diagonals of the longest macro sweep
     for (int b = 0; b < nblocks; ++b) steps = std::max(steps, 2L * (blocks[b].ni + blocks[b].nj - 1));
-    ctx->split_residual = residual_split((long)s.nc * s.nv, steps, ctx->fp32);
+    const char *e1 = getenv("UGKS_RESIDUAL_ONE_PASS");   // 1: the residual in one pass
+    ctx->split_residual = residual_split((long)s.nc * s.nv, steps, ctx->fp32) && !(e1 && atoi(e1) != 0);
   }
   {
     std::vector<int> wf;
