@@ -103,6 +103,7 @@ struct Dev {
   double *fsum;              // nf*NFS
   void *fpart;               // nsplit*NFS*nf (sum, error) pairs of the face reduction's CTAs (nsplit > 1)
   int nsplit;                // CTAs that share a tile's velocity chunks in the face kernels
+  int flux_pair;             // FP32 flux pass, joint form: two ranges of columns in turn
   double *fq12;              // nf*2 time integrals q1 / dts, q2 / dts of the faces
   void *fparT;               // nf*NFP in the arithmetic type
   double *fflux;             // nf*4 S * macro flux (L -> R / outward)

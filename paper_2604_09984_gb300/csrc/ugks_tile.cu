@@ -1096,12 +1096,13 @@ void launch_face_reduce(const Dev &d, cudaStream_t s, int fp32) {
   else if (d.fbf) k_face_reduce32<1><<<grid, NT32, sizeof(Smem32), s>>>(d);
   else k_face_reduce32<0><<<grid, NT32, sizeof(Smem32), s>>>(d);
 }
+// Pairs of ranges where a (cell, velocity) array exceeds the L2 (times at k_flux).
+bool flux_pairs(size_t items) { return 8.0 * (double)items > 120e6; }
 template <bool EVAL> static void flux(const Dev &d, cudaStream_t s, int fp32, double *eval) {
   const dim3 grid(d.ntiles, d.nsplit);
-  const bool pair = !EVAL && (double)d.nc * d.nvp * 8.0 > 120e6;         // beyond the L2
   if (!fp32) k_flux<double, true, false, EVAL><<<grid, NT, flux_smem<double>(), s>>>(d, eval);
   else if (d.nvx % 16 == 0) k_flux<float, true, false, EVAL><<<grid, NT, flux_smem<float>(), s>>>(d, eval);
-  else if (pair) k_flux<float, false, true, false><<<grid, NT, flux_smem<float>(), s>>>(d, nullptr);
+  else if (!EVAL && d.flux_pair) k_flux<float, false, true, false><<<grid, NT, flux_smem<float>(), s>>>(d, nullptr);
   else k_flux<float, false, false, EVAL><<<grid, NT, flux_smem<float>(), s>>>(d, eval);
 }
 void launch_flux(const Dev &d, cudaStream_t s, int fp32) { flux<false>(d, s, fp32, nullptr); }
