@@ -1021,7 +1021,7 @@ int ugks_init_mesh(ugks_ctx *ctx, int nblocks, const ugks_block_desc *blocks, co
   d.nsplit = s.nsplit;
   {
     const char *e = getenv("UGKS_FLUX_PAIR");        // 0 / 1: the flux pass's ranges of columns singly / in pairs
-    d.flux_pair = e ? atoi(e) != 0 : flux_pairs((size_t)s.nc * s.nvp);
+    d.flux_pair = e ? atoi(e) != 0 : flux_pairs((size_t)s.nc * s.nvp, s.nvx, s.nsplit);
   }
   d.vbox[0] = ctx->p.vx_min; d.vbox[1] = ctx->p.vx_max; d.vbox[2] = ctx->p.vy_min; d.vbox[3] = ctx->p.vy_max;
   {

@@ -56,7 +56,7 @@ void launch_residual(const Dev &d, cudaStream_t s, int first_iter, int fp32, int
 bool residual_split(long items, long steps, int fp32);
 void launch_face_reduce(const Dev &d, cudaStream_t s, int fp32);
 int face_splits(int ntiles, int nvx, int nv, int fp32);   // CTAs that share a tile's velocities
-bool flux_pairs(size_t items);                            // the flux pass in pairs of ranges; (cell, velocity) items
+bool flux_pairs(size_t items, int nvx, int nsplit);       // the flux pass in pairs of ranges; (cell, velocity) items
 size_t face_values(int ntiles, int nvp);                  // 4-vectors of the stored reconstruction
 void face_tile_shape(int fp32, int *vk, int *nh);         // velocities per chunk, threads per face slot
 }  // namespace ugks

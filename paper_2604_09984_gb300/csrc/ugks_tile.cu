@@ -724,11 +724,10 @@ template <typename T> static constexpr size_t flux_smem() {
 // that gathered the gradients and fluxes of its four faces from the cells:
 // 5.1 ms for 192 x 96 + 96 x 24 cells and 1024 velocities, 6.03 ms the call;
 // from the face values that the reduction leaves, 0.83 ms the call.)
-// PAIR (FP32 joint form, arrays beyond the L2): two ranges of columns in turn, row
-// by row, so that a cell's sums of both are stored close together (300x150 + 2 x
-// 120x30 cells, 33x33 velocities: 728 -> 649 us; within the L2 and in the separable
-// form the longer registers cost more: 128x64 + 64x16, 24x24: 56 -> 61,
-// 256x128 + 128x32, 32x32: 313 -> 431).
+// PAIR (FP32 joint form, by flux_pairs): two ranges of columns in turn, row by row,
+// so that a cell's sums of both are stored close together (300x150 + 2 x 120x30
+// cells, 33x33 velocities: 731 -> 649 us; in the separable form the longer
+// registers cost more: 256x128 + 128x32, 32x32: 313 -> 431).
 template <typename T, bool SEP, bool PAIR, bool EVAL>
 __global__ void __launch_bounds__(NT, FluxCfg<T>::CTAS) k_flux(Dev d, double *eval) {
   typedef typename PairOf<T>::type P;
@@ -1096,8 +1095,19 @@ void launch_face_reduce(const Dev &d, cudaStream_t s, int fp32) {
   else if (d.fbf) k_face_reduce32<1><<<grid, NT32, sizeof(Smem32), s>>>(d);
   else k_face_reduce32<0><<<grid, NT32, sizeof(Smem32), s>>>(d);
 }
-// Pairs of ranges where a (cell, velocity) array exceeds the L2 (times at k_flux).
-bool flux_pairs(size_t items) { return 8.0 * (double)items > 120e6; }
+// Pairs of ranges where neighbouring ranges share the 32-byte sectors of D (rows of
+// a multiple of four columns do not) and a sector written in part leaves the L2
+// before its other part comes: D exceeds it, and one CTA walks all rows of its
+// tile for a range, some 2.8 KB an item and 304 CTAs (126 MB and more from 21 rows
+// on; a few rows less each where CTAs share a tile).  Flux pass, us, single ranges
+// and pairs (MB of D): 256x128 + 128x32 cells, 17 columns 132 / 133 (90), 21: 194 /
+// 189 (132), 22: 177 / 180, 25: 294 / 265, 31: 445 / 361, 33: 565 / 457, 49: 1321 /
+// 995 (713); 300x150 + 2 x 120x30, 33: 731 / 649; multiples of four there, 24: 245
+// / 272, 40: 659 / 714; CTAs that share tiles, 192x96 + 96x24, 31: 205 / 220,
+// 300x150 + 120x30, 33: 579 / 596.
+bool flux_pairs(size_t items, int nvx, int nsplit) {
+  return nvx % 4 != 0 && nsplit == 1 && 8.0 * (double)items > 120e6;
+}
 template <bool EVAL> static void flux(const Dev &d, cudaStream_t s, int fp32, double *eval) {
   const dim3 grid(d.ntiles, d.nsplit);
   if (!fp32) k_flux<double, true, false, EVAL><<<grid, NT, flux_smem<double>(), s>>>(d, eval);
