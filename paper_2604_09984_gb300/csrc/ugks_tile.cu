@@ -1119,10 +1119,14 @@ void launch_flux(const Dev &d, cudaStream_t s, int fp32) { flux<false>(d, s, fp3
 void launch_flux_eval(const Dev &d, cudaStream_t s, double *D, int fp32) { flux<true>(d, s, fp32, D); }
 // Whether the macro sweep (steps: diagonals of its two passes, some 0.25 us each)
 // outlasts the flux pass and the residual's first pass (8.4 + 5.0 ps an item, a
-// cell and velocity).  128x64 + 64x16 cells, 576 velocities (1.4e4 items a
-// diagonal): a step of 10 iterations 5.03 ms in two passes, 5.13 in one;
-// 256x128 + 128x32 cells, 1024 velocities (4.9e4): 20.79 ms and 19.01.
-bool residual_split(long items, long steps, int fp32) { return fp32 && (double)items < 1.9e4 * (double)steps; }
+// cell and velocity).  A step of 10 iterations in two passes and in one, ms, by
+// the items a diagonal: 1.28e4 (128x64 + 64x16 cells, 23x23 velocities) 4.48 /
+// 4.54, 1.39e4 (24x24) 4.42 / 4.49, 1.51e4 (25x25) 4.79 / 4.79, 1.76e4 (27x27)
+// 5.16 / 5.05; 1.45e4 (192x96 + 96x24, 20x20) 7.51 / 7.35, 1.75e4 (22x22) 8.04 /
+// 7.79; 1.40e4 (64x32, 36x36) 2.57 / 2.59, 1.56e4 (38x38) 2.82 / 2.74; 1.46e4
+// (160x80 + 2 x 96x24, 20x20) 6.00 / 6.10; 2.8e4 (256x128 + 128x32, 24x24) 13.57 /
+// 12.96, 4.9e4 (32x32) 18.08 / 16.85: they meet near 1.5e4.
+bool residual_split(long items, long steps, int fp32) { return fp32 && (double)items < 1.5e4 * (double)steps; }
 
 template <typename T, int FB, int PART> static void residual(const Dev &d, cudaStream_t s, int first_iter) {
   const int n = (d.nv + 2 * ResPairs<T>::N - 1) / (2 * ResPairs<T>::N);      // threads a cell
