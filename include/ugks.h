@@ -294,9 +294,9 @@ int ugks_moments(ugks_ctx *ctx, double *W, double *q, int32_t *status,
 int ugks_sizes(const ugks_ctx *ctx, int *ncells, int *nfaces, int *nv,
                int *nv_stride);
 
-/* Read / write the distribution f (ncells x nv x 2, FP64, host or device
- * pointer, velocity index k = iy*nvx + ix) and W, q (FP64).  get synchronises
- * the stream; set overwrites the state (any pointer may be NULL). */
+/* Read / write the distribution f (ncells x nv x 2, FP64, DEVICE pointer,
+ * velocity index k = iy*nvx + ix) and W, q (FP64, host or device).  Both
+ * synchronise the stream; set overwrites the state (any pointer may be NULL). */
 int ugks_get_state(ugks_ctx *ctx, double *f, double *W, double *q);
 int ugks_set_state(ugks_ctx *ctx, const double *f, const double *W, const double *q);
 
@@ -320,8 +320,9 @@ int ugks_set_checkpoint(ugks_ctx *ctx, double t, const double *nodes, const int3
  * current state with the current geometry (after ugks_move_mesh) and write
  * D = sum_faces S F_hat (ncells x nv x 2, outward positive, Eq.
  * microscopicFlux summed per cell) and F = sum_k V_k Psi_k D_k (ncells x 4,
- * Eq. macroscopicFlux) to caller memory (host or device, FP64).  Receptors are
- * interpolated first.  Synchronises the stream. */
+ * Eq. macroscopicFlux) to caller memory (FP64; either may be NULL).  D is a DEVICE
+ * pointer, F host or device.  Receptors are interpolated first.  Synchronises the
+ * stream.  Errors: UGKS_ERR_ORDER, UGKS_ERR_ARG (D in host memory). */
 int ugks_eval_flux(ugks_ctx *ctx, double *D, double *F);
 
 /* Connectivity of the last assembly, HOST buffers: status (ncells int32),

@@ -1,8 +1,8 @@
-// ugks_internal.cuh -- device-side context of libugks and the per-(cell,
-// velocity) building blocks shared by the kernels: limited reconstruction
-// (Sec. 2.1, second-order initial distribution), the time-averaged interface
-// flux of one velocity (Eqs. microscopicFlux, fullSolution; wall condition
-// with Eq. maxWalldes) and its sum over the faces of a cell.
+// ugks_internal.cuh -- device-side context of libugks and what its kernels
+// share: record layouts, loads and stores of f in its storage type, pairs in
+// packed instructions, asynchronous copies, the error-free sums of the velocity
+// reductions, and the polynomials of the interface equilibrium (Eq.
+// fullSolution).
 #pragma once
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -90,7 +90,7 @@ struct Dev {
   // work
   void *Tn, *dfs;            // nc*nvp pairs: level-n term, forward-sweep result
   void *Dbuf;                // nc*nvp pairs: flux divergence of the inner iteration
-  void *fval;                // nf*nvp 4-vectors: upwind face value (h, b) and w.grad f (h, b) of the face pass
+  void *fval;                // ntiles*nvp*NSLOT 4-vectors: upwind face value (h, b) and w.grad f (h, b) of the face pass
   const double *stepc;       // [4]: dt, 1/dt, (float)(1/dt) as a float, of the pending step, on the device (the step's
                              // kernels read it there, so a captured step graph stays valid when dt changes)
   double *TW;                // nc*4 extensive level-n macro term
@@ -160,8 +160,7 @@ struct Dev {
 enum { MET_R2 = 0, MET_RMICRO2 = 1, MET_FIX2 = 2, MET_TOT = 3, MET_NQ = 7 };
 constexpr int MET_BLOCKS = 304, MET_THREADS = 256;
 
-// Polls of a bounded wait before it gives up; the drain of a CTA's own copies
-// after a timeout always uses the default.
+// Polls of a bounded wait before it gives up.
 constexpr int kWaitPolls = 1 << 21;
 
 // face geometry record / per-cell sweep record
@@ -348,58 +347,8 @@ template <int N> __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;\n" ::"n"(N));
 }
 
-// mbarrier and bulk (TMA engine) copies, shared::cta addresses
+// shared::cta address
 __device__ __forceinline__ unsigned smem_addr(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void mbar_init(unsigned long long *mb, unsigned count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(smem_addr(mb)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_fence_init() {
-  asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-}
-__device__ __forceinline__ void mbar_arrive_expect_tx(unsigned long long *mb, unsigned bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(smem_addr(mb)), "r"(bytes)
-               : "memory");
-}
-// raise the expected transaction bytes of the current phase (no arrival)
-__device__ __forceinline__ void mbar_expect_tx(unsigned long long *mb, unsigned bytes) {
-  asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;\n" ::"r"(smem_addr(mb)), "r"(bytes)
-               : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(unsigned long long *mb) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(smem_addr(mb)) : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(unsigned long long *mb, unsigned parity) {
-  unsigned ok;
-  asm volatile(
-      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-      : "=r"(ok)
-      : "r"(smem_addr(mb)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-// Wait for a phase of an mbarrier with at most `polls` polls; false (and
-// EF_TIMEOUT in *err) when the limit runs out.
-__device__ __forceinline__ bool mbar_wait(unsigned long long *mb, unsigned parity, int *err, int polls = kWaitPolls) {
-  for (int n = 0; n < polls; ++n)
-    if (mbar_try_wait(mb, parity)) return true;
-  atomicOr(err, EF_TIMEOUT);
-  return false;
-}
-// global -> shared bulk copy completing on an mbarrier (16-byte aligned
-// addresses, size a multiple of 16)
-__device__ __forceinline__ void bulk_g2s(void *dst, const void *src, unsigned bytes, unsigned long long *mb) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(
-          smem_addr(dst)),
-      "l"(src), "r"(bytes), "r"(smem_addr(mb))
-      : "memory");
-}
-__device__ __forceinline__ void fence_proxy_async_shared() {
-  asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-}
-__device__ __forceinline__ void fence_proxy_async_global() {
-  asm volatile("fence.proxy.async.global;\n" ::: "memory");
-}
 
 template <typename T> __device__ __forceinline__ T dvx(const Dev &d, int k);
 template <> __device__ __forceinline__ double dvx<double>(const Dev &d, int k) { return d.vx[k]; }
@@ -484,13 +433,6 @@ __device__ __forceinline__ R p2_sum(const Poly2<D, R> &x, const R *Mx, const R *
 #pragma unroll
     for (int b = 0; b <= t; ++b) s += x.c[Poly2<D, R>::idx(t - b, b)] * (Mx[t - b] * My[b]);
   return s;
-}
-// value at (x, y) of a cubic in the layout above (Horner, 9 fused multiply-adds)
-template <typename R> __device__ __forceinline__ R poly3_at(const R *c, R x, R y) {
-  R yy = c[0] + y * (c[2] + y * (c[5] + y * c[9]));
-  R u = c[1] + y * (c[4] + y * c[8]);
-  R w = c[3] + y * c[7] + x * c[6];
-  return yy + x * (u + x * w);
 }
 
 // Equilibrium factors of the time-integrated interface distribution (Eq.

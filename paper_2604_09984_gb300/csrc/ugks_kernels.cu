@@ -99,11 +99,6 @@ __device__ __forceinline__ double warp_sum(double v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
   return v;
 }
-__device__ __forceinline__ double warp_max(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_down_sync(0xffffffffu, v, o));
-  return v;
-}
 
 // Lane-local sum in the arithmetic type: plain for FP64, Neumaier-compensated
 // for FP32 (the mixed path keeps velocity sums accurate to a few FP32 ulps

@@ -6,7 +6,7 @@
 namespace ugks {
 int launch_upload(void *dst, const void *src, size_t n, cudaStream_t s);   // kernels launched
 void launch_move_nodes(const Dev &d, cudaStream_t s);
-void launch_geometry(const Dev &d, cudaStream_t s, int fp32);   // 4 kernels
+void launch_geometry(const Dev &d, cudaStream_t s, int fp32);   // 2 kernels
 void launch_slope_geo(const Dev &d, cudaStream_t s);
 void launch_ghost_gradW(const Dev &d, cudaStream_t s);                      // 2 kernels
 void launch_gradW(const Dev &d, cudaStream_t s);                            // the gradients alone
@@ -40,7 +40,7 @@ void launch_wall_loads(const Dev &d, cudaStream_t s);
 void launch_wall_torque(const Dev &d, cudaStream_t s, const double *ctr, double *out);
 void launch_f_convert(const Dev &d, cudaStream_t s, double *out, const double *in, int fp32);
 void launch_connect(const Dev &d, cudaStream_t s, int *prev_status, const int *blk_order,
-                    int *n_orphan);                           // 9 kernels
+                    int *n_orphan);                           // 10 kernels
 void launch_lists(const Dev &d, cudaStream_t s, const int *fresh_flag, const int *n_orphan);  // 2 kernels
 // parts: 1 the distributions, 2 W and q, 3 both
 void launch_interp(const Dev &d, cudaStream_t s, const int *list, const int *cnt, int nsm, int fp32,

@@ -315,19 +315,6 @@ UG_HD V2<R> shakhov_rec(const R *c, R vx, R vy, R Keff, R Kint) {
   return shakhov_exp<R>(c, vx, vy, c[SH_HPRE] * r_exp<R>(-c[SH_LAM] * (cx * cx + cy * cy)), Keff, Kint);
 }
 
-// Shakhov equilibrium f+ = g + g+ of a cell (Sec. 2.1), one velocity.
-template <typename R>
-UG_HD V2<R> shakhov(R rho, R ux, R uy, R lam, R qx, R qy, R vx, R vy, R Keff, R Kint, R Pr) {
-  R cx = vx - ux, cy = vy - uy;
-  R c2 = cx * cx + cy * cy;
-  R H = rho * (lam * R(M_1_PI)) * r_exp<R>(-lam * c2);
-  R il = R(1) / (R(2) * lam);
-  R pref = R(4) * (R(1) - Pr) * lam * lam / (R(5) * rho) * (cx * qx + cy * qy);
-  R Hp = pref * (R(2) * lam * c2 - R(4)) * H;
-  R Bp = pref * ((R(2) * lam * c2 - R(2)) * Keff - R(2) * Kint) * H * il;
-  return {H + Hp, Keff * il * H + Bp};
-}
-
 // van Leer limited slope of two centre differences
 template <typename R> UG_HD R vanleer(R a, R b) {
   R p = a * b;

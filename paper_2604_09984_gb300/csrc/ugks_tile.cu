@@ -86,10 +86,6 @@ __device__ __forceinline__ int g_of_region(int r) {
   return (ry - 1) * GW + (r - ry * RW) - 1;
 }
 
-template <typename T> struct Vec4;
-template <> struct Vec4<float> { typedef float4 type; };
-template <> struct Vec4<double> { typedef double4 type; };
-
 // a b + c d with one product rounded by itself (written out where results must
 // not depend on the compiler's choice)
 __device__ __forceinline__ float mul_add2(float a, float b, float c, float d) { return __fmaf_rn(a, b, __fmul_rn(c, d)); }
@@ -345,7 +341,7 @@ template <int FB> __global__ void __launch_bounds__(NT32, 2) k_face_reduce32(Dev
             dst[q] = pr_make(v.x, v.y);
           }
         } else {
-          // k < nv <= nvp, nvp a multiple of 4 and k even: the pair stays in
+          // k < nv <= nvp, nvp a multiple of 16 and k even: the pair stays in
           // the cell's row (padding velocities hold zero)
           cp_async<16>(dst, reinterpret_cast<const PairF *>(d.f) + (size_t)g * d.nvp + k);
         }
@@ -984,7 +980,7 @@ template <typename T, int FB, int PART> __global__ void __launch_bounds__(RES_NT
   constexpr bool SEP = sizeof(T) == 8;
   __shared__ ResTable<T> tp, tn0;
   // grid: cells x velocity chunks; a thread takes pairs of adjacent velocities
-  // (nvp is a multiple of 4, so a pair stays inside the cell's row)
+  // (nvp is a multiple of 16, so a pair stays inside the cell's row)
   constexpr int NP = ResPairs<T>::N;
   const int c = blockIdx.x, kc = 2 * NP * blockIdx.y * blockDim.x;
   if (!(d.cmask[c] & 1)) return;
@@ -1046,7 +1042,8 @@ template <typename T, int FB, int PART> __global__ void __launch_bounds__(RES_NT
   }
 }
 
-// CTAs that share a tile's velocity chunks: the share that ends a pass soonest
+// CTAs that share a tile's velocity chunks (by the sizes alone: the workspace is
+// laid out by them, without a device): the share that ends a pass soonest
 // on 152 SMs with two resident CTAs each (FP64: one), with ~4 us of set-up and
 // finish a CTA against ~7 us a pair of chunks (FP32, the fold's unit) or ~22 us
 // a chunk (FP64).  8 tiles at 16 x 16 velocities (32 x 16 cells): 8 CTAs a tile,
